@@ -58,22 +58,22 @@ struct LevelDev {
   int *mat_off = nullptr, *dmat_off = nullptr;
   double *Mloc = nullptr, *Dloc = nullptr, *w = nullptr;
   int *f_y0 = nullptr, *f_y1 = nullptr;            // per flux unknown: its slots in the per-cell buffer (-1)
-  int* own0 = nullptr;                             // per local slot: 1 if this cell is the first owner
+  int* loc_own = nullptr;                          // per local slot: loc where this cell is the first owner, else -1
   int* sad_off = nullptr;                          // per cell: offset of (nl+m)^2 inverse local saddle
   double* Sinv = nullptr;
-  int *if_off = nullptr, *if_slot = nullptr, *if_lam = nullptr;   // per cell: interface slots, their lambda
-  double* if_sign = nullptr;
+  int *if_off = nullptr, *if_slot = nullptr;       // per cell: interface slots
+  int* if_lams = nullptr;                          // ... their lambda, complemented (~) where the slot's sign is -1
   int* hc_off = nullptr;                           // per cell: nif x nif block of C S_ss C^T (kappa = 1)
   double* Hc = nullptr;
   int *lam_y0 = nullptr, *lam_y1 = nullptr;        // per lambda: its two entries in the per-interface buffer
   int* if_cell = nullptr;                          // per interface slot: its cell
   int* slot_cell = nullptr;                        // per local flux slot: its cell
   int* p_cell = nullptr;                           // per pressure unknown: its cell
-  // H over the lambdas as a SELL-32 matrix (for the memory-resident pipelined CG of large levels): per slice of 32
+  // H over the lambdas as a SELL-32 matrix (the hybridized CG's product): per slice of 32
   // lambdas its width and first entry; per entry (slice-major, lane fastest) the column lambda and the Hc indices of
   // its contributions from the row lambda's first and second slot (-1: none); per lambda the cells of its two slots.
   // Entry (l, m) = kappa_c0 Hc[i0] + kappa_c1 Hc[i1].
-  int hs_n = 0;
+  int hs_n = 0, hs_wmax = 0;   // entries with padding, longest row
   int *hs_w = nullptr, *hs_off = nullptr, *hs_col = nullptr, *hs_i0 = nullptr, *hs_i1 = nullptr;
   int *lam_c0 = nullptr, *lam_c1 = nullptr;
 };

@@ -102,13 +102,14 @@ struct CoarseStepResult {
 
 // One launch: [Algorithm 1 along a given correction], up to nsteps coarse Picard steps (frozen-kappa hybridized
 // solve, clamp on Pi~ dp, Algorithm 1), leaving the residual r = A(x) - b (and -r, kappa per cell) at the final x;
-// every decision is taken on the device. The hybridized CG runs on the assembled SELL form of H (B.hsv, L.hs_*) when
-// its pipelined form is memory resident on this grid; *sell (may be null) tells whether it did.
-template <class T>
-cudaError_t launch_coarse_step(cudaStream_t st, const LevelDev& L, const T* Hc, const T* Sinv,
-                               const CoarseStepBufs<T>& B, const CoarseStepParams& P, double* partial, GridSync gs,
+// every decision is taken on the device. *sell (may be null) tells whether the hybridized CG read the assembled SELL
+// form of H (B.hsv) in every iteration rather than a copy in shared memory.
+cudaError_t launch_coarse_step(cudaStream_t st, const LevelDev& L, const double* Hc, const double* Sinv,
+                               const CoarseStepBufs<double>& B, const CoarseStepParams& P, double* partial, GridSync gs,
                                CoarseStepResult* res, bool* sell = nullptr);
 
+// SMs a persistent kernel may use: all, or the launch's cap.
+int coop_sms(int sm_cap);
 
 // Failure-detection check: a cooperative launch of min(blocks, co-resident) blocks in which every block but `absent`
 // (absent < 0: none) waits at one bounded grid barrier (spin_limit polls); *passed (zeroed by the caller) counts the

@@ -342,7 +342,9 @@ void upload_level(nlmg_ctx* c, int l) {
     }
   D.f_y0 = c->upload(fy0);
   D.f_y1 = c->upload(fy1);
-  D.own0 = c->upload(own0);
+  std::vector<int> loc_own(L.loc.size());
+  for (size_t k = 0; k < loc_own.size(); ++k) loc_own[k] = own0[k] ? L.loc[k] : -1;
+  D.loc_own = c->upload(loc_own);
   // hybridization data
   std::vector<int> lam_of(L.n_flux, -1);
   int nlam = 0;
@@ -390,8 +392,9 @@ void upload_level(nlmg_ctx* c, int l) {
   D.Sinv = c->upload(Sinv);
   D.if_off = c->upload(if_off);
   D.if_slot = c->upload(if_slot);
-  D.if_lam = c->upload(if_lam);
-  D.if_sign = c->upload(if_sign);
+  std::vector<int> if_lams(if_lam.size());
+  for (size_t k = 0; k < if_lams.size(); ++k) if_lams[k] = if_sign[k] < 0.0 ? ~if_lam[k] : if_lam[k];
+  D.if_lams = c->upload(if_lams);
   D.hc_off = c->upload(hc_off);
   D.Hc = c->upload(Hc);
   D.lam_y0 = c->upload(ly0);
@@ -461,6 +464,7 @@ void upload_level(nlmg_ctx* c, int l) {
         }
       }
     D.hs_n = E;
+    D.hs_wmax = nsl ? *std::max_element(hw.begin(), hw.end()) : 0;
     D.hs_w = c->upload(hw);
     D.hs_off = c->upload(hoff);
     D.hs_col = c->upload(hcol);
@@ -1048,7 +1052,7 @@ void coarse_step(nlmg_ctx* c, int l, bool backtrack_first, int nsteps, bool coar
                             pipe ? HybPipeBufs<double>{B.hw, B.hz, B.hs, B.hma, B.hmb} : HybPipeBufs<double>{},
                             B.hsv};
   bool sell = false;
-  CK(launch_coarse_step<double>(c->st, L, L.Hc, L.Sinv, Bd, P, c->d_partial, gs, dres, &sell));
+  CK(launch_coarse_step(c->st, L, L.Hc, L.Sinv, Bd, P, c->d_partial, gs, dres, &sell));
   c->prof_end(pi);
   count_launch(1);
   CK(cudaMemcpyAsync(c->h_res, c->d_res, sizeof(PcgResult) + sizeof(CoarseStepResult), cudaMemcpyDeviceToHost,
