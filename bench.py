@@ -37,17 +37,15 @@ CPU_SAMPLE_SCALE = 24      # side of the cpu_baseline sample
 
 
 # DRAM bytes (read + write) per launch on the 64^3 workload with the default options, from ncu captures of the
-# kernels as they are now (averaged over the launches of one solve where they differ): valid for that kernel, that
-# workload and those options only, else the traffic is reported as null.
-DRAM_BYTES_64 = {0: 23.102e6,     # kp_fine_cg_reg<double, 4>, mean of the 8 launches of a solve
-                 1: 25.362e6,     # kp_coarse_step<double>, mean of the 15 launches (10 on level 1, 5 coarsest solves)
-                 3: 25.216e6}     # kp_fine_bicgstab, mean of the 3 launches
+# kernels as they are now: valid for that kernel, that workload and those options only, else the traffic is reported
+# as null (the register-resident kernels have no capture).
+DRAM_BYTES_64 = {}
 
-KERNELS = {0: ("kp_fine_cg_reg<double, 4> (persistent register-resident pipelined Jacobi-scaled CG of the level-0 "
+KERNELS = {0: ("kp_fine_cg_reg<double> (persistent register-resident pipelined Jacobi-scaled CG of the level-0 "
                "Picard step)", "kp_fine_cg* (level-0 Picard CG)"),
            1: ("kp_coarse_step<double> (fused coarse Picard step: coarse operator evaluations, pipelined hybridized "
                "CG, clamp and Algorithm 1 in one persistent launch)",) * 2,
-           3: ("kp_fine_bicgstab (persistent FP64 BiCGStab of the level-0 Newton step)",) * 2,
+           3: ("kp_fine_bicgstab* (persistent FP64 BiCGStab of the level-0 Newton step)",) * 2,
            5: ("level-0 CG preconditioned by the multigrid V-cycle (per-step Galerkin setup, then one CUDA graph "
                "with a device-side while loop: FP64 CG vectors, FP32 V-cycle kernels)",) * 2,
            6: ("level-0 BiCGStab of the Newton step preconditioned by the multigrid V-cycle (setup and CUDA "

@@ -283,24 +283,28 @@ __global__ void k_gmres_combine(int n, int nk, const double* __restrict__ V, con
   }
 }
 
-// Jacobi scaling of the Newton system, with the same safeguard as the Jacobi smoother: 1 / max(J_KK, d_K / 2)
+// Jacobi scaling of the Newton system, with the same safeguard as the Jacobi smoother: D = 1 / max(J_KK, d_K / 2) and
+// S = D^1/2
 __global__ void k_jacobi_dinv(int n, const double* __restrict__ jdiag, const double* __restrict__ diagT,
-                              double* __restrict__ out) {
-  GRID_STRIDE(i, n) out[i] = 1.0 / fmax(jdiag[i], 0.5 * diagT[i]);
+                              double* __restrict__ D, double* __restrict__ S) {
+  GRID_STRIDE(i, n) {
+    const double d = 1.0 / fmax(jdiag[i], 0.5 * diagT[i]);
+    D[i] = d;
+    S[i] = sqrt(d);
+  }
 }
 
-// Scaled Newton system of the level-0 BiCGStab: with D = jdinv = 1 / max(J_KK, d_K / 2) and S = D^1/2,
-// sS = S, jd = J_KK D_K on the diagonal and Js = S_K J_KL S_L off it (SELL layout; padding entries stay 0).
+// Scaled Newton system of the level-0 BiCGStab: jd = J_KK D_K on the diagonal and Js = S_K J_KL S_L off it (SELL layout;
+// padding entries stay 0).
 __global__ void k_scale_jac(FineDev F, const double* __restrict__ jdiag, const double* __restrict__ Joff,
-                            const double* __restrict__ jdinv, double* __restrict__ Js, double* __restrict__ jd,
-                            double* __restrict__ sS) {
+                            const double* __restrict__ D, const double* __restrict__ S, double* __restrict__ Js,
+                            double* __restrict__ jd) {
   GRID_STRIDE(K, F.N) {
-    const double sK = sqrt(jdinv[K]);
-    sS[K] = sK;
-    jd[K] = jdiag[K] * jdinv[K];
+    const double sK = S[K];
+    jd[K] = jdiag[K] * D[K];
     const int w = F.sell_w[K >> 5];
     int e = F.sell_off[K >> 5] + (K & 31);
-    for (int j = 0; j < w; ++j, e += 32) Js[e] = Joff[e] * sK * sqrt(jdinv[F.nbr[e]]);
+    for (int j = 0; j < w; ++j, e += 32) Js[e] = Joff[e] * sK * S[F.nbr[e]];
   }
 }
 
@@ -563,14 +567,14 @@ void launch_gmres_combine(cudaStream_t st, int n, int nk, const double* V, const
   COUNT(1);
   k_gmres_combine<<<grid_for(n), kThreads, 0, st>>>(n, nk, V, y, dinv, x);
 }
-void launch_jacobi_dinv(cudaStream_t st, int n, const double* jdiag, const double* diagT, double* out) {
+void launch_jacobi_dinv(cudaStream_t st, int n, const double* jdiag, const double* diagT, double* D, double* S) {
   COUNT(1);
-  k_jacobi_dinv<<<grid_for(n), kThreads, 0, st>>>(n, jdiag, diagT, out);
+  k_jacobi_dinv<<<grid_for(n), kThreads, 0, st>>>(n, jdiag, diagT, D, S);
 }
-void launch_scale_jac(cudaStream_t st, const FineDev& F, const double* jdiag, const double* Joff,
-                      const double* jdinv, double* Js, double* jd, double* sS) {
+void launch_scale_jac(cudaStream_t st, const FineDev& F, const double* jdiag, const double* Joff, const double* D,
+                      const double* S, double* Js, double* jd) {
   COUNT(1);
-  k_scale_jac<<<grid_for(F.N), kThreads, 0, st>>>(F, jdiag, Joff, jdinv, Js, jd, sS);
+  k_scale_jac<<<grid_for(F.N), kThreads, 0, st>>>(F, jdiag, Joff, D, S, Js, jd);
 }
 bool measure_fp64_peak(double* gflops) {
   int dev = 0, sms = 0;

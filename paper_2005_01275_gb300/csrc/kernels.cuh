@@ -23,7 +23,7 @@ struct Reduce {
 // ---------------------------------------------------------------------------------------------------------------
 // Fine level (reduced TPFA, Sec. 2.1)
 struct FineDev {
-  int N = 0, nnz = 0, nflux = 0, nslice = 0;
+  int N = 0, nnz = 0, nflux = 0, nslice = 0, wmax = 0;   // wmax: widest slice
   // interior neighbours per cell in SELL-32 layout: slice s = cells 32 s .. 32 s + 31, width sell_w[s]; entry j of
   // cell K sits at sell_off[s] + 32 j + (K & 31). Padding entries point to the cell itself with Ups = (1, 0).
   int *sell_off = nullptr, *sell_w = nullptr, *nbr = nullptr;
@@ -117,9 +117,9 @@ void launch_mdot(cudaStream_t st, int n, int nk, const double* V, const double* 
                  unsigned* counter, double* h);
 void launch_orth_update(cudaStream_t st, int n, int nk, const double* V, const double* h, double* w, Reduce red);
 void launch_scale_vec(cudaStream_t st, int n, const double* x, double s, double* y);
-void launch_jacobi_dinv(cudaStream_t st, int n, const double* jdiag, const double* diagT, double* out);
-void launch_scale_jac(cudaStream_t st, const FineDev& F, const double* jdiag, const double* Joff,
-                      const double* jdinv, double* Js, double* jd, double* sS);
+void launch_jacobi_dinv(cudaStream_t st, int n, const double* jdiag, const double* diagT, double* D, double* S);
+void launch_scale_jac(cudaStream_t st, const FineDev& F, const double* jdiag, const double* Joff, const double* D,
+                      const double* S, double* Js, double* jd);
 void launch_gmres_combine(cudaStream_t st, int n, int nk, const double* V, const double* y, const double* dinv,
                           double* x);
 void launch_jacobi_update(cudaStream_t st, int n, const double* q, const double* R, const double* jdiag,

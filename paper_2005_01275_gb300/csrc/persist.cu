@@ -1,17 +1,17 @@
-// Persistent (cooperative) kernels: one launch runs a whole level-0 linear solve (the Picard step's CG, the Newton
-// step's BiCGStab) or whole coarse Picard steps (hybridized CG, clamp, Algorithm 1), with device-side scalars,
-// decisions and convergence tests, so the iterations pay neither launch gaps nor host round trips.
+// Persistent (cooperative) kernels with their state in memory: one launch runs a whole level-0 linear solve (the Picard
+// step's CG, the Newton step's BiCGStab) with device-side scalars, decisions and convergence tests, so the iterations pay
+// neither launch gaps nor host round trips. Meshes whose cells fit the registers of the grid run fine_reg.cu instead.
 //
-// Grid-wide synchronisation uses a counter barrier whose wait is bounded: after ~2 s of spinning the
-// kernel records an error flag and every block leaves. The launch goes through cudaLaunchCooperativeKernel with at
-// most the co-resident number of blocks, so in a correct run every wait ends.
+// Grid-wide synchronisation uses a counter barrier whose wait is bounded: after ~2 s of polling the kernel records an
+// error flag and every block leaves. The launch goes through cudaLaunchCooperativeKernel with at most the co-resident
+// number of blocks, so in a correct run every wait ends.
 //
 // Data written by one block and read by another inside the same launch (CG vectors, per-interface buffers) is read
 // with ld.global.cg (L2, bypassing the non-coherent L1), after the barrier that orders the write.
 //
 // Reductions stay deterministic: each block writes one partial per value; after the barrier every block adds all
-// partials in block order with the same fixed tree and derives the step lengths once (one thread per block), so all
-// blocks take the same decisions from bit-identical scalars and a run is bitwise reproducible for a given grid.
+// partials (exactly, hence in no particular order) and derives the step lengths once, so all blocks take the same
+// decisions from bit-identical scalars and a run is bitwise reproducible for a given grid.
 #include <cmath>
 
 #include "kernels.cuh"
@@ -23,6 +23,9 @@ namespace nlmg {
 namespace {
 
 constexpr int kPThreads = 512;                           // threads per block of the persistent kernels
+
+// Cells over the grid, a block's threads side by side (these meshes fill every SM many times over).
+#define CSTRIDE(i, n) for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < (n); i += gridDim.x * blockDim.x)
 
 // ---- fine level: A dx = bscale * b with the frozen TPFA matrix --------------------------------------------------
 // CG on the symmetrically Jacobi-scaled system (S A S) y = S bscale b, dx = S y, S = diag(A)^-1/2, so the scaled
@@ -43,7 +46,7 @@ __global__ void __launch_bounds__(kPThreads) kp_fine_cg(FineDev F, const T* __re
   __shared__ double sm[kSmDoubles];
   Grid g{gs, partial, sm, 0u};
   T t1 = (T)0;   // per-thread partial sums in T (a thread holds one or two cells), block and grid sums in FP64
-  GSTRIDE(i, F.N) {
+  CSTRIDE(i, F.N) {
     const T ri = (T)(sdiag[i] * bscale * b[i]);
     y[i] = (T)0;
     r[i] = ri;
@@ -58,7 +61,7 @@ __global__ void __launch_bounds__(kPThreads) kp_fine_cg(FineDev F, const T* __re
   int it = 0;
   while (rr0 > 0.0 && rr > tol2 && it < maxit) {
     T tpq = (T)0;
-    GSTRIDE(K, F.N) {
+    CSTRIDE(K, F.N) {
       const int s = K >> 5, lane = K & 31;
       const T rK = __ldcg(&r[K]);
       T acc = rK;
@@ -92,7 +95,7 @@ __global__ void __launch_bounds__(kPThreads) kp_fine_cg(FineDev F, const T* __re
     const double alpha_d = pq[1];
     const T alpha = (T)alpha_d;
     T trn = (T)0;
-    GSTRIDE(i, F.N) {
+    CSTRIDE(i, F.N) {
       y[i] = alpha * p[i] + y[i];
       const T ri = r[i] - alpha * q[i];
       r[i] = ri;
@@ -106,7 +109,7 @@ __global__ void __launch_bounds__(kPThreads) kp_fine_cg(FineDev F, const T* __re
     ++it;
     if (!(alpha_d != 0.0)) break;   // breakdown (p.Ap = 0): stop with the current iterate
   }
-  GSTRIDE(i, F.N) dx[i] = sdiag[i] * (double)y[i];
+  CSTRIDE(i, F.N) dx[i] = sdiag[i] * (double)y[i];
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     res->iters = it;
     res->rr0 = rr0;
@@ -145,7 +148,7 @@ __device__ __forceinline__ T sell_apply(const FineDev& F, const T* __restrict__ 
 }
 
 template <class T>
-__global__ void __launch_bounds__(kPThreads) kp_fine_cg_pipe(FineDev F, const T* __restrict__ Ts,
+__global__ void __launch_bounds__(kPThreads, 2) kp_fine_cg_pipe(FineDev F, const T* __restrict__ Ts,
                                                              const double* __restrict__ sdiag,
                                                              const double* __restrict__ b, double bscale,
                                                              double* __restrict__ dx, T* __restrict__ y,
@@ -154,7 +157,7 @@ __global__ void __launch_bounds__(kPThreads) kp_fine_cg_pipe(FineDev F, const T*
                                                              GridSync gs, double tol, int maxit, PcgResult* res) {
   __shared__ double sm[kSmDoubles];
   Grid g{gs, partial, sm, 0u};
-  GSTRIDE(i, F.N) {
+  CSTRIDE(i, F.N) {
     r[i] = (T)(sdiag[i] * bscale * b[i]);
     y[i] = z[i] = sv[i] = p[i] = (T)0;
   }
@@ -162,7 +165,7 @@ __global__ void __launch_bounds__(kPThreads) kp_fine_cg_pipe(FineDev F, const T*
   // a4 = {gamma, delta, beta, alpha}: the sums and, from the last block's thread 0, the step lengths of the next
   // iteration (beta = gamma / gamma_old, alpha = gamma / (delta - beta gamma / alpha_old); first: 0, gamma / delta)
   double a4[4] = {0.0, 0.0, 0.0, 0.0};
-  GSTRIDE(K, F.N) {
+  CSTRIDE(K, F.N) {
     const T wK = sell_apply<T>(F, Ts, r, K);
     wa[K] = wK;
     const double rK = (double)r[K];
@@ -184,7 +187,7 @@ __global__ void __launch_bounds__(kPThreads) kp_fine_cg_pipe(FineDev F, const T*
     if (!(alpha_d != 0.0)) break;
     const T alpha = (T)alpha_d, beta = (T)beta_d;
     double n4[4] = {0.0, 0.0, 0.0, 0.0};
-    GSTRIDE(K, F.N) {
+    CSTRIDE(K, F.N) {
       const T nK = sell_apply<T>(F, Ts, wc, K);
       const T wK = wc[K];
       const T zK = nK + beta * z[K];
@@ -217,241 +220,7 @@ __global__ void __launch_bounds__(kPThreads) kp_fine_cg_pipe(FineDev F, const T*
     wn = t;
     ++it;
   }
-  GSTRIDE(i, F.N) dx[i] = sdiag[i] * (double)y[i];
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    res->iters = it;
-    res->rr0 = rr0;
-    res->rr = gamma;
-  }
-}
-
-// Register-resident pipelined CG. A persistent thread owns the same cells (at most R of them: K = k0 + u * stride)
-// for the whole solve, so y, r, p, s, z and w of its cells stay in FP64 registers; only w, which the neighbours
-// gather, is written to memory (double-buffered, type TM) each iteration. Per iteration: n = A w from the published
-// w, the recurrences of the pipelined CG above, the two dot products, one grid barrier. TM = double gives the FP64
-// path (bitwise the memory-resident kernel on the same grid). (TM = float, an FP32 matrix product inside FP64
-// recurrences, was measured to drift like the all-FP32 pipelined form and is not used.)
-template <class TM, int R>
-__global__ void __launch_bounds__(kPThreads) kp_fine_cg_reg(FineDev F, const TM* __restrict__ Ts,
-                                                            const double* __restrict__ sdiag,
-                                                            const double* __restrict__ b, double bscale,
-                                                            double* __restrict__ dx, TM* wa, TM* wb,
-                                                            double* partial, GridSync gs, double tol, int maxit,
-                                                            PcgResult* res) {
-  __shared__ double sm[kSmDoubles];
-  Grid g{gs, partial, sm, 0u};
-  const int stride = gridDim.x * blockDim.x;
-  const int k0 = blockIdx.x * blockDim.x + threadIdx.x;
-  double y[R], r[R], p[R], sv[R], z[R], w[R];
-#pragma unroll
-  for (int u = 0; u < R; ++u) {
-    const int K = k0 + u * stride;
-    y[u] = p[u] = sv[u] = z[u] = w[u] = 0.0;
-    r[u] = 0.0;
-    if (K < F.N) {
-      r[u] = sdiag[K] * bscale * b[K];
-      wa[K] = (TM)r[u];   // the first product is A r
-    }
-  }
-  if (!grid_barrier(g)) return;
-  double a4[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-  for (int u = 0; u < R; ++u) {
-    const int K = k0 + u * stride;
-    if (K < F.N) {
-      w[u] = (double)sell_apply<TM>(F, Ts, wa, K);
-      wb[K] = (TM)w[u];
-      a4[0] = fma(r[u], r[u], a4[0]);
-      a4[1] = fma(w[u], r[u], a4[1]);
-    }
-  }
-  if (!grid_sum_x<2, 2>(g, a4, [&](double* o) {
-        o[2] = 0.0;
-        o[3] = o[1] != 0.0 ? fast_div(o[0], o[1]) : 0.0;
-      }))
-    return;
-  double gamma = a4[0], beta = a4[2], alpha = a4[3];
-  const double rr0 = gamma;
-  const double tol2 = tol * tol * rr0;
-  TM* wc = wb;   // published w of the current iteration
-  TM* wn = wa;   // next w
-  int it = 0;
-  while (rr0 > 0.0 && gamma > tol2 && it < maxit) {
-    if (!(alpha != 0.0)) break;
-    double n4[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-    for (int u = 0; u < R; ++u) {
-      const int K = k0 + u * stride;
-      if (K < F.N) {
-        const double nK = (double)sell_apply<TM>(F, Ts, wc, K);
-        z[u] = nK + beta * z[u];
-        sv[u] = w[u] + beta * sv[u];
-        p[u] = r[u] + beta * p[u];
-        y[u] += alpha * p[u];
-        r[u] = r[u] - alpha * sv[u];
-        w[u] = w[u] - alpha * z[u];
-        wn[K] = (TM)w[u];
-        n4[0] = fma(r[u], r[u], n4[0]);
-        n4[1] = fma(w[u], r[u], n4[1]);
-      }
-    }
-    if (!grid_sum_x<2, 2>(g, n4, [&](double* o) {
-          const double g = o[0], d = o[1];
-          const double bn = gamma != 0.0 ? fast_div(g, gamma) : 0.0;
-          const double den = d - fast_div(bn * g, alpha);
-          o[2] = bn;
-          o[3] = den != 0.0 ? fast_div(g, den) : 0.0;
-        }))
-      return;
-    gamma = n4[0];
-    beta = n4[2];
-    alpha = n4[3];
-    TM* t = wc;
-    wc = wn;
-    wn = t;
-    ++it;
-  }
-#pragma unroll
-  for (int u = 0; u < R; ++u) {
-    const int K = k0 + u * stride;
-    if (K < F.N) dx[K] = sdiag[K] * y[u];
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    res->iters = it;
-    res->rr0 = rr0;
-    res->rr = gamma;
-  }
-}
-
-// FP32 pipelined CG with residual replacement. The recurrences of the pipelined CG (kp_fine_cg_reg) run in FP32
-// here, vectors and scaled matrix alike, a thread's cells in registers; in FP32 they drift away from the true
-// residual on the six-decade channelized field (the iteration count grew fivefold), so every `replace` iterations
-// the residual and the auxiliary vectors are recomputed from their definitions -- r = b - A y, s = A p, then
-// w = A r and z = A s (residual replacement, Cools and Vanroose) -- which costs four matrix products and two extra
-// synchronisations and keeps the iteration on the track of the FP64 one. Per-thread partial sums in FP32, block and
-// grid sums in FP64; the stopping test and the step lengths are those of kp_fine_cg_reg.
-template <int R>
-__global__ void __launch_bounds__(kPThreads) kp_fine_cg_rr32(FineDev F, const float* __restrict__ Ts,
-                                                             const double* __restrict__ sdiag,
-                                                             const double* __restrict__ b, double bscale,
-                                                             double* __restrict__ dx, float* wa, float* wb,
-                                                             float* ypub, float* ppub, float* rpub, float* spub,
-                                                             double* partial, GridSync gs, double tol, int maxit,
-                                                             int replace, PcgResult* res) {
-  __shared__ double sm[kSmDoubles];
-  Grid g{gs, partial, sm, 0u};
-  const int stride = gridDim.x * blockDim.x;
-  const int k0 = blockIdx.x * blockDim.x + threadIdx.x;
-  float y[R], r[R], p[R], sv[R], z[R], w[R];
-#pragma unroll
-  for (int u = 0; u < R; ++u) {
-    const int K = k0 + u * stride;
-    y[u] = p[u] = sv[u] = z[u] = w[u] = r[u] = 0.0f;
-    if (K < F.N) {
-      r[u] = (float)(sdiag[K] * bscale * b[K]);
-      wa[K] = r[u];   // the first product is A r
-    }
-  }
-  if (!grid_barrier(g)) return;
-  float t0 = 0.0f, t1 = 0.0f;
-#pragma unroll
-  for (int u = 0; u < R; ++u) {
-    const int K = k0 + u * stride;
-    if (K < F.N) {
-      w[u] = sell_apply<float>(F, Ts, wa, K);
-      wb[K] = w[u];
-      t0 = fmaf(r[u], r[u], t0);
-      t1 = fmaf(w[u], r[u], t1);
-    }
-  }
-  double a4[4] = {(double)t0, (double)t1, 0.0, 0.0};
-  if (!grid_sum_x<2, 2>(g, a4, [&](double* o) {
-        o[2] = 0.0;
-        o[3] = o[1] != 0.0 ? fast_div(o[0], o[1]) : 0.0;
-      }))
-    return;
-  double gamma = a4[0], beta = a4[2], alpha = a4[3];
-  const double rr0 = gamma;
-  const double tol2 = tol * tol * rr0;
-  float* wc = wb;   // published w of the current iteration
-  float* wn = wa;   // next w
-  int it = 0;
-  while (rr0 > 0.0 && gamma > tol2 && it < maxit) {
-    if (!(alpha != 0.0)) break;
-    const float af = (float)alpha, bf = (float)beta;
-    float n0 = 0.0f, n1 = 0.0f;
-#pragma unroll
-    for (int u = 0; u < R; ++u) {
-      const int K = k0 + u * stride;
-      if (K < F.N) {
-        const float nK = sell_apply<float>(F, Ts, wc, K);
-        z[u] = nK + bf * z[u];
-        sv[u] = w[u] + bf * sv[u];
-        p[u] = r[u] + bf * p[u];
-        y[u] += af * p[u];
-        r[u] = r[u] - af * sv[u];
-        w[u] = w[u] - af * z[u];
-        wn[K] = w[u];
-        n0 = fmaf(r[u], r[u], n0);
-        n1 = fmaf(w[u], r[u], n1);
-      }
-    }
-    if (replace > 0 && (it + 1) % replace == 0) {
-#pragma unroll
-      for (int u = 0; u < R; ++u) {
-        const int K = k0 + u * stride;
-        if (K < F.N) {
-          ypub[K] = y[u];
-          ppub[K] = p[u];
-        }
-      }
-      if (!grid_barrier(g)) return;
-#pragma unroll
-      for (int u = 0; u < R; ++u) {
-        const int K = k0 + u * stride;
-        if (K < F.N) {
-          r[u] = (float)(sdiag[K] * bscale * b[K]) - sell_apply<float>(F, Ts, ypub, K);
-          sv[u] = sell_apply<float>(F, Ts, ppub, K);
-          rpub[K] = r[u];
-          spub[K] = sv[u];
-        }
-      }
-      if (!grid_barrier(g)) return;
-      n0 = n1 = 0.0f;
-#pragma unroll
-      for (int u = 0; u < R; ++u) {
-        const int K = k0 + u * stride;
-        if (K < F.N) {
-          w[u] = sell_apply<float>(F, Ts, rpub, K);
-          z[u] = sell_apply<float>(F, Ts, spub, K);
-          wn[K] = w[u];
-          n0 = fmaf(r[u], r[u], n0);
-          n1 = fmaf(w[u], r[u], n1);
-        }
-      }
-    }
-    double n4[4] = {(double)n0, (double)n1, 0.0, 0.0};
-    if (!grid_sum_x<2, 2>(g, n4, [&](double* o) {
-          const double g = o[0], d = o[1];
-          const double bn = gamma != 0.0 ? fast_div(g, gamma) : 0.0;
-          const double den = d - fast_div(bn * g, alpha);
-          o[2] = bn;
-          o[3] = den != 0.0 ? fast_div(g, den) : 0.0;
-        }))
-      return;
-    gamma = n4[0];
-    beta = n4[2];
-    alpha = n4[3];
-    float* t = wc;
-    wc = wn;
-    wn = t;
-    ++it;
-  }
-#pragma unroll
-  for (int u = 0; u < R; ++u) {
-    const int K = k0 + u * stride;
-    if (K < F.N) dx[K] = sdiag[K] * (double)y[u];
-  }
+  CSTRIDE(i, F.N) dx[i] = sdiag[i] * (double)y[i];
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     res->iters = it;
     res->rr0 = rr0;
@@ -506,7 +275,7 @@ __global__ void __launch_bounds__(kPThreads) kp_fine_bicgstab(FineDev F, const d
   __shared__ double sm[kSmDoubles];
   Grid g{gs, partial, sm, 0u};
   double a1[1] = {0.0};
-  GSTRIDE(i, F.N) {
+  CSTRIDE(i, F.N) {
     const double ri = sS[i] * bscale * b[i];
     y[i] = 0.0;
     r[i] = ri;
@@ -521,7 +290,7 @@ __global__ void __launch_bounds__(kPThreads) kp_fine_bicgstab(FineDev F, const d
   int it = 0;
   while (rr0 > 0.0 && rr > tol2 && it < maxit) {
     double a2[2] = {0.0, 0.0};
-    GSTRIDE(K, F.N) {
+    CSTRIDE(K, F.N) {
       const double vK = jac_row(F, Js, jd[K], p, K);
       v[K] = vK;
       a2[0] = fma(rh[K], vK, a2[0]);
@@ -529,10 +298,10 @@ __global__ void __launch_bounds__(kPThreads) kp_fine_bicgstab(FineDev F, const d
     if (!grid_sum_x<1, 1>(g, a2, [&](double* o) { o[1] = o[0] != 0.0 ? fast_div(rho, o[0]) : 0.0; })) return;
     const double alpha = a2[1];
     if (!(alpha != 0.0)) break;
-    GSTRIDE(K, F.N) s[K] = r[K] - alpha * v[K];
+    CSTRIDE(K, F.N) s[K] = r[K] - alpha * v[K];
     if (!grid_barrier(g)) return;
     double a3[3] = {0.0, 0.0, 0.0};
-    GSTRIDE(K, F.N) {
+    CSTRIDE(K, F.N) {
       const double tK = jac_row(F, Js, jd[K], s, K);
       const double sK = s[K];
       t[K] = tK;
@@ -542,7 +311,7 @@ __global__ void __launch_bounds__(kPThreads) kp_fine_bicgstab(FineDev F, const d
     if (!grid_sum_x<2, 1>(g, a3, [&](double* o) { o[2] = o[1] != 0.0 ? fast_div(o[0], o[1]) : 0.0; })) return;
     const double omega = a3[2];
     double a4[3] = {0.0, 0.0, 0.0};
-    GSTRIDE(K, F.N) {
+    CSTRIDE(K, F.N) {
       const double sK = s[K];
       y[K] += alpha * p[K] + omega * sK;
       const double rK = sK - omega * t[K];
@@ -560,10 +329,10 @@ __global__ void __launch_bounds__(kPThreads) kp_fine_bicgstab(FineDev F, const d
     const bool stop = !(omega != 0.0) || !(a4[0] != 0.0);
     rho = a4[0];
     if (stop) break;
-    GSTRIDE(K, F.N) p[K] = r[K] + beta * (p[K] - omega * v[K]);
+    CSTRIDE(K, F.N) p[K] = r[K] + beta * (p[K] - omega * v[K]);
     if (!grid_barrier(g)) return;
   }
-  GSTRIDE(i, F.N) dx[i] = sS[i] * y[i];
+  CSTRIDE(i, F.N) dx[i] = sS[i] * y[i];
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     res->iters = it;
     res->rr0 = rr0;
@@ -617,27 +386,6 @@ cudaError_t launch_fine_cg_pipe(cudaStream_t st, const FineDev& F, const T* Ts, 
                   (void*)&tol, (void*)&maxit, (void*)&res};
   return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kPThreads), args, 0, st);
 }
-// FP32 pipelined CG with residual replacement if every thread holds at most 8 cells on the grid the launch gets;
-// returns cudaErrorNotSupported (nothing launched) otherwise.
-cudaError_t launch_fine_cg_rr32(cudaStream_t st, const FineDev& F, const float* Ts, const double* sdiag,
-                                const double* b, double bscale, double* dx, float* wa, float* wb, float* ypub,
-                                float* ppub, float* rpub, float* spub, double* partial, GridSync gs, double tol,
-                                int maxit, int replace, PcgResult* res) {
-  const void* fns[4] = {(const void*)kp_fine_cg_rr32<1>, (const void*)kp_fine_cg_rr32<2>,
-                        (const void*)kp_fine_cg_rr32<4>, (const void*)kp_fine_cg_rr32<8>};
-  const int Rs[4] = {1, 2, 4, 8};
-  for (int i = 0; i < 4; ++i) {
-    const int grid = coop_grid(fns[i], F.N, gs.sm_cap);
-    const long cap = (long)grid * kPThreads * Rs[i];
-    if (cap < F.N) continue;
-    void* args[] = {(void*)&F, (void*)&Ts, (void*)&sdiag, (void*)&b, (void*)&bscale, (void*)&dx, (void*)&wa,
-                    (void*)&wb, (void*)&ypub, (void*)&ppub, (void*)&rpub, (void*)&spub, (void*)&partial,
-                    (void*)&gs, (void*)&tol, (void*)&maxit, (void*)&replace, (void*)&res};
-    return cudaLaunchCooperativeKernel(fns[i], dim3(grid), dim3(kPThreads), args, 0, st);
-  }
-  return cudaErrorNotSupported;
-}
-
 cudaError_t launch_fine_bicgstab(cudaStream_t st, const FineDev& F, const double* Js, const double* jd,
                                  const double* sS, const double* b, double bscale, double* dx, double* work,
                                  double* partial, GridSync gs, double tol, int maxit, PcgResult* res) {
@@ -651,28 +399,6 @@ cudaError_t launch_fine_bicgstab(cudaStream_t st, const FineDev& F, const double
                   (void*)&gs, (void*)&tol, (void*)&maxit, (void*)&res};
   return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kPThreads), args, 0, st);
 }
-// Register-resident pipelined CG if every thread holds at most 4 cells on the grid the launch gets; returns
-// cudaErrorNotSupported (nothing launched) otherwise.
-template <class TM>
-cudaError_t launch_fine_cg_reg(cudaStream_t st, const FineDev& F, const TM* Ts, const double* sdiag, const double* b,
-                               double bscale, double* dx, TM* wa, TM* wb, double* partial, GridSync gs, double tol,
-                               int maxit, PcgResult* res) {
-  const void* fns[3] = {(const void*)kp_fine_cg_reg<TM, 1>, (const void*)kp_fine_cg_reg<TM, 2>,
-                        (const void*)kp_fine_cg_reg<TM, 4>};
-  const int Rs[3] = {1, 2, 4};
-  for (int i = 0; i < 3; ++i) {
-    const int grid = coop_grid(fns[i], F.N, gs.sm_cap);
-    const long cap = (long)grid * kPThreads * Rs[i];
-    if (cap < F.N) continue;
-    void* args[] = {(void*)&F, (void*)&Ts, (void*)&sdiag, (void*)&b, (void*)&bscale, (void*)&dx, (void*)&wa,
-                    (void*)&wb, (void*)&partial, (void*)&gs, (void*)&tol, (void*)&maxit, (void*)&res};
-    return cudaLaunchCooperativeKernel(fns[i], dim3(grid), dim3(kPThreads), args, 0, st);
-  }
-  return cudaErrorNotSupported;
-}
-template cudaError_t launch_fine_cg_reg<double>(cudaStream_t, const FineDev&, const double*, const double*,
-                                                const double*, double, double*, double*, double*, double*, GridSync,
-                                                double, int, PcgResult*);
 template cudaError_t launch_fine_cg_pipe<double>(cudaStream_t, const FineDev&, const double*, const double*,
                                                  const double*, double, double*, double*, double*, double*, double*,
                                                  double*, double*, double*, double*, GridSync, double, int,

@@ -32,25 +32,34 @@ cudaError_t launch_fine_cg_pipe(cudaStream_t st, const FineDev& F, const T* Ts, 
                                 double bscale, double* dx, T* y, T* r, T* wa, T* wb, T* z, T* sv, T* p,
                                 double* partial, GridSync gs, double tol, int maxit, PcgResult* res);
 
-// Register-resident pipelined CG (TM = type of the matrix and of the exchanged vector, double; recurrences in FP64).
-// Returns cudaErrorNotSupported without launching when a thread would have to hold more than 4 cells.
-template <class TM>
-cudaError_t launch_fine_cg_reg(cudaStream_t st, const FineDev& F, const TM* Ts, const double* sdiag, const double* b,
-                               double bscale, double* dx, TM* wa, TM* wb, double* partial, GridSync gs, double tol,
-                               int maxit, PcgResult* res);
+// Vectors the register-resident CG publishes: w double-buffered, and (T = float) y, p, r and s at a replacement.
+template <class T>
+struct FineCgBufs {
+  T *wa = nullptr, *wb = nullptr, *y = nullptr, *p = nullptr, *r = nullptr, *s = nullptr;
+};
 
-// Register-resident FP32 pipelined CG with residual replacement every `replace` iterations (0: never). Returns
-// cudaErrorNotSupported without launching when a thread would have to hold more than 8 cells.
-cudaError_t launch_fine_cg_rr32(cudaStream_t st, const FineDev& F, const float* Ts, const double* sdiag,
-                                const double* b, double bscale, double* dx, float* wa, float* wb, float* ypub,
-                                float* ppub, float* rpub, float* spub, double* partial, GridSync gs, double tol,
-                                int maxit, int replace, PcgResult* res);
+// Register-resident pipelined CG on the frozen matrix Tval scaled by sdiag (Ts: room for the scaled entries, used when
+// the rows do not fit in shared memory); T = float with residual replacement every `replace` iterations (0: never).
+// Returns cudaErrorNotSupported without launching when a thread would have to hold more than 5 (FP32: 9) cells.
+template <class T>
+cudaError_t launch_fine_cg_reg(cudaStream_t st, const FineDev& F, const double* Tval, T* Ts, const double* sdiag,
+                               const double* b, double bscale, double* dx, const FineCgBufs<T>& B, double* partial,
+                               GridSync gs, double tol, int maxit, int replace, PcgResult* res);
 
 // Persistent FP64 BiCGStab for the level-0 Newton system J dx = bscale b on the scaled Jacobian (Js off the
 // diagonal in the SELL layout, jd on it, sS = S per cell); work holds 7 n_cells doubles.
 cudaError_t launch_fine_bicgstab(cudaStream_t st, const FineDev& F, const double* Js, const double* jd,
                                  const double* sS, const double* b, double bscale, double* dx, double* work,
                                  double* partial, GridSync gs, double tol, int maxit, PcgResult* res);
+
+// The same with the cells' state in registers, on the unscaled Jacobian (Joff off the diagonal, jdiag on it) and the
+// Jacobi weights D with S = D^1/2 (Js: room for the scaled entries, used when the rows do not fit in shared memory);
+// work holds 2 n_cells doubles. Returns cudaErrorNotSupported without launching when a thread would have to hold more
+// than 4 cells.
+cudaError_t launch_fine_bicgstab_reg(cudaStream_t st, const FineDev& F, const double* Joff, double* Js,
+                                     const double* jdiag, const double* D, const double* S, const double* b,
+                                     double bscale, double* dx, double* work, double* partial, GridSync gs, double tol,
+                                     int maxit, PcgResult* res);
 
 // Extra per-lambda vectors of the pipelined hybridized CG (w = H u, z, s, and m = M w double-buffered).
 template <class T>

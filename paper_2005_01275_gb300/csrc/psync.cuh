@@ -194,7 +194,7 @@ __device__ __forceinline__ bool grid_barrier(Grid& g, unsigned long long spin_li
 
 // Grid sums of NV values, in two halves, for a block whose warp `server` does the serial part (it may hold values too).
 // grid_sum_arrive: warp sums, the block's sums to the partial buffer, then the grid barrier; on return every block's
-// earlier writes and partials are visible. grid_sum_finish, by the server warp alone: every block's partials added
+// earlier writes and partials are visible. The other warps run `meanwhile` (on registers) while the server waits. grid_sum_finish, by the server warp alone: every block's partials added
 // (all blocks get bit-identical sums, so they take the same decisions); every lane of that warp returns the sums.
 // Consecutive reductions use the two partial buffers in turn: a block can only overwrite a buffer after every block
 // has passed the next barrier, i.e. has finished reading it.
@@ -202,8 +202,8 @@ template <int NV>
 __device__ __forceinline__ constexpr int part_stride() {   // doubles of a block's partials: whole double2
   return NV <= 2 ? 2 : NV <= 4 ? 4 : 8;
 }
-template <int NV>
-__device__ __forceinline__ bool grid_sum_arrive(Grid& g, const double (&v)[NV], int server) {
+template <int NV, class Work>
+__device__ __forceinline__ bool grid_sum_arrive(Grid& g, const double (&v)[NV], int server, Work&& meanwhile) {
   static_assert(NV >= 1 && NV <= kMaxNV, "grid sums: the shared scratch holds kMaxNV values per warp");
   __shared__ int ok;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -242,10 +242,16 @@ __device__ __forceinline__ bool grid_sum_arrive(Grid& g, const double (&v)[NV], 
       ok = grid_wait(g, kSpinLimit) ? 1 : 0;
     }
     __syncwarp();
+  } else {
+    meanwhile();
   }
   g.phase ^= 0x80000000u;
   __syncthreads();
   return ok != 0;
+}
+template <int NV>
+__device__ __forceinline__ bool grid_sum_arrive(Grid& g, const double (&v)[NV], int server) {
+  return grid_sum_arrive<NV>(g, v, server, [] {});
 }
 template <int NV>
 __device__ __forceinline__ void grid_sum_finish(const Grid& g, double (&s)[NV]) {

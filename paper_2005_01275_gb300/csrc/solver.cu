@@ -282,6 +282,7 @@ void upload_fine(nlmg_ctx* c) {
     }
   }
   F.nnz = soff[F.nslice];
+  F.wmax = *std::max_element(sw.begin(), sw.end());
   c->sh->nnz_real = (long long)nbr.size();
   F.sell_off = c->upload(soff);
   F.sell_w = c->upload(sw);
@@ -684,49 +685,46 @@ int fine_pcg(nlmg_ctx* c, const double* R, const double* kap) {
   launch_sdiag(c->st, c->F.N, c->diagT, c->sdiag);
   const bool fp32 = c->opt.lin_precision == 1;
   // FP64 at loose tolerances: pipelined CG (one grid barrier per iteration), register-resident when every thread
-  // holds at most 4 cells. FP32: the pipelined CG with residual replacement every kReplace iterations (without it
+  // holds at most 5 cells. FP32: the pipelined CG with residual replacement every kReplace iterations (without it
   // the FP32 recurrences drift: measured 10,768 instead of 3,466 fine iterations on the 64^3 workload), registers
-  // for at most 8 cells per thread; else the two-barrier CG in memory. Tight FP64 tolerances: the two-barrier CG, whose
+  // for at most 9 cells per thread; else the two-barrier CG in memory. Tight FP64 tolerances: the two-barrier CG, whose
   // updated residual tracks the true one more closely.
   constexpr int kReplace = 50;
   const bool pipe = !fp32 && c->lin_tol_eff >= 1e-6;
   int kind = 0;   // 0 two-barrier, 1 pipelined in memory, 2 pipelined in registers, 4 FP32 pipelined with
                   // residual replacement
-  int pi;
+  const int pi = c->prof_begin(0);
   if (fp32) {
-    launch_scale_sell<float>(c->st, c->F, c->Tval, c->sdiag, c->Ts32);
-    pi = c->prof_begin(0);
-    cudaError_t e = launch_fine_cg_rr32(c->st, c->F, c->Ts32, c->sdiag, R, -1.0, c->cx, c->fpa, c->fpb, c->fy,
-                                        c->fq, c->fr, c->fs, c->d_partial, gs, std::max(c->lin_tol_eff, 1e-6),
-                                        c->opt.lin_maxit, kReplace, c->d_res);
+    const double tol = std::max(c->lin_tol_eff, 1e-6);
+    const FineCgBufs<float> B{c->fpa, c->fpb, c->fy, c->fq, c->fr, c->fs};
+    cudaError_t e = launch_fine_cg_reg<float>(c->st, c->F, c->Tval, c->Ts32, c->sdiag, R, -1.0, c->cx, B, c->d_partial,
+                                              gs, tol, c->opt.lin_maxit, kReplace, c->d_res);
     kind = 4;
     if (e == cudaErrorNotSupported) {
       kind = 0;
-      CK(launch_fine_cg<float>(c->st, c->F, c->Ts32, c->sdiag, R, -1.0, c->cx, c->fy, c->fr, c->fpa, c->fpb, c->fq,
-                               c->d_partial, gs, std::max(c->lin_tol_eff, 1e-6), c->opt.lin_maxit, c->d_res));
-    } else {
-      CK(e);
+      launch_scale_sell<float>(c->st, c->F, c->Tval, c->sdiag, c->Ts32);
+      e = launch_fine_cg<float>(c->st, c->F, c->Ts32, c->sdiag, R, -1.0, c->cx, c->fy, c->fr, c->fpa, c->fpb, c->fq,
+                                c->d_partial, gs, tol, c->opt.lin_maxit, c->d_res);
     }
+    CK(e);
   } else {
-    launch_scale_sell<double>(c->st, c->F, c->Tval, c->sdiag, c->Ts64);
-    pi = c->prof_begin(0);
     cudaError_t e = cudaErrorNotSupported;
-    if (pipe)
-      e = launch_fine_cg_reg<double>(c->st, c->F, c->Ts64, c->sdiag, R, -1.0, c->cx, c->dv1, c->dv2, c->d_partial,
-                                     gs, c->lin_tol_eff, c->opt.lin_maxit, c->d_res);
-    if (e == cudaSuccess) {
+    if (pipe) {
+      const FineCgBufs<double> B{c->dv1, c->dv2};
+      e = launch_fine_cg_reg<double>(c->st, c->F, c->Tval, c->Ts64, c->sdiag, R, -1.0, c->cx, B, c->d_partial, gs,
+                                     c->lin_tol_eff, c->opt.lin_maxit, 0, c->d_res);
       kind = 2;
-    } else if (e != cudaErrorNotSupported) {
-      CK(e);
-    } else if (pipe) {
-      kind = 1;
-      CK(launch_fine_cg_pipe<double>(c->st, c->F, c->Ts64, c->sdiag, R, -1.0, c->cx, c->cz, c->cr, c->cpa, c->cpb,
-                                     c->cq, c->dv1, c->dv2, c->d_partial, gs, c->lin_tol_eff, c->opt.lin_maxit,
-                                     c->d_res));
-    } else {
-      CK(launch_fine_cg<double>(c->st, c->F, c->Ts64, c->sdiag, R, -1.0, c->cx, c->cz, c->cr, c->cpa, c->cpb,
-                                c->cq, c->d_partial, gs, c->lin_tol_eff, c->opt.lin_maxit, c->d_res));
     }
+    if (e == cudaErrorNotSupported) {
+      launch_scale_sell<double>(c->st, c->F, c->Tval, c->sdiag, c->Ts64);
+      kind = pipe ? 1 : 0;
+      e = pipe ? launch_fine_cg_pipe<double>(c->st, c->F, c->Ts64, c->sdiag, R, -1.0, c->cx, c->cz, c->cr, c->cpa,
+                                             c->cpb, c->cq, c->dv1, c->dv2, c->d_partial, gs, c->lin_tol_eff,
+                                             c->opt.lin_maxit, c->d_res)
+               : launch_fine_cg<double>(c->st, c->F, c->Ts64, c->sdiag, R, -1.0, c->cx, c->cz, c->cr, c->cpa, c->cpb,
+                                        c->cq, c->d_partial, gs, c->lin_tol_eff, c->opt.lin_maxit, c->d_res);
+    }
+    CK(e);
   }
   c->last_fine_kind = kind;
   c->prof_end(pi);
@@ -784,7 +782,7 @@ void newton_linearize(nlmg_ctx* c) {
   launch_residual(c->st, c->F, c->cur.p, c->t2.kap, c->dkap, c->g, c->rhs, c->t2.R,
                   c->opt.lin_precond == 1 ? c->Tval : nullptr, nullptr, c->diagT, c->jdiag, c->red(S_NORM2B),
                   c->Joff);
-  launch_jacobi_dinv(c->st, N, c->jdiag, c->diagT, c->jdinv);
+  launch_jacobi_dinv(c->st, N, c->jdiag, c->diagT, c->jdinv, c->jsS);
 }
 
 // Persistent FP64 BiCGStab on the Jacobi-scaled Newton system J dx = -R (J from newton_linearize) to newton_tol_eff;
@@ -794,10 +792,16 @@ int fine_bicgstab(nlmg_ctx* c, const double* R) {
   GridSync gs{c->d_bar, &c->d_res->err, c->sm_cap};
   CK(cudaMemsetAsync(c->d_bar, 0, sizeof(unsigned), c->st));
   CK(cudaMemsetAsync(c->d_res, 0, sizeof(PcgResult), c->st));
-  launch_scale_jac(c->st, c->F, c->jdiag, c->Joff, c->jdinv, c->Js, c->jdS, c->jsS);
   const int pi = c->prof_begin(3);
-  CK(launch_fine_bicgstab(c->st, c->F, c->Js, c->jdS, c->jsS, R, -1.0, c->cx, c->gV, c->d_partial, gs,
-                          c->newton_tol_eff, c->opt.lin_maxit, c->d_res));
+  cudaError_t e = launch_fine_bicgstab_reg(c->st, c->F, c->Joff, c->Js, c->jdiag, c->jdinv, c->jsS, R, -1.0, c->cx,
+                                           c->gV, c->d_partial, gs, c->newton_tol_eff, c->opt.lin_maxit, c->d_res);
+  const bool reg = e != cudaErrorNotSupported;
+  if (!reg) {
+    launch_scale_jac(c->st, c->F, c->jdiag, c->Joff, c->jdinv, c->jsS, c->Js, c->jdS);
+    e = launch_fine_bicgstab(c->st, c->F, c->Js, c->jdS, c->jsS, R, -1.0, c->cx, c->gV, c->d_partial, gs,
+                             c->newton_tol_eff, c->opt.lin_maxit, c->d_res);
+  }
+  CK(e);
   c->prof_end(pi);
   count_launch(1);
   CK(cudaMemcpyAsync(c->h_res, c->d_res, sizeof(PcgResult), cudaMemcpyDeviceToHost, c->st));
@@ -809,11 +813,11 @@ int fine_bicgstab(nlmg_ctx* c, const double* R) {
     // Algorithmic bytes: once, b and S read, y, r, rh, p written, then S and y read and dx written (10 vectors).
     // Per iteration the scaled Jacobian (values, indices, diagonal) twice, and the vectors of the five passes:
     // p gathered, rh read, v written; r, v read, s written; s gathered, t written; s, y, p, t, rh read, y, r
-    // written; r, p, v read, p written (19 vectors). Flops: two products (2 per stored entry, diagonal included)
-    // and 11 FMAs per cell per iteration.
+    // written; r, p, v read, p written (19 vectors); in registers only p and s written and gathered (4 vectors). Flops:
+    // two products (2 per stored entry, diagonal included) and 11 FMAs (in registers 12) per cell per iteration.
     const double N = c->F.N, nnz = (double)c->sh->nnz_real;
-    c->prof.bytes[3] += 10.0 * 8.0 * N + it * (2.0 * (12.0 * nnz + 8.0 * N) + 19.0 * 8.0 * N);
-    c->prof.flops[3] += it * (4.0 * (nnz + N) + 22.0 * N);
+    c->prof.bytes[3] += 10.0 * 8.0 * N + it * (2.0 * (12.0 * nnz + 8.0 * N) + (reg ? 4.0 : 19.0) * 8.0 * N);
+    c->prof.flops[3] += it * (4.0 * (nnz + N) + (reg ? 24.0 : 22.0) * N);
   }
   c->lin_iters += it;
   c->lin_iters_level[0] += it;
