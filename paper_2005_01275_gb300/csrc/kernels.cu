@@ -1,13 +1,14 @@
 // Device kernels of the FAS path (sm_103a, FP64). See kernels.cuh for the data layout.
 //
 // All kernels are memory-bound sparse or per-cell work with little arithmetic per byte; on this part FP64 ALU
-// throughput is low, so each kernel does the minimum FP64 work: kappa is evaluated once per cell (k_kappa) and read
+// throughput is low, so each kernel does the minimum FP64 work: 1 / kappa is evaluated once per cell (k_kappa) and read
 // back by the residual, and the Picard steps freeze the face transmissibilities once (k_residual with Tval) so
 // that the CG iterations only stream the frozen matrix.
 #include <algorithm>
 #include <atomic>
 #include <cmath>
 
+#include "fp64.cuh"
 #include "kernels.cuh"
 
 namespace nlmg {
@@ -83,13 +84,15 @@ __device__ __forceinline__ bool grid_reduce(double (&v)[NV], const Reduce& red) 
 // ---- fine level ------------------------------------------------------------------------------------------------
 
 __global__ void k_kappa(int n, const double* __restrict__ p, const double* __restrict__ dp, double s,
-                        double* __restrict__ q, double* __restrict__ kap, double* __restrict__ dkap, int kind,
-                        double a) {
+                        double* __restrict__ q, double* __restrict__ r, double* __restrict__ dr, int kind, double a,
+                        unsigned* zero) {
+  if (zero && blockIdx.x == 0 && threadIdx.x == 0) *zero = 0u;
   GRID_STRIDE(i, n) {
-    double v = dp ? fma(s, dp[i], p[i]) : p[i];
+    const double v = dp ? fma(s, dp[i], p[i]) : p[i];
     if (q != p) q[i] = v;
-    kap[i] = kappa_of(v, kind, a);
-    if (dkap) dkap[i] = dkappa_of(v, kind, a);
+    const double ri = level0_r(v, kind, a);
+    r[i] = ri;
+    if (dr) dr[i] = level0_dr(v, ri, kind, a);
   }
 }
 
@@ -101,53 +104,62 @@ __global__ void k_rhs(FineDev F, const double* __restrict__ f, const double* __r
   }
 }
 
-// R_K = sum_faces Ups_f (q_K - q_L) + sum_Dirichlet kappa_K Ups_K (q_K - g) - [f]_K  (eqs. TPFA_flux, FV_matrix)
-// Optionally: frozen matrix entries Tval (= Ups_f), its diagonal diagT and inverse, and the exact Jacobian diagonal.
+// The transmissibility 1 / d of a face, d = r_K / Ups_K + r_L / Ups_L (rare: a d at the ends of the exponent range, where
+// two vanishing kappas have no harmonic mean).
+__device__ __noinline__ double face_rare(double d, double rK, double rL) {
+  return isinf(rK) && isinf(rL) ? __longlong_as_double(0x7ff8000000000000ll) : 1.0 / d;
+}
+
+// R_K = sum_faces Ups_f (q_K - q_L) + sum_Dirichlet kappa_K Ups_K (q_K - g) - [f]_K  (eqs. TPFA_flux, FV_matrix).
+// MAT: also the frozen matrix entries Tval (= Ups_f) and its diagonal diagT; JAC: the exact Jacobian's diagonal jdiag and
+// entries Joff (null: not wanted), with diagT.
+// Bounded by FP64 issue: 7 operations an entry (2 for d, 3 for its reciprocal, the difference, the flux) and 1 for the
+// diagonal. 10^6 cells: with a division, and a diagonal nobody asked for, an entry: 200 us; now about 110; its 125 MB would take 19.
+template <bool MAT, bool JAC>
 __global__ void __launch_bounds__(kThreads) k_residual(FineDev F, const double* __restrict__ q,
-                                                       const double* __restrict__ kap,
-                                                       const double* __restrict__ dkap,
+                                                       const double* __restrict__ r, const double* __restrict__ dr,
                                                        const double* __restrict__ g,
                                                        const double* __restrict__ rhs, double* __restrict__ R,
-                                                       double* __restrict__ Tval, double* __restrict__ dinv,
-                                                       double* __restrict__ diagT, double* __restrict__ jdiag,
-                                                       double* __restrict__ Joff, Reduce red) {
+                                                       double* __restrict__ Tval, double* __restrict__ diagT,
+                                                       double* __restrict__ jdiag, double* __restrict__ Joff,
+                                                       Reduce red) {
   double acc[1] = {0.0};
   GRID_STRIDE(K, F.N) {
-    const double qK = q[K], kK = kap[K];
-    const double dkK = jdiag ? dkap[K] : 0.0;
+    const double qK = q[K], rK = r[K];
+    const double drK = JAC ? dr[K] : 0.0;
     double flux = 0.0, dsum = 0.0, jd = 0.0;
     const int w = F.sell_w[K >> 5];
     int e = F.sell_off[K >> 5] + (K & 31);
+#pragma unroll 2
     for (int j = 0; j < w; ++j, e += 32) {
       const int L = F.nbr[e];
-      const double us = F.ups_s[e];
-      const double ha = kK * us, hb = kap[L] * F.ups_n[e];
-      const double t = hb / (ha + hb);           // Ups / ha
-      const double T = ha * t;                   // harmonic mean of the two kappa-scaled halves
+      const double is = F.iu_s[e], in = F.iu_n[e], rL = r[L];
+      const double d = fma(rK, is, rL * in);
+      double T = rcp_in_range(d) ? rcp_core(d) : face_rare(d, rK, rL);
+      if (L == K) T = 0.0;   // padding
       const double diff = qK - q[L];
       flux = fma(T, diff, flux);
-      dsum += T;
-      if (Tval) Tval[e] = T;
-      if (jdiag) jd += T + t * t * dkK * us * diff;
-      // dR_K/dp_L = -Ups + (Ups/hb)^2 kappa'(p_L) Ups_bar_L (p_K - p_L), Ups/hb = ha / (ha + hb)
-      if (Joff) {
-        const double tb = ha / (ha + hb);
-        Joff[e] = -T + tb * tb * dkap[L] * F.ups_n[e] * diff;
+      if (MAT || JAC) dsum += T;
+      if (MAT) Tval[e] = T;
+      if (JAC) {
+        // dT/dp_K = -T^2 r_K' / Ups_K, so dR_K/dp_K = T - T^2 r_K' / Ups_K (p_K - p_L), dR_K/dp_L likewise
+        const double w2 = T * T * diff;
+        jd += fma(-w2 * is, drK, T);
+        if (Joff) Joff[e] = L == K ? 0.0 : -fma(w2 * in, dr[L], T);
       }
     }
     for (int e = F.dir_off[K]; e < F.dir_off[K + 1]; ++e) {
-      const double h = kK * F.dir_ups[e];
+      const double h = fast_div(F.dir_ups[e], rK);
       const double diff = qK - g[F.dir_face[e]];
       flux = fma(h, diff, flux);
-      dsum += h;
-      if (jdiag) jd += dkK * F.dir_ups[e] * diff + h;
+      if (MAT || JAC) dsum += h;
+      if (JAC) jd += fma(-fast_div(h, rK) * drK, diff, h);
     }
-    const double r = flux - rhs[K];
-    R[K] = r;
-    acc[0] = fma(r, r, acc[0]);
-    if (diagT) diagT[K] = dsum;
-    if (dinv) dinv[K] = 1.0 / dsum;
-    if (jdiag) jdiag[K] = jd;
+    const double res = flux - rhs[K];
+    R[K] = res;
+    acc[0] = fma(res, res, acc[0]);
+    if (MAT || JAC) diagT[K] = dsum;
+    if (JAC) jdiag[K] = jd;
   }
   grid_reduce<1, false>(acc, red);
 }
@@ -193,20 +205,14 @@ __global__ void k_sub(int n, const double* __restrict__ y, const double* __restr
 }
 
 // TPFA flux on each level-0 flux unknown, oriented out of K (eq. TPFA_flux).
-__global__ void k_fine_flux(FineDev F, const double* __restrict__ p, const double* __restrict__ kap,
+__global__ void k_fine_flux(FineDev F, const double* __restrict__ p, const double* __restrict__ r,
                             const double* __restrict__ g, double* __restrict__ sigma) {
   GRID_STRIDE(j, F.nflux) {
     const int K = F.fl_k[j], L = F.fl_l[j];
-    const double ha = kap[K] * F.fl_u0[j];
-    double s;
-    if (L >= 0) {
-      const double hb = kap[L] * F.fl_u1[j];
-      const double T = ha * (hb / (ha + hb));
-      s = T * (p[K] - p[L]);
-    } else {
-      s = ha * (p[K] - g[F.fl_face[j]]);
-    }
-    sigma[j] = s;
+    const double rK = r[K], rL = L >= 0 ? r[L] : 0.0;
+    const double d = L >= 0 ? fma(rK, F.fl_u0[j], rL * F.fl_u1[j]) : rK * F.fl_u0[j];
+    const double T = rcp_in_range(d) ? rcp_core(d) : face_rare(d, rK, rL);
+    sigma[j] = T * (p[K] - (L >= 0 ? p[L] : g[F.fl_face[j]]));
   }
 }
 
@@ -485,20 +491,22 @@ void count_launch(int n) {
 }
 #define COUNT(n) count_launch(n)
 
-void launch_kappa(cudaStream_t st, int n, const double* p, const double* dp, double s, double* q, double* kap,
-                  double* dkap, int kind, double a) {
+void launch_kappa(cudaStream_t st, int n, const double* p, const double* dp, double s, double* q, double* r,
+                  double* dr, int kind, double a, unsigned* zero) {
   COUNT(1);
-  k_kappa<<<grid_for(n), kThreads, 0, st>>>(n, p, dp, s, q, kap, dkap, kind, a);
+  k_kappa<<<grid_for(n), kThreads, 0, st>>>(n, p, dp, s, q, r, dr, kind, a, zero);
 }
 void launch_rhs(cudaStream_t st, const FineDev& F, const double* f, const double* g, double* rhs) {
   COUNT(1);
   k_rhs<<<grid_for(F.N), kThreads, 0, st>>>(F, f, g, rhs);
 }
-void launch_residual(cudaStream_t st, const FineDev& F, const double* q, const double* kap, const double* dkap,
-                     const double* g, const double* rhs, double* R, double* Tval, double* dinv, double* diagT,
-                     double* jdiag, Reduce red, double* Joff) {
+void launch_residual(cudaStream_t st, const FineDev& F, const double* q, const double* r, const double* dr,
+                     const double* g, const double* rhs, double* R, double* Tval, double* diagT, double* jdiag,
+                     Reduce red, double* Joff) {
   COUNT(1);
-  k_residual<<<grid_for(F.N), kThreads, 0, st>>>(F, q, kap, dkap, g, rhs, R, Tval, dinv, diagT, jdiag, Joff, red);
+  const auto k = jdiag ? (Tval ? k_residual<true, true> : k_residual<false, true>)
+                       : (Tval ? k_residual<true, false> : k_residual<false, false>);
+  k<<<grid_for(F.N), kThreads, 0, st>>>(F, q, r, dr, g, rhs, R, Tval, diagT, jdiag, Joff, red);
 }
 void launch_jacobi_update(cudaStream_t st, int n, const double* q, const double* R, const double* jdiag,
                           const double* diagT, double omega, double* qnew) {
@@ -517,10 +525,10 @@ void launch_sub(cudaStream_t st, int n, const double* y, const double* x, double
   COUNT(1);
   k_sub<<<grid_for(n), kThreads, 0, st>>>(n, y, x, out);
 }
-void launch_fine_flux(cudaStream_t st, const FineDev& F, const double* p, const double* kap, const double* g,
+void launch_fine_flux(cudaStream_t st, const FineDev& F, const double* p, const double* r, const double* g,
                       double* sigma) {
   COUNT(1);
-  k_fine_flux<<<grid_for(F.nflux), kThreads, 0, st>>>(F, p, kap, g, sigma);
+  k_fine_flux<<<grid_for(F.nflux), kThreads, 0, st>>>(F, p, r, g, sigma);
 }
 void launch_restrict_p(cudaStream_t st, const TransferDev& T, const double* in1, double* out1, double scale1,
                        const double* in2, double* out2) {

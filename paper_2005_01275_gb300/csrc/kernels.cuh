@@ -25,16 +25,16 @@ struct Reduce {
 struct FineDev {
   int N = 0, nnz = 0, nflux = 0, nslice = 0, wmax = 0;   // wmax: widest slice
   // interior neighbours per cell in SELL-32 layout: slice s = cells 32 s .. 32 s + 31, width sell_w[s]; entry j of
-  // cell K sits at sell_off[s] + 32 j + (K & 31). Padding entries point to the cell itself with Ups = (1, 0).
+  // cell K sits at sell_off[s] + 32 j + (K & 31). Padding entries point to the cell itself (no face does).
   int *sell_off = nullptr, *sell_w = nullptr, *nbr = nullptr;
-  double *ups_s = nullptr, *ups_n = nullptr;       // own / neighbour half transmissibility per entry
+  double *iu_s = nullptr, *iu_n = nullptr;         // 1 / own and 1 / neighbour half transmissibility per entry
   int *dir_off = nullptr, *dir_face = nullptr;     // Dirichlet faces per cell (CSR)
   double* dir_ups = nullptr;
   int *neu_off = nullptr, *neu_face = nullptr;     // Neumann faces per cell (CSR)
   double* neu_area = nullptr;
   double* vol = nullptr;
   int *fl_k = nullptr, *fl_l = nullptr, *fl_face = nullptr;   // level-0 flux unknowns
-  double *fl_u0 = nullptr, *fl_u1 = nullptr;
+  double *fl_u0 = nullptr, *fl_u1 = nullptr;       // 1 / half transmissibilities (fl_u1: 0 on Dirichlet faces)
 };
 
 // The nonlinearity: kind 0 kappa = exp(a p), kind 1 kappa = (1 + p^2)^-1 (Sec. 4 examples), and its derivative.
@@ -45,10 +45,15 @@ __device__ __forceinline__ double kappa_of(double p, int kind, double a) {
 __device__ __forceinline__ double inv_kappa_of(double p, int kind, double a) {
   return kind == 0 ? exp(-a * p) : fma(p, p, 1.0);
 }
-__device__ __forceinline__ double dkappa_of(double p, int kind, double a) {
-  if (kind == 0) return a * exp(a * p);
-  double t = 1.0 + p * p;
-  return -2.0 * p / (t * t);
+// What the level-0 kernels carry per cell: r = 1 / kappa(p), whose face transmissibility 1 / (r_K / Ups_K + r_L / Ups_L)
+// needs one reciprocal and seven FP64 operations an entry (a division of kappas took sixteen), and r' = dr/dp where the
+// Jacobian is formed. A kappa that overflows is not a number here, as its transmissibilities are.
+__device__ __forceinline__ double level0_r(double p, int kind, double a) {
+  const double r = inv_kappa_of(p, kind, a);
+  return r < 0x1p-1024 ? __longlong_as_double(0x7ff8000000000000ll) : r;   // 1 / DBL_MAX rounds to 2^-1024
+}
+__device__ __forceinline__ double level0_dr(double p, double r, int kind, double a) {
+  return kind == 0 ? -a * r : 2.0 * p;
 }
 
 // Coarse level (mixed, cell-by-cell: Prop. 1)
@@ -105,12 +110,15 @@ long long launch_count_thread();   // issued by the calling host thread
 void count_launch(int n);
 
 // launchers (kernels.cu)
-void launch_kappa(cudaStream_t st, int n, const double* p, const double* dp, double s, double* q, double* kap,
-                  double* dkap, int kind, double a);
+// q = p + s dp (dp may be null), r = 1 / kappa(q) and, if dr, its derivative; zeroes *zero (if not null)
+void launch_kappa(cudaStream_t st, int n, const double* p, const double* dp, double s, double* q, double* r,
+                  double* dr, int kind, double a, unsigned* zero = nullptr);
 void launch_rhs(cudaStream_t st, const FineDev& F, const double* f, const double* g, double* rhs);
-void launch_residual(cudaStream_t st, const FineDev& F, const double* q, const double* kap, const double* dkap,
-                     const double* g, const double* rhs, double* R, double* Tval, double* dinv, double* diagT,
-                     double* jdiag, Reduce red, double* Joff = nullptr);
+// R and ||R||^2 at q (r from launch_kappa). Tval, diagT (both or neither): the frozen matrix; jdiag, Joff (with dr and
+// diagT): the exact Jacobian.
+void launch_residual(cudaStream_t st, const FineDev& F, const double* q, const double* r, const double* dr,
+                     const double* g, const double* rhs, double* R, double* Tval, double* diagT, double* jdiag,
+                     Reduce red, double* Joff = nullptr);
 void launch_jac_apply(cudaStream_t st, const FineDev& F, const double* jdiag, const double* Joff,
                       const double* dinv, const double* v, double* w);
 void launch_mdot(cudaStream_t st, int n, int nk, const double* V, const double* w, double* partial,
@@ -127,7 +135,7 @@ void launch_jacobi_update(cudaStream_t st, int n, const double* q, const double*
 void launch_max_abs(cudaStream_t st, int n, const double* x, Reduce red);
 void launch_axpy(cudaStream_t st, int n, const double* x, double s, const double* dx, double* out);
 void launch_sub(cudaStream_t st, int n, const double* y, const double* x, double* out);
-void launch_fine_flux(cudaStream_t st, const FineDev& F, const double* p, const double* kap, const double* g,
+void launch_fine_flux(cudaStream_t st, const FineDev& F, const double* p, const double* r, const double* g,
                       double* sigma);
 void launch_restrict_p(cudaStream_t st, const TransferDev& T, const double* in1, double* out1, double scale1,
                        const double* in2, double* out2);

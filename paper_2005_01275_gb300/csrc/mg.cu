@@ -13,6 +13,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "fp64.cuh"
 #include "mg.cuh"
 
 namespace nlmg {
@@ -181,10 +182,10 @@ __global__ void k_fine_vals(FineDev F, const double* __restrict__ Tval, const do
 // block's list and accumulates the whole MB x MB block; a fixed shuffle tree then adds the lanes' blocks. The
 // contributions (K, L, e, type): 0 interior face inside the aggregate, T (P_K - P_L)(P_K - P_L)^T; 1 face to another
 // aggregate seen from this one's cell K, T P_K P_K^T; 2 the off-diagonal part, -T P_K P_L^T; 3 Dirichlet face (L = its
-// entry in the Dirichlet list), h P_K P_K^T with h = kappa_K Ups_K.
+// entry in the Dirichlet list), h P_K P_K^T with h = Ups_K / r_K, r = 1 / kappa.
 template <int MB, class PT>
 __global__ void k_asm1(int nblk, const int* __restrict__ off, const int4* __restrict__ list,
-                       const PT* __restrict__ P0, const double* __restrict__ Tval, const double* __restrict__ kap,
+                       const PT* __restrict__ P0, const double* __restrict__ Tval, const double* __restrict__ r,
                        const double* __restrict__ dir_ups, float* __restrict__ aval) {
   pdl_start();
   const int lane = threadIdx.x & 31;
@@ -201,7 +202,7 @@ __global__ void k_asm1(int nblk, const int* __restrict__ off, const int4* __rest
       for (int j = 0; j < MB; ++j) pk[j] = pval(P0, (size_t)t.x * MB + j);
       float w;
       if (t.w == 3) {
-        w = (float)(kap[t.x] * dir_ups[t.y]);
+        w = (float)fast_div(dir_ups[t.y], r[t.x]);
 #pragma unroll
         for (int j = 0; j < MB; ++j) pl[j] = pk[j];
       } else {
@@ -1481,17 +1482,17 @@ void res_level(cudaStream_t st, const MgDev& M, const MgWork& W, int l, int cur,
 }  // namespace
 
 void mg_enqueue_setup(cudaStream_t st, const MgDev& M, const FineDev& F, const MgWork& W, const double* Tval,
-                      const double* diagT, const double* kap) {
+                      const double* diagT, const double* r) {
   cudaMemsetAsync(W.lam, 0, kMgMaxLevels * sizeof(float), st);
   launchk(st, blocks_for(M.N, 4096), kT, 0, k_fine_vals, F, Tval, diagT, W.a0off, W.a0diag, W.a0dinv, W.lam);
   if (W.bf16) {
     MG_MB_SWITCH(M.mb[1], launchk(st, warps_grid(M.nblk[1]), kT, 0, k_asm1<MB, __nv_bfloat16>, M.nblk[1],
                                   (const int*)M.asm_off[1], (const int4*)M.asm_list[1],
-                                  (const __nv_bfloat16*)M.Pb[0], Tval, kap, (const double*)F.dir_ups, W.aval[1]));
+                                  (const __nv_bfloat16*)M.Pb[0], Tval, r, (const double*)F.dir_ups, W.aval[1]));
   } else {
     MG_MB_SWITCH(M.mb[1], launchk(st, warps_grid(M.nblk[1]), kT, 0, k_asm1<MB, float>, M.nblk[1],
-                                  (const int*)M.asm_off[1], (const int4*)M.asm_list[1], (const float*)M.P[0], Tval,
-                                  kap, (const double*)F.dir_ups, W.aval[1]));
+                                  (const int*)M.asm_off[1], (const int4*)M.asm_list[1], (const float*)M.P[0], Tval, r,
+                                  (const double*)F.dir_ups, W.aval[1]));
   }
   launchk(st, blocks_for(M.nc[1]), kT, 0, k_pad_diag, M.nc[1], M.mb[1], (const int*)M.dpos[1],
           (const int*)M.mcnt[1], W.aval[1]);

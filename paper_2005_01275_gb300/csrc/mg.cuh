@@ -117,7 +117,7 @@ int mg_levels_for(const Hierarchy& H);
 // Enqueues, on stream st, the per-Picard-step setup: FP32 fine values, Galerkin operators, block-diagonal inverses,
 // Gershgorin bounds and the coarsest inverse, from the frozen matrix (Tval, diagT) and kappa per cell.
 void mg_enqueue_setup(cudaStream_t st, const MgDev& M, const FineDev& F, const MgWork& W, const double* Tval,
-                      const double* diagT, const double* kap);
+                      const double* diagT, const double* r);
 
 // Enqueues one V-cycle z = B r on stream st for an FP32 right-hand side already in W.b[0] with the first pre-smoothing
 // step fused by the caller (x[0][0], d[0] hold it); returns the index i of the level-0 buffer W.x[0][i] that holds z;

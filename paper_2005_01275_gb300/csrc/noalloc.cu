@@ -17,7 +17,7 @@ namespace nlmg {
 namespace {
 
 struct NoallocScratch {
-  double kap[kNoallocMaxCells];     // kappa(p) per cell
+  double kap[kNoallocMaxCells];     // 1 / kappa(p) per cell
   double partial[kMaxBlocks * 4];   // per-block partial sums of the reduction
   unsigned counter;                 // arrivals of the last-block reduction (must be 0 when a launch starts)
 };
@@ -33,7 +33,7 @@ NoallocScratch* g_addr[kMaxDevices] = {nullptr};
 
 // Device address of the scratch array on the current device, resolved once per device. Nothing in the array needs
 // clearing here: kappa and the partial sums are written before they are read, and the arrival counter is zeroed on
-// the caller's stream before every launch (and left at zero by the reduction's last block).
+// the caller's stream by the kernel before the reduction (and left at zero by the reduction's last block).
 bool noalloc_scratch_address(void** out, std::string& err) {
   int dev = -1;
   cudaError_t e = cudaGetDevice(&dev);
@@ -58,15 +58,10 @@ bool noalloc_scratch_address(void** out, std::string& err) {
 bool noalloc_residual(cudaStream_t st, void* scratch, const FineDev& F, const double* p, const double* g,
                       const double* rhs, double* r, double* norm2, int kind, double a, std::string& err) {
   NoallocScratch* S = (NoallocScratch*)scratch;
-  cudaError_t e = cudaMemsetAsync(&S->counter, 0, sizeof(unsigned), st);
-  if (e != cudaSuccess) {
-    err = std::string("cudaMemsetAsync: ") + cudaGetErrorString(e);
-    return false;
-  }
-  launch_kappa(st, F.N, p, nullptr, 0.0, const_cast<double*>(p), S->kap, nullptr, kind, a);
+  launch_kappa(st, F.N, p, nullptr, 0.0, const_cast<double*>(p), S->kap, nullptr, kind, a, &S->counter);
   Reduce red{S->partial, &S->counter, norm2};
-  launch_residual(st, F, p, S->kap, nullptr, g, rhs, r, nullptr, nullptr, nullptr, nullptr, red);
-  e = cudaGetLastError();
+  launch_residual(st, F, p, S->kap, nullptr, g, rhs, r, nullptr, nullptr, nullptr, red);
+  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     err = std::string("kernel launch: ") + cudaGetErrorString(e);
     return false;

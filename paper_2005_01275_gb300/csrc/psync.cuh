@@ -11,6 +11,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "fp64.cuh"
 #include "persist.cuh"
 
 namespace nlmg {
@@ -28,34 +29,6 @@ __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
 
 __device__ __forceinline__ void red_add_release_gpu(unsigned* p, unsigned v) {
   asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
-// 1 / x from the hardware's approximation (about 20 bits) and one third-order step, r (1 + e + e^2) with e = 1 - x r
-// (the truncated geometric series: the remaining error e^3 is below 2^-60); x away from the ends of the exponent range.
-__device__ __forceinline__ double rcp_core(double x) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  const double e = fma(-x, r, 1.0);
-  return fma(r, fma(e, e, e), r);
-}
-// 2^-960 <= |x| <= 2^960: the core's range (a zero, an infinity or a NaN is outside)
-__device__ __forceinline__ bool rcp_in_range(double x) {
-  const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
-  return ex - 63u < 1921u;
-}
-__device__ __forceinline__ double fast_rcp(double x) { return rcp_in_range(x) ? rcp_core(x) : 1.0 / x; }
-// a / b: the reciprocal's quotient with its residual added back (about half a division's chain of operations)
-__device__ __forceinline__ double fast_div(double a, double b) {
-  if (!rcp_in_range(b) || !rcp_in_range(a)) return a / b;
-  const double r = rcp_core(b), q = a * r;
-  return fma(fma(-b, q, a), r, q);
-}
-
-// Exact double of a float, by its bits (a conversion instruction takes as long as an FP64 addition).
-__device__ __forceinline__ double widen(float f) {
-  const unsigned b = __float_as_uint(f), ex = (b >> 23) & 0xffu;
-  if (ex == 0u || ex == 255u) return (double)f;
-  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
 }
 
 // A sum in integer form: t 2^(mx - 1077), or, with mx < 0, the double whose bits t are (special values, see above).

@@ -64,9 +64,9 @@ struct Prof {
   double flops[8] = {0};
 };
 
-// Fine-level state: iterate, its kappa and residual.
+// Fine-level state: iterate, its 1 / kappa and residual.
 struct FineState {
-  double *p = nullptr, *kap = nullptr, *R = nullptr;
+  double *p = nullptr, *r = nullptr, *R = nullptr;
   double rn = 0.0;
 };
 
@@ -121,7 +121,7 @@ struct nlmg_ctx {
   double* d_sc = nullptr;
   double* h_sc = nullptr;   // pinned
   // fine buffers
-  double *f = nullptr, *g = nullptr, *rhs = nullptr, *dkap = nullptr, *Tval = nullptr, *dinv = nullptr,
+  double *f = nullptr, *g = nullptr, *rhs = nullptr, *dr = nullptr, *Tval = nullptr,
          *diagT = nullptr, *jdiag = nullptr, *sig0 = nullptr, *ptr_e = nullptr, *fdp = nullptr;
   double *cx = nullptr, *cr = nullptr, *cz = nullptr, *cpa = nullptr, *cpb = nullptr, *cq = nullptr;
   double *sdiag = nullptr, *Ts64 = nullptr, *dv1 = nullptr, *dv2 = nullptr;
@@ -267,17 +267,17 @@ void upload_fine(nlmg_ctx* c) {
     soff[sl + 1] = soff[sl] + 32 * w;
   }
   std::vector<int> snbr(soff[F.nslice], 0);
-  std::vector<double> sus(soff[F.nslice], 1.0), sun(soff[F.nslice], 0.0);
+  std::vector<double> sus(soff[F.nslice], 1.0), sun(soff[F.nslice], 1.0);   // reciprocals
   for (int K = 0; K < N; ++K) {
     int sl = K >> 5, lane = K & 31, deg = off[K + 1] - off[K];
     for (int j = 0; j < sw[sl]; ++j) {
       int e = soff[sl] + 32 * j + lane;
       if (j < deg) {
         snbr[e] = nbr[off[K] + j];
-        sus[e] = us[off[K] + j];
-        sun[e] = un[off[K] + j];
+        sus[e] = 1.0 / us[off[K] + j];
+        sun[e] = 1.0 / un[off[K] + j];
       } else {
-        snbr[e] = K;   // padding: Ups = (1, 0) gives a zero transmissibility
+        snbr[e] = K;   // padding: the cell itself
       }
     }
   }
@@ -287,8 +287,8 @@ void upload_fine(nlmg_ctx* c) {
   F.sell_off = c->upload(soff);
   F.sell_w = c->upload(sw);
   F.nbr = c->upload(snbr);
-  F.ups_s = c->upload(sus);
-  F.ups_n = c->upload(sun);
+  F.iu_s = c->upload(sus);
+  F.iu_n = c->upload(sun);
   F.dir_off = c->upload(doff);
   F.dir_face = c->upload(dface);
   F.dir_ups = c->upload(dups);
@@ -304,8 +304,8 @@ void upload_fine(nlmg_ctx* c) {
     flk.push_back(fm.fk[f]);
     fll.push_back(fm.bc[f] == 0 ? fm.fl[f] : -1);
     flf.push_back(f);
-    u0.push_back(fm.ups0[f]);
-    u1.push_back(fm.bc[f] == 0 ? fm.ups1[f] : 0.0);
+    u0.push_back(1.0 / fm.ups0[f]);
+    u1.push_back(fm.bc[f] == 0 ? 1.0 / fm.ups1[f] : 0.0);
   }
   F.nflux = L0.n_flux;
   F.fl_k = c->upload(flk);
@@ -640,10 +640,9 @@ void upload_mg(nlmg_ctx* c, int levels) {
 // level 0
 
 double fine_eval(nlmg_ctx* c, const double* p, const double* dp, double s, FineState& out) {
-  launch_kappa(c->st, c->F.N, p, dp, s, out.p, out.kap, nullptr, c->kind, c->a);
+  launch_kappa(c->st, c->F.N, p, dp, s, out.p, out.r, nullptr, c->kind, c->a);
   int pi = c->prof_begin(2);
-  launch_residual(c->st, c->F, out.p, out.kap, nullptr, c->g, c->rhs, out.R, nullptr, nullptr, nullptr, nullptr,
-                  c->red(S_NORM2));
+  launch_residual(c->st, c->F, out.p, out.r, nullptr, c->g, c->rhs, out.R, nullptr, nullptr, nullptr, c->red(S_NORM2));
   c->prof_end(pi);
   c->fine_evals++;
   out.rn = std::sqrt(c->read_sc(S_NORM2));
@@ -674,11 +673,11 @@ void backtrack0(nlmg_ctx* c, const double* dp, double s0) {
 // Persistent CG on the frozen fine matrix (Tval, diagT): A dx = -R with symmetric Jacobi scaling; dx -> c->cx.
 // lin_precision 0 runs it in FP64, 1 in FP32 (vectors and matrix; per-thread partial sums in FP32, block and grid
 // sums in FP64).
-int mg_pcg(nlmg_ctx* c, const double* R, const double* kap);
-int mg_bicgstab(nlmg_ctx* c, const double* R, const double* kap);
+int mg_pcg(nlmg_ctx* c, const double* R, const double* r);
+int mg_bicgstab(nlmg_ctx* c, const double* R, const double* r);
 
-int fine_pcg(nlmg_ctx* c, const double* R, const double* kap) {
-  if (c->opt.lin_precond == 1) return mg_pcg(c, R, kap);
+int fine_pcg(nlmg_ctx* c, const double* R, const double* r) {
+  if (c->opt.lin_precond == 1) return mg_pcg(c, R, r);
   GridSync gs{c->d_bar, &c->d_res->err, c->sm_cap};
   CK(cudaMemsetAsync(c->d_bar, 0, sizeof(unsigned), c->st));
   CK(cudaMemsetAsync(c->d_res, 0, sizeof(PcgResult), c->st));
@@ -772,15 +771,15 @@ void alloc_newton(nlmg_ctx* c) {
   c->jsS = c->dalloc<double>(N);
 }
 
-// The exact Jacobian at c->cur.p (Sec. 3.3.2 on level 0): kappa and kappa' per cell, the residual kernel's
+// The exact Jacobian at c->cur.p (Sec. 3.3.2 on level 0): 1 / kappa and its derivative per cell, the residual kernel's
 // Jacobian diagonal and off-diagonal entries (SELL layout), the frozen diagonal d and the Jacobi weights
 // 1 / max(J_KK, d_K / 2).
 void newton_linearize(nlmg_ctx* c) {
   alloc_newton(c);
   const int N = c->F.N;
-  launch_kappa(c->st, N, c->cur.p, nullptr, 0.0, c->cur.p, c->t2.kap, c->dkap, c->kind, c->a);
-  launch_residual(c->st, c->F, c->cur.p, c->t2.kap, c->dkap, c->g, c->rhs, c->t2.R,
-                  c->opt.lin_precond == 1 ? c->Tval : nullptr, nullptr, c->diagT, c->jdiag, c->red(S_NORM2B),
+  launch_kappa(c->st, N, c->cur.p, nullptr, 0.0, c->cur.p, c->t2.r, c->dr, c->kind, c->a);
+  launch_residual(c->st, c->F, c->cur.p, c->t2.r, c->dr, c->g, c->rhs, c->t2.R,
+                  c->opt.lin_precond == 1 ? c->Tval : nullptr, c->diagT, c->jdiag, c->red(S_NORM2B),
                   c->Joff);
   launch_jacobi_dinv(c->st, N, c->jdiag, c->diagT, c->jdinv, c->jsS);
 }
@@ -788,7 +787,7 @@ void newton_linearize(nlmg_ctx* c) {
 // Persistent FP64 BiCGStab on the Jacobi-scaled Newton system J dx = -R (J from newton_linearize) to newton_tol_eff;
 // dx -> c->cx.
 int fine_bicgstab(nlmg_ctx* c, const double* R) {
-  if (c->opt.lin_precond == 1) return mg_bicgstab(c, R, c->t2.kap);
+  if (c->opt.lin_precond == 1) return mg_bicgstab(c, R, c->t2.r);
   GridSync gs{c->d_bar, &c->d_res->err, c->sm_cap};
   CK(cudaMemsetAsync(c->d_bar, 0, sizeof(unsigned), c->st));
   CK(cudaMemsetAsync(c->d_res, 0, sizeof(PcgResult), c->st));
@@ -949,9 +948,9 @@ void smooth0(nlmg_ctx* c, int nu) {
     dp = c->cx;
     c->newton_steps++;
   } else if (o.smoother == NLMG_SMOOTH_PICARD || o.smoother == NLMG_SMOOTH_PICARD_NEWTON) {
-    launch_residual(c->st, c->F, c->cur.p, c->cur.kap, nullptr, c->g, c->rhs, c->t2.R, c->Tval, c->dinv, c->diagT,
-                    nullptr, c->red(S_NORM2B));
-    fine_pcg(c, c->cur.R, c->cur.kap);
+    launch_residual(c->st, c->F, c->cur.p, c->cur.r, nullptr, c->g, c->rhs, c->t2.R, c->Tval, c->diagT, nullptr,
+                    c->red(S_NORM2B));
+    fine_pcg(c, c->cur.R, c->cur.r);
     dp = c->cx;
   } else {
     // nu sweeps q <- q - omega R(q) / max(J_qq, d_q / 2) from q = p, then dp = q - p
@@ -959,9 +958,9 @@ void smooth0(nlmg_ctx* c, int nu) {
     double* qn = c->cpb;
     CK(cudaMemcpyAsync(q, c->cur.p, N * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
     for (int k = 0; k < nu; ++k) {
-      launch_kappa(c->st, N, q, nullptr, 0.0, q, c->t2.kap, c->dkap, c->kind, c->a);
-      launch_residual(c->st, c->F, q, c->t2.kap, c->dkap, c->g, c->rhs, c->t2.R, nullptr, nullptr, c->diagT,
-                      c->jdiag, c->red(S_NORM2B));
+      launch_kappa(c->st, N, q, nullptr, 0.0, q, c->t2.r, c->dr, c->kind, c->a);
+      launch_residual(c->st, c->F, q, c->t2.r, c->dr, c->g, c->rhs, c->t2.R, nullptr, c->diagT, c->jdiag,
+                      c->red(S_NORM2B));
       launch_jacobi_update(c->st, N, q, c->t2.R, c->jdiag, c->diagT, o.omega, qn);
       std::swap(q, qn);
       c->fine_evals++;
@@ -1000,8 +999,7 @@ void make_coarse_problem(nlmg_ctx* c, int l) {
   const LevelDev& C = c->LD[l + 1];
   CoarseBuf& Bc = c->CB[l + 1];
   if (l == 0) {
-    launch_kappa(c->st, c->F.N, c->cur.p, nullptr, 0.0, c->cur.p, c->cur.kap, nullptr, c->kind, c->a);
-    launch_fine_flux(c->st, c->F, c->cur.p, c->cur.kap, c->g, c->sig0);
+    launch_fine_flux(c->st, c->F, c->cur.p, c->cur.r, c->g, c->sig0);   // cur.r: of the evaluation that made cur
     launch_csr(c->st, T.qs_n, T.qs_off, T.qs_col, T.qs_val, c->sig0, Bc.x, 1.0, 0.0);
     // projection of p and restriction of the mixed pressure residual -R
     launch_restrict_p(c->st, T, c->cur.p, Bc.x + C.nflux, 1.0, c->cur.R, Bc.ptmp + C.nflux);
@@ -1159,9 +1157,8 @@ void alloc_fine(nlmg_ctx* c) {
   c->f = c->dalloc<double>(N);
   c->g = c->dalloc<double>(c->fm().n_faces);
   c->rhs = c->dalloc<double>(N);
-  c->dkap = c->dalloc<double>(N);
+  c->dr = c->dalloc<double>(N);
   c->Tval = c->dalloc<double>(c->F.nnz);
-  c->dinv = c->dalloc<double>(N);
   c->diagT = c->dalloc<double>(N);
   c->jdiag = c->dalloc<double>(N);
   c->sig0 = c->dalloc<double>(c->F.nflux);
@@ -1180,7 +1177,7 @@ void alloc_fine(nlmg_ctx* c) {
   for (float** pp : {&c->fy, &c->fr, &c->fpa, &c->fpb, &c->fq, &c->fs}) *pp = c->dalloc<float>(N);
   for (FineState* s : {&c->cur, &c->t1, &c->t2}) {
     s->p = c->dalloc<double>(N);
-    s->kap = c->dalloc<double>(N);
+    s->r = c->dalloc<double>(N);
     s->R = c->dalloc<double>(N);
   }
 }
@@ -1263,15 +1260,15 @@ void mg_set_limits(nlmg_ctx* c, double tol) {
   CK(cudaMemcpyAsync(&W.sc->maxit, &W.h_sc->maxit, sizeof(int), cudaMemcpyHostToDevice, c->st));
 }
 
-// Level-0 Picard system A(kappa(p)) dx = -R (A from the last residual launch with Tval / diagT; kappa per cell in
-// kap for the Dirichlet terms of the Galerkin operators) by CG preconditioned with one multigrid V-cycle; dx -> c->cx.
+// Level-0 Picard system A(kappa(p)) dx = -R (A from the last residual launch with Tval / diagT; 1 / kappa per cell in
+// r for the Dirichlet terms of the Galerkin operators) by CG preconditioned with one multigrid V-cycle; dx -> c->cx.
 // Stops at ||S r|| <= lin_tol ||S r_0|| (S = diag(A)^-1/2, the test of the Jacobi-preconditioned CG) or lin_maxit.
-int mg_pcg(nlmg_ctx* c, const double* R, const double* kap) {
+int mg_pcg(nlmg_ctx* c, const double* R, const double* r) {
   const MgDev& M = c->sh->MG;
   MgWork& W = c->mg;
   mg_select_precision(c);
   const int ps = c->prof_begin(7);
-  mg_enqueue_setup(c->st, M, c->F, W, c->Tval, c->diagT, kap);
+  mg_enqueue_setup(c->st, M, c->F, W, c->Tval, c->diagT, r);
   c->prof_end(ps);
   const int pi = c->prof_begin(5);
   CK(cudaMemcpyAsync(W.kb, R, (size_t)c->F.N * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
@@ -1295,12 +1292,12 @@ int mg_pcg(nlmg_ctx* c, const double* R, const double* kap) {
 // Level-0 Newton system J dx = -R (J from newton_linearize, preconditioner from the Picard matrix at the same point)
 // by right-preconditioned BiCGStab with one V-cycle per preconditioning; stops at ||W r|| <= newton_lin_tol ||W r_0||
 // with W^2 = 1 / max(J_KK, d_K / 2), the test of the Jacobi-scaled BiCGStab; dx -> c->cx.
-int mg_bicgstab(nlmg_ctx* c, const double* R, const double* kap) {
+int mg_bicgstab(nlmg_ctx* c, const double* R, const double* r) {
   const MgDev& M = c->sh->MG;
   MgWork& W = c->mg;
   mg_select_precision(c);
   const int ps = c->prof_begin(7);
-  mg_enqueue_setup(c->st, M, c->F, W, c->Tval, c->diagT, kap);
+  mg_enqueue_setup(c->st, M, c->F, W, c->Tval, c->diagT, r);
   c->prof_end(ps);
   const int pi = c->prof_begin(6);
   CK(cudaMemcpyAsync(W.kb, R, (size_t)c->F.N * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
@@ -1908,8 +1905,8 @@ nlmg_status nlmg_fine_flux(nlmg_ctx* c, const double* p, double* sigma_out) {
   return guarded(c, [&]() -> nlmg_status {
     need_data(c);
     CK(cudaMemcpyAsync(c->cpa, p, (size_t)c->F.N * sizeof(double), cudaMemcpyHostToDevice, c->st));
-    launch_kappa(c->st, c->F.N, c->cpa, nullptr, 0.0, c->cpa, c->t1.kap, nullptr, c->kind, c->a);
-    launch_fine_flux(c->st, c->F, c->cpa, c->t1.kap, c->g, c->sig0);
+    launch_kappa(c->st, c->F.N, c->cpa, nullptr, 0.0, c->cpa, c->t1.r, nullptr, c->kind, c->a);
+    launch_fine_flux(c->st, c->F, c->cpa, c->t1.r, c->g, c->sig0);
     CK(cudaMemcpyAsync(sigma_out, c->sig0, (size_t)c->F.nflux * sizeof(double), cudaMemcpyDeviceToHost, c->st));
     CK(cudaStreamSynchronize(c->st));
     return NLMG_OK;
@@ -1949,8 +1946,8 @@ nlmg_status nlmg_transfer(nlmg_ctx* c, int32_t level, int32_t op, const double* 
       if (op == NLMG_PROJECT) {
         if (level == 0) {
           need_data(c);
-          launch_kappa(c->st, c->F.N, fin, nullptr, 0.0, fin, c->t1.kap, nullptr, c->kind, c->a);
-          launch_fine_flux(c->st, c->F, fin, c->t1.kap, c->g, c->sig0);
+          launch_kappa(c->st, c->F.N, fin, nullptr, 0.0, fin, c->t1.r, nullptr, c->kind, c->a);
+          launch_fine_flux(c->st, c->F, fin, c->t1.r, c->g, c->sig0);
           launch_csr(c->st, T.qs_n, T.qs_off, T.qs_col, T.qs_val, c->sig0, Bc.xt2, 1.0, 0.0);
         } else {
           launch_csr(c->st, T.qs_n, T.qs_off, T.qs_col, T.qs_val, fin, Bc.xt2, 1.0, 0.0);
@@ -1987,9 +1984,9 @@ nlmg_status nlmg_picard_update(nlmg_ctx* c, int32_t level, const double* x, cons
       need_data(c);
       CK(cudaMemcpyAsync(c->cpa, x, (size_t)c->F.N * sizeof(double), cudaMemcpyHostToDevice, c->st));
       fine_eval(c, c->cpa, nullptr, 0.0, c->t1);
-      launch_residual(c->st, c->F, c->t1.p, c->t1.kap, nullptr, c->g, c->rhs, c->t2.R, c->Tval, c->dinv, c->diagT,
-                      nullptr, c->red(S_NORM2B));
-      it = fine_pcg(c, c->t1.R, c->t1.kap);
+      launch_residual(c->st, c->F, c->t1.p, c->t1.r, nullptr, c->g, c->rhs, c->t2.R, c->Tval, c->diagT, nullptr,
+                    c->red(S_NORM2B));
+      it = fine_pcg(c, c->t1.R, c->t1.r);
       CK(cudaMemcpyAsync(dx_out, c->cx, (size_t)c->F.N * sizeof(double), cudaMemcpyDeviceToHost, c->st));
     } else {
       const LevelDev& L = c->LD[level];
@@ -2020,10 +2017,10 @@ nlmg_status nlmg_precond_apply(nlmg_ctx* c, const double* p, const double* r, do
     const size_t N = (size_t)c->F.N;
     CK(cudaMemcpyAsync(c->cpa, p, N * sizeof(double), cudaMemcpyHostToDevice, c->st));
     fine_eval(c, c->cpa, nullptr, 0.0, c->t1);
-    launch_residual(c->st, c->F, c->t1.p, c->t1.kap, nullptr, c->g, c->rhs, c->t2.R, c->Tval, c->dinv, c->diagT,
-                    nullptr, c->red(S_NORM2B));
+    launch_residual(c->st, c->F, c->t1.p, c->t1.r, nullptr, c->g, c->rhs, c->t2.R, c->Tval, c->diagT, nullptr,
+                    c->red(S_NORM2B));
     mg_select_precision(c);
-    mg_enqueue_setup(c->st, M, c->F, W, c->Tval, c->diagT, c->t1.kap);
+    mg_enqueue_setup(c->st, M, c->F, W, c->Tval, c->diagT, c->t1.r);
     CK(cudaMemcpyAsync(W.kb, r, N * sizeof(double), cudaMemcpyHostToDevice, c->st));
     if (!W.g_apply) CK(mg_capture_apply(c->st, M, c->F, W, &W.g_apply));
     CK(cudaGraphLaunch(W.g_apply, c->st));
@@ -2151,7 +2148,7 @@ nlmg_status nlmg_profile_read(nlmg_ctx* c, int32_t kernel, int64_t* launches, do
     const double N = c->F.N, nnz = (double)c->sh->nnz_real;
     double b = 0.0;
     if (kernel != 2) b = c->prof.n[kernel] ? c->prof.bytes[kernel] / c->prof.n[kernel] : 0.0;
-    if (kernel == 2) b = 20.0 * nnz + 8.0 * N * 4;                          // nbr + 2 ups, q, kap, rhs, R
+    if (kernel == 2) b = 20.0 * nnz + 8.0 * N * 4;                          // nbr + 2 reciprocal halves, q, r, rhs, R
     if (bytes_per_launch) *bytes_per_launch = b;
     if (flops_per_launch) *flops_per_launch = c->prof.n[kernel] ? c->prof.flops[kernel] / c->prof.n[kernel] : 0.0;
     return NLMG_OK;
