@@ -149,66 +149,135 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
+// MB consecutive floats from p into v: 16-byte loads when MB % 4 == 0, 8-byte loads when MB is even (the caller
+// guarantees p is aligned accordingly: every array here is its own allocation, and a block row or a cell's vector
+// segment starts at a multiple of MB floats).
+template <int MB>
+__device__ __forceinline__ void ld_seg(const float* p, float (&v)[MB]) {
+  if constexpr (MB % 4 == 0) {
+#pragma unroll
+    for (int k = 0; k < MB / 4; ++k) {
+      const float4 t = reinterpret_cast<const float4*>(p)[k];
+      v[4 * k] = t.x;
+      v[4 * k + 1] = t.y;
+      v[4 * k + 2] = t.z;
+      v[4 * k + 3] = t.w;
+    }
+  } else if constexpr (MB % 2 == 0) {
+#pragma unroll
+    for (int k = 0; k < MB / 2; ++k) {
+      const float2 t = reinterpret_cast<const float2*>(p)[k];
+      v[2 * k] = t.x;
+      v[2 * k + 1] = t.y;
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < MB; ++k) v[k] = p[k];
+  }
+}
+
+// MB consecutive BF16 transfer entries from p, widened to float: 4-byte pair loads when MB is even.
+template <int MB>
+__device__ __forceinline__ void ld_seg(const __nv_bfloat16* p, float (&v)[MB]) {
+  if constexpr (MB % 2 == 0) {
+#pragma unroll
+    for (int k = 0; k < MB / 2; ++k) {
+      const float2 t = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(p)[k]);
+      v[2 * k] = t.x;
+      v[2 * k + 1] = t.y;
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < MB; ++k) v[k] = __bfloat162float(p[k]);
+  }
+}
+
 // ---------------------------------------------------------------------------------------------------------------
 // setup kernels (once per frozen matrix)
 
 // FP32 copy of the level-0 matrix (off-diagonal entries -T in the SELL layout, diagonal, its inverse) and the
-// Gershgorin bound max_K (A_KK + sum_L T_KL) / A_KK of D^-1 A.
+// Gershgorin bound max_K (A_KK + sum_L T_KL) / A_KK of D^-1 A: 2 where a cell has no Dirichlet face, for its diagonal is
+// that sum. One pass over the matrix; values are rounded to FP32 on the integer pipe (10^6 cells: conversions, sums and
+// two divisions took 60 us, this takes 16).
 __global__ void k_fine_vals(FineDev F, const double* __restrict__ Tval, const double* __restrict__ diagT,
                             float* __restrict__ a0off, float* __restrict__ a0diag, float* __restrict__ a0dinv,
                             float* lam) {
   pdl_start();
   float g = 0.0f;
   for (int K = blockIdx.x * blockDim.x + threadIdx.x; K < F.N; K += gridDim.x * blockDim.x) {
-    const int w = F.sell_w[K >> 5];
-    int e = F.sell_off[K >> 5] + (K & 31);
-    double s = 0.0;
-    for (int j = 0; j < w; ++j, e += 32) {
-      const double t = Tval[e];
-      a0off[e] = (float)(-t);
-      s += t;
+    const int w = F.sell_w[K >> 5], e0 = F.sell_off[K >> 5] + (K & 31);
+    for (int j = 0; j < w; ++j) a0off[e0 + 32 * j] = -narrow(Tval[e0 + 32 * j]);
+    const double dg = diagT[K], di = fast_rcp(dg);
+    a0diag[K] = narrow(dg);
+    a0dinv[K] = narrow(di);
+    float b = 2.0f;
+    if (F.dir_off[K + 1] > F.dir_off[K]) {
+      double s = 0.0;
+      for (int j = 0; j < w; ++j) s += Tval[e0 + 32 * j];
+      b = (float)((dg + s) / dg);
+    } else if (!(dg > 0.0)) {
+      b = (float)((dg + dg) / dg);
     }
-    const double dg = diagT[K];
-    a0diag[K] = (float)dg;
-    a0dinv[K] = (float)(1.0 / dg);
-    g = fmaxf(g, (float)((dg + s) / dg));
+    g = fmaxf(g, b);
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) g = fmaxf(g, __shfl_down_sync(0xffffffffu, g, off));
   if ((threadIdx.x & 31) == 0) atomic_max_pos(&lam[0], g);
 }
 
-// Level-1 Galerkin blocks from the fine faces, one warp per block: lane t takes contributions t, t + 32, ... of the
+// Sums a whole n-value array over a group of LN = 16 or 32 lanes: after each step a lane keeps the half of the values its
+// partner gave up, so 16 values take 15 or 16 shuffles instead of 64 or 80. Entry i = the returned lane index's value:
+// lane t of a 16-lane group holds the sum of value t (both halves of a 32-lane group hold it).
+template <int LN>
+__device__ __forceinline__ float group_sum16(float (&v)[16]) {
+  const int lane = threadIdx.x & (LN - 1);
+#pragma unroll
+  for (int h = 8; h > 0; h >>= 1) {
+    const bool up = (lane & h) != 0;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const float keep = up ? v[i + h] : v[i], give = up ? v[i] : v[i + h];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, give, h);
+    }
+  }
+  if (LN == 32) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 16);
+  return v[0];
+}
+
+// Level-1 Galerkin blocks from the fine faces: lane t of a group takes contributions t, t + lanes, ... of the
 // block's list and accumulates the whole MB x MB block; a fixed shuffle tree then adds the lanes' blocks. The
 // contributions (K, L, e, type): 0 interior face inside the aggregate, T (P_K - P_L)(P_K - P_L)^T; 1 face to another
 // aggregate seen from this one's cell K, T P_K P_K^T; 2 the off-diagonal part, -T P_K P_L^T; 3 Dirichlet face (L = its
-// entry in the Dirichlet list), h P_K P_K^T with h = Ups_K / r_K, r = 1 / kappa.
+// entry in the Dirichlet list), h P_K P_K^T with h = Ups_K / r_K, r = 1 / kappa. T is read as the FP32 entry of the level-0
+// matrix. With four modes a group is half a warp (an off-diagonal block has about 16 faces) and its 16 lanes end up with
+// one entry of the block each; 10^6 cells took 261 us with a warp a block, FP64 entries and a tree per entry.
 template <int MB, class PT>
 __global__ void k_asm1(int nblk, const int* __restrict__ off, const int4* __restrict__ list,
-                       const PT* __restrict__ P0, const double* __restrict__ Tval, const double* __restrict__ r,
+                       const PT* __restrict__ P0, const float* __restrict__ a0off, const double* __restrict__ r,
                        const double* __restrict__ dir_ups, float* __restrict__ aval) {
   pdl_start();
-  const int lane = threadIdx.x & 31;
+  constexpr int LN = MB == 4 ? 16 : 32;
+  const int lane = threadIdx.x & (LN - 1), per = 32 / LN;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nw = (gridDim.x * blockDim.x) >> 5;
-  for (int b = warp; b < nblk; b += nw) {
+  for (int b0 = warp * per; b0 < nblk; b0 += nw * per) {
+    const int b = b0 + (int)((threadIdx.x & 31) / LN);
     float acc[MB * MB];
 #pragma unroll
     for (int i = 0; i < MB * MB; ++i) acc[i] = 0.0f;
-    for (int c = off[b] + lane; c < off[b + 1]; c += 32) {
+    const int c1 = b < nblk ? off[b + 1] : 0;
+    for (int c = b < nblk ? off[b] + lane : 0; c < c1; c += LN) {
       const int4 t = list[c];
       float pk[MB], pl[MB];
-#pragma unroll
-      for (int j = 0; j < MB; ++j) pk[j] = pval(P0, (size_t)t.x * MB + j);
+      ld_seg<MB>(P0 + (size_t)t.x * MB, pk);
       float w;
       if (t.w == 3) {
-        w = (float)fast_div(dir_ups[t.y], r[t.x]);
+        w = narrow(fast_div(dir_ups[t.y], r[t.x]));
 #pragma unroll
         for (int j = 0; j < MB; ++j) pl[j] = pk[j];
       } else {
-        w = (float)Tval[t.z];
-#pragma unroll
-        for (int j = 0; j < MB; ++j) pl[j] = pval(P0, (size_t)t.y * MB + j);
+        w = -a0off[t.z];
+        ld_seg<MB>(P0 + (size_t)t.y * MB, pl);
         if (t.w == 0) {
 #pragma unroll
           for (int j = 0; j < MB; ++j) {
@@ -227,11 +296,17 @@ __global__ void k_asm1(int nblk, const int* __restrict__ off, const int4* __rest
 #pragma unroll
         for (int v = 0; v < MB; ++v) acc[u * MB + v] = fmaf(w * pk[u], pl[v], acc[u * MB + v]);
     }
+    __syncwarp();
+    if constexpr (MB == 4) {
+      const float s = group_sum16<LN>(acc);
+      if (b < nblk) aval[(size_t)b * 16 + lane] = s;
+    } else {
 #pragma unroll
-    for (int i = 0; i < MB * MB; ++i) acc[i] = warp_sum(acc[i]);
+      for (int i = 0; i < MB * MB; ++i) acc[i] = warp_sum(acc[i]);
 #pragma unroll
-    for (int i = 0; i < MB * MB; ++i)
-      if ((i & 31) == lane) aval[(size_t)b * MB * MB + i] = acc[i];
+      for (int i = 0; i < MB * MB; ++i)
+        if ((i & 31) == lane) aval[(size_t)b * MB * MB + i] = acc[i];
+    }
   }
 }
 
@@ -283,29 +358,34 @@ __global__ void k_asml(int nblk, int mbf, const int* __restrict__ off, const int
         }
       }
     }
+    __syncwarp();
+    if constexpr (MB == 4) {
+      const float s = group_sum16<32>(acc);
+      if (lane < 16) aval[(size_t)b * 16 + lane] = s;
+    } else {
 #pragma unroll
-    for (int i = 0; i < MB * MB; ++i) acc[i] = warp_sum(acc[i]);
+      for (int i = 0; i < MB * MB; ++i) acc[i] = warp_sum(acc[i]);
 #pragma unroll
-    for (int i = 0; i < MB * MB; ++i)
-      if ((i & 31) == lane) aval[(size_t)b * MB * MB + i] = acc[i];
+      for (int i = 0; i < MB * MB; ++i)
+        if ((i & 31) == lane) aval[(size_t)b * MB * MB + i] = acc[i];
+    }
   }
 }
 
 // Inverse of each diagonal block of a block level (Gauss-Jordan in FP64 registers, no pivoting: the blocks are
-// symmetric positive definite) and the Gershgorin bound max over rows of sum |D^-1 A| (one thread per cell).
+// symmetric positive definite), one thread per cell; conversions on the integer pipe, short reciprocals.
 template <int MB>
-__global__ void k_block_inv(int nc, const int* __restrict__ rowptr, const int* __restrict__ dpos,
-                            const float* __restrict__ aval, float* __restrict__ dinv, float* lam) {
+__global__ void k_block_inv(int nc, const int* __restrict__ dpos, const float* __restrict__ aval,
+                            float* __restrict__ dinv) {
   pdl_start();
-  float g = 0.0f;
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += gridDim.x * blockDim.x) {
     double A[MB * MB];
     const float* B = aval + (size_t)dpos[c] * MB * MB;
 #pragma unroll
-    for (int i = 0; i < MB * MB; ++i) A[i] = B[i];
+    for (int i = 0; i < MB * MB; ++i) A[i] = widen(B[i]);
 #pragma unroll
     for (int k = 0; k < MB; ++k) {
-      const double dk = 1.0 / A[k * MB + k];
+      const double dk = fast_rcp(A[k * MB + k]);
       A[k * MB + k] = 1.0;
 #pragma unroll
       for (int j = 0; j < MB; ++j) A[k * MB + j] *= dk;
@@ -318,20 +398,30 @@ __global__ void k_block_inv(int nc, const int* __restrict__ rowptr, const int* _
         for (int j = 0; j < MB; ++j) A[i * MB + j] -= f * A[k * MB + j];
       }
     }
-    float Di[MB * MB];
 #pragma unroll
-    for (int i = 0; i < MB * MB; ++i) {
-      Di[i] = (float)A[i];
-      dinv[(size_t)c * MB * MB + i] = Di[i];
-    }
-    float rs[MB];
+    for (int i = 0; i < MB * MB; ++i) dinv[(size_t)c * MB * MB + i] = narrow(A[i]);
+  }
+}
+
+// The Gershgorin bound max over rows of sum |D^-1 A| of a block level, one warp per cell, a lane per block of its row (a
+// thread per cell walked its 27 blocks one memory round trip after another, with the inverse: 37 us on any level).
+template <int MB>
+__global__ void k_block_bound(int nc, const int* __restrict__ rowptr, const float* __restrict__ aval,
+                              const float* __restrict__ dinv, float* lam) {
+  pdl_start();
+  const int lane = threadIdx.x & 31;
+  float g = 0.0f;
+  for (int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < nc; c += (gridDim.x * blockDim.x) >> 5) {
+    float Di[MB * MB], rs[MB];
+#pragma unroll
+    for (int u = 0; u < MB; ++u) ld_seg<MB>(dinv + ((size_t)c * MB + u) * MB, *(float(*)[MB])(Di + u * MB));
 #pragma unroll
     for (int u = 0; u < MB; ++u) rs[u] = 0.0f;
-    for (int q = rowptr[c]; q < rowptr[c + 1]; ++q) {
-      const float* Bq = aval + (size_t)q * MB * MB;
+    const int q1 = rowptr[c + 1];
+    for (int q = rowptr[c] + lane; q < q1; q += 32) {
       float Bl[MB * MB];
 #pragma unroll
-      for (int i = 0; i < MB * MB; ++i) Bl[i] = Bq[i];
+      for (int u = 0; u < MB; ++u) ld_seg<MB>(aval + ((size_t)q * MB + u) * MB, *(float(*)[MB])(Bl + u * MB));
 #pragma unroll
       for (int u = 0; u < MB; ++u)
 #pragma unroll
@@ -343,11 +433,9 @@ __global__ void k_block_inv(int nc, const int* __restrict__ rowptr, const int* _
         }
     }
 #pragma unroll
-    for (int u = 0; u < MB; ++u) g = fmaxf(g, rs[u]);
+    for (int u = 0; u < MB; ++u) g = fmaxf(g, warp_sum(rs[u]));
   }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) g = fmaxf(g, __shfl_down_sync(0xffffffffu, g, off));
-  if ((threadIdx.x & 31) == 0) atomic_max_pos(lam, g);
+  if (lane == 0) atomic_max_pos(lam, g);
 }
 
 // Chebyshev coefficient table of every level and step from the Gershgorin bounds (one thread per entry).
@@ -362,46 +450,77 @@ __global__ void k_cheb_table(const float* __restrict__ lam, float* __restrict__ 
   tab[2 * t + 1] = c2;
 }
 
-// Dense inverse of the coarsest level (n = nc * mb <= kMgMaxCoarse) in one block: the blocks assembled into an
-// n x n FP64 matrix in shared memory, in-place Gauss-Jordan (symmetric positive definite, no pivoting).
-__global__ void k_coarse_inv(int nc, int mb, const int* __restrict__ rowptr, const int* __restrict__ col,
-                             const float* __restrict__ aval, float* __restrict__ cinv) {
+// Dense inverse of the coarsest level (n = nc * mb <= kMgMaxCoarse) by one cluster of kInvCtas blocks: FP64 Gauss-Jordan
+// (symmetric positive definite, no pivoting), column j in block j % kInvCtas. Step k needs column k of its owner; the
+// owner updates column k + 1 first, publishes a copy of it with its pivot's reciprocal in its shared memory and arrives
+// at the cluster's barrier before the rest of its update, which hides the barrier. n^3 FP64 multiply-adds on one SM take
+// 0.5 ms at n = 128 (1.16 ms with a step's serial part), a cluster of eight a tenth of that.
+constexpr int kInvCtas = 8;
+constexpr int kInvCols = kMgMaxCoarse / kInvCtas;
+constexpr int kInvThreads = 256;
+__device__ __forceinline__ double ld_cluster(const double* p, unsigned rank) {   // p in block `rank`'s shared memory
+  unsigned a;
+  double v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+  return v;
+}
+__global__ void __cluster_dims__(kInvCtas, 1, 1) __launch_bounds__(kInvThreads)
+    k_coarse_inv(int nc, int mb, const int* __restrict__ rowptr, const int* __restrict__ col,
+                 const float* __restrict__ aval, float* __restrict__ cinv) {
   pdl_start();
-  extern __shared__ double S[];   // n * n + n
-  const int n = nc * mb;
-  double* colk = S + n * n;
-  __shared__ double piv;
-  for (int i = threadIdx.x; i < n * n; i += blockDim.x) S[i] = 0.0;
+  __shared__ double S[kInvCols][kMgMaxCoarse];        // own columns
+  __shared__ double pub[2][kMgMaxCoarse + 1];         // a published column and its pivot's reciprocal
+  __shared__ double f[kMgMaxCoarse + 1], p[kInvCols]; // the step's column, and the pivot row on the own columns
+  const int n = nc * mb, rank = (int)blockIdx.x, tid = threadIdx.x;
+  for (int i = tid; i < kInvCols * kMgMaxCoarse; i += kInvThreads) S[i / kMgMaxCoarse][i % kMgMaxCoarse] = 0.0;
   __syncthreads();
-  for (int c = 0; c < nc; ++c)
-    for (int q = rowptr[c]; q < rowptr[c + 1]; ++q) {
-      const int d = col[q];
-      for (int idx = threadIdx.x; idx < mb * mb; idx += blockDim.x) {
-        const int u = idx / mb, v = idx % mb;
-        S[(c * mb + u) * n + d * mb + v] = aval[(size_t)q * mb * mb + idx];
+  for (int c = tid >> 5; c < nc; c += kInvThreads / 32)   // a warp per block row
+    for (int q = rowptr[c]; q < rowptr[c + 1]; ++q)
+      for (int idx = tid & 31; idx < mb * mb; idx += 32) {
+        const int j = col[q] * mb + idx % mb;
+        if (j % kInvCtas == rank) S[j / kInvCtas][c * mb + idx / mb] = (double)aval[(size_t)q * mb * mb + idx];
       }
-    }
   __syncthreads();
-  for (int k = 0; k < n; ++k) {
-    if (threadIdx.x == 0) {
-      piv = 1.0 / S[k * n + k];
-      S[k * n + k] = 1.0;
+  auto publish = [&](int k) {   // by the owner of column k (none beyond n), whose column is up to date in the whole block
+    if (k < n && k % kInvCtas == rank) {
+      for (int i = tid; i < n; i += kInvThreads) pub[k & 1][i] = S[k / kInvCtas][i];
+      if (tid == 0) pub[k & 1][kMgMaxCoarse] = fast_rcp(S[k / kInvCtas][k]);
     }
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  };
+  // one column's update: S_ij -= f_i p_j, row k becomes p, column k -f piv
+  auto update = [&](int jl, int k, int i) {
+    const int j = jl * kInvCtas + rank;
+    const double pj = p[jl];
+    if (j == k) S[jl][i] = i == k ? f[kMgMaxCoarse] : -f[i] * f[kMgMaxCoarse];
+    else S[jl][i] = i == k ? pj : fma(-f[i], pj, S[jl][i]);
+  };
+  publish(0);
+  for (int k = 0; k < n; ++k) {
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    for (int i = tid; i <= kMgMaxCoarse; i += kInvThreads)
+      if (i < n || i == kMgMaxCoarse) f[i] = ld_cluster(&pub[k & 1][i], (unsigned)(k % kInvCtas));
     __syncthreads();
-    for (int j = threadIdx.x; j < n; j += blockDim.x) S[k * n + j] *= piv;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) colk[i] = i == k ? 0.0 : S[i * n + k];
+    if (tid < kInvCols) p[tid] = S[tid][k] * f[kMgMaxCoarse];
     __syncthreads();
-    for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
-      const int i = idx / n, j = idx % n;
-      if (i == k) continue;
-      if (j == k)
-        S[idx] = -colk[i] * S[k * n + k];
-      else
-        S[idx] -= colk[i] * S[k * n + j];
+    const int next = k + 1 < n && (k + 1) % kInvCtas == rank ? (k + 1) / kInvCtas : -1;
+    if (next >= 0) {   // the same in the whole block
+      for (int i = tid; i < n; i += kInvThreads) update(next, k, i);
+      __syncthreads();
+    }
+    publish(k + 1);
+    for (int e = tid; e < kInvCols * kMgMaxCoarse; e += kInvThreads) {
+      const int jl = e / kMgMaxCoarse, i = e % kMgMaxCoarse;
+      if (i < n && jl * kInvCtas + rank < n && jl != next) update(jl, k, i);
     }
     __syncthreads();
   }
-  for (int i = threadIdx.x; i < n * n; i += blockDim.x) cinv[i] = (float)S[i];
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");   // nobody reads this block's memory any more
+  for (int e = tid; e < kInvCols * kMgMaxCoarse; e += kInvThreads) {
+    const int jl = e / kMgMaxCoarse, i = e % kMgMaxCoarse, j = jl * kInvCtas + rank;
+    if (i < n && j < n) cinv[(size_t)i * n + j] = (float)S[jl][i];
+  }
 }
 
 // ---------------------------------------------------------------------------------------------------------------
@@ -718,49 +837,6 @@ __global__ void k_prol(int nc, int mbf, int mb, const PT* __restrict__ Pl, const
   if (stop(done)) return;
   prol_body<PT, false>((long)blockIdx.x * blockDim.x + threadIdx.x, (long)gridDim.x * blockDim.x, nc, mbf, mb, Pl,
                        agg, e, x);
-}
-
-// MB consecutive floats from p into v: 16-byte loads when MB % 4 == 0, 8-byte loads when MB is even (the caller
-// guarantees p is aligned accordingly: every array here is its own allocation, and a block row or a cell's vector
-// segment starts at a multiple of MB floats).
-template <int MB>
-__device__ __forceinline__ void ld_seg(const float* p, float (&v)[MB]) {
-  if constexpr (MB % 4 == 0) {
-#pragma unroll
-    for (int k = 0; k < MB / 4; ++k) {
-      const float4 t = reinterpret_cast<const float4*>(p)[k];
-      v[4 * k] = t.x;
-      v[4 * k + 1] = t.y;
-      v[4 * k + 2] = t.z;
-      v[4 * k + 3] = t.w;
-    }
-  } else if constexpr (MB % 2 == 0) {
-#pragma unroll
-    for (int k = 0; k < MB / 2; ++k) {
-      const float2 t = reinterpret_cast<const float2*>(p)[k];
-      v[2 * k] = t.x;
-      v[2 * k + 1] = t.y;
-    }
-  } else {
-#pragma unroll
-    for (int k = 0; k < MB; ++k) v[k] = p[k];
-  }
-}
-
-// MB consecutive BF16 transfer entries from p, widened to float: 4-byte pair loads when MB is even.
-template <int MB>
-__device__ __forceinline__ void ld_seg(const __nv_bfloat16* p, float (&v)[MB]) {
-  if constexpr (MB % 2 == 0) {
-#pragma unroll
-    for (int k = 0; k < MB / 2; ++k) {
-      const float2 t = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(p)[k]);
-      v[2 * k] = t.x;
-      v[2 * k + 1] = t.y;
-    }
-  } else {
-#pragma unroll
-    for (int k = 0; k < MB; ++k) v[k] = __bfloat162float(p[k]);
-  }
 }
 
 // Row-parallel forms of the block-level smoothing step and residual (the per-level kernels of the V-cycle; the
@@ -1310,6 +1386,7 @@ bool mg_build_host(const FineMesh& fm, const Hierarchy& H, int levels, MgHost& M
     }
     M.mb[l] = mb;
     M.mcnt[l] = Lv.m;
+    M.padded[l] = std::any_of(Lv.m.begin(), Lv.m.end(), [&](int k) { return k < mb; });
   }
   if ((long)M.nc[levels - 1] * M.mb[levels - 1] > kMgMaxCoarse) {
     err = "multigrid preconditioner: the coarsest level has more than " + std::to_string(kMgMaxCoarse) +
@@ -1485,18 +1562,25 @@ void mg_enqueue_setup(cudaStream_t st, const MgDev& M, const FineDev& F, const M
                       const double* diagT, const double* r) {
   cudaMemsetAsync(W.lam, 0, kMgMaxLevels * sizeof(float), st);
   launchk(st, blocks_for(M.N, 4096), kT, 0, k_fine_vals, F, Tval, diagT, W.a0off, W.a0diag, W.a0dinv, W.lam);
+  int n = 2;
+  const int per = M.mb[1] == 4 ? 2 : 1;   // blocks a warp of k_asm1
   if (W.bf16) {
-    MG_MB_SWITCH(M.mb[1], launchk(st, warps_grid(M.nblk[1]), kT, 0, k_asm1<MB, __nv_bfloat16>, M.nblk[1],
+    MG_MB_SWITCH(M.mb[1], launchk(st, warps_grid((M.nblk[1] + per - 1) / per), kT, 0, k_asm1<MB, __nv_bfloat16>, M.nblk[1],
                                   (const int*)M.asm_off[1], (const int4*)M.asm_list[1],
-                                  (const __nv_bfloat16*)M.Pb[0], Tval, r, (const double*)F.dir_ups, W.aval[1]));
+                                  (const __nv_bfloat16*)M.Pb[0], (const float*)W.a0off, r, (const double*)F.dir_ups,
+                                  W.aval[1]));
   } else {
-    MG_MB_SWITCH(M.mb[1], launchk(st, warps_grid(M.nblk[1]), kT, 0, k_asm1<MB, float>, M.nblk[1],
-                                  (const int*)M.asm_off[1], (const int4*)M.asm_list[1], (const float*)M.P[0], Tval, r,
-                                  (const double*)F.dir_ups, W.aval[1]));
+    MG_MB_SWITCH(M.mb[1], launchk(st, warps_grid((M.nblk[1] + per - 1) / per), kT, 0, k_asm1<MB, float>, M.nblk[1],
+                                  (const int*)M.asm_off[1], (const int4*)M.asm_list[1], (const float*)M.P[0],
+                                  (const float*)W.a0off, r, (const double*)F.dir_ups, W.aval[1]));
   }
-  launchk(st, blocks_for(M.nc[1]), kT, 0, k_pad_diag, M.nc[1], M.mb[1], (const int*)M.dpos[1],
-          (const int*)M.mcnt[1], W.aval[1]);
-  int n = 3;
+  auto pad = [&](int l) {
+    if (!M.padded[l]) return;
+    launchk(st, blocks_for(M.nc[l]), kT, 0, k_pad_diag, M.nc[l], M.mb[l], (const int*)M.dpos[l], (const int*)M.mcnt[l],
+            W.aval[l]);
+    ++n;
+  };
+  pad(1);
   for (int l = 2; l < M.L; ++l) {
     if (W.bf16) {
       MG_MB_SWITCH(M.mb[l], launchk(st, warps_grid(M.nblk[l]), kT, 0, k_asml<MB, __nv_bfloat16>, M.nblk[l],
@@ -1507,22 +1591,21 @@ void mg_enqueue_setup(cudaStream_t st, const MgDev& M, const FineDev& F, const M
                                     (const int*)M.asm_off[l], (const int4*)M.asm_list[l], (const float*)M.P[l - 1],
                                     (const float*)W.aval[l - 1], W.aval[l]));
     }
-    launchk(st, blocks_for(M.nc[l]), kT, 0, k_pad_diag, M.nc[l], M.mb[l], (const int*)M.dpos[l],
-            (const int*)M.mcnt[l], W.aval[l]);
-    n += 2;
+    ++n;
+    pad(l);
   }
   for (int l = 1; l + 1 < M.L; ++l) {
-    MG_MB_SWITCH(M.mb[l], launchk(st, blocks_for(M.nc[l]), 128, 0, k_block_inv<MB>, M.nc[l],
-                                  (const int*)M.rowptr[l], (const int*)M.dpos[l], (const float*)W.aval[l], W.dinv[l],
-                                  W.lam + l));
-    ++n;
+    MG_MB_SWITCH(M.mb[l], launchk(st, (M.nc[l] + 31) / 32, 32, 0, k_block_inv<MB>, M.nc[l], (const int*)M.dpos[l],
+                                  (const float*)W.aval[l], W.dinv[l]));
+    MG_MB_SWITCH(M.mb[l], launchk(st, warps_grid(M.nc[l]), kT, 0, k_block_bound<MB>, M.nc[l], (const int*)M.rowptr[l],
+                                  (const float*)W.aval[l], (const float*)W.dinv[l], W.lam + l));
+    n += 2;
   }
   launchk(st, 1, 32, 0, k_cheb_table, (const float*)W.lam, W.coef);
-  ++n;
-  const int C = M.L - 1, nco = M.nc[C] * M.mb[C];
-  launchk(st, 1, 512, (size_t)(nco * nco + nco) * sizeof(double), k_coarse_inv, M.nc[C], M.mb[C],
-          (const int*)M.rowptr[C], (const int*)M.col[C], (const float*)W.aval[C], W.cinv);
-  count_launch(n + 1);
+  const int C = M.L - 1;
+  launchk(st, kInvCtas, kInvThreads, 0, k_coarse_inv, M.nc[C], M.mb[C], (const int*)M.rowptr[C], (const int*)M.col[C],
+          (const float*)W.aval[C], W.cinv);
+  count_launch(n + 2);
 }
 
 namespace {
@@ -1852,8 +1935,6 @@ cudaError_t mg_capture_apply(cudaStream_t st, const MgDev& M, const FineDev& F, 
 
 void mg_set_smem_limits() {
   static const bool once = [] {   // thread-safe one-time initialisation
-    cudaFuncSetAttribute(k_coarse_inv, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (kMgMaxCoarse * kMgMaxCoarse + kMgMaxCoarse) * (int)sizeof(double));
     cudaFuncSetAttribute(k_small<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmem);
     cudaFuncSetAttribute(k_small<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmem);
     return true;

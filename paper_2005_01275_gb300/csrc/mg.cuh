@@ -34,6 +34,7 @@ constexpr int kTailMaxCopies = 8 * kMgMaxLevels;
 struct MgHost {
   int L = 0, N = 0;
   int nc[kMgMaxLevels] = {0}, mb[kMgMaxLevels] = {0}, nblk[kMgMaxLevels] = {0};
+  int padded[kMgMaxLevels] = {0};                       // some cell has fewer modes than mb
   std::vector<int> rowptr[kMgMaxLevels], col[kMgMaxLevels], dpos[kMgMaxLevels], mcnt[kMgMaxLevels];
   std::vector<int> asm_off[kMgMaxLevels];
   std::vector<int4> asm_list[kMgMaxLevels];
@@ -45,6 +46,7 @@ struct MgHost {
 struct MgDev {
   int L = 0, N = 0;
   int nc[kMgMaxLevels] = {0}, mb[kMgMaxLevels] = {0}, nblk[kMgMaxLevels] = {0};
+  int padded[kMgMaxLevels] = {0};
   int *rowptr[kMgMaxLevels] = {nullptr}, *col[kMgMaxLevels] = {nullptr}, *dpos[kMgMaxLevels] = {nullptr},
       *mcnt[kMgMaxLevels] = {nullptr};
   int* asm_off[kMgMaxLevels] = {nullptr};
@@ -146,7 +148,7 @@ cudaError_t mg_capture_bicgstab(cudaStream_t st, const MgDev& M, const FineDev& 
                                 const double* Joff, const double* wgt, cudaGraphExec_t* out);
 cudaError_t mg_capture_apply(cudaStream_t st, const MgDev& M, const FineDev& F, MgWork& W, cudaGraphExec_t* out);
 
-// Raises the dynamic shared-memory limit of the coarsest-level inversion (once per process).
+// Raises the dynamic shared-memory limit of the small-level kernel (once per process).
 void mg_set_smem_limits();
 
 }  // namespace nlmg

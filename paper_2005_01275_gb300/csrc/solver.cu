@@ -598,6 +598,7 @@ void upload_mg(nlmg_ctx* c, int levels) {
     M.nc[l] = mh.nc[l];
     M.mb[l] = mh.mb[l];
     M.nblk[l] = mh.nblk[l];
+    M.padded[l] = mh.padded[l];
     if (l >= 1) {
       M.rowptr[l] = c->upload(mh.rowptr[l]);
       M.col[l] = c->upload(mh.col[l]);
