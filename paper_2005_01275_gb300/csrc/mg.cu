@@ -135,6 +135,9 @@ __device__ __forceinline__ bool stop(const int* done) { return done && *((volati
 // Programmatic dependent launch: wait until the preceding kernel of the stream (or graph edge) has finished and its
 // writes are visible, then let the next kernel start its launch (it waits the same way before it reads anything).
 // Without a programmatic predecessor the wait returns at once.
+// What a kernel loads before that (the matrix entries, indices and transfers of its first items) is older than its
+// predecessor: a kernel only starts once its predecessor has waited for the one before, and setup and hierarchy are
+// several kernels back. So those loads overlap the predecessor, and what is left after the wait is the vectors.
 __device__ __forceinline__ void pdl_start() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -526,56 +529,104 @@ __global__ void __cluster_dims__(kInvCtas, 1, 1) __launch_bounds__(kInvThreads)
 // ---------------------------------------------------------------------------------------------------------------
 // V-cycle kernels
 
+// The entries of a level-0 row: up to eight in registers (loaded before the wait for the first cell of a thread), the
+// rest, if any, read in the product.
+struct Row0 {
+  int nb[8];
+  float a[8];
+  int w, e;
+};
+__device__ __forceinline__ Row0 row0(const FineDev& F, const float* __restrict__ a0off, int K) {
+  Row0 R;
+  R.w = K < F.N ? F.sell_w[K >> 5] : 0;
+  R.e = K < F.N ? F.sell_off[K >> 5] + (K & 31) : 0;
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    if (j < R.w) {
+      R.nb[j] = F.nbr[R.e + 32 * j];
+      R.a[j] = a0off[R.e + 32 * j];
+    }
+  return R;
+}
+__device__ __forceinline__ float row0_ax(const FineDev& F, const float* __restrict__ a0off, const Row0& R, float ax,
+                                         const float* __restrict__ x) {
+  float xv[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    if (j < R.w) xv[j] = x[R.nb[j]];
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    if (j < R.w) ax = fmaf(R.a[j], xv[j], ax);
+  for (int j = 8; j < R.w; ++j) ax = fmaf(a0off[R.e + 32 * j], x[F.nbr[R.e + 32 * j]], ax);
+  return ax;
+}
+
 // One Chebyshev step on level 0: res = b - A x_in, d = c1 d + c2 D^-1 res, x_out = x_in + d (x_in is gathered by the
 // neighbours, so the new iterate goes to the other buffer).
-__device__ __forceinline__ float cheb0_cell(const FineDev& F, const float* __restrict__ a0off,
-                                            const float* __restrict__ a0diag, const float* __restrict__ a0dinv,
-                                            const float* __restrict__ b, const float* __restrict__ xin,
+__device__ __forceinline__ float cheb0_cell(const FineDev& F, const float* __restrict__ a0off, const Row0& R, float diag,
+                                            float dinv, const float* __restrict__ b, const float* __restrict__ xin,
                                             float* __restrict__ xout, float* __restrict__ d, float c1, float c2, int k,
                                             int K) {
-  const int w = F.sell_w[K >> 5];
-  int e = F.sell_off[K >> 5] + (K & 31);
   const float xk = xin[K];
-  float ax = a0diag[K] * xk;
-  for (int j = 0; j < w; ++j, e += 32) ax = fmaf(a0off[e], xin[F.nbr[e]], ax);
+  const float ax = row0_ax(F, a0off, R, diag * xk, xin);
   const float res = b[K] - ax;
-  const float dn = (k == 0 ? 0.0f : c1 * d[K]) + c2 * a0dinv[K] * res;
+  const float dn = (k == 0 ? 0.0f : c1 * d[K]) + c2 * dinv * res;
   d[K] = dn;
   const float xn = xk + dn;
   xout[K] = xn;
   return xn;
 }
 
-__global__ void k_cheb0(FineDev F, const float* __restrict__ a0off, const float* __restrict__ a0diag,
+__global__ void __launch_bounds__(kT, 6) k_cheb0(FineDev F, const float* __restrict__ a0off, const float* __restrict__ a0diag,
                         const float* __restrict__ a0dinv, const float* __restrict__ b, const float* __restrict__ xin,
                         float* __restrict__ xout, float* __restrict__ d, const float* __restrict__ lam, int k,
                         const int* done) {
-  pdl_start();
-  if (stop(done)) return;
+  int K = blockIdx.x * blockDim.x + threadIdx.x;
+  Row0 R = row0(F, a0off, K);
+  float dg = K < F.N ? a0diag[K] : 0.0f, di = K < F.N ? a0dinv[K] : 0.0f;
   float c1, c2;
   cheb_tab(lam, 0, k, c1, c2);
-  for (int K = blockIdx.x * blockDim.x + threadIdx.x; K < F.N; K += gridDim.x * blockDim.x)
-    (void)cheb0_cell(F, a0off, a0diag, a0dinv, b, xin, xout, d, c1, c2, k, K);
+  pdl_start();
+  if (stop(done)) return;
+  while (K < F.N) {
+    (void)cheb0_cell(F, a0off, R, dg, di, b, xin, xout, d, c1, c2, k, K);
+    K += gridDim.x * blockDim.x;
+    if (K < F.N) {
+      R = row0(F, a0off, K);
+      dg = a0diag[K];
+      di = a0dinv[K];
+    }
+  }
 }
 
 // The last Chebyshev step of level 0 (z = xout) fused with the flexible CG step length: rz_new = (r, z),
 // beta = (r, z - z_old) / rz (0 on the first step), which equals the plain rz_new / rz for a fixed linear
 // preconditioner and tolerates the FP32 rounding of the V-cycle. At most kMaxRedBlocks blocks.
-__global__ void k_cheb0_beta(FineDev F, const float* __restrict__ a0off, const float* __restrict__ a0diag,
+__global__ void __launch_bounds__(kT, 6) k_cheb0_beta(FineDev F, const float* __restrict__ a0off, const float* __restrict__ a0diag,
                              const float* __restrict__ a0dinv, const float* __restrict__ b,
                              const float* __restrict__ xin, float* __restrict__ xout, float* __restrict__ d,
                              const float* __restrict__ lam, int k, const double* __restrict__ r,
                              const float* __restrict__ zold, double* part, MgScal* sc) {
-  pdl_start();
-  if (stop(&sc->done)) return;
+  int K = blockIdx.x * blockDim.x + threadIdx.x;
+  Row0 R = row0(F, a0off, K);
+  float dg = K < F.N ? a0diag[K] : 0.0f, di = K < F.N ? a0dinv[K] : 0.0f;
   float c1, c2;
   cheb_tab(lam, 0, k, c1, c2);
+  pdl_start();
+  if (stop(&sc->done)) return;
   const bool first = sc->it == 0;
   double v[2] = {0.0, 0.0};
-  for (int K = blockIdx.x * blockDim.x + threadIdx.x; K < F.N; K += gridDim.x * blockDim.x) {
-    const float z = cheb0_cell(F, a0off, a0diag, a0dinv, b, xin, xout, d, c1, c2, k, K);
-    v[0] = fma(r[K], (double)z, v[0]);
-    if (!first) v[1] = fma(r[K], (double)zold[K], v[1]);
+  while (K < F.N) {
+    const float z = cheb0_cell(F, a0off, R, dg, di, b, xin, xout, d, c1, c2, k, K);
+    const double rK = r[K];
+    v[0] = fma(rK, widen(z), v[0]);
+    if (!first) v[1] = fma(rK, widen(zold[K]), v[1]);
+    K += gridDim.x * blockDim.x;
+    if (K < F.N) {
+      R = row0(F, a0off, K);
+      dg = a0diag[K];
+      di = a0dinv[K];
+    }
   }
   __shared__ double out[2];
   if (reduce_last<2>(v, part, &sc->cnt[1], out) && threadIdx.x == 0) {
@@ -596,41 +647,59 @@ __device__ __forceinline__ float ldv(const float* p) {
 // the row; a shuffle tree adds the slots, so every lane with component u < MB holds (A x)_u. The blocks are taken in
 // batches of RB per slot whose column indices, then matrix and vector entries, are all loaded before the first
 // product: on the small levels few warps are in flight, and a row costs two dependent memory round trips per batch
-// instead of two per block. The products are added in block order either way.
-template <int MB, bool CG>
-__device__ __forceinline__ float row_ax(int c, int lane, const int* __restrict__ rowptr, const int* __restrict__ col,
-                                        const float* __restrict__ aval, const float* x) {
-  constexpr int RB = MB >= 8 ? 2 : (MB >= 4 ? 4 : 8);
-  const int slot = lane >> 3, u = lane & 7;
-  float ax = 0.0f;
-  if (u < MB) {
-    const int q1 = rowptr[c + 1];
-    for (int qb = rowptr[c] + slot; qb < q1; qb += 4 * RB) {
-      int cq[RB];
+// instead of two per block. The products are added in block order either way. A row's first batch can be loaded ahead.
+template <int MB>
+struct RowBatch {
+  static constexpr int RB = MB >= 8 ? 2 : (MB >= 4 ? 4 : 8);
+  int cq[RB];
+  float bv[RB][MB];
+  __device__ __forceinline__ void load(int qb, int q1, int u, const int* __restrict__ col, const float* __restrict__ aval) {
 #pragma unroll
-      for (int j = 0; j < RB; ++j) cq[j] = qb + 4 * j < q1 ? col[qb + 4 * j] : -1;
-      float bv[RB][MB], xv[RB][MB];
+    for (int j = 0; j < RB; ++j) cq[j] = u < MB && qb + 4 * j < q1 ? col[qb + 4 * j] : -1;
 #pragma unroll
-      for (int j = 0; j < RB; ++j) {
-        const float* Bq = aval + (size_t)(qb + 4 * j) * MB * MB + u * MB;
-        const float* xd = x + (size_t)(cq[j] < 0 ? 0 : cq[j]) * MB;
+    for (int j = 0; j < RB; ++j) {
+      const float* Bq = aval + (size_t)(qb + 4 * j) * MB * MB + u * MB;
 #pragma unroll
-        for (int v = 0; v < MB; ++v) {
-          bv[j][v] = cq[j] >= 0 ? Bq[v] : 0.0f;
-          xv[j][v] = cq[j] >= 0 ? ldv<CG>(xd + v) : 0.0f;
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < RB; ++j)
-        if (cq[j] >= 0) {
-#pragma unroll
-          for (int v = 0; v < MB; ++v) ax = fmaf(bv[j][v], xv[j][v], ax);
-        }
+      for (int v = 0; v < MB; ++v) bv[j][v] = cq[j] >= 0 ? Bq[v] : 0.0f;
     }
   }
+};
+template <int MB, bool CG>
+__device__ __forceinline__ float row_ax(RowBatch<MB>& A, int q0, int q1, int lane, const int* __restrict__ col,
+                                        const float* __restrict__ aval, const float* x) {
+  constexpr int RB = RowBatch<MB>::RB;
+  const int slot = lane >> 3, u = lane & 7;
+  float ax = 0.0f;
+  for (int qb = q0 + slot;;) {   // A holds the batch at qb
+    float xv[RB][MB];
+#pragma unroll
+    for (int j = 0; j < RB; ++j) {
+      const float* xd = x + (size_t)(A.cq[j] < 0 ? 0 : A.cq[j]) * MB;
+#pragma unroll
+      for (int v = 0; v < MB; ++v) xv[j][v] = A.cq[j] >= 0 ? ldv<CG>(xd + v) : 0.0f;
+    }
+#pragma unroll
+    for (int j = 0; j < RB; ++j)
+      if (A.cq[j] >= 0) {
+#pragma unroll
+        for (int v = 0; v < MB; ++v) ax = fmaf(A.bv[j][v], xv[j][v], ax);
+      }
+    qb += 4 * RB;
+    if (u >= MB || qb >= q1) break;
+    A.load(qb, q1, u, col, aval);
+  }
+  __syncwarp();
   ax += __shfl_xor_sync(0xffffffffu, ax, 8);
   ax += __shfl_xor_sync(0xffffffffu, ax, 16);
   return ax;
+}
+template <int MB, bool CG>
+__device__ __forceinline__ float row_ax(int c, int lane, const int* __restrict__ rowptr, const int* __restrict__ col,
+                                        const float* __restrict__ aval, const float* x) {
+  RowBatch<MB> A;
+  const int q0 = rowptr[c], q1 = rowptr[c + 1];
+  A.load(q0 + (lane >> 3), q1, lane & 7, col, aval);
+  return row_ax<MB, CG>(A, q0, q1, lane, col, aval, x);
 }
 
 // One Chebyshev step on block level l (coefficients c1, c2 of step k): res = b - A x_in, d = c1 d + c2 D^-1 res,
@@ -762,25 +831,74 @@ __device__ __forceinline__ void coarse_solve_body(int i0, int ni, int n, const f
 __device__ __forceinline__ int gwarp() { return (blockIdx.x * blockDim.x + threadIdx.x) >> 5; }
 __device__ __forceinline__ int nwarps() { return (gridDim.x * blockDim.x) >> 5; }
 
+// One Chebyshev step of a block level, a warp per cell; the row's first batch, its place and the block inverse are loaded
+// before the wait.
 template <int MB>
 __global__ void k_chebl(int nc, const int* __restrict__ rowptr, const int* __restrict__ col,
                         const float* __restrict__ aval, const float* __restrict__ dinv, const float* __restrict__ b,
                         const float* __restrict__ xin, float* __restrict__ xout, float* __restrict__ d,
                         const float* __restrict__ lam, int l, int k, const int* done) {
-  pdl_start();
-  if (stop(done)) return;
+  const int lane = threadIdx.x & 31, u = lane & 7;
+  int c = gwarp();
+  RowBatch<MB> A;
+  int q0 = 0, q1 = 0;
+  float dv[MB];
+  auto ahead = [&]() {
+    q0 = rowptr[c];
+    q1 = rowptr[c + 1];
+    A.load(q0 + (lane >> 3), q1, u, col, aval);
+#pragma unroll
+    for (int v = 0; v < MB; ++v) dv[v] = u < MB ? dinv[(size_t)c * MB * MB + u * MB + v] : 0.0f;
+  };
+  if (c < nc) ahead();
   float c1, c2;
   cheb_tab(lam, l, k, c1, c2);
-  chebl_body<MB, false>(gwarp(), nwarps(), nc, rowptr, col, aval, dinv, b, xin, xout, d, c1, c2, k);
+  pdl_start();
+  if (stop(done)) return;
+  while (c < nc) {
+    const size_t i = (size_t)c * MB + u;
+    const bool own = lane < MB;
+    const float bi = u < MB ? b[i] : 0.0f, di = own && k > 0 ? d[i] : 0.0f, xi = own ? xin[i] : 0.0f;
+    const float res = bi - row_ax<MB, false>(A, q0, q1, lane, col, aval, xin);
+    float s = 0.0f;
+#pragma unroll
+    for (int v = 0; v < MB; ++v) {
+      const float rv = __shfl_sync(0xffffffffu, res, v);
+      if (u < MB) s = fmaf(dv[v], rv, s);
+    }
+    if (own) {
+      const float dn = (k == 0 ? 0.0f : c1 * di) + c2 * s;
+      d[i] = dn;
+      xout[i] = xi + dn;
+    }
+    c += nwarps();
+    if (c < nc) ahead();
+  }
 }
 
 template <int MB>
 __global__ void k_resl(int nc, const int* __restrict__ rowptr, const int* __restrict__ col,
                        const float* __restrict__ aval, const float* __restrict__ b, const float* __restrict__ x,
                        float* __restrict__ res, const int* done) {
+  const int lane = threadIdx.x & 31;
+  int c = gwarp();
+  RowBatch<MB> A;
+  int q0 = 0, q1 = 0;
+  auto ahead = [&]() {
+    q0 = rowptr[c];
+    q1 = rowptr[c + 1];
+    A.load(q0 + (lane >> 3), q1, lane & 7, col, aval);
+  };
+  if (c < nc) ahead();
   pdl_start();
   if (stop(done)) return;
-  resl_body<MB, false>(gwarp(), nwarps(), nc, rowptr, col, aval, b, x, res);
+  while (c < nc) {
+    const float bi = lane < MB ? b[(size_t)c * MB + lane] : 0.0f;
+    const float ax = row_ax<MB, false>(A, q0, q1, lane, col, aval, x);
+    if (lane < MB) res[(size_t)c * MB + lane] = bi - ax;
+    c += nwarps();
+    if (c < nc) ahead();
+  }
 }
 
 template <class PT>
@@ -796,17 +914,21 @@ __global__ void k_restr(int mbf, const float* __restrict__ res, const PT* __rest
 }
 
 // Level-0 residual b - A x (FP32), one thread per cell.
-__global__ void k_res0(FineDev F, const float* __restrict__ a0off, const float* __restrict__ a0diag,
+__global__ void __launch_bounds__(kT, 6) k_res0(FineDev F, const float* __restrict__ a0off, const float* __restrict__ a0diag,
                        const float* __restrict__ b, const float* __restrict__ x, float* __restrict__ res,
                        const int* done) {
+  int K = blockIdx.x * blockDim.x + threadIdx.x;
+  Row0 R = row0(F, a0off, K);
+  float dg = K < F.N ? a0diag[K] : 0.0f;
   pdl_start();
   if (stop(done)) return;
-  for (int K = blockIdx.x * blockDim.x + threadIdx.x; K < F.N; K += gridDim.x * blockDim.x) {
-    const int w = F.sell_w[K >> 5];
-    int e = F.sell_off[K >> 5] + (K & 31);
-    float ax = a0diag[K] * x[K];
-    for (int j = 0; j < w; ++j, e += 32) ax = fmaf(a0off[e], x[F.nbr[e]], ax);
-    res[K] = b[K] - ax;
+  while (K < F.N) {
+    res[K] = b[K] - row0_ax(F, a0off, R, dg * x[K], x);
+    K += gridDim.x * blockDim.x;
+    if (K < F.N) {
+      R = row0(F, a0off, K);
+      dg = a0diag[K];
+    }
   }
 }
 
@@ -817,30 +939,64 @@ __global__ void k_coarse_solve(int n, const float* __restrict__ cinv, const floa
   coarse_solve_body<false>(threadIdx.x, blockDim.x, n, cinv, b, x);
 }
 
-// x_0 += P e on level 0 (per fine cell) and on a block level (per cell and component).
+// x_0 += P e on level 0 (per fine cell) and on a block level (per cell and component); the first item's transfer row and
+// aggregate are loaded before the wait.
 template <class PT>
 __global__ void k_pro0(int N, int mb, const PT* __restrict__ P0, const int* __restrict__ agg,
                        const float* __restrict__ e, float* __restrict__ x, const int* done) {
+  int K = blockIdx.x * blockDim.x + threadIdx.x;
+  float P[kMaxM];
+  int A = 0;
+  auto ahead = [&]() {
+    A = agg[K];
+#pragma unroll
+    for (int j = 0; j < kMaxM; ++j)
+      if (j < mb) P[j] = pval(P0, (size_t)K * mb + j);
+  };
+  if (K < N) ahead();
   pdl_start();
   if (stop(done)) return;
-  for (int K = blockIdx.x * blockDim.x + threadIdx.x; K < N; K += gridDim.x * blockDim.x) {
-    const float* ea = e + (size_t)agg[K] * mb;
+  while (K < N) {
+    const float* ea = e + (size_t)A * mb;
     float s = x[K];
-    for (int j = 0; j < mb; ++j) s = fmaf(pval(P0, (size_t)K * mb + j), ea[j], s);
+#pragma unroll
+    for (int j = 0; j < kMaxM; ++j)
+      if (j < mb) s = fmaf(P[j], ea[j], s);
     x[K] = s;
+    K += gridDim.x * blockDim.x;
+    if (K < N) ahead();
   }
 }
 template <class PT>
 __global__ void k_prol(int nc, int mbf, int mb, const PT* __restrict__ Pl, const int* __restrict__ agg,
                        const float* __restrict__ e, float* __restrict__ x, const int* done) {
+  const long total = (long)nc * mbf;
+  long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  float P[kMaxM];
+  int A = 0;
+  auto ahead = [&]() {
+    A = agg[(int)(i / mbf)];
+#pragma unroll
+    for (int j = 0; j < kMaxM; ++j)
+      if (j < mb) P[j] = pval(Pl, (size_t)i * mb + j);
+  };
+  if (i < total) ahead();
   pdl_start();
   if (stop(done)) return;
-  prol_body<PT, false>((long)blockIdx.x * blockDim.x + threadIdx.x, (long)gridDim.x * blockDim.x, nc, mbf, mb, Pl,
-                       agg, e, x);
+  while (i < total) {
+    const float* ea = e + (size_t)A * mb;
+    float s = x[i];
+#pragma unroll
+    for (int j = 0; j < kMaxM; ++j)
+      if (j < mb) s = fmaf(P[j], ea[j], s);
+    x[i] = s;
+    i += (long)gridDim.x * blockDim.x;
+    if (i < total) ahead();
+  }
 }
 
 // Row-parallel forms of the block-level smoothing step and residual (the per-level kernels of the V-cycle; the
-// shared-memory tail keeps the warp-per-cell bodies above): one thread per cell component, cell c = 32 g + t / MB and
+// small levels' map is formed with the warp-per-cell bodies above): one thread per cell component, cell c = 32 g + t / MB and
 // component u = t % MB for thread t of a block of 32 MB threads, so a block holds whole cells; blocks take groups g
 // gridDim.x apart. A thread reads row u of each block of the cell's row in block order and the block column's x
 // segment, with vector loads, the column indices of kRowBatch blocks before their entries. The warp-per-cell form
@@ -980,16 +1136,14 @@ __global__ void k_restr0(const float* __restrict__ res, const PT* __restrict__ P
   }
 }
 
-// The small levels of one V-cycle in one launch of one thread block, out of shared memory: from the restriction of
-// level t-1's residual (W.d[t-1], global) to the prolongation into level t-1 (W.x[t-1][cur_prev], global), the
-// smoothing, residuals and transfers of levels t .. C-1 and the coarsest solve run as phases separated by
-// __syncthreads on copies of their matrices, transfers and vectors held in shared memory, instead of one dependent
-// kernel (a few L2 round trips) per phase. The copy-in is one pass of 16-byte loads, eight in flight per thread, from
-// the table's copy list (every source array is allocated in whole 16-byte units). The phases are the bodies of the
-// per-level kernels with the same work split per cell and the same order of operations, so the result does not depend
-// on which form ran.
+// The small levels t .. C of a V-cycle are a linear map of level t's restricted residual, so the setup forms it: block j
+// runs their smoothing, residuals, transfers and coarsest solve on the unit vector e_j, out of shared memory (phases
+// separated by __syncthreads on copies of the levels' matrices and transfers, with the bodies of the per-level kernels),
+// prolongs the result to level t-1 and writes column j of E = P B, n_t x n_(t-1) (column j contiguous). A V-cycle then
+// applies E (k_tail_apply) with every SM. Run as phases of one block in every V-cycle instead, the same levels took 25.6 us
+// of a 127 us CG iteration on 229,360 cells; forming E takes about as much once per setup.
 template <class PT>
-__global__ void __launch_bounds__(kTailThreads, 1) k_small(const MgTailTab* __restrict__ Tg, int cur_prev) {
+__global__ void __launch_bounds__(kTailThreads, 1) k_tail_cols(const MgTailTab* __restrict__ Tg, float* __restrict__ E) {
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ MgTailTab T_;   // the table itself, read by every phase
   static_assert(sizeof(MgTailTab) % 4 == 0, "table copied in words");
@@ -1037,10 +1191,19 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_small(const MgTailTab* __re
   constexpr int kDown = (kMgDegCoarse - 1) & 1, kUp = (2 * kMgDegCoarse - 1) & 1;
   const float* coef = F32(T->o_coef);
   float c1, c2 = 0.0f;
-  if (t < C) cheb_tab(coef, t, 0, c1, c2);
-  restr_body<PT, false>(w0, nw, M.mb[t - 1], T->d[t - 1], PL(t - 1), I32(T->o_choff[t - 1]), I32(T->o_ch[t - 1]),
-                        M.nc[t], M.mb[t], F32(T->o_b[t]), F32(T->o_dinv[t]), F32(T->o_x[t][0]), F32(T->o_d[t]), c2,
-                        t < C ? 1 : 0);
+  const int nt = M.nc[t] * M.mb[t], j = blockIdx.x;
+  {   // b = e_j and the first smoothing step on it
+    if (t < C) cheb_tab(coef, t, 0, c1, c2);
+    const int mb = M.mb[t];
+    for (int i = i0; i < nt; i += ni) {
+      F32(T->o_b[t])[i] = i == j ? 1.0f : 0.0f;
+      if (t < C) {
+        const float dn = i / mb == j / mb ? c2 * F32(T->o_dinv[t])[(size_t)i * mb + j % mb] : 0.0f;
+        F32(T->o_d[t])[i] = dn;
+        F32(T->o_x[t][0])[i] = dn;
+      }
+    }
+  }
   __syncthreads();
   for (int l = t; l < C; ++l) {
     const int *rp = I32(T->o_rowptr[l]), *cl = I32(T->o_col[l]);
@@ -1078,21 +1241,58 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_small(const MgTailTab* __re
       __syncthreads();
     }
   }
-  prol_body<PT, false>(i0, ni, M.nc[t - 1], M.mb[t - 1], M.mb[t], PL(t - 1), I32(T->o_agg[t - 1]),
-                       F32(T->o_x[t][t == C ? 0 : kUp]), T->x[t - 1][cur_prev]);
+  const float* xt = F32(T->o_x[t][t == C ? 0 : kUp]);
+  const int mbf = M.mb[t - 1], mb = M.mb[t], rows = M.nc[t - 1] * mbf;
+  const int* agg = I32(T->o_agg[t - 1]);
+  for (int i = i0; i < rows; i += ni) {
+    const float* ea = xt + (size_t)agg[i / mbf] * mb;
+    float s = 0.0f;
+    for (int q = 0; q < mb; ++q) s = fmaf(pval(PL(t - 1), (size_t)i * mb + q), ea[q], s);
+    E[(size_t)j * rows + i] = s;
+  }
+}
+
+// x_(t-1) += E b_t: a block takes 32 rows, each of its kApplyWarps warps an equal run of the columns (coalesced reads, all of
+// a lane's entries independent), then the warps' sums are added in order.
+constexpr int kApplyWarps = 16;
+__global__ void __launch_bounds__(32 * kApplyWarps) k_tail_apply(int rows, int nt, const float* __restrict__ E,
+                                                                 const float* __restrict__ b, float* __restrict__ x,
+                                                                 const int* done) {
+  __shared__ float s[kApplyWarps][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
+  const int j0 = nt * warp / kApplyWarps, j1 = nt * (warp + 1) / kApplyWarps;
+  float e[16];   // the run's first entries: older than the predecessor
+#pragma unroll
+  for (int q = 0; q < 16; ++q) e[q] = j0 + q < j1 && i < rows ? E[(size_t)(j0 + q) * rows + i] : 0.0f;
+  pdl_start();
+  if (stop(done)) return;
+  float a = 0.0f;
+#pragma unroll
+  for (int q = 0; q < 16; ++q)
+    if (j0 + q < j1) a = fmaf(e[q], b[j0 + q], a);
+#pragma unroll 8
+  for (int j = j0 + 16; j < j1; ++j) a = fmaf(i < rows ? E[(size_t)j * rows + i] : 0.0f, b[j], a);
+  s[warp][lane] = a;
+  __syncthreads();
+  if (warp == 0 && i < rows) {
+    float t = 0.0f;
+#pragma unroll
+    for (int w = 0; w < kApplyWarps; ++w) t += s[w][lane];
+    x[i] += t;
+  }
 }
 
 // ---------------------------------------------------------------------------------------------------------------
 // Krylov kernels (FP64 outer iteration)
 
-// A v with the frozen FP64 matrix (diagT, Tval) at cell K, v of type T.
-template <class T>
+// A v with the frozen FP64 matrix (diagT, Tval) at cell K, v in FP32 (widened on the integer pipe: as conversions the
+// seven values cost as much FP64 issue as the products).
 __device__ __forceinline__ double amul(const FineDev& F, const double* __restrict__ Tval,
-                                       const double* __restrict__ diagT, const T* __restrict__ v, int K) {
+                                       const double* __restrict__ diagT, const float* __restrict__ v, int K) {
   const int w = F.sell_w[K >> 5];
   int e = F.sell_off[K >> 5] + (K & 31);
-  double s = diagT[K] * (double)v[K];
-  for (int j = 0; j < w; ++j, e += 32) s = fma(-Tval[e], (double)v[F.nbr[e]], s);
+  double s = diagT[K] * widen(v[K]);
+  for (int j = 0; j < w; ++j, e += 32) s = fma(-Tval[e], widen(v[F.nbr[e]]), s);
   return s;
 }
 
@@ -1117,9 +1317,10 @@ __global__ void k_pcg_init(int N, const double* __restrict__ b, double bscale, c
     const double ri = bscale * b[K];
     x[K] = 0.0;
     r[K] = ri;
-    r32[K] = (float)ri;
-    first_step0(K, (float)ri, a0dinv, c2, x0, d0);
-    v[0] = fma(ri * ri, (double)a0dinv[K], v[0]);   // ||S r||^2 with S^2 = 1 / A_KK
+    const float rf = narrow(ri);
+    r32[K] = rf;
+    first_step0(K, rf, a0dinv, c2, x0, d0);
+    v[0] = fma(ri * ri, widen(a0dinv[K]), v[0]);   // ||S r||^2 with S^2 = 1 / A_KK
   }
   __shared__ double out[1];
   if (reduce_last<1>(v, part, &sc->cnt[0], out) && threadIdx.x == 0) {
@@ -1142,12 +1343,14 @@ __global__ void k_pcg_pq(FineDev F, const double* __restrict__ Tval, const doubl
   const bool first = sc->it == 0;
   double v[1] = {0.0};
   for (int K = blockIdx.x * blockDim.x + threadIdx.x; K < F.N; K += gridDim.x * blockDim.x) {
-    const double az = amul<float>(F, Tval, diagT, z, K);
-    const double pk = first ? (double)z[K] : fma(beta, p[K], (double)z[K]);
+    const double az = amul(F, Tval, diagT, z, K);
+    const float zf = z[K];
+    const double zk = widen(zf);
+    const double pk = first ? zk : fma(beta, p[K], zk);
     const double qk = first ? az : fma(beta, q[K], az);
     p[K] = pk;
     q[K] = qk;
-    zold[K] = z[K];
+    zold[K] = zf;
     v[0] = fma(pk, qk, v[0]);
   }
   __shared__ double out[1];
@@ -1174,9 +1377,10 @@ __global__ void k_pcg_update(int N, const double* __restrict__ p, const double* 
     x[K] = fma(alpha, p[K], x[K]);
     const double ri = fma(-alpha, q[K], r[K]);
     r[K] = ri;
-    r32[K] = (float)ri;
-    first_step0(K, (float)ri, a0dinv, c2, x0, d0);
-    v[0] = fma(ri * ri, (double)a0dinv[K], v[0]);   // ||S r||^2 with S^2 = 1 / A_KK
+    const float rf = narrow(ri);
+    r32[K] = rf;
+    first_step0(K, rf, a0dinv, c2, x0, d0);
+    v[0] = fma(ri * ri, widen(a0dinv[K]), v[0]);   // ||S r||^2 with S^2 = 1 / A_KK
   }
   __shared__ double out[1];
   if (reduce_last<1>(v, part, &sc->cnt[3], out) && threadIdx.x == 0) {
@@ -1191,13 +1395,12 @@ __global__ void k_pcg_update(int N, const double* __restrict__ p, const double* 
 }
 
 // ---- BiCGStab (right-preconditioned) for J dx = bscale b with the Newton Jacobian (jd diagonal, Joff SELL) ------
-template <class T>
 __device__ __forceinline__ double jmul(const FineDev& F, const double* __restrict__ Joff,
-                                       const double* __restrict__ jd, const T* __restrict__ v, int K) {
+                                       const double* __restrict__ jd, const float* __restrict__ v, int K) {
   const int w = F.sell_w[K >> 5];
   int e = F.sell_off[K >> 5] + (K & 31);
-  double s = jd[K] * (double)v[K];
-  for (int j = 0; j < w; ++j, e += 32) s = fma(Joff[e], (double)v[F.nbr[e]], s);
+  double s = jd[K] * widen(v[K]);
+  for (int j = 0; j < w; ++j, e += 32) s = fma(Joff[e], widen(v[F.nbr[e]]), s);
   return s;
 }
 
@@ -1218,8 +1421,9 @@ __global__ void k_bicg_init(int N, const double* __restrict__ b, double bscale, 
     r[K] = ri;
     rh[K] = ri;
     p[K] = ri;
-    r32[K] = (float)ri;
-    first_step0(K, (float)ri, a0dinv, c2, x0, d0);
+    const float f32 = narrow(ri);
+    r32[K] = f32;
+    first_step0(K, f32, a0dinv, c2, x0, d0);
     v[0] = fma(ri, ri, v[0]);
     v[1] = fma(ri * ri, wgt[K], v[1]);
   }
@@ -1243,8 +1447,8 @@ __global__ void k_bicg_v(FineDev F, const double* __restrict__ Joff, const doubl
   if (stop(&sc->done)) return;
   double a[1] = {0.0};
   for (int K = blockIdx.x * blockDim.x + threadIdx.x; K < F.N; K += gridDim.x * blockDim.x) {
-    pp[K] = (double)zp[K];
-    const double vk = jmul<float>(F, Joff, jd, zp, K);
+    pp[K] = widen(zp[K]);
+    const double vk = jmul(F, Joff, jd, zp, K);
     v[K] = vk;
     a[0] = fma(rh[K], vk, a[0]);
   }
@@ -1262,8 +1466,9 @@ __global__ void k_bicg_s(int N, const double* __restrict__ r, const double* __re
   for (int K = blockIdx.x * blockDim.x + threadIdx.x; K < N; K += gridDim.x * blockDim.x) {
     const double sk = fma(-alpha, v[K], r[K]);
     s[K] = sk;
-    r32[K] = (float)sk;
-    first_step0(K, (float)sk, a0dinv, c2, x0, d0);
+    const float f32 = narrow(sk);
+    r32[K] = f32;
+    first_step0(K, f32, a0dinv, c2, x0, d0);
   }
 }
 // t = J s^ (s^ = B s from the V-cycle), omega = (t, s) / (t, t).
@@ -1274,7 +1479,7 @@ __global__ void k_bicg_t(FineDev F, const double* __restrict__ Joff, const doubl
   if (stop(&sc->done)) return;
   double a[2] = {0.0, 0.0};
   for (int K = blockIdx.x * blockDim.x + threadIdx.x; K < F.N; K += gridDim.x * blockDim.x) {
-    const double tk = jmul<float>(F, Joff, jd, zs, K);
+    const double tk = jmul(F, Joff, jd, zs, K);
     t[K] = tk;
     a[0] = fma(tk, s[K], a[0]);
     a[1] = fma(tk, tk, a[1]);
@@ -1295,7 +1500,7 @@ __global__ void k_bicg_x(int N, const double* __restrict__ pp, const float* __re
   const double alpha = sc->alpha, omega = sc->omega;
   double a[2] = {0.0, 0.0};
   for (int K = blockIdx.x * blockDim.x + threadIdx.x; K < N; K += gridDim.x * blockDim.x) {
-    x[K] = fma(omega, (double)zs[K], fma(alpha, pp[K], x[K]));
+    x[K] = fma(omega, widen(zs[K]), fma(alpha, pp[K], x[K]));
     const double rk = fma(-omega, t[K], s[K]);
     r[K] = rk;
     a[0] = fma(rh[K], rk, a[0]);
@@ -1328,8 +1533,9 @@ __global__ void k_bicg_p(int N, const double* __restrict__ r, const double* __re
   for (int K = blockIdx.x * blockDim.x + threadIdx.x; K < N; K += gridDim.x * blockDim.x) {
     const double pk = fma(beta, fma(-omega, v[K], p[K]), r[K]);
     p[K] = pk;
-    r32[K] = (float)pk;
-    first_step0(K, (float)pk, a0dinv, c2, x0, d0);
+    const float f32 = narrow(pk);
+    r32[K] = f32;
+    first_step0(K, f32, a0dinv, c2, x0, d0);
   }
 }
 
@@ -1341,13 +1547,14 @@ __global__ void k_apply_in(int N, const double* __restrict__ b, float* __restric
   float c1, c2;
   cheb_tab(lam, 0, 0, c1, c2);
   for (int K = blockIdx.x * blockDim.x + threadIdx.x; K < N; K += gridDim.x * blockDim.x) {
-    r32[K] = (float)b[K];
-    first_step0(K, (float)b[K], a0dinv, c2, x0, d0);
+    const float f32 = narrow(b[K]);
+    r32[K] = f32;
+    first_step0(K, f32, a0dinv, c2, x0, d0);
   }
 }
 __global__ void k_apply_out(int N, const float* __restrict__ z, double* __restrict__ out) {
   pdl_start();
-  for (int K = blockIdx.x * blockDim.x + threadIdx.x; K < N; K += gridDim.x * blockDim.x) out[K] = (double)z[K];
+  for (int K = blockIdx.x * blockDim.x + threadIdx.x; K < N; K += gridDim.x * blockDim.x) out[K] = widen(z[K]);
 }
 
 }  // namespace
@@ -1605,6 +1812,13 @@ void mg_enqueue_setup(cudaStream_t st, const MgDev& M, const FineDev& F, const M
   const int C = M.L - 1;
   launchk(st, kInvCtas, kInvThreads, 0, k_coarse_inv, M.nc[C], M.mb[C], (const int*)M.rowptr[C], (const int*)M.col[C],
           (const float*)W.aval[C], W.cinv);
+  const int t = mg_tail_level(M);
+  if (t > 0) {
+    const int nt = M.nc[t] * M.mb[t];
+    if (W.bf16) launchk(st, nt, kTailThreads, W.tail_smem, k_tail_cols<__nv_bfloat16>, (const MgTailTab*)W.tail, W.tailE);
+    else launchk(st, nt, kTailThreads, W.tail_smem, k_tail_cols<float>, (const MgTailTab*)W.tail, W.tailE);
+    ++n;
+  }
   count_launch(n + 2);
 }
 
@@ -1648,7 +1862,7 @@ size_t small_layout(const MgDev& M, int t, MgTailTab* T) {
 int mg_tail_level(const MgDev& M) {
   const int C = M.L - 1;
   for (int l = 2; l <= C; ++l)
-    if (M.nc[l] <= kTailMaxCells && small_layout(M, l, nullptr) <= kTailSmem) return l;
+    if (M.nc[l] * M.mb[l] <= kTailMaxUnknowns && small_layout(M, l, nullptr) <= kTailSmem) return l;
   return 0;
 }
 
@@ -1656,11 +1870,6 @@ void mg_fill_tail(cudaStream_t st, const MgDev& M, MgWork& W) {
   MgTailTab h;
   h.M = M;
   h.t = mg_tail_level(M);
-  for (int l = 0; l < kMgMaxLevels; ++l) {
-    h.d[l] = W.d[l];
-    h.x[l][0] = W.x[l][0];
-    h.x[l][1] = W.x[l][1];
-  }
   W.tail_smem = 0;
   if (h.t > 0) {
     const int t = h.t, C = M.L - 1;
@@ -1701,27 +1910,8 @@ void mg_fill_tail(cudaStream_t st, const MgDev& M, MgWork& W) {
   cudaMemcpyAsync(W.tail, &h, sizeof(MgTailTab), cudaMemcpyHostToDevice, st);
 }
 
-namespace {
-
-template <class PT>
-void launch_small(cudaStream_t st, const MgWork& W, int cur_prev) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(1);
-  cfg.blockDim = dim3(kTailThreads);
-  cfg.dynamicSmemBytes = W.tail_smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, k_small<PT>, (const MgTailTab*)W.tail, cur_prev);
-}
-
-}  // namespace
-
 // The V-cycle after the fused first step of level 0 (x[0][0], d[0] set from b[0]); returns the index of the level-0
-// buffer that holds z. Levels from mg_tail_level on run in one launch of k_small.
+// buffer that holds z. Levels from mg_tail_level on are one precomputed map (k_tail_cols).
 int mg_enqueue_vcycle(cudaStream_t st, const MgDev& M, const FineDev& F, const MgWork& W, const int* flag,
                       bool cg_beta) {
   const int L = M.L, C = L - 1;
@@ -1755,7 +1945,7 @@ int mg_enqueue_vcycle(cudaStream_t st, const MgDev& M, const FineDev& F, const M
       cur[l] ^= 1;
     }
     res_level(st, M, W, l, cur[l], flag);
-    if (l == top) break;   // the tail restricts from here
+    if (l == top) break;
     if (W.bf16)
       launchk(st, warps_grid(M.nc[l + 1]), kT, 0, k_restr<__nv_bfloat16>, M.mb[l], (const float*)W.d[l],
               (const __nv_bfloat16*)M.Pb[l], (const int*)M.ch_off[l], (const int*)M.ch[l], M.nc[l + 1],
@@ -1767,11 +1957,19 @@ int mg_enqueue_vcycle(cudaStream_t st, const MgDev& M, const FineDev& F, const M
               W.b[l + 1], (const float*)W.dinv[l + 1], W.x[l + 1][0], W.d[l + 1], (const float*)W.coef, l + 1,
               l + 1 < C ? 1 : 0, flag);
   }
-  if (tl > 0) {
+  if (tl > 0) {   // restriction to level tl, then the small levels' map back to level tl - 1
+    const int nt = M.nc[tl] * M.mb[tl], rows = M.nc[tl - 1] * M.mb[tl - 1];
     if (W.bf16)
-      launch_small<__nv_bfloat16>(st, W, cur[tl - 1]);
+      launchk(st, warps_grid(M.nc[tl]), kT, 0, k_restr<__nv_bfloat16>, M.mb[tl - 1], (const float*)W.d[tl - 1],
+              (const __nv_bfloat16*)M.Pb[tl - 1], (const int*)M.ch_off[tl - 1], (const int*)M.ch[tl - 1], M.nc[tl],
+              M.mb[tl], W.b[tl], (const float*)nullptr, (float*)nullptr, (float*)nullptr, (const float*)W.coef, tl, 0,
+              flag);
     else
-      launch_small<float>(st, W, cur[tl - 1]);
+      launchk(st, warps_grid(M.nc[tl]), kT, 0, k_restr<float>, M.mb[tl - 1], (const float*)W.d[tl - 1],
+              (const float*)M.P[tl - 1], (const int*)M.ch_off[tl - 1], (const int*)M.ch[tl - 1], M.nc[tl], M.mb[tl],
+              W.b[tl], (const float*)nullptr, (float*)nullptr, (float*)nullptr, (const float*)W.coef, tl, 0, flag);
+    launchk(st, (rows + 31) / 32, 32 * kApplyWarps, 0, k_tail_apply, rows, nt, (const float*)W.tailE,
+            (const float*)W.b[tl], W.x[tl - 1][cur[tl - 1]], flag);
   } else {
     launchk(st, 1, kMgMaxCoarse, 0, k_coarse_solve, M.nc[C] * M.mb[C], (const float*)W.cinv, (const float*)W.b[C],
             W.x[C][0], flag);
@@ -1819,9 +2017,9 @@ int mg_vcycle_kernels(const MgDev& M) {
   const int level0 = (kMgDegFine - 1) + 2 + 1 + kMgDegFine;   // smoothing, residual, restriction, prolongation
   if (tl == 0) return level0 + (C - 1) * (kMgDegCoarse + 1) + 1 + (C - 1) * (1 + kMgDegCoarse);
   // levels 1 .. tl-1 run their own kernels: down smoothing and residual, the restrictions between them, and on the
-  // way up the prolongations between them and the smoothing; the tail is one more
+  // way up the prolongations between them and the smoothing; the tail is two more (restriction, map)
   const int own = tl - 1;
-  return level0 + 2 * own * kMgDegCoarse + 2 * (own - 1) + 1;
+  return level0 + 2 * own * kMgDegCoarse + 2 * (own - 1) + 2;
 }
 
 namespace {
@@ -1935,8 +2133,8 @@ cudaError_t mg_capture_apply(cudaStream_t st, const MgDev& M, const FineDev& F, 
 
 void mg_set_smem_limits() {
   static const bool once = [] {   // thread-safe one-time initialisation
-    cudaFuncSetAttribute(k_small<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmem);
-    cudaFuncSetAttribute(k_small<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmem);
+    cudaFuncSetAttribute(k_tail_cols<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmem);
+    cudaFuncSetAttribute(k_tail_cols<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmem);
     return true;
   }();
   (void)once;

@@ -25,8 +25,8 @@ constexpr int kMgDegFine = 2;       // Chebyshev steps before and after the coar
 constexpr int kMgDegCoarse = 2;     // the same on levels 1 .. L-2
 constexpr double kMgAlpha = 4.0;    // Chebyshev interval [lam / alpha, lam]
 constexpr int kMgMaxDeg = 4;        // Chebyshev steps per smoothing at most (coefficient table size)
-constexpr int kTailThreads = 1024;  // threads of the small-level kernel (k_small, one block)
-constexpr int kTailMaxCells = 1024; // it starts at the first level l >= 2 with at most this many cells ...
+constexpr int kTailThreads = 1024;  // threads of a block of the small levels' setup (k_tail_cols)
+constexpr int kTailMaxUnknowns = 512;   // the small levels start at the first l >= 2 with at most this many unknowns ...
 constexpr size_t kTailSmem = 200 * 1024;   // ... whose data from there on fit this much shared memory
 constexpr int kTailMaxCopies = 8 * kMgMaxLevels;
 
@@ -63,17 +63,16 @@ struct MgScal {
   unsigned cnt[8];   // arrival counters of the reductions (each reset by its last block)
 };
 
-// One contiguous source array of the small-level kernel's copy-in: 16-byte chunks c0 .. to shared byte offset dst.
+// One contiguous source array of the small levels' copy-in: 16-byte chunks c0 .. to shared byte offset dst.
 struct MgTailCopy {
   const void* src;
   unsigned dst, c0;
 };
 
-// What the small-level kernel reads, as one device-resident table per context: the level data, its shared-memory
+// What the small levels' setup reads, as one device-resident table per context: the level data, its shared-memory
 // layout (byte offsets) and copy list (index 0 with FP32 transfers, 1 with BF16).
 struct MgTailTab {
   MgDev M;
-  float *d[kMgMaxLevels] = {nullptr}, *x[kMgMaxLevels][2] = {{nullptr}};   // global vectors (level t-1 is used)
   int t = 0;
   unsigned o_P[kMgMaxLevels] = {0}, o_choff[kMgMaxLevels] = {0}, o_ch[kMgMaxLevels] = {0}, o_agg[kMgMaxLevels] = {0};
   unsigned o_rowptr[kMgMaxLevels] = {0}, o_col[kMgMaxLevels] = {0}, o_aval[kMgMaxLevels] = {0},
@@ -99,11 +98,12 @@ struct MgWork {
   MgScal* sc = nullptr;
   MgScal* h_sc = nullptr;                                // pinned copy
   cudaGraphExec_t g_pcg[2] = {nullptr, nullptr}, g_bicg[2] = {nullptr, nullptr}, g_apply = nullptr;
-  MgTailTab* tail = nullptr;   // device copy for the small-level kernel (mg_fill_tail)
+  MgTailTab* tail = nullptr;   // device copy for the small levels' setup (mg_fill_tail)
+  float* tailE = nullptr;      // their map: n_t columns of level t-1's length
   size_t tail_smem = 0;        // its dynamic shared memory
   int bf16 = 0;            // transfers in BF16 (FP32 accumulation) in the setup and V-cycle enqueued next
   int graphs_bf16 = -1;    // the transfer type the captured graphs use (-1: none captured)
-  int grid0 = 4096;        // blocks of the level-0 streaming kernels: one full wave, SMs x 8 blocks of 256 threads
+  int grid0 = 4096;        // blocks of the level-0 streaming kernels: one full wave, SMs x 6 blocks of 256 threads
   int row_cells = 16384;   // block levels with at least this many cells run the row-parallel kernels
   int graphs_row_cells = -1;   // the row_cells the captured graphs use (-1: none captured)
 };
@@ -132,8 +132,8 @@ int mg_enqueue_vcycle(cudaStream_t st, const MgDev& M, const FineDev& F, const M
 // W.tail_smem. Every array it lists must be allocated in whole 16-byte units.
 void mg_fill_tail(cudaStream_t st, const MgDev& M, MgWork& W);
 
-// First level the small-level kernel takes over (levels t .. L-1 and the transfers to and from t-1 in one launch of
-// one thread block, out of shared memory), or 0 if the V-cycle runs one kernel per phase throughout.
+// First of the small levels (t .. L-1, whose part of the V-cycle is one precomputed map from level t's residual to level
+// t-1's correction), or 0 if the V-cycle runs one kernel per phase throughout.
 int mg_tail_level(const MgDev& M);
 
 // Kernels in one V-cycle after its fused first step (for the launch counts of graph replays).
@@ -148,7 +148,7 @@ cudaError_t mg_capture_bicgstab(cudaStream_t st, const MgDev& M, const FineDev& 
                                 const double* Joff, const double* wgt, cudaGraphExec_t* out);
 cudaError_t mg_capture_apply(cudaStream_t st, const MgDev& M, const FineDev& F, MgWork& W, cudaGraphExec_t* out);
 
-// Raises the dynamic shared-memory limit of the small-level kernel (once per process).
+// Raises the dynamic shared-memory limit of the small levels' setup (once per process).
 void mg_set_smem_limits();
 
 }  // namespace nlmg

@@ -1193,7 +1193,7 @@ void alloc_mg(nlmg_ctx* c) {
     int dev = 0, sms = 0;
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    W.grid0 = std::max(1, sms) * 8;   // the level-0 kernels use at most 32 registers: 8 blocks of 256 per SM
+    W.grid0 = std::max(1, sms) * 6;   // the level-0 kernels are compiled for 6 blocks of 256 per SM
   }
   W.a0off = c->dalloc<float>(c->F.nnz);
   W.a0diag = c->dalloc<float>(N);
@@ -1220,6 +1220,7 @@ void alloc_mg(nlmg_ctx* c) {
   W.sc = c->dalloc<MgScal>(1);
   CK(cudaMemsetAsync(W.sc, 0, sizeof(MgScal), c->st));
   CK(cudaMallocHost(&W.h_sc, sizeof(MgScal)));
+  if (const int t = mg_tail_level(M)) W.tailE = c->dalloc<float>((size_t)M.nc[t] * M.mb[t] * M.nc[t - 1] * M.mb[t - 1]);
   W.tail = c->dalloc<MgTailTab>(1);
   mg_fill_tail(c->st, M, W);
   CK(cudaGetLastError());
