@@ -774,14 +774,20 @@ cudaError_t launch_coarse_step(cudaStream_t st, const LevelDev& L, const double*
   }();
   (void)once;
   const int sms = coop_sms(gs.sm_cap);
+  // A small level runs as one cluster of up to eight blocks, whose barrier costs a quarter of the grid's: worth it while
+  // the CG's FP64 work on eight SMs (row entries and 13 operations a lambda, 19 clocks a warp operation) stays below
+  // about 3,500 clocks.
+  const bool small = (long)L.nlam * (L.hs_wmax + 13) <= 48000;
+  const int most = small ? std::min(sms, kClusterBlocks) : sms;
   // lanes per lambda: as many as leave one warp of rows per sub-partition (four per SM)
   int gsz = 4;
-  while (gsz > 1 && (long)L.nlam * gsz > 128L * sms) gsz /= 2;
+  while (gsz > 1 && (long)L.nlam * gsz > 128L * most) gsz /= 2;
   // blocks: four warps' worth of the level's largest item count each
   long items = (long)L.nlam * gsz;
   for (long v : {(long)L.nif, (long)L.nyl, (long)L.np, (long)L.nflux + L.np, (long)L.nc})
     if (v > items) items = v;
-  const int grid = (int)std::max(1L, std::min((long)sms, (items + 127) / 128));
+  int grid = (int)std::max(1L, std::min((long)most, (items + 127) / 128));
+  gs.cluster = cluster_grid(grid, sms) ? 1 : 0;
   // form: registers when every lambda gets lanes in at most kMaxU passes of the grid (kept with its entries in shared
   // memory when they fit, else streamed, one lane a row), else memory; two synchronisations when a tight solve is
   // asked for
@@ -805,7 +811,7 @@ cudaError_t launch_coarse_step(cudaStream_t st, const LevelDev& L, const double*
   const void* fn = fns[U - 1];
   void* args[] = {(void*)&L, (void*)&Hc, (void*)&Sinv, (void*)&B, (void*)&P, (void*)&partial, (void*)&gs,
                   (void*)&form, (void*)&gsz, (void*)&staged, (void*)&res};
-  return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kCThreads), args, (size_t)staged * 12, st);
+  return launch_persistent(fn, grid, kCThreads, args, (size_t)staged * 12, gs.cluster != 0, st);
 }
 
 }  // namespace nlmg

@@ -545,10 +545,15 @@ __global__ void __launch_bounds__(kFThreads, 1) kp_fine_bicgstab_reg(FineDev F, 
 // block (one per sub-partition) before a second block's worth, then more warps, then more slices a warp.
 struct FShape {
   int grid, warps, R;   // R: slices a warp
+  bool cluster;
 };
 FShape fine_shape(const FineDev& F, int sm_cap) {
   FShape s;
   s.grid = std::max(1, std::min(coop_sms(sm_cap), (F.nslice + 3) / 4));
+  // up to 64 slices: one cluster (an iteration's 14 FP64 operations of eight slices an SM take 2.1k clocks, its barrier
+  // saves more)
+  if (F.nslice <= 64) s.grid = std::min(s.grid, kClusterBlocks);
+  s.cluster = cluster_grid(s.grid, coop_sms(sm_cap));
   const int per = (F.nslice + s.grid - 1) / s.grid;
   s.warps = std::max(1, std::min(kFWarps, per));
   s.R = (per + s.warps - 1) / s.warps;
@@ -571,12 +576,13 @@ cudaError_t launch_cg(cudaStream_t st, const FShape& s, const FineDev& F, const 
   }();
   (void)once;
   const size_t eb = sizeof(T) + sizeof(int);
+  gs.cluster = s.cluster ? 1 : 0;
   int staged = staged_entries(F, s, eb);
   if (!staged) launch_scale_sell<T>(st, F, Tval, sdiag, Ts);
   void* args[] = {(void*)&F, (void*)&Tval, (void*)&Ts, (void*)&sdiag, (void*)&b, (void*)&bscale, (void*)&dx, (void*)&B,
                   (void*)&partial, (void*)&gs, (void*)&tol, (void*)&maxit, (void*)&replace, (void*)&staged, (void*)&res};
-  return cudaLaunchCooperativeKernel(fn, dim3(s.grid), dim3(32 * (s.warps + 1)), args,
-                                     staged ? (size_t)staged * eb + (size_t)s.warps * s.R * 32 * sizeof(T) : 0, st);
+  return launch_persistent(fn, s.grid, 32 * (s.warps + 1), args,
+                           staged ? (size_t)staged * eb + (size_t)s.warps * s.R * 32 * sizeof(T) : 0, s.cluster, st);
 }
 
 template <int R>
@@ -589,6 +595,7 @@ cudaError_t launch_bicg(cudaStream_t st, const FShape& s, const FineDev& F, cons
     return true;
   }();
   (void)once;
+  gs.cluster = s.cluster ? 1 : 0;
   const size_t own = (size_t)3 * R * 32 * (s.warps + 1) * sizeof(double);
   int staged = staged_entries(F, s, sizeof(double) + sizeof(int), own);
   if (!staged) launch_scale_sell<double>(st, F, Joff, S, Js);
@@ -596,8 +603,8 @@ cudaError_t launch_bicg(cudaStream_t st, const FShape& s, const FineDev& F, cons
   void* args[] = {(void*)&F, (void*)&Joff, (void*)&Js, (void*)&jdiag, (void*)&D, (void*)&S, (void*)&b, (void*)&bscale,
                   (void*)&dx, (void*)&pg, (void*)&sg, (void*)&partial, (void*)&gs, (void*)&tol, (void*)&maxit,
                   (void*)&staged, (void*)&res};
-  return cudaLaunchCooperativeKernel(fn, dim3(s.grid), dim3(32 * (s.warps + 1)), args,
-                                     own + (staged ? (size_t)staged * 12 + (size_t)s.warps * s.R * 32 * 8 : 0), st);
+  return launch_persistent(fn, s.grid, 32 * (s.warps + 1), args,
+                           own + (staged ? (size_t)staged * 12 + (size_t)s.warps * s.R * 32 * 8 : 0), s.cluster, st);
 }
 
 }  // namespace

@@ -353,6 +353,32 @@ int coop_grid(const void* fn, int n_items, int sm_cap) {
 
 }  // namespace
 
+bool cluster_grid(int& grid, int sms) {
+  if (grid > kClusterBlocks) return false;
+  int g = 1;
+  while (g < grid) g *= 2;
+  if (g > sms) return false;
+  grid = g;
+  return true;
+}
+
+cudaError_t launch_persistent(const void* fn, int grid, int threads, void** args, size_t smem, bool cluster,
+                              cudaStream_t st) {
+  if (!cluster) return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(threads), args, smem, st);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = grid;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelExC(&cfg, fn, args);
+}
+
 int coop_sms(int sm_cap) {
   static const int sms = [] {
     int dev = 0, n = 0;

@@ -20,7 +20,16 @@ struct GridSync {
   unsigned* count;   // barrier arrival counter (0 at launch); own 128-byte line
   int* err;          // set when a wait gives up
   int sm_cap;        // host side: at most this many SMs for the launch (0 = all)
+  int cluster = 0;   // the grid is one thread-block cluster (set by the launch)
 };
+
+// Whether a grid of this size runs as one cluster; it is then rounded up to a power of two (within sms).
+constexpr int kClusterBlocks = 8;
+bool cluster_grid(int& grid, int sms);
+
+// Launches a persistent kernel of `grid` blocks: as one cluster if `cluster`, else cooperatively.
+cudaError_t launch_persistent(const void* fn, int grid, int threads, void** args, size_t smem, bool cluster, cudaStream_t st);
+
 
 template <class T>
 cudaError_t launch_fine_cg(cudaStream_t st, const FineDev& F, const T* Ts, const double* sdiag, const double* b,

@@ -133,6 +133,12 @@ struct Grid {
   unsigned phase = 0u;   // the counter's top bit after the last barrier (0 at launch)
 };
 
+// A grid of at most kClusterBlocks blocks is launched as one thread-block cluster (gs.cluster), whose hardware barrier takes
+// the place of the counter: it orders the same writes at cluster scope, needs no polling and cannot be left waiting by a
+// block that was never scheduled.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
 // One arrival and the bounded wait for all others, by one thread: every block adds 1 to gs.count except block 0, which
 // adds 2^31 - (gridDim.x - 1), so the counter's top bit flips exactly when the last block arrives and its low bits
 // return to 0 (barriers follow one another without a reset). The arrival is a release without a return value, the
@@ -154,6 +160,11 @@ __device__ __forceinline__ bool grid_wait(Grid& g, unsigned long long spin_limit
 
 // Bounded grid barrier: thread 0 arrives after __syncthreads (its release covers the block's earlier writes).
 __device__ __forceinline__ bool grid_barrier(Grid& g, unsigned long long spin_limit = kSpinLimit) {
+  if (g.gs.cluster) {
+    cluster_arrive();
+    cluster_wait();
+    return true;
+  }
   __shared__ int ok;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -210,14 +221,19 @@ __device__ __forceinline__ bool grid_sum_arrive(Grid& g, const double (&v)[NV], 
       g.partial[((g.seq - 1u) & 1u) * kPartStride + blockIdx.x * part_stride<NV>() + lane] = mine;
     }
     __syncwarp();
-    if (lane == 0) {
+    if (lane == 0 && !g.gs.cluster) {
       grid_arrive(g);
       ok = grid_wait(g, kSpinLimit) ? 1 : 0;
     }
     __syncwarp();
-  } else {
-    meanwhile();
   }
+  if (g.gs.cluster) {
+    cluster_arrive();
+    if (warp != server) meanwhile();
+    cluster_wait();
+    return true;
+  }
+  if (warp != server) meanwhile();
   g.phase ^= 0x80000000u;
   __syncthreads();
   return ok != 0;
