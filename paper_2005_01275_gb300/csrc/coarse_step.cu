@@ -446,32 +446,22 @@ __device__ bool hyb_solve_dev(const LevelDev& L, const double* __restrict__ Hc, 
     }
   }
   // recovery: sigma^c = kappa A w + B b_p, p_c = B^T w + C b_p / kappa with w = bhat - C^T lambda: four lanes per owned
-  // local flux slot, then per pressure unknown
-  QSTRIDE(y, L.nyl) {
-    const int i = y < L.nyl ? L.loc_own[y] : -1;
+  // local flux slot (rows y < nyl) and per pressure unknown (the rest)
+  QSTRIDE(y, L.nyl + L.np) {
+    const bool press = y >= L.nyl;
+    const int i = y >= L.nyl + L.np ? -1 : press ? y - L.nyl : L.loc_own[y];
     double v = 0.0;
     if (i >= 0) {
-      const int c = L.slot_cell[y];
+      const int c = press ? L.p_cell[i] : L.slot_cell[y];
       const int mc = L.m[c], lo = L.loc_off[c], nl = L.loc_off[c + 1] - lo, po = L.p_off[c];
-      const double* Su = Sinv + L.sad_off[c] + (size_t)(y - lo) * (nl + mc);
+      const double* Su = Sinv + L.sad_off[c] + (size_t)(press ? nl + i - po : y - lo) * (nl + mc);
       const double kp = __ldcg(&kapc[c]);
-      v = saddle_row(L, Su, lo, nl, po, mc, bs, bp, kp, 1.0, lane & 3) - kp * lambda_row(L, Su, c, lam, lane & 3);
+      const double w = lambda_row(L, Su, c, lam, lane & 3);
+      v = press ? saddle_row(L, Su, lo, nl, po, mc, bs, bp, 1.0, fast_rcp(kp), lane & 3) - w
+                : saddle_row(L, Su, lo, nl, po, mc, bs, bp, kp, 1.0, lane & 3) - kp * w;
     }
     v = quad_sum(v);
-    if (i >= 0 && (lane & 3) == 0) dsig[i] = v;
-  }
-  QSTRIDE(i, L.np) {
-    const bool act = i < L.np;
-    double v = 0.0;
-    if (act) {
-      const int c = L.p_cell[i];
-      const int mc = L.m[c], lo = L.loc_off[c], nl = L.loc_off[c + 1] - lo, po = L.p_off[c];
-      const double* Sr = Sinv + L.sad_off[c] + (size_t)(nl + i - po) * (nl + mc);
-      v = saddle_row(L, Sr, lo, nl, po, mc, bs, bp, 1.0, fast_rcp(__ldcg(&kapc[c])), lane & 3) -
-          lambda_row(L, Sr, c, lam, lane & 3);
-    }
-    v = quad_sum(v);
-    if (act && (lane & 3) == 0) dp[i] = v;
+    if (i >= 0 && (lane & 3) == 0) (press ? dp : dsig)[i] = v;
   }
   iters = it;
   return true;
@@ -489,6 +479,7 @@ __device__ bool hyb_solve_dev(const LevelDev& L, const double* __restrict__ Hc, 
 // Linear parts of v (read through L2: v may have been written earlier in the launch). With shift != 0 the parts
 // `acc` first take acc += shift * out (the previous step's accepted trial; the same lane owns both entries).
 __device__ void lin_parts_pass(const LevelDev& L, const double* v, LinParts out, LinParts acc, double shift) {
+  const bool fold = nonzero(shift);
   const double* vs = v;
   const double* vp = v + L.nflux;
   const int gi = threadIdx.x & 3;
@@ -509,54 +500,48 @@ __device__ void lin_parts_pass(const LevelDev& L, const double* v, LinParts out,
     }
     return m;
   };
-  QSTRIDE(y, L.nyl) {
-    const bool act = y < L.nyl;
+  // rows y < nyl: local flux slots; the rest: pressure unknowns
+  QSTRIDE(y, L.nyl + L.np) {
+    const bool act = y < L.nyl + L.np, press = y >= L.nyl;
+    const int i = y - L.nyl;
     double m = 0.0, d = 0.0;
     if (act) {
-      const int c = L.slot_cell[y];
+      const int c = press ? L.p_cell[i] : L.slot_cell[y];
       const int lo = L.loc_off[c], nl = L.loc_off[c + 1] - lo, mc = L.m[c], po = L.p_off[c];
-      const int u = y - lo;
+      const int u = press ? i - po : y - lo;
       const double* D = L.Dloc + L.dmat_off[c];
-      m = flux_row(L.Mloc + L.mat_off[c] + (size_t)u * nl, lo, nl);
-      for (int q = gi; q < mc; q += 4) d = fma(D[q * nl + u], __ldcg(&vp[po + q]), d);
+      m = flux_row(press ? D + (size_t)u * nl : L.Mloc + L.mat_off[c] + (size_t)u * nl, lo, nl);
+      if (!press)
+        for (int q = gi; q < mc; q += 4) d = fma(D[q * nl + u], __ldcg(&vp[po + q]), d);
     }
     m = quad_sum(m);
     d = quad_sum(d);
     if (act && gi == 0) {
-      if (shift != 0.0) {
-        acc.ms[y] = fma(shift, out.ms[y], acc.ms[y]);
-        acc.ds[y] = fma(shift, out.ds[y], acc.ds[y]);
+      if (press) {
+        if (fold) acc.dr[i] = fma(shift, out.dr[i], acc.dr[i]);
+        out.dr[i] = m;
+      } else {
+        if (fold) {
+          acc.ms[y] = fma(shift, out.ms[y], acc.ms[y]);
+          acc.ds[y] = fma(shift, out.ds[y], acc.ds[y]);
+        }
+        out.ms[y] = m;
+        out.ds[y] = d;
       }
-      out.ms[y] = m;
-      out.ds[y] = d;
     }
   }
-  QSTRIDE(i, L.np) {
-    const bool act = i < L.np;
-    double d = 0.0;
-    if (act) {
-      const int c = L.p_cell[i];
-      const int lo = L.loc_off[c], nl = L.loc_off[c + 1] - lo, po = L.p_off[c];
-      d = flux_row(L.Dloc + L.dmat_off[c] + (size_t)(i - po) * nl, lo, nl);
-    }
-    d = quad_sum(d);
-    if (act && gi == 0) {
-      if (shift != 0.0) acc.dr[i] = fma(shift, out.dr[i], acc.dr[i]);
-      out.dr[i] = d;
-    }
-  }
-  GSTRIDE(c, L.nc) {
+  TSTRIDE(c, L.nc) {
     const int po = L.p_off[c];
     double pb = 0.0;
     for (int q = 0; q < L.m[c]; ++q) pb = fma(L.w[po + q], __ldcg(&vp[po + q]), pb);
-    if (shift != 0.0) acc.pb[c] = fma(shift, out.pb[c], acc.pb[c]);
+    if (fold) acc.pb[c] = fma(shift, out.pb[c], acc.pb[c]);
     out.pb[c] = pb;
   }
 }
 
 // A(x + s dx) - b from the linear parts (dir is not read when s == 0), for flux unknown i / pressure unknown i.
 __device__ __forceinline__ double trial_flux_row(const LevelDev& L, const LinParts& bx, const LinParts& dx, double s,
-                                                 const double* b, int kind, double a, int i) {
+                                                 bool nz, const double* b, int kind, double a, int i) {
   double v = 0.0;
 #pragma unroll
   for (int side = 0; side < 2; ++side) {
@@ -564,7 +549,7 @@ __device__ __forceinline__ double trial_flux_row(const LevelDev& L, const LinPar
     if (y < 0) continue;
     const int c = L.slot_cell[y];
     double pb = __ldcg(&bx.pb[c]), m = __ldcg(&bx.ms[y]), d = __ldcg(&bx.ds[y]);
-    if (s != 0.0) {
+    if (nz) {
       pb = fma(s, __ldcg(&dx.pb[c]), pb);
       m = fma(s, __ldcg(&dx.ms[y]), m);
       d = fma(s, __ldcg(&dx.ds[y]), d);
@@ -573,87 +558,109 @@ __device__ __forceinline__ double trial_flux_row(const LevelDev& L, const LinPar
   }
   return v - __ldcg(&b[i]);
 }
-__device__ __forceinline__ double trial_p_row(const LevelDev& L, const LinParts& bx, const LinParts& dx, double s,
+__device__ __forceinline__ double trial_p_row(const LevelDev& L, const LinParts& bx, const LinParts& dx, double s, bool nz,
                                               const double* b, int i) {
   double d = __ldcg(&bx.dr[i]);
-  if (s != 0.0) d = fma(s, __ldcg(&dx.dr[i]), d);
+  if (nz) d = fma(s, __ldcg(&dx.dr[i]), d);
   return d - __ldcg(&b[L.nflux + i]);
 }
 
-// ||A(x + s dx) - b|| (one pass, one reduction).
-__device__ bool trial_norm(const LevelDev& L, const LinParts& bx, const LinParts& dx, double s, const double* b,
-                           int kind, double a, Grid& g, double& rn) {
+// r = A(x + s dx) - b and nb = -r at a trial point; returns this thread's share of ||r||^2.
+__device__ double trial_pass(const LevelDev& L, const CoarseStepBufs<double>& B, double s, int kind, double a) {
+  const bool nz = nonzero(s);
   double acc = 0.0;
   GSTRIDE(i, L.nflux) {
-    const double v = trial_flux_row(L, bx, dx, s, b, kind, a, i);
-    acc = fma(v, v, acc);
-  }
-  GSTRIDE(i, L.np) {
-    const double v = trial_p_row(L, bx, dx, s, b, i);
-    acc = fma(v, v, acc);
-  }
-  double s1[1] = {acc};
-  if (!grid_sum<1>(g, s1)) return false;
-  rn = sqrt(s1[0]);
-  return true;
-}
-
-// Makes x + s dx the iterate: r = A(x) - b, nb = -r and kappa per cell at the new point, x += s dx; returns this
-// thread's share of ||r||^2 (the same sum as the trial's). The linear parts of x are left as they were (the next
-// pass over the step's direction adds s times the old direction's).
-__device__ double accept_pass(const LevelDev& L, const CoarseStepBufs<double>& B, double s, int kind, double a) {
-  double acc = 0.0;
-  GSTRIDE(i, L.nflux) {
-    const double v = trial_flux_row(L, B.base, B.dir, s, B.b, kind, a, i);
+    const double v = trial_flux_row(L, B.base, B.dir, s, nz, B.b, kind, a, i);
     B.r[i] = v;
-    B.nb[i] = -v;
+    B.nb[i] = flip(v, 1);
     acc = fma(v, v, acc);
   }
-  GSTRIDE(i, L.np) {
-    const double v = trial_p_row(L, B.base, B.dir, s, B.b, i);
+  TSTRIDE(i, L.np) {
+    const double v = trial_p_row(L, B.base, B.dir, s, nz, B.b, i);
     B.r[L.nflux + i] = v;
-    B.nb[L.nflux + i] = -v;
+    B.nb[L.nflux + i] = flip(v, 1);
     acc = fma(v, v, acc);
-  }
-  GSTRIDE(c, L.nc) {
-    double pb = __ldcg(&B.base.pb[c]);
-    if (s != 0.0) pb = fma(s, __ldcg(&B.dir.pb[c]), pb);
-    B.kapc[c] = kappa_of(pb, kind, a);
-  }
-  if (s != 0.0) {
-    const int nx = L.nflux + L.np;
-    GSTRIDE(i, nx) B.x[i] = fma(s, __ldcg(&B.dx[i]), B.x[i]);
   }
   return acc;
 }
 
-// Algorithm 1 from x (residual norm rn) along s0 dx, with trial norms from the linear parts. Returns the accepted
-// scaling s * s0 in `step` (0: every trial was non-finite, x is kept; a non-finite trial counts as +infinity) and its
-// residual norm in rn.
-__device__ bool backtrack_lin(const LevelDev& L, const LinParts& bx, const LinParts& dx, const CoarseStepParams& P,
-                              const double* b, double s0, double& rn, double& step, int& trials, Grid& g) {
-  double s = 1.0, r_s = 0.0;
-  if (!trial_norm(L, bx, dx, s * s0, b, P.kind, P.a, g, r_s)) return false;
-  ++trials;
-  if (!isfinite(r_s)) r_s = HUGE_VAL;
-  int n = 0;
-  while (r_s > rn && n < P.bt_nmax) {
-    double r_half = 0.0;
-    if (!trial_norm(L, bx, dx, 0.5 * s * s0, b, P.kind, P.a, g, r_half)) return false;
+// Makes x + s dx the iterate: kappa per cell at the new point, x += s dx, and r and nb unless the last trial was there
+// (`at_trial`). The linear parts of x are left as they were (the next pass over the step's direction adds s times the
+// old direction's).
+__device__ void accept_pass(const LevelDev& L, const CoarseStepBufs<double>& B, double s, bool at_trial, int kind,
+                            double a) {
+  const bool nz = nonzero(s);
+  if (!at_trial) (void)trial_pass(L, B, s, kind, a);
+  TSTRIDE(c, L.nc) {
+    double pb = __ldcg(&B.base.pb[c]);
+    if (nz) pb = fma(s, __ldcg(&B.dir.pb[c]), pb);
+    B.kapc[c] = kappa_of(pb, kind, a);
+  }
+  if (nz) {
+    const int nx = L.nflux + L.np;
+    GSTRIDE(i, nx) B.x[i] = fma(s, __ldcg(&B.dx[i]), B.x[i]);
+  }
+}
+
+// The scalars of a coarse step. Only warp 0 computes with them (a scalar FP64 operation in all sixteen warps costs the SM
+// 300 clocks, a square root 2,800: together a third of a step on a small level); the others follow the outcome it
+// publishes with each sum.
+struct StepScalars {
+  double rn, r0;   // ||A(x) - b||, and at the start of the Picard steps (warp 0)
+  double step;     // the accepted scaling (0: every trial was non-finite, x is kept)
+  bool at_trial;   // the last trial evaluated is the accepted one
+  bool done;       // the coarsest level's stopping test holds at x
+};
+
+__device__ __forceinline__ bool step_done(const CoarseStepParams& P, double rn, double r0) {
+  return P.coarsest && (rn <= P.tol_rel * r0 || rn <= P.tol_abs);
+}
+
+// Algorithm 1 from x (residual norm S.rn) along s0 dx, with trial residuals from the linear parts; a non-finite trial counts
+// as +infinity. `first`: S.rn at the accepted point is also the start value of the stopping test.
+__device__ bool backtrack_lin(const LevelDev& L, const CoarseStepBufs<double>& B, const CoarseStepParams& P, double s0,
+                              bool first, StepScalars& S, int& trials, Grid& g) {
+  double s = 1.0, r_s = HUGE_VAL;   // accepted so far (warp 0)
+  double s_try = s0;
+  int n = -1;                       // halvings accepted (-1: the full step is being tried)
+  while (true) {
+    // {sum, step to try or accepted, outcome: bit 0 decided, bit 1 the last trial is the accepted one, bit 2 done}
+    double v[3] = {trial_pass(L, B, s_try, P.kind, P.a), 0.0, 0.0};
     ++trials;
-    if (!isfinite(r_half)) r_half = HUGE_VAL;
-    if (r_half > P.bt_theta * r_s) break;
-    s *= 0.5;
-    ++n;
-    r_s = r_half;
+    if (!grid_sum_x<1, 2>(g, v, [&](double* o) {
+          double r = sqrt(o[0]);
+          if (!finite_bits(r)) r = HUGE_VAL;
+          int code = 0;
+          if (n < 0 || !(r > P.bt_theta * r_s)) {   // the full step, or a halving Algorithm 1 keeps
+            if (n >= 0) s *= 0.5;
+            ++n;
+            r_s = r;
+            if (!(r_s > S.rn && n < P.bt_nmax)) code = 3;
+          } else {
+            code = 1;
+          }
+          double next = 0.5 * s * s0;
+          if (code) {
+            const bool none = r_s == HUGE_VAL;
+            next = none ? 0.0 : s * s0;
+            if (none) code = 1;
+            else S.rn = r_s;
+            if (first) S.r0 = S.rn;
+            if (step_done(P, S.rn, S.r0)) code |= 4;
+          }
+          o[1] = next;
+          o[2] = __hiloint2double(0, code);
+        }))
+      return false;
+    s_try = v[1];
+    const int code = __double2loint(v[2]);
+    if (code) {
+      S.step = s_try;
+      S.at_trial = (code & 2) != 0;
+      S.done = (code & 4) != 0;
+      return true;
+    }
   }
-  if (r_s == HUGE_VAL) {
-    step = 0.0;
-    return true;
-  }
-  step = s * s0;
-  rn = r_s;
-  return true;
 }
 
 // One launch. On entry x (and, with backtrack_first, the correction in dx and ||A(x) - b|| in rn_in); on exit x, r,
@@ -696,7 +703,7 @@ __global__ void __launch_bounds__(kCThreads, 1) kp_coarse_step(LevelDev L, const
     }
   }
   int iters = 0, steps = 0, evals = 0, trials = 0, bad = 0;
-  double rn = P.rn_in;
+  StepScalars S{P.rn_in, P.rn_in, 0.0, false, false};
   double pending = 0.0;   // accepted step not yet added to the linear parts of x
   // linear parts of x (and of the given correction)
   lin_parts_pass(L, B.x, B.base, B.base, 0.0);
@@ -706,29 +713,30 @@ __global__ void __launch_bounds__(kCThreads, 1) kp_coarse_step(LevelDev L, const
     ++evals;
   }
   if (!grid_barrier(g)) return;
-  double step = 0.0;
   if (P.backtrack_first) {
-    if (!backtrack_lin(L, B.base, B.dir, P, B.b, 1.0, rn, step, trials, g)) return;
+    if (!backtrack_lin(L, B, P, 1.0, true, S, trials, g)) return;
+    accept_pass(L, B, S.step, S.at_trial, P.kind, P.a);   // r, nb, kappa at the new x
+    pending = S.step;
+    if (!grid_barrier(g)) return;
+  } else {
+    double v[2] = {trial_pass(L, B, 0.0, P.kind, P.a), 0.0};
+    accept_pass(L, B, 0.0, true, P.kind, P.a);
+    if (!grid_sum_x<1, 1>(g, v, [&](double* o) {
+          S.rn = S.r0 = sqrt(o[0]);
+          o[1] = __hiloint2double(0, (finite_bits(S.rn) ? 0 : 1) | (step_done(P, S.rn, S.r0) ? 4 : 0));
+        }))
+      return;
+    const int code = __double2loint(v[1]);
+    bad = code & 1;
+    S.done = (code & 4) != 0;
   }
-  const double acc = accept_pass(L, B, step, P.kind, P.a);   // r, nb, kappa at the (new) x
-  pending = step;
-  if (!P.backtrack_first) {
-    double s1[1] = {acc};
-    if (!grid_sum<1>(g, s1)) return;
-    rn = sqrt(s1[0]);
-    if (!isfinite(rn)) bad = 1;
-  } else if (!grid_barrier(g)) {
-    return;
-  }
-  const double r0 = rn;
-  for (int k = 0; k < P.nsteps && !bad; ++k) {
-    if (P.coarsest && (rn <= P.tol_rel * r0 || rn <= P.tol_abs)) break;
+  for (int k = 0; k < P.nsteps && !bad && !S.done; ++k) {
     int it = 0;
     double rr0 = 0.0, rr = 0.0;
     if (!hyb_solve_dev<U>(L, Hc, Sinv, B, R, form, gsz, dyn, (int*)(dyn + staged), g, P.lin_tol, P.maxit, it, rr0, rr))
       return;
     iters += it;
-    if (!isfinite(rr)) {
+    if (!finite_bits(rr)) {
       bad = 2;
       break;
     }
@@ -739,20 +747,20 @@ __global__ void __launch_bounds__(kCThreads, 1) kp_coarse_step(LevelDev L, const
     double s0 = 1.0;
     if (P.dp_clamp > 0.0) {
       double m = 0.0;
-      GSTRIDE(c, L.nc) m = fmax(m, fabs(B.dir.pb[c]));   // written by this thread just above
-      if (!grid_max(g, m)) return;
-      if (m > P.dp_clamp) s0 = P.dp_clamp / m;
+      TSTRIDE(c, L.nc) m = fmax(m, fabs(B.dir.pb[c]));   // written by this thread just above
+      if (!grid_max(g, m, [&](double v) { return v > P.dp_clamp ? fast_div(P.dp_clamp, v) : 1.0; })) return;
+      s0 = m;
     } else if (!grid_barrier(g)) {
       return;
     }
-    if (!backtrack_lin(L, B.base, B.dir, P, B.b, s0, rn, step, trials, g)) return;
-    (void)accept_pass(L, B, step, P.kind, P.a);
-    pending = step;
+    if (!backtrack_lin(L, B, P, s0, false, S, trials, g)) return;
+    accept_pass(L, B, S.step, S.at_trial, P.kind, P.a);
+    pending = S.step;
     if (!grid_barrier(g)) return;   // r, nb, kappa and x complete
     ++steps;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
-    res->rn = rn;
+    res->rn = S.rn;
     res->iters = iters;
     res->steps = steps;
     res->res_evals = evals;
@@ -775,9 +783,9 @@ cudaError_t launch_coarse_step(cudaStream_t st, const LevelDev& L, const double*
   (void)once;
   const int sms = coop_sms(gs.sm_cap);
   // A small level runs as one cluster of up to eight blocks, whose barrier costs a quarter of the grid's: worth it while
-  // the CG's FP64 work on eight SMs (row entries and 13 operations a lambda, 19 clocks a warp operation) stays below
-  // about 3,500 clocks.
-  const bool small = (long)L.nlam * (L.hs_wmax + 13) <= 48000;
+  // the FP64 work on eight SMs stays small beside it. In row entries and operations a lambda: 163 lambdas of a 2D level
+  // (3.7k) gain, 900 (21k: 262 -> 282 us a step) and 482 of a 3D level (28k: 1,046 -> 1,171 us a solve) lose.
+  const bool small = (long)L.nlam * (L.hs_wmax + 13) <= 12000;
   const int most = small ? std::min(sms, kClusterBlocks) : sms;
   // lanes per lambda: as many as leave one warp of rows per sub-partition (four per SM)
   int gsz = 4;

@@ -305,8 +305,10 @@ __device__ __forceinline__ double warp_max(double m) {
   return __hiloint2double((int)mh, (int)ml);
 }
 
-// Max over the grid of one non-negative value per thread (exact, hence deterministic), by the same protocol.
-__device__ __forceinline__ bool grid_max(Grid& g, double& v) {
+// post(max over the grid of one non-negative value per thread) (exact, hence deterministic), by the same protocol; post
+// runs in warp 0.
+template <class PostFn>
+__device__ __forceinline__ bool grid_max(Grid& g, double& v, PostFn&& post) {
   __shared__ double o;
   double* part = g.partial + (g.seq & 1u) * kPartStride;
   ++g.seq;
@@ -322,7 +324,7 @@ __device__ __forceinline__ bool grid_max(Grid& g, double& v) {
   if (warp == 0) {
     m = 0.0;
     for (int b = lane; b < (int)gridDim.x; b += 32) m = fmax(m, __ldcg(&part[b]));
-    m = warp_max(m);
+    m = post(warp_max(m));
     if (lane == 0) o = m;
   }
   __syncthreads();
@@ -338,6 +340,11 @@ __device__ __forceinline__ bool grid_max(Grid& g, double& v) {
   for (int i = (int)(((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32u + (threadIdx.x & 31u)); i < (n); \
        i += (int)(gridDim.x * blockDim.x))
 
+// The same from the last warp down: for a second set of items in the same pass, on the warps the first set leaves idle.
+#define TSTRIDE(i, n)                                                                                         \
+  for (int i = (int)((((blockDim.x - 1u - threadIdx.x) >> 5) * gridDim.x + blockIdx.x) * 32u + (threadIdx.x & 31u)); \
+       i < (n); i += (int)(gridDim.x * blockDim.x))
+
 // Rows 0 .. n-1 of short sums, four lanes (part of a warp) a row: lane gi = 0 .. 3 of a row's group takes its entries gi,
 // gi + 4, ..., and quad_sum adds the four. A thread a row walks one chain of dependent loads and 64-clock FP64
 // operations as long as the row; four lanes a row cut it to a quarter, read the row's entries side by side, and still
@@ -351,7 +358,10 @@ __device__ __forceinline__ double quad_sum(double v) {
   return v;
 }
 
-// v, or -v when neg is 1, on the integer pipe.
+// Tests and signs of a double on the integer pipe.
+__device__ __forceinline__ bool nonzero(double v) { return ((__double2hiint(v) << 1) | __double2loint(v)) != 0; }
+__device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+// v, or -v when neg is 1
 __device__ __forceinline__ double flip(double v, int neg) {
   return __hiloint2double(__double2hiint(v) ^ (neg << 31), __double2loint(v));
 }
