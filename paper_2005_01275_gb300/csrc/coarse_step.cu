@@ -673,7 +673,7 @@ __global__ void __launch_bounds__(kCThreads, 1) kp_coarse_step(LevelDev L, const
   __shared__ double sm[kSmDoubles];
   __shared__ int ew[U * kCWarps];
   extern __shared__ double dyn[];   // the staged entries: values, then columns
-  Grid g{gs, partial, sm, 0u};
+  Grid g = grid_start(gs, partial, sm);
   HRows<U> R;
   {
     // rows of this thread: item i = ((warp + kCWarps u) gridDim + block) 32 + lane, gsz consecutive items a lambda
@@ -760,6 +760,7 @@ __global__ void __launch_bounds__(kCThreads, 1) kp_coarse_step(LevelDev L, const
     ++steps;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
+    res->err = 0;
     res->rn = S.rn;
     res->iters = iters;
     res->steps = steps;

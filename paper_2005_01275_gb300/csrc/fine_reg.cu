@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(kFThreads, 1) kp_fine_cg_reg(FineDev F, const 
   __shared__ int stop;
   extern __shared__ double dyn[];
   const int server = (blockDim.x >> 5) - 1, warp = threadIdx.x >> 5;
-  Grid g{gs, partial, sm, 0u};
+  Grid g = grid_start(gs, partial, sm);
   FRows<R, T> X;
   rows_init(X, F, server);
   X.staged = staged > 0;
@@ -331,6 +331,7 @@ __global__ void __launch_bounds__(kFThreads, 1) kp_fine_cg_reg(FineDev F, const 
   for (int u = 0; u < R; ++u)
     if (X.K[u] >= 0) dx[X.K[u]] = sdiag[X.K[u]] * (double)y[u];
   if (blockIdx.x == 0 && threadIdx.x == 0) {
+    res->err = 0;
     res->iters = it;
     res->rr0 = sc[3];
     res->rr = sc[2];
@@ -362,7 +363,7 @@ __global__ void __launch_bounds__(kFThreads, 1) kp_fine_bicgstab_reg(FineDev F, 
   __shared__ int state;      // 0 go on, 1 stop, 2 sum (rh, r) and (r, r) from the vectors
   extern __shared__ double dyn[];
   const int server = (blockDim.x >> 5) - 1, warp = threadIdx.x >> 5;
-  Grid g{gs, partial, sm, 0u};
+  Grid g = grid_start(gs, partial, sm);
   FRows<R, double> X;
   rows_init(X, F, server);
   X.staged = staged > 0;
@@ -535,6 +536,7 @@ __global__ void __launch_bounds__(kFThreads, 1) kp_fine_bicgstab_reg(FineDev F, 
   for (int u = 0; u < R; ++u)
     if (X.K[u] >= 0) dx[X.K[u]] = S[X.K[u]] * ys[u * T];
   if (blockIdx.x == 0 && threadIdx.x == 32 * server) {
+    res->err = 0;
     res->iters = it;
     res->rr0 = sv[0];
     res->rr = sv[1];

@@ -8,7 +8,7 @@
 #include <atomic>
 #include <cmath>
 
-#include "fp64.cuh"
+#include "isum.cuh"
 #include "kernels.cuh"
 
 namespace nlmg {
@@ -44,13 +44,21 @@ __device__ __forceinline__ void block_reduce(double (&v)[NV], double* sm) {
   __syncthreads();
 }
 
-// Grid-wide deterministic reduction; returns true in the last block (thread 0 then holds the result in v, which is
-// also stored to red.out[0..NV)).
+// Grid-wide deterministic reduction; returns true in the last block's warp 0 (whose lanes then hold the result in v, which
+// is also stored to red.out[0..NV)). Sums run on the integer pipes (isum.cuh), maxima as a tree.
 template <int NV, bool MAX>
 __device__ __forceinline__ bool grid_reduce(double (&v)[NV], const Reduce& red) {
   __shared__ double sm[NV * 32];
+  __shared__ ISum si[MAX ? 1 : NV * 32];
   __shared__ int am_last;
-  block_reduce<NV, MAX>(v, sm);
+  if constexpr (MAX) {
+    block_reduce<NV, MAX>(v, sm);
+  } else {
+    double a[NV][1];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) a[k][0] = v[k];
+    block_sums<NV, 1>(a, v, si, kThreads / 32);
+  }
   if (threadIdx.x == 0) {
 #pragma unroll
     for (int k = 0; k < NV; ++k) red.partial[blockIdx.x * NV + k] = v[k];
@@ -61,22 +69,34 @@ __device__ __forceinline__ bool grid_reduce(double (&v)[NV], const Reduce& red) 
   __syncthreads();
   if (!am_last) return false;
   __threadfence();
-  double acc[NV];
+  if constexpr (MAX) {
+    double acc[NV];
 #pragma unroll
-  for (int k = 0; k < NV; ++k) acc[k] = 0.0;
-  for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x)
+    for (int k = 0; k < NV; ++k) acc[k] = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x)
 #pragma unroll
-    for (int k = 0; k < NV; ++k) acc[k] = comb<MAX>(acc[k], __ldcg(&red.partial[b * NV + k]));
-  block_reduce<NV, MAX>(acc, sm);
+      for (int k = 0; k < NV; ++k) acc[k] = comb<MAX>(acc[k], __ldcg(&red.partial[b * NV + k]));
+    block_reduce<NV, MAX>(acc, sm);
+#pragma unroll
+    for (int k = 0; k < NV; ++k) v[k] = acc[k];
+  } else {
+    constexpr int M = 4;   // partials a thread in the exact sum; beyond 1,024 blocks they are added onto those first
+    double p[NV][M];
+#pragma unroll
+    for (int j = 0; j < M; ++j)
+#pragma unroll
+      for (int k = 0; k < NV; ++k) {
+        p[k][j] = 0.0;
+        for (int b = threadIdx.x + kThreads * j; b < (int)gridDim.x; b += kThreads * M) p[k][j] += __ldcg(&red.partial[b * NV + k]);
+      }
+    block_sums<NV, M>(p, v, si, kThreads / 32);
+  }
   if (threadIdx.x == 0) {
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      red.out[k] = acc[k];
-      v[k] = acc[k];
-    }
+    for (int k = 0; k < NV; ++k) red.out[k] = v[k];
     *red.counter = 0u;
   }
-  return true;
+  return threadIdx.x < 32;
 }
 
 #define GRID_STRIDE(i, n) for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < (n); i += gridDim.x * blockDim.x)
@@ -85,7 +105,8 @@ __device__ __forceinline__ bool grid_reduce(double (&v)[NV], const Reduce& red) 
 
 __global__ void k_kappa(int n, const double* __restrict__ p, const double* __restrict__ dp, double s,
                         double* __restrict__ q, double* __restrict__ r, double* __restrict__ dr, int kind, double a,
-                        unsigned* zero) {
+                        unsigned* zero, const double* __restrict__ scale) {
+  if (scale) s *= *scale;
   if (zero && blockIdx.x == 0 && threadIdx.x == 0) *zero = 0u;
   GRID_STRIDE(i, n) {
     const double v = dp ? fma(s, dp[i], p[i]) : p[i];
@@ -189,10 +210,11 @@ __global__ void k_jacobi_update(int n, const double* __restrict__ q, const doubl
   }
 }
 
-__global__ void k_max_abs(int n, const double* __restrict__ x, Reduce red) {
+// red.out = clamp / max |x| where that is below 1, else 1: the scaling the pressure-change clamp asks for
+__global__ void k_clamp_scale(int n, const double* __restrict__ x, double clamp, Reduce red) {
   double acc[1] = {0.0};
   GRID_STRIDE(i, n) acc[0] = fmax(acc[0], fabs(x[i]));
-  grid_reduce<1, true>(acc, red);
+  if (grid_reduce<1, true>(acc, red) && threadIdx.x == 0) *red.out = acc[0] > clamp ? clamp / acc[0] : 1.0;
 }
 
 __global__ void k_axpy(int n, const double* __restrict__ x, double s, const double* __restrict__ dx,
@@ -492,9 +514,9 @@ void count_launch(int n) {
 #define COUNT(n) count_launch(n)
 
 void launch_kappa(cudaStream_t st, int n, const double* p, const double* dp, double s, double* q, double* r,
-                  double* dr, int kind, double a, unsigned* zero) {
+                  double* dr, int kind, double a, unsigned* zero, const double* scale) {
   COUNT(1);
-  k_kappa<<<grid_for(n), kThreads, 0, st>>>(n, p, dp, s, q, r, dr, kind, a, zero);
+  k_kappa<<<grid_for(n), kThreads, 0, st>>>(n, p, dp, s, q, r, dr, kind, a, zero, scale);
 }
 void launch_rhs(cudaStream_t st, const FineDev& F, const double* f, const double* g, double* rhs) {
   COUNT(1);
@@ -513,9 +535,9 @@ void launch_jacobi_update(cudaStream_t st, int n, const double* q, const double*
   COUNT(1);
   k_jacobi_update<<<grid_for(n), kThreads, 0, st>>>(n, q, R, jdiag, diagT, omega, qnew);
 }
-void launch_max_abs(cudaStream_t st, int n, const double* x, Reduce red) {
+void launch_clamp_scale(cudaStream_t st, int n, const double* x, double clamp, Reduce red) {
   COUNT(1);
-  k_max_abs<<<grid_for(n), kThreads, 0, st>>>(n, x, red);
+  k_clamp_scale<<<grid_for(n), kThreads, 0, st>>>(n, x, clamp, red);
 }
 void launch_axpy(cudaStream_t st, int n, const double* x, double s, const double* dx, double* out) {
   COUNT(1);

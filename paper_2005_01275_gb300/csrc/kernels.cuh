@@ -17,7 +17,7 @@ enum Scalar { S_RZ = 0, S_ALPHA, S_BETA, S_RR, S_RR0, S_PQ, S_NORM2, S_NORM2B, S
 struct Reduce {
   double* partial;    // kMaxBlocks * 4
   unsigned* counter;  // one counter per reduction call site
-  double* out;        // result slot(s)
+  double* out;        // result slot(s), device or pinned host memory
 };
 
 // ---------------------------------------------------------------------------------------------------------------
@@ -110,9 +110,10 @@ long long launch_count_thread();   // issued by the calling host thread
 void count_launch(int n);
 
 // launchers (kernels.cu)
-// q = p + s dp (dp may be null), r = 1 / kappa(q) and, if dr, its derivative; zeroes *zero (if not null)
+// q = p + s dp (dp may be null; s times *scale if not null), r = 1 / kappa(q) and, if dr, its derivative; zeroes *zero (if
+// not null)
 void launch_kappa(cudaStream_t st, int n, const double* p, const double* dp, double s, double* q, double* r,
-                  double* dr, int kind, double a, unsigned* zero = nullptr);
+                  double* dr, int kind, double a, unsigned* zero = nullptr, const double* scale = nullptr);
 void launch_rhs(cudaStream_t st, const FineDev& F, const double* f, const double* g, double* rhs);
 // R and ||R||^2 at q (r from launch_kappa). Tval, diagT (both or neither): the frozen matrix; jdiag, Joff (with dr and
 // diagT): the exact Jacobian.
@@ -132,7 +133,7 @@ void launch_gmres_combine(cudaStream_t st, int n, int nk, const double* V, const
                           double* x);
 void launch_jacobi_update(cudaStream_t st, int n, const double* q, const double* R, const double* jdiag,
                           const double* diagT, double omega, double* qnew);
-void launch_max_abs(cudaStream_t st, int n, const double* x, Reduce red);
+void launch_clamp_scale(cudaStream_t st, int n, const double* x, double clamp, Reduce red);
 void launch_axpy(cudaStream_t st, int n, const double* x, double s, const double* dx, double* out);
 void launch_sub(cudaStream_t st, int n, const double* y, const double* x, double* out);
 void launch_fine_flux(cudaStream_t st, const FineDev& F, const double* p, const double* r, const double* g,

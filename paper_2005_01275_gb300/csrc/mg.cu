@@ -1,8 +1,8 @@
 // Linear multigrid preconditioner for the level-0 Krylov solves (see mg.cuh), and the preconditioned CG / BiCGStab
 // that use it, each captured once per context as CUDA graphs with a device-side conditional while loop.
 //
-// Every reduction is deterministic: per-block partial sums in a fixed tree, then the grid's last block adds the
-// partials in block order (the arrival counter is reset by that block, so graphs replay). Maxima are exact.
+// Every reduction is deterministic: per-block partial sums, then the grid's last block adds the partials, both exactly
+// (the arrival counter is reset by that block, so graphs replay). Maxima are exact.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -13,7 +13,7 @@
 #include <type_traits>
 #include <vector>
 
-#include "fp64.cuh"
+#include "isum.cuh"
 #include "mg.cuh"
 
 namespace nlmg {
@@ -48,55 +48,43 @@ inline int blocks_for(long n, int cap = 1 << 20) {
 // ---------------------------------------------------------------------------------------------------------------
 // reductions
 
-// Sums NV values over the grid: block tree sums to part[block][k]; the last block to arrive adds the partials in block
-// order (thread t takes partials t, t + blockDim, ...; then a fixed tree) and returns true in every one of its
-// threads with the sums in out (shared). The counter is left at zero.
+// Sums NV values over the grid: block sums to part[block][k]; the last block to arrive adds the partials (exactly, hence
+// in no particular order; at most kMaxRedBlocks) and returns true in its warp 0 with the sums in out. The counter is left
+// at zero. On the integer pipes (isum.cuh): block trees, 1,024 partials and their trees took 2 us at the end of a kernel.
 template <int NV>
-__device__ bool reduce_last(double (&v)[NV], double* part, unsigned* cnt, double* out) {
-  __shared__ double sh[NV][kT / 32];
+__device__ bool reduce_last(double (&v)[NV], double* part, unsigned* cnt, double (&out)[NV]) {
+  __shared__ ISum sh[NV * 32];
   __shared__ int last;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int M = kMaxRedBlocks / kT;
+  const int lane = threadIdx.x & 31;
+  double a[NV][1], s[NV];
 #pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    double a = v[k];
+  for (int k = 0; k < NV; ++k) a[k][0] = v[k];
+  block_sums<NV, 1>(a, s, sh, kT / 32);
+  if (threadIdx.x < NV) {
+    double mine = s[0];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) a += __shfl_down_sync(0xffffffffu, a, off);
-    if (lane == 0) sh[k][warp] = a;
+    for (int k = 1; k < NV; ++k) mine = lane == k ? s[k] : mine;
+    part[(size_t)blockIdx.x * NV + lane] = mine;
   }
-  __syncthreads();
+  __syncwarp();
   if (threadIdx.x == 0) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      double a = 0.0;
-      for (int w = 0; w < kT / 32; ++w) a += sh[k][w];
-      part[(size_t)blockIdx.x * NV + k] = a;
-    }
     __threadfence();
     last = atomicAdd(cnt, 1u) == gridDim.x - 1 ? 1 : 0;
   }
   __syncthreads();
   if (!last) return false;
   __threadfence();
+  double p[NV][M];
 #pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    double a = 0.0;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += kT) a += __ldcg(&part[(size_t)b * NV + k]);
+  for (int j = 0; j < M; ++j) {
+    const int b = (int)threadIdx.x + kT * j;
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) a += __shfl_down_sync(0xffffffffu, a, off);
-    if (lane == 0) sh[k][warp] = a;
+    for (int k = 0; k < NV; ++k) p[k][j] = b < (int)gridDim.x ? __ldcg(&part[(size_t)b * NV + k]) : 0.0;
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      double a = 0.0;
-      for (int w = 0; w < kT / 32; ++w) a += sh[k][w];
-      out[k] = a;
-    }
-    *cnt = 0u;
-  }
-  __syncthreads();
-  return true;
+  block_sums<NV, M>(p, out, sh, kT / 32);
+  if (threadIdx.x == 0) *cnt = 0u;
+  return threadIdx.x < 32;
 }
 
 __device__ __forceinline__ void atomic_max_pos(float* addr, float v) {
@@ -628,9 +616,9 @@ __global__ void __launch_bounds__(kT, 6) k_cheb0_beta(FineDev F, const float* __
       di = a0dinv[K];
     }
   }
-  __shared__ double out[2];
+  double out[2];
   if (reduce_last<2>(v, part, &sc->cnt[1], out) && threadIdx.x == 0) {
-    sc->beta = first ? 0.0 : (out[0] - out[1]) / sc->rz;
+    sc->beta = first ? 0.0 : fast_div(out[0] - out[1], sc->rz);
     sc->rz = out[0];
   }
 }
@@ -1322,7 +1310,7 @@ __global__ void k_pcg_init(int N, const double* __restrict__ b, double bscale, c
     first_step0(K, rf, a0dinv, c2, x0, d0);
     v[0] = fma(ri * ri, widen(a0dinv[K]), v[0]);   // ||S r||^2 with S^2 = 1 / A_KK
   }
-  __shared__ double out[1];
+  double out[1];
   if (reduce_last<1>(v, part, &sc->cnt[0], out) && threadIdx.x == 0) {
     sc->rr0 = out[0];
     sc->rr = out[0];
@@ -1353,8 +1341,8 @@ __global__ void k_pcg_pq(FineDev F, const double* __restrict__ Tval, const doubl
     zold[K] = zf;
     v[0] = fma(pk, qk, v[0]);
   }
-  __shared__ double out[1];
-  if (reduce_last<1>(v, part, &sc->cnt[2], out) && threadIdx.x == 0) sc->alpha = sc->rz / out[0];
+  double out[1];
+  if (reduce_last<1>(v, part, &sc->cnt[2], out) && threadIdx.x == 0) sc->alpha = fast_div(sc->rz, out[0]);
 }
 
 // x += alpha p, r -= alpha q, r32 = r with the first smoothing step of the next V-cycle; ||S r||^2 decides: the
@@ -1382,7 +1370,7 @@ __global__ void k_pcg_update(int N, const double* __restrict__ p, const double* 
     first_step0(K, rf, a0dinv, c2, x0, d0);
     v[0] = fma(ri * ri, widen(a0dinv[K]), v[0]);   // ||S r||^2 with S^2 = 1 / A_KK
   }
-  __shared__ double out[1];
+  double out[1];
   if (reduce_last<1>(v, part, &sc->cnt[3], out) && threadIdx.x == 0) {
     sc->rr = out[0];
     sc->it += 1;
@@ -1427,7 +1415,7 @@ __global__ void k_bicg_init(int N, const double* __restrict__ b, double bscale, 
     v[0] = fma(ri, ri, v[0]);
     v[1] = fma(ri * ri, wgt[K], v[1]);
   }
-  __shared__ double out[2];
+  double out[2];
   if (reduce_last<2>(v, part, &sc->cnt[0], out) && threadIdx.x == 0) {
     sc->rho = out[0];
     sc->rr0 = out[1];
@@ -1452,8 +1440,8 @@ __global__ void k_bicg_v(FineDev F, const double* __restrict__ Joff, const doubl
     v[K] = vk;
     a[0] = fma(rh[K], vk, a[0]);
   }
-  __shared__ double out[1];
-  if (reduce_last<1>(a, part, &sc->cnt[1], out) && threadIdx.x == 0) sc->alpha = sc->rho / out[0];
+  double out[1];
+  if (reduce_last<1>(a, part, &sc->cnt[1], out) && threadIdx.x == 0) sc->alpha = fast_div(sc->rho, out[0]);
 }
 __global__ void k_bicg_s(int N, const double* __restrict__ r, const double* __restrict__ v, double* __restrict__ s,
                          float* __restrict__ r32, const float* __restrict__ a0dinv, float* __restrict__ x0,
@@ -1484,8 +1472,8 @@ __global__ void k_bicg_t(FineDev F, const double* __restrict__ Joff, const doubl
     a[0] = fma(tk, s[K], a[0]);
     a[1] = fma(tk, tk, a[1]);
   }
-  __shared__ double out[2];
-  if (reduce_last<2>(a, part, &sc->cnt[2], out) && threadIdx.x == 0) sc->omega = out[1] != 0.0 ? out[0] / out[1] : 0.0;
+  double out[2];
+  if (reduce_last<2>(a, part, &sc->cnt[2], out) && threadIdx.x == 0) sc->omega = out[1] != 0.0 ? fast_div(out[0], out[1]) : 0.0;
 }
 // x += alpha p^ + omega s^, r = s - omega t, rho_new = (rh, r), ||W r||^2; beta = (rho_new / rho)(alpha / omega).
 __global__ void k_bicg_x(int N, const double* __restrict__ pp, const float* __restrict__ zs,
@@ -1506,14 +1494,14 @@ __global__ void k_bicg_x(int N, const double* __restrict__ pp, const float* __re
     a[0] = fma(rh[K], rk, a[0]);
     a[1] = fma(rk * rk, wgt[K], a[1]);
   }
-  __shared__ double out[2];
+  double out[2];
   if (reduce_last<2>(a, part, &sc->cnt[3], out) && threadIdx.x == 0) {
     sc->rr = out[1];
     sc->it += 1;
     const bool fin = isfinite(out[1]) && isfinite(alpha) && isfinite(omega);
     if (!fin) sc->bad = 1;
     const bool breakdown = omega == 0.0 || sc->rho == 0.0;
-    sc->beta = breakdown ? 0.0 : (out[0] / sc->rho) * (alpha / omega);
+    sc->beta = breakdown ? 0.0 : fast_div(out[0], sc->rho) * fast_div(alpha, omega);
     sc->rho = out[0];
     const int d = (!fin || breakdown || out[1] <= sc->tol2 * sc->rr0 || sc->it >= sc->maxit) ? 1 : 0;
     sc->done = d;

@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(kPThreads) kp_fine_cg(FineDev F, const T* __re
                                                         double* partial, GridSync gs, double tol, int maxit,
                                                         PcgResult* res) {
   __shared__ double sm[kSmDoubles];
-  Grid g{gs, partial, sm, 0u};
+  Grid g = grid_start(gs, partial, sm);
   T t1 = (T)0;   // per-thread partial sums in T (a thread holds one or two cells), block and grid sums in FP64
   CSTRIDE(i, F.N) {
     const T ri = (T)(sdiag[i] * bscale * b[i]);
@@ -111,6 +111,7 @@ __global__ void __launch_bounds__(kPThreads) kp_fine_cg(FineDev F, const T* __re
   }
   CSTRIDE(i, F.N) dx[i] = sdiag[i] * (double)y[i];
   if (blockIdx.x == 0 && threadIdx.x == 0) {
+    res->err = 0;
     res->iters = it;
     res->rr0 = rr0;
     res->rr = rr;
@@ -156,7 +157,7 @@ __global__ void __launch_bounds__(kPThreads, 2) kp_fine_cg_pipe(FineDev F, const
                                                              T* __restrict__ sv, T* __restrict__ p, double* partial,
                                                              GridSync gs, double tol, int maxit, PcgResult* res) {
   __shared__ double sm[kSmDoubles];
-  Grid g{gs, partial, sm, 0u};
+  Grid g = grid_start(gs, partial, sm);
   CSTRIDE(i, F.N) {
     r[i] = (T)(sdiag[i] * bscale * b[i]);
     y[i] = z[i] = sv[i] = p[i] = (T)0;
@@ -222,6 +223,7 @@ __global__ void __launch_bounds__(kPThreads, 2) kp_fine_cg_pipe(FineDev F, const
   }
   CSTRIDE(i, F.N) dx[i] = sdiag[i] * (double)y[i];
   if (blockIdx.x == 0 && threadIdx.x == 0) {
+    res->err = 0;
     res->iters = it;
     res->rr0 = rr0;
     res->rr = gamma;
@@ -273,7 +275,7 @@ __global__ void __launch_bounds__(kPThreads) kp_fine_bicgstab(FineDev F, const d
                                                               double* __restrict__ t, double* partial, GridSync gs,
                                                               double tol, int maxit, PcgResult* res) {
   __shared__ double sm[kSmDoubles];
-  Grid g{gs, partial, sm, 0u};
+  Grid g = grid_start(gs, partial, sm);
   double a1[1] = {0.0};
   CSTRIDE(i, F.N) {
     const double ri = sS[i] * bscale * b[i];
@@ -334,6 +336,7 @@ __global__ void __launch_bounds__(kPThreads) kp_fine_bicgstab(FineDev F, const d
   }
   CSTRIDE(i, F.N) dx[i] = sS[i] * y[i];
   if (blockIdx.x == 0 && threadIdx.x == 0) {
+    res->err = 0;
     res->iters = it;
     res->rr0 = rr0;
     res->rr = rr;
@@ -444,7 +447,7 @@ template cudaError_t launch_fine_cg<float>(cudaStream_t, const FineDev&, const f
 __global__ void __launch_bounds__(kPThreads) kp_barrier_probe(GridSync gs, double* partial, int absent,
                                                               unsigned long long spin_limit, int* passed) {
   __shared__ double sm[kSmDoubles];
-  Grid g{gs, partial, sm, 0u};
+  Grid g = grid_start(gs, partial, sm);
   if ((int)blockIdx.x == absent) return;
   const bool ok = grid_barrier(g, spin_limit);
   if (ok && threadIdx.x == 0) atomicAdd(passed, 1);

@@ -6,6 +6,8 @@
 
 namespace nlmg {
 
+// Results of a launch, in pinned host memory the kernel writes itself: the host sets err before the launch, and only a
+// launch whose barriers all completed clears it.
 struct PcgResult {
   int iters;      // CG iterations taken
   int err;        // 1 if a grid barrier gave up waiting
@@ -17,7 +19,7 @@ struct PcgResult {
 constexpr int kPartStride = 8192;
 
 struct GridSync {
-  unsigned* count;   // barrier arrival counter (0 at launch); own 128-byte line
+  unsigned* count;   // barrier arrival counter (0 but for its top bit between launches); own 128-byte line
   int* err;          // set when a wait gives up
   int sm_cap;        // host side: at most this many SMs for the launch (0 = all)
   int cluster = 0;   // the grid is one thread-block cluster (set by the launch)
@@ -116,6 +118,7 @@ struct CoarseStepResult {
   int res_evals;    // evaluations of the operator's linear parts (one per Picard step and one on entry)
   int bad;          // 0, or where a non-finite value appeared: 1 residual, 2 hybridized CG
   int trials;       // residual norms of Algorithm 1's trial points (from the linear parts)
+  int err;          // 1 if a grid barrier gave up waiting
 };
 
 // One launch: [Algorithm 1 along a given correction], up to nsteps coarse Picard steps (frozen-kappa hybridized

@@ -1,17 +1,11 @@
 // Synchronisation and sums of the persistent (cooperative) kernels: the bounded grid barrier, deterministic grid sums
 // and the division that derives step lengths from them.
 //
-// What a sum costs on this part is a chain of dependent FP64 operations: one takes 64 clocks, and a warp issues one
-// every 64 clocks whatever its lanes do (measured; an FP64 division 560, a shuffle tree over a warp 546). So the sums
-// here run on the integer pipes. A warp's values are aligned to their largest exponent as 64-bit integers and added
-// exactly in three limbs by warp-wide integer reductions: 236 clocks, an error of at most 2^-54 of the largest value
-// after the last rounding (below the rounding of a floating-point tree), and no order dependence at all. Values no
-// such window holds (subnormal sums, infinities, NaN, sums next to overflow) go through the floating-point
-// tree, so they mean what they meant there.
+// What the sums cost, and why they run on the integer pipes, stands in isum.cuh.
 #pragma once
 #include <cuda_runtime.h>
 
-#include "fp64.cuh"
+#include "isum.cuh"
 #include "persist.cuh"
 
 namespace nlmg {
@@ -31,97 +25,6 @@ __device__ __forceinline__ void red_add_release_gpu(unsigned* p, unsigned v) {
   asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// A sum in integer form: t 2^(mx - 1077), or, with mx < 0, the double whose bits t are (special values, see above).
-struct ISum {
-  long long t;
-  int mx;
-};
-__device__ __forceinline__ double isum_value(const ISum& s) {
-  if (s.mx < 0) return __longlong_as_double(s.t);
-  const long long d = __double_as_longlong((double)s.t);
-  return s.t == 0 ? 0.0 : __longlong_as_double(d + ((long long)(s.mx - 1077) << 52));
-}
-
-// s[k] = the sum over the warp of v[k][0..M) (see above), in every lane; all 32 lanes take part.
-template <int NV, int M>
-__device__ __forceinline__ void warp_sums(const double (&v)[NV][M], ISum (&s)[NV]) {
-  int mx[NV];
-  bool odd = false;
-#pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    unsigned m = 0u;
-#pragma unroll
-    for (int j = 0; j < M; ++j) m = max(m, (unsigned)__double2hiint(v[k][j]) & 0x7fffffffu);
-    mx[k] = (int)(__reduce_max_sync(0xffffffffu, m) >> 20);
-    odd = odd || (mx[k] < 64 && __any_sync(0xffffffffu, m != 0u)) || mx[k] > 2032;
-  }
-  if (odd) {   // the same in every lane
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      double a = v[k][0];
-#pragma unroll
-      for (int j = 1; j < M; ++j) a += v[k][j];
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
-      s[k].t = __double_as_longlong(a);
-      s[k].mx = -1;
-    }
-    return;
-  }
-#pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    int lo = 0, mi = 0, hi = 0;   // limbs of 22, 21 and 21 bits: at most 32 M <= 224 terms, no limb overflows
-#pragma unroll
-    for (int j = 0; j < M; ++j) {
-      const unsigned long long b = (unsigned long long)__double_as_longlong(v[k][j]);
-      const int ex = (int)((b >> 52) & 0x7ffu), sh = mx[k] - ex;
-      unsigned long long x = (b << 11) | 0x8000000000000000ull;
-      x = ex != 0 && sh < 64 ? x >> sh : 0ull;   // (a subnormal is far below the window)
-      const int sg = (int)((long long)b >> 63);
-      lo += ((int)(x & 0x3fffffu) ^ sg) - sg;
-      mi += ((int)((x >> 22) & 0x1fffffu) ^ sg) - sg;
-      hi += ((int)(x >> 43) ^ sg) - sg;
-    }
-    static_assert(M <= 7, "limbs sized for 224 terms");
-    lo = __reduce_add_sync(0xffffffffu, lo);
-    mi = __reduce_add_sync(0xffffffffu, mi);
-    hi = __reduce_add_sync(0xffffffffu, hi);
-    // the window's bits from 2^9 up: |t| < 2^63; its unit is 2^(mx - 1077)
-    s[k].t = ((long long)hi << 34) + ((long long)mi << 13) + (long long)(lo >> 9);
-    s[k].mx = mx[k];
-  }
-}
-
-// The sum over the warp of one integer sum per lane, as a double in every lane; all 32 lanes take part.
-template <int NV>
-__device__ __forceinline__ void warp_sums_i(const ISum (&v)[NV], double (&s)[NV]) {
-  bool odd = false;
-#pragma unroll
-  for (int k = 0; k < NV; ++k) odd = odd || v[k].mx < 0;
-  if (__any_sync(0xffffffffu, odd)) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      double a = isum_value(v[k]);
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
-      s[k] = a;
-    }
-    return;
-  }
-#pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    const int mx = (int)__reduce_max_sync(0xffffffffu, (unsigned)v[k].mx), sh = mx - v[k].mx;
-    const long long x = sh < 63 ? v[k].t >> sh : 0ll;
-    const int lo = __reduce_add_sync(0xffffffffu, (int)(x & 0x3fffff));
-    const int mi = __reduce_add_sync(0xffffffffu, (int)((x >> 22) & 0x1fffff));
-    const int hi = __reduce_add_sync(0xffffffffu, (int)(x >> 43));
-    ISum r;   // six bits of room for 32 terms
-    r.t = ((long long)hi << 37) + ((long long)mi << 16) + (long long)(lo >> 6);
-    r.mx = mx + 6;
-    s[k] = isum_value(r);
-  }
-}
-
 // The synchronisation state one thread of a persistent kernel carries: the launch's barrier words, the two
 // buffers of per-block partial sums (used alternately by consecutive reductions), kSmDoubles doubles of shared
 // memory, the number of reductions so far and the barrier phase (both the same in every block).
@@ -130,7 +33,7 @@ struct Grid {
   double* partial;
   double* sm;
   unsigned seq;
-  unsigned phase = 0u;   // the counter's top bit after the last barrier (0 at launch)
+  unsigned phase;   // the counter's top bit after the last barrier
 };
 
 // A grid of at most kClusterBlocks blocks is launched as one thread-block cluster (gs.cluster), whose hardware barrier takes
@@ -138,6 +41,15 @@ struct Grid {
 // block that was never scheduled.
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
+// The state at the start of a launch. The counter's top bit is wherever the last launch left it; no block can have
+// completed a barrier of this launch before this block's first arrival, so every block reads the same bit.
+__device__ __forceinline__ Grid grid_start(const GridSync& gs, double* partial, double* sm) {
+  __shared__ unsigned phase;
+  if (threadIdx.x == 0) phase = gs.cluster ? 0u : ld_acquire_gpu(gs.count) & 0x80000000u;
+  __syncthreads();
+  return Grid{gs, partial, sm, 0u, phase};
+}
 
 // One arrival and the bounded wait for all others, by one thread: every block adds 1 to gs.count except block 0, which
 // adds 2^31 - (gridDim.x - 1), so the counter's top bit flips exactly when the last block arrives and its low bits

@@ -49,7 +49,7 @@ struct CoarseBuf {
   double *hw = nullptr, *hz = nullptr, *hs = nullptr, *hma = nullptr, *hmb = nullptr;   // pipelined hybridized CG
   double* hsv = nullptr;    // values of the SELL form of H
   LinParts base{}, dir{};   // linear parts of the operator at x and along dx (fused coarse step)
-  double rn = 0.0;  // ||A(x) - b|| at the current x (valid after coarse_res)
+  double rn = 0.0;  // ||A(x) - b|| at the current x
 };
 
 // Optional CUDA-event timing of selected kernels on the context stream (pairs of events around each launch).
@@ -156,9 +156,9 @@ struct nlmg_ctx {
   long long fine_evals = 0, lin_iters = 0;
   long long lin_iters_level[8] = {0};
   Prof prof;
-  PcgResult* d_res = nullptr;   // device result of the persistent CG kernels
-  PcgResult* h_res = nullptr;   // pinned copy
-  unsigned* d_bar = nullptr;    // grid barrier count / generation
+  PcgResult* d_res = nullptr;   // the persistent kernels' error word (and the barrier check's result)
+  PcgResult* h_res = nullptr;   // pinned: results of the persistent kernels, written by them
+  unsigned* d_bar = nullptr;    // grid barrier count
   int prof_begin(int k) {
     if (!prof.on) return -1;
     if (prof.used * 2 + 2 > (int)prof.ev.size()) prof_flush();
@@ -205,17 +205,17 @@ struct nlmg_ctx {
     CK(cudaStreamSynchronize(st));
     return (T*)p;
   }
-  Reduce red(int slot) { return Reduce{d_partial, d_cnt, d_sc + slot}; }
+  // sums go to pinned host memory (no copy of their own), scalings the next kernel reads stay on the device
+  Reduce red(int slot) { return Reduce{d_partial, d_cnt, h_sc + slot}; }
+  Reduce red_dev(int slot) { return Reduce{d_partial, d_cnt, d_sc + slot}; }
   double read_sc(int slot) {
-    CK(cudaMemcpyAsync(h_sc, d_sc + slot, sizeof(double), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    return *h_sc;
+    return h_sc[slot];
   }
-  void read_sc2(int s0, double& v0, double& v1) {  // two consecutive slots
-    CK(cudaMemcpyAsync(h_sc, d_sc + s0, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    v0 = h_sc[0];
-    v1 = h_sc[1];
+  // A persistent launch whose barrier gave up leaves its counter anywhere.
+  void reset_barrier() {
+    CK(cudaMemsetAsync(d_bar, 0, sizeof(unsigned), st));
+    CK(cudaMemsetAsync(d_res, 0, sizeof(PcgResult), st));
   }
   int nlev() const { return sh->n_fas; }
   MgWork mg;               // multigrid preconditioner work buffers and graphs (when sh->MG.L > 0)
@@ -640,8 +640,9 @@ void upload_mg(nlmg_ctx* c, int levels) {
 // ---------------------------------------------------------------------------------------------------------------
 // level 0
 
-double fine_eval(nlmg_ctx* c, const double* p, const double* dp, double s, FineState& out) {
-  launch_kappa(c->st, c->F.N, p, dp, s, out.p, out.r, nullptr, c->kind, c->a);
+// The level-0 residual at p + s dp (s times *scale, on the device, if not null) into `out`; returns its norm.
+double fine_eval(nlmg_ctx* c, const double* p, const double* dp, double s, FineState& out, const double* scale = nullptr) {
+  launch_kappa(c->st, c->F.N, p, dp, s, out.p, out.r, nullptr, c->kind, c->a, nullptr, scale);
   int pi = c->prof_begin(2);
   launch_residual(c->st, c->F, out.p, out.r, nullptr, c->g, c->rhs, out.R, nullptr, nullptr, nullptr, c->red(S_NORM2));
   c->prof_end(pi);
@@ -650,17 +651,17 @@ double fine_eval(nlmg_ctx* c, const double* p, const double* dp, double s, FineS
   return out.rn;
 }
 
-// Algorithm 1 on level 0 from c->cur along dp (scaled by s0); the accepted trial becomes c->cur.
-// Algorithm 1 on level 0. A trial whose residual norm is not finite counts as +infinity; if the trial the algorithm
-// returns is not finite, the iterate is kept.
-void backtrack0(nlmg_ctx* c, const double* dp, double s0) {
+// Algorithm 1 on level 0 from c->cur along dp (times *s0, a device scalar, if not null); the accepted trial becomes
+// c->cur. A trial whose residual norm is not finite counts as +infinity; if the trial the algorithm returns is not
+// finite, the iterate is kept.
+void backtrack0(nlmg_ctx* c, const double* dp, const double* s0) {
   const nlmg_options& o = c->opt;
   auto fin = [](double v) { return std::isfinite(v) ? v : HUGE_VAL; };
   double s = 1.0;
   int n = 0;
-  double r_s = fin(fine_eval(c, c->cur.p, dp, s * s0, c->t1));
+  double r_s = fin(fine_eval(c, c->cur.p, dp, s, c->t1, s0));
   while (r_s > c->cur.rn && n < o.bt_nmax) {
-    double r_half = fin(fine_eval(c, c->cur.p, dp, 0.5 * s * s0, c->t2));
+    double r_half = fin(fine_eval(c, c->cur.p, dp, 0.5 * s, c->t2, s0));
     if (r_half > o.bt_theta * r_s) break;
     s *= 0.5;
     ++n;
@@ -669,6 +670,13 @@ void backtrack0(nlmg_ctx* c, const double* dp, double s0) {
   }
   if (r_s == HUGE_VAL) return;
   std::swap(c->cur, c->t1);
+}
+
+// The scaling of a step dp by the pressure-change clamp (Sec. 4.1), left on the device; null without a clamp.
+const double* clamp_scale(nlmg_ctx* c, const double* dp) {
+  if (!(c->opt.dp_clamp > 0)) return nullptr;
+  launch_clamp_scale(c->st, c->F.N, dp, c->opt.dp_clamp, c->red_dev(S_MAX));
+  return c->d_sc + S_MAX;
 }
 
 // Persistent CG on the frozen fine matrix (Tval, diagT): A dx = -R with symmetric Jacobi scaling; dx -> c->cx.
@@ -680,8 +688,7 @@ int mg_bicgstab(nlmg_ctx* c, const double* R, const double* r);
 int fine_pcg(nlmg_ctx* c, const double* R, const double* r) {
   if (c->opt.lin_precond == 1) return mg_pcg(c, R, r);
   GridSync gs{c->d_bar, &c->d_res->err, c->sm_cap};
-  CK(cudaMemsetAsync(c->d_bar, 0, sizeof(unsigned), c->st));
-  CK(cudaMemsetAsync(c->d_res, 0, sizeof(PcgResult), c->st));
+  c->h_res->err = 1;
   launch_sdiag(c->st, c->F.N, c->diagT, c->sdiag);
   const bool fp32 = c->opt.lin_precision == 1;
   // FP64 at loose tolerances: pipelined CG (one grid barrier per iteration), register-resident when every thread
@@ -698,13 +705,13 @@ int fine_pcg(nlmg_ctx* c, const double* R, const double* r) {
     const double tol = std::max(c->lin_tol_eff, 1e-6);
     const FineCgBufs<float> B{c->fpa, c->fpb, c->fy, c->fq, c->fr, c->fs};
     cudaError_t e = launch_fine_cg_reg<float>(c->st, c->F, c->Tval, c->Ts32, c->sdiag, R, -1.0, c->cx, B, c->d_partial,
-                                              gs, tol, c->opt.lin_maxit, kReplace, c->d_res);
+                                              gs, tol, c->opt.lin_maxit, kReplace, c->h_res);
     kind = 4;
     if (e == cudaErrorNotSupported) {
       kind = 0;
       launch_scale_sell<float>(c->st, c->F, c->Tval, c->sdiag, c->Ts32);
       e = launch_fine_cg<float>(c->st, c->F, c->Ts32, c->sdiag, R, -1.0, c->cx, c->fy, c->fr, c->fpa, c->fpb, c->fq,
-                                c->d_partial, gs, tol, c->opt.lin_maxit, c->d_res);
+                                c->d_partial, gs, tol, c->opt.lin_maxit, c->h_res);
     }
     CK(e);
   } else {
@@ -712,7 +719,7 @@ int fine_pcg(nlmg_ctx* c, const double* R, const double* r) {
     if (pipe) {
       const FineCgBufs<double> B{c->dv1, c->dv2};
       e = launch_fine_cg_reg<double>(c->st, c->F, c->Tval, c->Ts64, c->sdiag, R, -1.0, c->cx, B, c->d_partial, gs,
-                                     c->lin_tol_eff, c->opt.lin_maxit, 0, c->d_res);
+                                     c->lin_tol_eff, c->opt.lin_maxit, 0, c->h_res);
       kind = 2;
     }
     if (e == cudaErrorNotSupported) {
@@ -720,18 +727,20 @@ int fine_pcg(nlmg_ctx* c, const double* R, const double* r) {
       kind = pipe ? 1 : 0;
       e = pipe ? launch_fine_cg_pipe<double>(c->st, c->F, c->Ts64, c->sdiag, R, -1.0, c->cx, c->cz, c->cr, c->cpa,
                                              c->cpb, c->cq, c->dv1, c->dv2, c->d_partial, gs, c->lin_tol_eff,
-                                             c->opt.lin_maxit, c->d_res)
+                                             c->opt.lin_maxit, c->h_res)
                : launch_fine_cg<double>(c->st, c->F, c->Ts64, c->sdiag, R, -1.0, c->cx, c->cz, c->cr, c->cpa, c->cpb,
-                                        c->cq, c->d_partial, gs, c->lin_tol_eff, c->opt.lin_maxit, c->d_res);
+                                        c->cq, c->d_partial, gs, c->lin_tol_eff, c->opt.lin_maxit, c->h_res);
     }
     CK(e);
   }
   c->last_fine_kind = kind;
   c->prof_end(pi);
   count_launch(1);
-  CK(cudaMemcpyAsync(c->h_res, c->d_res, sizeof(PcgResult), cudaMemcpyDeviceToHost, c->st));
   CK(cudaStreamSynchronize(c->st));
-  if (c->h_res->err) throw Error(NLMG_ETIMEOUT, "grid barrier wait gave up in the fine CG kernel");
+  if (c->h_res->err) {
+    c->reset_barrier();
+    throw Error(NLMG_ETIMEOUT, "grid barrier wait gave up in the fine CG kernel");
+  }
   if (!std::isfinite(c->h_res->rr)) throw Error(NLMG_EDIVERGED, "non-finite value in the level-0 linear solve");
   const int it = c->h_res->iters;
   if (pi >= 0) {
@@ -790,23 +799,24 @@ void newton_linearize(nlmg_ctx* c) {
 int fine_bicgstab(nlmg_ctx* c, const double* R) {
   if (c->opt.lin_precond == 1) return mg_bicgstab(c, R, c->t2.r);
   GridSync gs{c->d_bar, &c->d_res->err, c->sm_cap};
-  CK(cudaMemsetAsync(c->d_bar, 0, sizeof(unsigned), c->st));
-  CK(cudaMemsetAsync(c->d_res, 0, sizeof(PcgResult), c->st));
+  c->h_res->err = 1;
   const int pi = c->prof_begin(3);
   cudaError_t e = launch_fine_bicgstab_reg(c->st, c->F, c->Joff, c->Js, c->jdiag, c->jdinv, c->jsS, R, -1.0, c->cx,
-                                           c->gV, c->d_partial, gs, c->newton_tol_eff, c->opt.lin_maxit, c->d_res);
+                                           c->gV, c->d_partial, gs, c->newton_tol_eff, c->opt.lin_maxit, c->h_res);
   const bool reg = e != cudaErrorNotSupported;
   if (!reg) {
     launch_scale_jac(c->st, c->F, c->jdiag, c->Joff, c->jdinv, c->jsS, c->Js, c->jdS);
     e = launch_fine_bicgstab(c->st, c->F, c->Js, c->jdS, c->jsS, R, -1.0, c->cx, c->gV, c->d_partial, gs,
-                             c->newton_tol_eff, c->opt.lin_maxit, c->d_res);
+                             c->newton_tol_eff, c->opt.lin_maxit, c->h_res);
   }
   CK(e);
   c->prof_end(pi);
   count_launch(1);
-  CK(cudaMemcpyAsync(c->h_res, c->d_res, sizeof(PcgResult), cudaMemcpyDeviceToHost, c->st));
   CK(cudaStreamSynchronize(c->st));
-  if (c->h_res->err) throw Error(NLMG_ETIMEOUT, "grid barrier wait gave up in the fine BiCGStab kernel");
+  if (c->h_res->err) {
+    c->reset_barrier();
+    throw Error(NLMG_ETIMEOUT, "grid barrier wait gave up in the fine BiCGStab kernel");
+  }
   if (!std::isfinite(c->h_res->rr)) throw Error(NLMG_EDIVERGED, "non-finite value in the level-0 Newton solve");
   const int it = c->h_res->iters;
   if (pi >= 0) {
@@ -920,13 +930,7 @@ void newton_step(nlmg_ctx* c) {
   const int N = c->F.N;
   newton_linearize(c);
   fine_gmres(c, c->cur.R);
-  double s0 = 1.0;
-  if (c->opt.dp_clamp > 0) {
-    launch_max_abs(c->st, N, c->cx, c->red(S_MAX));
-    double mx = c->read_sc(S_MAX);
-    if (mx > c->opt.dp_clamp) s0 = c->opt.dp_clamp / mx;
-  }
-  backtrack0(c, c->cx, s0);
+  backtrack0(c, c->cx, clamp_scale(c, c->cx));
 }
 
 // A Newton smoothing step that leaves more than this fraction of the residual it started from shows that the
@@ -969,29 +973,26 @@ void smooth0(nlmg_ctx* c, int nu) {
     launch_sub(c->st, N, q, c->cur.p, c->cx);
     dp = c->cx;
   }
-  double s0 = 1.0;
-  if (o.dp_clamp > 0) {
-    launch_max_abs(c->st, N, dp, c->red(S_MAX));
-    double mx = c->read_sc(S_MAX);
-    if (mx > o.dp_clamp) s0 = o.dp_clamp / mx;
-  }
-  backtrack0(c, dp, s0);
+  backtrack0(c, dp, clamp_scale(c, dp));
   if (newton && !(c->cur.rn <= kNewtonKeep * rn_in)) c->newton_off = true;
 }
 
 // ---------------------------------------------------------------------------------------------------------------
 // coarse levels
 
-// r = A^l(x) - b (b may be null), kapc; returns ||r||.
-double coarse_res(nlmg_ctx* c, int l, const double* x, const double* b, double* r) {
+// r = A^l(x) - b (b may be null), kapc.
+void coarse_res(nlmg_ctx* c, int l, const double* x, const double* b, double* r) {
   const LevelDev& L = c->LD[l];
   CoarseBuf& B = c->CB[l];
   launch_coarse_cell(c->st, L, x, x + L.nflux, b ? b + L.nflux : nullptr, B.yl, r + L.nflux, B.kapc, c->kind, c->a,
                      c->red(S_NORM2));
   launch_coarse_flux(c->st, L, B.yl, b, r, c->red(S_NORM2B));
-  double v0, v1;
-  c->read_sc2(S_NORM2, v0, v1);
-  return std::sqrt(v0 + v1);
+}
+
+// The norm of the last coarse_res.
+double coarse_res_norm(nlmg_ctx* c) {
+  const double v0 = c->read_sc(S_NORM2);
+  return std::sqrt(v0 + c->h_sc[S_NORM2B]);
 }
 
 // x_{l+1} = Q x_l, b_{l+1} = A_{l+1}(x_{l+1}) - P^T r_l (r_l = [r_sigma; r_p] of level l >= 1 in CB[l].r)
@@ -1040,10 +1041,8 @@ void coarse_step(nlmg_ctx* c, int l, bool backtrack_first, int nsteps, bool coar
   P.tol_abs = c->tol_abs;
   P.maxit = c->opt.lin_maxit;
   GridSync gs{c->d_bar, &c->d_res->err, c->sm_cap};
-  CK(cudaMemsetAsync(c->d_bar, 0, sizeof(unsigned), c->st));
-  CK(cudaMemsetAsync(c->d_res, 0, sizeof(PcgResult), c->st));
-  CoarseStepResult* dres = (CoarseStepResult*)(c->d_res + 1);
-  CK(cudaMemsetAsync(dres, 0, sizeof(CoarseStepResult), c->st));
+  CoarseStepResult* res = (CoarseStepResult*)(c->h_res + 1);
+  res->err = 1;
   const int kid = coarsest ? 4 : 1;   // profile id: the coarsest solve apart from the other coarse steps
   int pi = c->prof_begin(kid);
   // FP64 whatever lin_precision is: the coarse levels are latency bound, FP32 would save nothing there. Pipelined
@@ -1055,14 +1054,15 @@ void coarse_step(nlmg_ctx* c, int l, bool backtrack_first, int nsteps, bool coar
                             pipe ? HybPipeBufs<double>{B.hw, B.hz, B.hs, B.hma, B.hmb} : HybPipeBufs<double>{},
                             B.hsv};
   bool sell = false;
-  CK(launch_coarse_step(c->st, L, L.Hc, L.Sinv, Bd, P, c->d_partial, gs, dres, &sell));
+  CK(launch_coarse_step(c->st, L, L.Hc, L.Sinv, Bd, P, c->d_partial, gs, res, &sell));
   c->prof_end(pi);
   count_launch(1);
-  CK(cudaMemcpyAsync(c->h_res, c->d_res, sizeof(PcgResult) + sizeof(CoarseStepResult), cudaMemcpyDeviceToHost,
-                     c->st));
   CK(cudaStreamSynchronize(c->st));
-  if (c->h_res->err) throw Error(NLMG_ETIMEOUT, "grid barrier wait gave up in the coarse step kernel");
-  const CoarseStepResult& R = *(const CoarseStepResult*)(c->h_res + 1);
+  const CoarseStepResult& R = *res;
+  if (R.err) {
+    c->reset_barrier();
+    throw Error(NLMG_ETIMEOUT, "grid barrier wait gave up in the coarse step kernel");
+  }
   if (R.bad)
     throw Error(NLMG_EDIVERGED, std::string("non-finite value in the ") +
                                     (R.bad == 1 ? "residual" : "hybridized linear solve") + " of coarse level " +
@@ -1114,7 +1114,7 @@ bool vcycle(nlmg_ctx* c, double r0, double tol_rel, double tol_abs) {
     CoarseBuf& Bc = c->CB[1];
     launch_sub(c->st, C.nflux + C.np, Bc.x, Bc.xc, Bc.ptmp);
     launch_prolong_p(c->st, c->TD[0], Bc.ptmp + C.nflux, c->fdp);
-    backtrack0(c, c->fdp, 1.0);
+    backtrack0(c, c->fdp, nullptr);
   }
   smooth0(c, o.nu_post);
   return false;
@@ -1131,7 +1131,8 @@ void cascade(nlmg_ctx* c) {
   make_coarse_problem(c, 0);
   for (int l = 1; l + 1 < nl; ++l) {
     CoarseBuf& B = c->CB[l];
-    B.rn = coarse_res(c, l, B.x, B.b, B.r);   // r = A(x) - b at the projected x, restricted below
+    coarse_res(c, l, B.x, B.b, B.r);   // r = A(x) - b at the projected x, restricted below
+    B.rn = coarse_res_norm(c);
     make_coarse_problem(c, l);
   }
   coarse_step(c, nl - 1, false, o.coarsest_steps, true);
@@ -1150,7 +1151,7 @@ void cascade(nlmg_ctx* c) {
   CoarseBuf& Bc = c->CB[1];
   launch_sub(c->st, C.nflux + C.np, Bc.x, Bc.xc, Bc.ptmp);
   launch_prolong_p(c->st, c->TD[0], Bc.ptmp + C.nflux, c->fdp);
-  backtrack0(c, c->fdp, 1.0);
+  backtrack0(c, c->fdp, nullptr);
 }
 
 void alloc_fine(nlmg_ctx* c) {
@@ -1520,10 +1521,11 @@ static void init_work(nlmg_ctx* c) {
   CK(cudaMemsetAsync(c->d_cnt, 0, 16 * sizeof(unsigned), c->st));
   c->d_sc = c->dalloc<double>(64);
   static_assert(sizeof(CoarseStepResult) <= 2 * sizeof(PcgResult), "result slots");
-  c->d_res = c->dalloc<PcgResult>(3);   // the CG result, then the coarse-step result (two slots)
-  c->d_bar = c->dalloc<unsigned>(64);   // count and generation on separate 128-byte lines
+  c->d_res = c->dalloc<PcgResult>(3);
+  c->d_bar = c->dalloc<unsigned>(64);   // the counter on its own 128-byte line
   CK(cudaMemsetAsync(c->d_bar, 0, 64 * sizeof(unsigned), c->st));
-  CK(cudaMallocHost(&c->h_res, 3 * sizeof(PcgResult)));
+  CK(cudaMemsetAsync(c->d_res, 0, 3 * sizeof(PcgResult), c->st));
+  CK(cudaMallocHost(&c->h_res, 3 * sizeof(PcgResult)));   // the CG result, then the coarse-step result (two slots)
   CK(cudaMemsetAsync(c->d_sc, 0, 64 * sizeof(double), c->st));
   c->reset_inner_tols();
   alloc_fine(c);
@@ -2192,12 +2194,12 @@ nlmg_status nlmg_check_grid_barrier(nlmg_ctx* c, int32_t blocks, int32_t absent_
       throw Error(NLMG_EINVAL, "nlmg_check_grid_barrier: blocks >= 1, absent_block < blocks and a spin limit in "
                                "[1024, 2^26] are required");
     GridSync gs{c->d_bar, &c->d_res->err, c->sm_cap};
-    CK(cudaMemsetAsync(c->d_bar, 0, sizeof(unsigned), c->st));
-    CK(cudaMemsetAsync(c->d_res, 0, sizeof(PcgResult), c->st));
+    c->reset_barrier();
     CK(launch_barrier_probe(c->st, gs, c->d_partial, blocks, absent_block, (unsigned long long)spin_limit,
                             &c->d_res->iters));
     count_launch(1);
     CK(cudaMemcpyAsync(c->h_res, c->d_res, sizeof(PcgResult), cudaMemcpyDeviceToHost, c->st));
+    c->reset_barrier();
     CK(cudaStreamSynchronize(c->st));
     if (passed) *passed = c->h_res->iters;
     if (c->h_res->err) {
