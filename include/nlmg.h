@@ -353,7 +353,7 @@ nlmg_status nlmg_profile_read(nlmg_ctx* ctx, int32_t kernel, int64_t* launches, 
  * they call: an application whose caching allocator already holds the device memory it may use (a cudaMalloc
  * there fails or forces the pool to give memory back), code under a fixed device-memory budget, and loops that must
  * not stall other streams (cudaFree, and often cudaMalloc, synchronize the device). It allocates nothing: the
- * per-cell kappa values and the reduction partial sums live in one fixed device array of this library (about
+ * per-cell values of 1 / kappa and the reduction partial sums live in one fixed device array of this library (about
  * 8.1 MiB, held on every device that loads the library until the process exits), and p_dev, r_dev, norm2_dev are
  * caller-owned device pointers. It computes exactly what nlmg_fine_residual computes, with the same kernels, on the
  * context's mesh and the context's current problem data: those of the last nlmg_set_data, or of the last solve
@@ -364,7 +364,7 @@ nlmg_status nlmg_profile_read(nlmg_ctx* ctx, int32_t kernel, int64_t* launches, 
  *   - the first call on a device resolves the array's device address (cudaGetSymbolAddress, checked), so make that
  *     first call before any stream capture.
  *   - every call reuses the same array, which keeps the last call's contents (the reduction's arrival counter is
- *     zeroed on the given stream by every call); calls that overlap on the GPU (on different streams, or from
+ *     zeroed by the first kernel of every call); calls that overlap on the GPU (on different streams, or from
  *     different contexts on the same device) race on it and must be serialized. */
 nlmg_status nlmg_fine_residual_noalloc(nlmg_ctx* ctx, const double* p_dev, double* r_dev, double* norm2_dev,
                                        void* stream);
@@ -378,7 +378,8 @@ nlmg_status nlmg_device_bytes(const nlmg_ctx* ctx, size_t* shared_bytes, size_t*
  * kernels is bounded: a block that has polled the barrier spin_limit times (about 2 s in the solver kernels) records
  * an error and every block leaves, so a solve returns NLMG_ETIMEOUT instead of hanging. This call runs that barrier
  * alone on the context's stream, in a cooperative launch of min(blocks, co-resident) blocks of which block
- * absent_block (< 0: none) leaves without arriving, with the given spin limit (1024 .. 2^26 polls of ~32 ns sleeps).
+ * absent_block (< 0: none) leaves without arriving, with the given spin limit (1024 .. 2^26 polls of about 0.2 us).
+ * Solver launches of at most 8 blocks are one thread-block cluster and wait in the hardware's cluster barrier instead.
  * Returns NLMG_ETIMEOUT when a wait gave up (the expected outcome with an absent block), NLMG_OK when every block
  * passed; *passed (may be NULL) receives the number of blocks whose wait completed. The context stays usable.
  * Errors: NLMG_EINVAL (bad arguments, host-only context), NLMG_ECUDA. */
