@@ -33,17 +33,14 @@ __device__ __forceinline__ void warp_sums(const double (&v)[NV][M], ISum (&s)[NV
   bool odd = false;
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
-    unsigned m = 0u;
+    unsigned m = 0u;   // the high word, its last bit set where only the low one holds a value
 #pragma unroll
-    for (int j = 0; j < M; ++j) m = max(m, (unsigned)__double2hiint(v[k][j]) & 0x7fffffffu);
-    mx[k] = (int)(__reduce_max_sync(0xffffffffu, m) >> 20);
-    if (mx[k] < 64) {   // zeros (an idle warp), or values next to the subnormals
-      bool nz = false;
-#pragma unroll
-      for (int j = 0; j < M; ++j) nz = nz || ((__double2hiint(v[k][j]) << 1) | __double2loint(v[k][j])) != 0;
-      odd = odd || __any_sync(0xffffffffu, nz);
-    }
-    odd = odd || mx[k] > 2032;
+    for (int j = 0; j < M; ++j)
+      m = max(m, ((unsigned)__double2hiint(v[k][j]) & 0x7fffffffu) | min((unsigned)__double2loint(v[k][j]), 1u));
+    m = __reduce_max_sync(0xffffffffu, m);
+    mx[k] = (int)(m >> 20);
+    // not zeros (an idle warp), but values next to the subnormals or to overflow
+    odd = odd || m - 1u < (64u << 20) - 1u || mx[k] > 2032;
   }
   if (odd) {   // the same in every lane
 #pragma unroll
@@ -107,12 +104,13 @@ __device__ __forceinline__ void warp_sums_i(const ISum (&v)[NV], double (&s)[NV]
     const int lo = __reduce_add_sync(0xffffffffu, (int)(x & 0x3fffff));
     const int mi = __reduce_add_sync(0xffffffffu, (int)((x >> 22) & 0x1fffff));
     const int hi = __reduce_add_sync(0xffffffffu, (int)(x >> 43));
-    // all bits of the sum in two exact parts, so that it is rounded once
+    // the sum in 63 bits: all of it, or, from 2^62 up, without its last six (an eighth of its rounding at most)
     const long long up = ((long long)hi << 21) + (long long)mi + (long long)(lo >> 22);
-    const double d = fma((double)up, 0x1p22, (double)(lo & 0x3fffff));
-    s[k] = up == 0 && (lo & 0x3fffff) == 0
-               ? 0.0
-               : __longlong_as_double(__double_as_longlong(d) + ((long long)(mx - 1077) << 52));
+    const int sh6 = (up >> 40) == (up >> 63) ? 0 : 6;
+    ISum r;
+    r.t = (up << (22 - sh6)) + (long long)((lo & 0x3fffff) >> sh6);
+    r.mx = mx + sh6;
+    s[k] = isum_value(r);
   }
 }
 
