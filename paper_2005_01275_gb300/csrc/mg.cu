@@ -901,6 +901,79 @@ __global__ void k_restr(int mbf, const float* __restrict__ res, const PT* __rest
   restr_body<PT, false>(gwarp(), nwarps(), mbf, res, Pl, ch_off, ch, ncc, mb, bc, dinvc, xc, dc, c2, first);
 }
 
+// The residual of a block level and its restriction in one pass: a block per cell A of the next level, a warp per child;
+// a child's residual stays in the lanes of its components, which take their terms of P^T res, and the warps' sums are
+// added in order. `first` adds the first Chebyshev step of the next level. What bounds these levels is the chain of
+// dependent kernels of a few microseconds each, so one launch less, and no way through memory for the residual: a CG
+// iteration on 229,360 cells 85.1 -> 81.3 us, on 64,000 cells 59.7 -> 56.7 us, of which two such pairs. (The same on
+// level 0, whose cells an aggregate reads out of order, loses: 81.3 -> 83.3 us, 10^6 cells 253.9 -> 263.2 us.)
+template <class PT, int MB>
+__global__ void __launch_bounds__(kT) k_res_restr(const int* __restrict__ rowptr, const int* __restrict__ col,
+                                                  const float* __restrict__ aval, const float* __restrict__ b,
+                                                  const float* __restrict__ x, const PT* __restrict__ Pl,
+                                                  const int* __restrict__ ch_off, const int* __restrict__ ch, int mb,
+                                                  float* __restrict__ bc, const float* __restrict__ dinvc,
+                                                  float* __restrict__ xc, float* __restrict__ dc,
+                                                  const float* __restrict__ lam, int lc, int first, const int* done) {
+  constexpr int NW = kT / 32;
+  __shared__ float s[NW][kMaxM];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, A = blockIdx.x;
+  const int t1 = ch_off[A + 1];
+  int t = ch_off[A] + warp, c = 0, q0 = 0, q1 = 0;
+  RowBatch<MB> R;
+  float P[kMaxM], acc[kMaxM], dv[kMaxM];
+  auto ahead = [&]() {
+    c = ch[t];
+    q0 = rowptr[c];
+    q1 = rowptr[c + 1];
+    R.load(q0 + (lane >> 3), q1, lane & 7, col, aval);
+#pragma unroll
+    for (int j = 0; j < kMaxM; ++j) P[j] = j < mb && lane < MB ? pval(Pl, ((size_t)c * MB + lane) * mb + j) : 0.0f;
+  };
+  if (t < t1) ahead();
+#pragma unroll
+  for (int j = 0; j < kMaxM; ++j) {
+    acc[j] = 0.0f;
+    dv[j] = first && warp == 0 && lane < mb && j < mb ? dinvc[((size_t)A * mb + lane) * mb + j] : 0.0f;
+  }
+  pdl_start();
+  if (stop(done)) return;
+  while (t < t1) {
+    const float bi = lane < MB ? b[(size_t)c * MB + lane] : 0.0f;
+    const float ax = row_ax<MB, false>(R, q0, q1, lane, col, aval, x);
+    const float res = lane < MB ? bi - ax : 0.0f;
+#pragma unroll
+    for (int j = 0; j < kMaxM; ++j) acc[j] = fmaf(P[j], res, acc[j]);
+    t += NW;
+    if (t < t1) ahead();
+  }
+#pragma unroll
+  for (int j = 0; j < kMaxM; ++j)
+    if (j < mb) {
+      acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], 1);
+      acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], 2);
+      acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], 4);
+      if (lane == 0) s[warp][j] = acc[j];
+    }
+  __syncthreads();
+  if (warp > 0) return;
+  float bj = 0.0f, dn = 0.0f;
+  if (lane < mb)
+#pragma unroll
+    for (int w = 0; w < NW; ++w) bj += s[w][lane];
+#pragma unroll
+  for (int j = 0; j < kMaxM; ++j) dn = fmaf(dv[j], __shfl_sync(0xffffffffu, bj, j), dn);
+  if (lane < mb) {
+    const size_t i = (size_t)A * mb + lane;
+    bc[i] = bj;
+    if (first) {
+      float c1, c2;
+      cheb_tab(lam, lc, 0, c1, c2);
+      xc[i] = dc[i] = c2 * dn;
+    }
+  }
+}
+
 // Level-0 residual b - A x (FP32), one thread per cell.
 __global__ void __launch_bounds__(kT, 6) k_res0(FineDev F, const float* __restrict__ a0off, const float* __restrict__ a0diag,
                        const float* __restrict__ b, const float* __restrict__ x, float* __restrict__ res,
@@ -1751,6 +1824,33 @@ void res_level(cudaStream_t st, const MgDev& M, const MgWork& W, int l, int cur,
   }
 }
 
+// Whether level l's residual and restriction are one kernel: where the residual takes a warp per cell, the blocks (one
+// per cell of level l+1) are at most a wave, four an SM, beyond which they lose their early loads and more than they save
+// (10^6 cells, 1,935 blocks: the CG iteration 250.8 -> 251.8 us; 64^3, 508 blocks: 98.0 -> 95.5), and aggregates are small
+// (with more than two children a warp few blocks walk a long chain).
+bool fused_restr(const MgDev& M, const MgWork& W, int l) {
+  return M.nc[l] < W.row_cells && M.nc[l + 1] <= kFusedMaxBlocks && M.nc[l] <= 16L * M.nc[l + 1];
+}
+
+// b_(l+1) = P^T (b_l - A x_l), and (first) level l+1's first smoothing step.
+template <class PT>
+void restrict_level(cudaStream_t st, const MgDev& M, const MgWork& W, int l, int cur, const PT* P, int first,
+                    const int* flag) {
+  const float* dinv = first ? W.dinv[l + 1] : nullptr;
+  float *xc = first ? W.x[l + 1][0] : nullptr, *dc = first ? W.d[l + 1] : nullptr;
+  if (fused_restr(M, W, l)) {
+    MG_MB_SWITCH(M.mb[l], launchk(st, M.nc[l + 1], kT, 0, k_res_restr<PT, MB>, (const int*)M.rowptr[l],
+                                  (const int*)M.col[l], (const float*)W.aval[l], (const float*)W.b[l],
+                                  (const float*)W.x[l][cur], P, (const int*)M.ch_off[l], (const int*)M.ch[l],
+                                  M.mb[l + 1], W.b[l + 1], dinv, xc, dc, (const float*)W.coef, l + 1, first, flag));
+  } else {
+    res_level(st, M, W, l, cur, flag);
+    launchk(st, warps_grid(M.nc[l + 1]), kT, 0, k_restr<PT>, M.mb[l], (const float*)W.d[l], P,
+            (const int*)M.ch_off[l], (const int*)M.ch[l], M.nc[l + 1], M.mb[l + 1], W.b[l + 1], dinv, xc, dc,
+            (const float*)W.coef, l + 1, first, flag);
+  }
+}
+
 }  // namespace
 
 void mg_enqueue_setup(cudaStream_t st, const MgDev& M, const FineDev& F, const MgWork& W, const double* Tval,
@@ -1932,30 +2032,12 @@ int mg_enqueue_vcycle(cudaStream_t st, const MgDev& M, const FineDev& F, const M
       cheb_level(st, M, W, l, k, cur[l], flag);
       cur[l] ^= 1;
     }
-    res_level(st, M, W, l, cur[l], flag);
-    if (l == top) break;
-    if (W.bf16)
-      launchk(st, warps_grid(M.nc[l + 1]), kT, 0, k_restr<__nv_bfloat16>, M.mb[l], (const float*)W.d[l],
-              (const __nv_bfloat16*)M.Pb[l], (const int*)M.ch_off[l], (const int*)M.ch[l], M.nc[l + 1],
-              M.mb[l + 1], W.b[l + 1], (const float*)W.dinv[l + 1], W.x[l + 1][0], W.d[l + 1],
-              (const float*)W.coef, l + 1, l + 1 < C ? 1 : 0, flag);
-    else
-      launchk(st, warps_grid(M.nc[l + 1]), kT, 0, k_restr<float>, M.mb[l], (const float*)W.d[l],
-              (const float*)M.P[l], (const int*)M.ch_off[l], (const int*)M.ch[l], M.nc[l + 1], M.mb[l + 1],
-              W.b[l + 1], (const float*)W.dinv[l + 1], W.x[l + 1][0], W.d[l + 1], (const float*)W.coef, l + 1,
-              l + 1 < C ? 1 : 0, flag);
+    const int first = l != top && l + 1 < C ? 1 : 0;   // (the map holds level top + 1's own)
+    if (W.bf16) restrict_level(st, M, W, l, cur[l], (const __nv_bfloat16*)M.Pb[l], first, flag);
+    else restrict_level(st, M, W, l, cur[l], (const float*)M.P[l], first, flag);
   }
-  if (tl > 0) {   // restriction to level tl, then the small levels' map back to level tl - 1
+  if (tl > 0) {   // the small levels' map back to level tl - 1
     const int nt = M.nc[tl] * M.mb[tl], rows = M.nc[tl - 1] * M.mb[tl - 1];
-    if (W.bf16)
-      launchk(st, warps_grid(M.nc[tl]), kT, 0, k_restr<__nv_bfloat16>, M.mb[tl - 1], (const float*)W.d[tl - 1],
-              (const __nv_bfloat16*)M.Pb[tl - 1], (const int*)M.ch_off[tl - 1], (const int*)M.ch[tl - 1], M.nc[tl],
-              M.mb[tl], W.b[tl], (const float*)nullptr, (float*)nullptr, (float*)nullptr, (const float*)W.coef, tl, 0,
-              flag);
-    else
-      launchk(st, warps_grid(M.nc[tl]), kT, 0, k_restr<float>, M.mb[tl - 1], (const float*)W.d[tl - 1],
-              (const float*)M.P[tl - 1], (const int*)M.ch_off[tl - 1], (const int*)M.ch[tl - 1], M.nc[tl], M.mb[tl],
-              W.b[tl], (const float*)nullptr, (float*)nullptr, (float*)nullptr, (const float*)W.coef, tl, 0, flag);
     launchk(st, (rows + 31) / 32, 32 * kApplyWarps, 0, k_tail_apply, rows, nt, (const float*)W.tailE,
             (const float*)W.b[tl], W.x[tl - 1][cur[tl - 1]], flag);
   } else {
@@ -2000,14 +2082,14 @@ int mg_enqueue_vcycle(cudaStream_t st, const MgDev& M, const FineDev& F, const M
   return cur[0];
 }
 
-int mg_vcycle_kernels(const MgDev& M) {
+int mg_vcycle_kernels(const MgDev& M, const MgWork& W) {
   const int C = M.L - 1, tl = mg_tail_level(M);
-  const int level0 = (kMgDegFine - 1) + 2 + 1 + kMgDegFine;   // smoothing, residual, restriction, prolongation
-  if (tl == 0) return level0 + (C - 1) * (kMgDegCoarse + 1) + 1 + (C - 1) * (1 + kMgDegCoarse);
-  // levels 1 .. tl-1 run their own kernels: down smoothing and residual, the restrictions between them, and on the
-  // way up the prolongations between them and the smoothing; the tail is two more (restriction, map)
-  const int own = tl - 1;
-  return level0 + 2 * own * kMgDegCoarse + 2 * (own - 1) + 2;
+  int n = (kMgDegFine - 1) + 2 + 1 + kMgDegFine;   // level 0: smoothing, residual, restriction, prolongation
+  // levels with their own kernels: smoothing, residual and restriction (one or two), and on the way up the prolongations
+  // between them; then the map, or the coarsest solve and the prolongation from it
+  const int own = tl > 0 ? tl - 1 : C - 1;
+  for (int l = 1; l <= own; ++l) n += (kMgDegCoarse - 1) + (fused_restr(M, W, l) ? 1 : 2) + kMgDegCoarse;
+  return n + (tl > 0 ? std::max(own - 1, 0) : own) + 1;
 }
 
 namespace {

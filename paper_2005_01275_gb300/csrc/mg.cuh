@@ -25,6 +25,7 @@ constexpr int kMgDegFine = 2;       // Chebyshev steps before and after the coar
 constexpr int kMgDegCoarse = 2;     // the same on levels 1 .. L-2
 constexpr double kMgAlpha = 4.0;    // Chebyshev interval [lam / alpha, lam]
 constexpr int kMgMaxDeg = 4;        // Chebyshev steps per smoothing at most (coefficient table size)
+constexpr int kFusedMaxBlocks = 608;  // largest grid of the fused residual and restriction (see fused_restr)
 constexpr int kTailThreads = 1024;  // threads of a block of the small levels' setup (k_tail_cols)
 constexpr int kTailMaxUnknowns = 512;   // the small levels start at the first l >= 2 with at most this many unknowns ...
 constexpr size_t kTailSmem = 200 * 1024;   // ... whose data from there on fit this much shared memory
@@ -137,7 +138,7 @@ void mg_fill_tail(cudaStream_t st, const MgDev& M, MgWork& W);
 int mg_tail_level(const MgDev& M);
 
 // Kernels in one V-cycle after its fused first step (for the launch counts of graph replays).
-int mg_vcycle_kernels(const MgDev& M);
+int mg_vcycle_kernels(const MgDev& M, const MgWork& W);
 
 // The preconditioned Krylov solves as graphs captured once per context (out[0] the start, out[1] a conditional
 // while loop over the iterations; tolerance tol2 and cap maxit read from W.sc at run time), and one V-cycle for the

@@ -1281,7 +1281,7 @@ int mg_pcg(nlmg_ctx* c, const double* R, const double* r) {
   CK(cudaGraphLaunch(W.g_pcg[1], c->st));
   c->prof_end(pi);
   const int it = mg_finish(c, "multigrid-preconditioned CG");
-  const int V = mg_vcycle_kernels(M);
+  const int V = mg_vcycle_kernels(M, W);
   count_launch(1 + std::max(it, 1) * (2 + V));   // the start, then one loop body per iteration
   if (pi >= 0) {
     c->prof.bytes[5] += (double)it * (c->sh->mg_bytes_vcycle + c->sh->mg_bytes_iter);
@@ -1310,7 +1310,7 @@ int mg_bicgstab(nlmg_ctx* c, const double* R, const double* r) {
   CK(cudaGraphLaunch(W.g_bicg[1], c->st));
   c->prof_end(pi);
   const int it = mg_finish(c, "multigrid-preconditioned BiCGStab");
-  const int V = mg_vcycle_kernels(M);
+  const int V = mg_vcycle_kernels(M, W);
   count_launch(1 + std::max(it, 1) * (5 + 2 * V));
   if (pi >= 0) {
     c->prof.bytes[6] += (double)(2 * it) * c->sh->mg_bytes_vcycle + (double)it * 2.0 * c->sh->mg_bytes_iter;
@@ -2028,7 +2028,7 @@ nlmg_status nlmg_precond_apply(nlmg_ctx* c, const double* p, const double* r, do
     CK(cudaMemcpyAsync(W.kb, r, N * sizeof(double), cudaMemcpyHostToDevice, c->st));
     if (!W.g_apply) CK(mg_capture_apply(c->st, M, c->F, W, &W.g_apply));
     CK(cudaGraphLaunch(W.g_apply, c->st));
-    count_launch(2 + mg_vcycle_kernels(M));
+    count_launch(2 + mg_vcycle_kernels(M, W));
     CK(cudaMemcpyAsync(z_out, W.kx, N * sizeof(double), cudaMemcpyDeviceToHost, c->st));
     CK(cudaStreamSynchronize(c->st));
     return NLMG_OK;

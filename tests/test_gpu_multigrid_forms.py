@@ -1,13 +1,14 @@
 """The multigrid preconditioner's kernels over the mode counts and level sizes that choose between them.
 
 A cell's block takes one to eight modes (a group of lanes a block, padded where a level's mode counts differ), the
-levels of at most 512 unknowns are one precomputed map, and the coarsest level's inverse is formed by a cluster whatever
-its order. The cases put the map's boundary on both sides of level 1 (63 cells of 8 modes are 504 unknowns, 213 cells of
-3 are 639), leave it nothing but the coarsest level (63 cells of one mode end the cycle at level 1), and have odd and
-mixed mode counts. One application is compared with the oracle's FP64 cycle: FP32 rounding (6e-8) times the conditioning
-of the cell blocks (at most 5.3e3 here) or of the coarsest matrix (at most 2.2e4) is at most 1.3e-3, and 2e-3 is taken; a
-wrong index or a lost term shows at 1e-1. The Picard update must meet its own tolerance on the oracle's matrix, in the
-oracle's number of steps to a tenth.
+levels of at most 512 unknowns are one precomputed map, and the coarsest level's inverse is formed by a cluster
+whatever its order. The cases put the map's boundary on both sides of level 1 (63 cells of 8 modes are 504 unknowns,
+213 cells of 3 are 639), leave it nothing but the coarsest level (63 cells of one mode end the cycle at level 1), have
+odd and mixed mode counts, and aggregates of level-1 cells both small (residual and restriction in one kernel) and
+large (two kernels). One application is compared with the oracle's FP64 cycle: FP32 rounding (6e-8) times the
+conditioning of the cell blocks (at most 5.3e3 here) or of the coarsest matrix (at most 2.2e4) is at most 1.3e-3, and
+2e-3 is taken; a wrong index or a lost term shows at 1e-1. The Picard update must meet its own tolerance on the
+oracle's matrix, in the oracle's number of steps to a tenth.
 """
 import numpy as np
 import pytest
@@ -24,6 +25,7 @@ pytestmark = pytest.mark.gpu
                                                   ("chan3d_64", 24, [64, 8, 8], [3, 3, 3]),
                                                   ("chan3d_64", 24, [64, 8, 8], [6, 5, 2]),
                                                   ("chan3d_64", 21, [48, 6, 6], [7, 4, 4]),
+                                                  ("chan3d_64", 24, [8, 27, 8], [2, 2, 2]),
                                                   ("cart2d_32", 32, [16, 4, 4], [2, 3, 2])])
 def test_mode_counts_and_level_sizes(nlmg_lib, name, scale, agg, modes):
     pr = problem_config(name, scale=scale)
