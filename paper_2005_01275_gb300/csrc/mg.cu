@@ -1,8 +1,8 @@
 // Linear multigrid preconditioner for the level-0 Krylov solves (see mg.cuh), and the preconditioned CG / BiCGStab
 // that use it, each captured once per context as CUDA graphs with a device-side conditional while loop.
 //
-// Every reduction is deterministic: per-block partial sums, then the grid's last block adds the partials, both exactly
-// (the arrival counter is reset by that block, so graphs replay). Maxima are exact.
+// Every reduction is deterministic: per-block partial sums, then the grid's last block adds the partials, both in
+// integers (isum.cuh; the arrival counter is reset by that block, so graphs replay). Maxima are exact.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -48,9 +48,8 @@ inline int blocks_for(long n, int cap = 1 << 20) {
 // ---------------------------------------------------------------------------------------------------------------
 // reductions
 
-// Sums NV values over the grid: block sums to part[block][k]; the last block to arrive adds the partials (exactly, hence
-// in no particular order; at most kMaxRedBlocks) and returns true in its warp 0 with the sums in out. The counter is left
-// at zero. On the integer pipes (isum.cuh): block trees, 1,024 partials and their trees took 2 us at the end of a kernel.
+// Sums NV values over the grid: block sums to part[block][k]; the last block to arrive adds the partials (at most
+// kMaxRedBlocks) and returns true in its warp 0 with the sums in out. The counter is left at zero. On the integer pipes (isum.cuh): block trees, 1,024 partials and their trees took 2 us at the end of a kernel.
 template <int NV>
 __device__ bool reduce_last(double (&v)[NV], double* part, unsigned* cnt, double (&out)[NV]) {
   __shared__ ISum sh[NV * 32];

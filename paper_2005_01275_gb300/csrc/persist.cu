@@ -10,7 +10,7 @@
 // with ld.global.cg (L2, bypassing the non-coherent L1), after the barrier that orders the write.
 //
 // Reductions stay deterministic: each block writes one partial per value; after the barrier every block adds all
-// partials (exactly, hence in no particular order) and derives the step lengths once, so all blocks take the same
+// partials (in integers, isum.cuh) and derives the step lengths once, so all blocks take the same
 // decisions from bit-identical scalars and a run is bitwise reproducible for a given grid.
 #include <cmath>
 

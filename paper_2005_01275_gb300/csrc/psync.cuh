@@ -171,7 +171,9 @@ __device__ __forceinline__ void grid_sum_finish(const Grid& g, double (&s)[NV]) 
       if (k + 1 < NV) a[k + 1][j] = x.y;
     }
   }
-  for (int b = 32 * M + lane; b < G; b += 32)   // larger grids: the rest onto the lane's first value
+  // larger grids (the memory-resident kernels put two blocks on an SM): the rest onto the lane's first value in double, in
+  // block order
+  for (int b = 32 * M + lane; b < G; b += 32)
 #pragma unroll
     for (int k = 0; k < NV; ++k) a[k][0] += __ldcg((const double*)part + b * ST + k);
   warp_sums<NV, M>(a, t);
