@@ -125,10 +125,49 @@ __global__ void k_rhs(FineDev F, const double* __restrict__ f, const double* __r
   }
 }
 
-// The transmissibility 1 / d of a face, d = r_K / Ups_K + r_L / Ups_L (rare: a d at the ends of the exponent range, where
-// two vanishing kappas have no harmonic mean).
-__device__ __noinline__ double face_rare(double d, double rK, double rL) {
-  return isinf(rK) && isinf(rL) ? __longlong_as_double(0x7ff8000000000000ll) : 1.0 / d;
+// The transmissibility T = ha hb / (ha + hb) of a face from its kappa-scaled halves, and the w_K, w_L of dT/dp = -T w (T / ha
+// and T / hb times the kappas' rates): where 1 / kappa leaves the range of its reciprocal (see level0_r).
+struct FaceRare {
+  double T, wK, wL;
+};
+__device__ __forceinline__ FaceRare face_rare(double pK, double pL, double us, double un, int kind, double a) {
+  const double ha = kappa_of(pK, kind, a) * us, hb = kappa_of(pL, kind, a) * un, t = hb / (ha + hb);
+  return FaceRare{ha * t, -t * kappa_rate(pK, kind, a), -(ha / (ha + hb)) * kappa_rate(pL, kind, a)};
+}
+__device__ __noinline__ double face_rare_T(double pK, double pL, double us, double un, int kind, double a) {
+  return face_rare(pK, pL, us, un, kind, a).T;
+}
+// A row of k_residual in that form. A call for the whole row, after its loop, in a kernel compiled for five blocks an SM
+// (48 registers): a call for a face in the loop, and its 64 registers, took 168 us for 10^6 cells instead of 139.
+struct RowRare {
+  double flux, dsum, jd;
+};
+template <bool MAT, bool JAC>
+__device__ __noinline__ RowRare row_rare(const FineDev& F, int K, const double* __restrict__ q,
+                                         const double* __restrict__ g, double* __restrict__ Tval,
+                                         double* __restrict__ Joff, int kind, double a) {
+  RowRare s{0.0, 0.0, 0.0};
+  const double qK = q[K];
+  const int w = F.sell_w[K >> 5];
+  int e = F.sell_off[K >> 5] + (K & 31);
+  for (int j = 0; j < w; ++j, e += 32) {
+    const int L = F.nbr[e];
+    FaceRare f{0.0, 0.0, 0.0};
+    if (L != K) f = face_rare(qK, q[L], 1.0 / F.iu_s[e], 1.0 / F.iu_n[e], kind, a);
+    const double td = f.T * (qK - q[L]);
+    s.flux += td;
+    s.dsum += f.T;
+    if (MAT) Tval[e] = f.T;
+    if (JAC) s.jd += fma(-td, f.wK, f.T);
+    if (JAC && Joff) Joff[e] = -fma(td, f.wL, f.T);
+  }
+  for (int e = F.dir_off[K]; e < F.dir_off[K + 1]; ++e) {
+    const double h = kappa_of(qK, kind, a) * F.dir_ups[e], hd = h * (qK - g[F.dir_face[e]]);
+    s.flux += hd;
+    s.dsum += h;
+    s.jd += fma(hd, kappa_rate(qK, kind, a), h);
+  }
+  return s;
 }
 
 // R_K = sum_faces Ups_f (q_K - q_L) + sum_Dirichlet kappa_K Ups_K (q_K - g) - [f]_K  (eqs. TPFA_flux, FV_matrix).
@@ -137,18 +176,20 @@ __device__ __noinline__ double face_rare(double d, double rK, double rL) {
 // Bounded by FP64 issue: 7 operations an entry (2 for d, 3 for its reciprocal, the difference, the flux) and 1 for the
 // diagonal. 10^6 cells: with a division, and a diagonal nobody asked for, an entry: 200 us; now about 110; its 125 MB would take 19.
 template <bool MAT, bool JAC>
-__global__ void __launch_bounds__(kThreads) k_residual(FineDev F, const double* __restrict__ q,
+__global__ void __launch_bounds__(kThreads, 5) k_residual(const __grid_constant__ FineDev F,
+                                                       const double* __restrict__ q,
                                                        const double* __restrict__ r, const double* __restrict__ dr,
                                                        const double* __restrict__ g,
                                                        const double* __restrict__ rhs, double* __restrict__ R,
                                                        double* __restrict__ Tval, double* __restrict__ diagT,
                                                        double* __restrict__ jdiag, double* __restrict__ Joff,
-                                                       Reduce red) {
+                                                       Reduce red, int kind, double a) {
   double acc[1] = {0.0};
   GRID_STRIDE(K, F.N) {
     const double qK = q[K], rK = r[K];
     const double drK = JAC ? dr[K] : 0.0;
     double flux = 0.0, dsum = 0.0, jd = 0.0;
+    bool rare = false;   // some face's 1 / kappa is out of range
     const int w = F.sell_w[K >> 5];
     int e = F.sell_off[K >> 5] + (K & 31);
 #pragma unroll 2
@@ -156,25 +197,35 @@ __global__ void __launch_bounds__(kThreads) k_residual(FineDev F, const double* 
       const int L = F.nbr[e];
       const double is = F.iu_s[e], in = F.iu_n[e], rL = r[L];
       const double d = fma(rK, is, rL * in);
-      double T = rcp_in_range(d) ? rcp_core(d) : face_rare(d, rK, rL);
+      rare |= !rcp_in_range(d);
+      double T = rcp_core(d);
       if (L == K) T = 0.0;   // padding
       const double diff = qK - q[L];
       flux = fma(T, diff, flux);
       if (MAT || JAC) dsum += T;
       if (MAT) Tval[e] = T;
       if (JAC) {
-        // dT/dp_K = -T^2 r_K' / Ups_K, so dR_K/dp_K = T - T^2 r_K' / Ups_K (p_K - p_L), dR_K/dp_L likewise
-        const double w2 = T * T * diff;
-        jd += fma(-w2 * is, drK, T);
-        if (Joff) Joff[e] = L == K ? 0.0 : -fma(w2 * in, dr[L], T);
+        // dT/dp_K = -T w_K with w_K = T r_K' / Ups_K (bounded by the kappa's rate, where T^2 leaves the range for kappas
+        // beyond 10^+-154), so dR_K/dp_K = T - T w_K (p_K - p_L), dR_K/dp_L = -T - T w_L (p_K - p_L)
+        const double td = T * diff;
+        jd += fma(-td, T * is * drK, T);
+        if (Joff) Joff[e] = L == K ? 0.0 : -fma(td, T * in * dr[L], T);
       }
     }
-    for (int e = F.dir_off[K]; e < F.dir_off[K + 1]; ++e) {
+    const int d0 = F.dir_off[K], d1 = F.dir_off[K + 1];
+    rare |= d1 > d0 && !rcp_in_range(rK);
+    for (int e = d0; e < d1; ++e) {
       const double h = fast_div(F.dir_ups[e], rK);
       const double diff = qK - g[F.dir_face[e]];
       flux = fma(h, diff, flux);
       if (MAT || JAC) dsum += h;
-      if (JAC) jd += fma(-fast_div(h, rK) * drK, diff, h);
+      if (JAC) jd += fma(-h * fast_div(drK, rK), diff, h);
+    }
+    if (rare) {
+      const RowRare s = row_rare<MAT, JAC>(F, K, q, g, Tval, Joff, kind, a);
+      flux = s.flux;
+      dsum = s.dsum;
+      jd = s.jd;
     }
     const double res = flux - rhs[K];
     R[K] = res;
@@ -227,14 +278,16 @@ __global__ void k_sub(int n, const double* __restrict__ y, const double* __restr
 }
 
 // TPFA flux on each level-0 flux unknown, oriented out of K (eq. TPFA_flux).
-__global__ void k_fine_flux(FineDev F, const double* __restrict__ p, const double* __restrict__ r,
-                            const double* __restrict__ g, double* __restrict__ sigma) {
+__global__ void __launch_bounds__(kThreads, 6) k_fine_flux(FineDev F, const double* __restrict__ p, const double* __restrict__ r,
+                            const double* __restrict__ g, double* __restrict__ sigma, int kind, double a) {
   GRID_STRIDE(j, F.nflux) {
     const int K = F.fl_k[j], L = F.fl_l[j];
-    const double rK = r[K], rL = L >= 0 ? r[L] : 0.0;
-    const double d = L >= 0 ? fma(rK, F.fl_u0[j], rL * F.fl_u1[j]) : rK * F.fl_u0[j];
-    const double T = rcp_in_range(d) ? rcp_core(d) : face_rare(d, rK, rL);
-    sigma[j] = T * (p[K] - (L >= 0 ? p[L] : g[F.fl_face[j]]));
+    const double rK = r[K], pK = p[K], pL = L >= 0 ? p[L] : g[F.fl_face[j]];
+    const double d = L >= 0 ? fma(rK, F.fl_u0[j], r[L] * F.fl_u1[j]) : rK * F.fl_u0[j];
+    double T = rcp_core(d);
+    if (!rcp_in_range(d))
+      T = L >= 0 ? face_rare_T(pK, pL, 1.0 / F.fl_u0[j], 1.0 / F.fl_u1[j], kind, a) : kappa_of(pK, kind, a) / F.fl_u0[j];
+    sigma[j] = T * (pK - pL);
   }
 }
 
@@ -524,11 +577,11 @@ void launch_rhs(cudaStream_t st, const FineDev& F, const double* f, const double
 }
 void launch_residual(cudaStream_t st, const FineDev& F, const double* q, const double* r, const double* dr,
                      const double* g, const double* rhs, double* R, double* Tval, double* diagT, double* jdiag,
-                     Reduce red, double* Joff) {
+                     Reduce red, int kind, double a, double* Joff) {
   COUNT(1);
   const auto k = jdiag ? (Tval ? k_residual<true, true> : k_residual<false, true>)
                        : (Tval ? k_residual<true, false> : k_residual<false, false>);
-  k<<<grid_for(F.N), kThreads, 0, st>>>(F, q, r, dr, g, rhs, R, Tval, diagT, jdiag, Joff, red);
+  k<<<grid_for(F.N), kThreads, 0, st>>>(F, q, r, dr, g, rhs, R, Tval, diagT, jdiag, Joff, red, kind, a);
 }
 void launch_jacobi_update(cudaStream_t st, int n, const double* q, const double* R, const double* jdiag,
                           const double* diagT, double omega, double* qnew) {
@@ -548,9 +601,9 @@ void launch_sub(cudaStream_t st, int n, const double* y, const double* x, double
   k_sub<<<grid_for(n), kThreads, 0, st>>>(n, y, x, out);
 }
 void launch_fine_flux(cudaStream_t st, const FineDev& F, const double* p, const double* r, const double* g,
-                      double* sigma) {
+                      double* sigma, int kind, double a) {
   COUNT(1);
-  k_fine_flux<<<grid_for(F.nflux), kThreads, 0, st>>>(F, p, r, g, sigma);
+  k_fine_flux<<<grid_for(F.nflux), kThreads, 0, st>>>(F, p, r, g, sigma, kind, a);
 }
 void launch_restrict_p(cudaStream_t st, const TransferDev& T, const double* in1, double* out1, double scale1,
                        const double* in2, double* out2) {

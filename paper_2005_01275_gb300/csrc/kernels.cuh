@@ -45,9 +45,14 @@ __device__ __forceinline__ double kappa_of(double p, int kind, double a) {
 __device__ __forceinline__ double inv_kappa_of(double p, int kind, double a) {
   return kind == 0 ? exp(-a * p) : fma(p, p, 1.0);
 }
+// kappa'(p) / kappa(p)
+__device__ __forceinline__ double kappa_rate(double p, int kind, double a) {
+  return kind == 0 ? a : -2.0 * p / fma(p, p, 1.0);
+}
 // What the level-0 kernels carry per cell: r = 1 / kappa(p), whose face transmissibility 1 / (r_K / Ups_K + r_L / Ups_L)
 // needs one reciprocal and seven FP64 operations an entry (a division of kappas took sixteen), and r' = dr/dp where the
-// Jacobian is formed. A kappa that overflows is not a number here, as its transmissibilities are.
+// Jacobian is formed. Faces whose sum leaves the reciprocal's range (a kappa beyond 10^+-289) are formed from the kappas
+// instead; r is not a number where kappa overflows, so that those are among them.
 __device__ __forceinline__ double level0_r(double p, int kind, double a) {
   const double r = inv_kappa_of(p, kind, a);
   return r < 0x1p-1024 ? __longlong_as_double(0x7ff8000000000000ll) : r;   // 1 / DBL_MAX rounds to 2^-1024
@@ -119,7 +124,7 @@ void launch_rhs(cudaStream_t st, const FineDev& F, const double* f, const double
 // diagT): the exact Jacobian.
 void launch_residual(cudaStream_t st, const FineDev& F, const double* q, const double* r, const double* dr,
                      const double* g, const double* rhs, double* R, double* Tval, double* diagT, double* jdiag,
-                     Reduce red, double* Joff = nullptr);
+                     Reduce red, int kind, double a, double* Joff = nullptr);
 void launch_jac_apply(cudaStream_t st, const FineDev& F, const double* jdiag, const double* Joff,
                       const double* dinv, const double* v, double* w);
 void launch_mdot(cudaStream_t st, int n, int nk, const double* V, const double* w, double* partial,
@@ -137,7 +142,7 @@ void launch_clamp_scale(cudaStream_t st, int n, const double* x, double clamp, R
 void launch_axpy(cudaStream_t st, int n, const double* x, double s, const double* dx, double* out);
 void launch_sub(cudaStream_t st, int n, const double* y, const double* x, double* out);
 void launch_fine_flux(cudaStream_t st, const FineDev& F, const double* p, const double* r, const double* g,
-                      double* sigma);
+                      double* sigma, int kind, double a);
 void launch_restrict_p(cudaStream_t st, const TransferDev& T, const double* in1, double* out1, double scale1,
                        const double* in2, double* out2);
 void launch_prolong_p(cudaStream_t st, const TransferDev& T, const double* e, double* out);

@@ -49,7 +49,8 @@ inline int blocks_for(long n, int cap = 1 << 20) {
 // reductions
 
 // Sums NV values over the grid: block sums to part[block][k]; the last block to arrive adds the partials (at most
-// kMaxRedBlocks) and returns true in its warp 0 with the sums in out. The counter is left at zero. On the integer pipes (isum.cuh): block trees, 1,024 partials and their trees took 2 us at the end of a kernel.
+// kMaxRedBlocks) and returns true in its warp 0 with the sums in out. The counter is left at zero. On
+// the integer pipes (isum.cuh): block trees, 1,024 partials and their trees took 2 us at the end of a kernel.
 template <int NV>
 __device__ bool reduce_last(double (&v)[NV], double* part, unsigned* cnt, double (&out)[NV]) {
   __shared__ ISum sh[NV * 32];

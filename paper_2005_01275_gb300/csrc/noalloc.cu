@@ -60,7 +60,7 @@ bool noalloc_residual(cudaStream_t st, void* scratch, const FineDev& F, const do
   NoallocScratch* S = (NoallocScratch*)scratch;
   launch_kappa(st, F.N, p, nullptr, 0.0, const_cast<double*>(p), S->kap, nullptr, kind, a, &S->counter);
   Reduce red{S->partial, &S->counter, norm2};
-  launch_residual(st, F, p, S->kap, nullptr, g, rhs, r, nullptr, nullptr, nullptr, red);
+  launch_residual(st, F, p, S->kap, nullptr, g, rhs, r, nullptr, nullptr, nullptr, red, kind, a);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     err = std::string("kernel launch: ") + cudaGetErrorString(e);

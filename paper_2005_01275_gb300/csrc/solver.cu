@@ -644,7 +644,8 @@ void upload_mg(nlmg_ctx* c, int levels) {
 double fine_eval(nlmg_ctx* c, const double* p, const double* dp, double s, FineState& out, const double* scale = nullptr) {
   launch_kappa(c->st, c->F.N, p, dp, s, out.p, out.r, nullptr, c->kind, c->a, nullptr, scale);
   int pi = c->prof_begin(2);
-  launch_residual(c->st, c->F, out.p, out.r, nullptr, c->g, c->rhs, out.R, nullptr, nullptr, nullptr, c->red(S_NORM2));
+  launch_residual(c->st, c->F, out.p, out.r, nullptr, c->g, c->rhs, out.R, nullptr, nullptr, nullptr, c->red(S_NORM2),
+                  c->kind, c->a);
   c->prof_end(pi);
   c->fine_evals++;
   out.rn = std::sqrt(c->read_sc(S_NORM2));
@@ -789,8 +790,8 @@ void newton_linearize(nlmg_ctx* c) {
   const int N = c->F.N;
   launch_kappa(c->st, N, c->cur.p, nullptr, 0.0, c->cur.p, c->t2.r, c->dr, c->kind, c->a);
   launch_residual(c->st, c->F, c->cur.p, c->t2.r, c->dr, c->g, c->rhs, c->t2.R,
-                  c->opt.lin_precond == 1 ? c->Tval : nullptr, c->diagT, c->jdiag, c->red(S_NORM2B),
-                  c->Joff);
+                  c->opt.lin_precond == 1 ? c->Tval : nullptr, c->diagT, c->jdiag, c->red(S_NORM2B), c->kind,
+                  c->a, c->Joff);
   launch_jacobi_dinv(c->st, N, c->jdiag, c->diagT, c->jdinv, c->jsS);
 }
 
@@ -954,7 +955,7 @@ void smooth0(nlmg_ctx* c, int nu) {
     c->newton_steps++;
   } else if (o.smoother == NLMG_SMOOTH_PICARD || o.smoother == NLMG_SMOOTH_PICARD_NEWTON) {
     launch_residual(c->st, c->F, c->cur.p, c->cur.r, nullptr, c->g, c->rhs, c->t2.R, c->Tval, c->diagT, nullptr,
-                    c->red(S_NORM2B));
+                    c->red(S_NORM2B), c->kind, c->a);
     fine_pcg(c, c->cur.R, c->cur.r);
     dp = c->cx;
   } else {
@@ -965,7 +966,7 @@ void smooth0(nlmg_ctx* c, int nu) {
     for (int k = 0; k < nu; ++k) {
       launch_kappa(c->st, N, q, nullptr, 0.0, q, c->t2.r, c->dr, c->kind, c->a);
       launch_residual(c->st, c->F, q, c->t2.r, c->dr, c->g, c->rhs, c->t2.R, nullptr, c->diagT, c->jdiag,
-                      c->red(S_NORM2B));
+                      c->red(S_NORM2B), c->kind, c->a);
       launch_jacobi_update(c->st, N, q, c->t2.R, c->jdiag, c->diagT, o.omega, qn);
       std::swap(q, qn);
       c->fine_evals++;
@@ -1001,7 +1002,8 @@ void make_coarse_problem(nlmg_ctx* c, int l) {
   const LevelDev& C = c->LD[l + 1];
   CoarseBuf& Bc = c->CB[l + 1];
   if (l == 0) {
-    launch_fine_flux(c->st, c->F, c->cur.p, c->cur.r, c->g, c->sig0);   // cur.r: of the evaluation that made cur
+    launch_fine_flux(c->st, c->F, c->cur.p, c->cur.r, c->g, c->sig0, c->kind,
+                     c->a);   // cur.r: of the evaluation that made cur
     launch_csr(c->st, T.qs_n, T.qs_off, T.qs_col, T.qs_val, c->sig0, Bc.x, 1.0, 0.0);
     // projection of p and restriction of the mixed pressure residual -R
     launch_restrict_p(c->st, T, c->cur.p, Bc.x + C.nflux, 1.0, c->cur.R, Bc.ptmp + C.nflux);
@@ -1910,7 +1912,7 @@ nlmg_status nlmg_fine_flux(nlmg_ctx* c, const double* p, double* sigma_out) {
     need_data(c);
     CK(cudaMemcpyAsync(c->cpa, p, (size_t)c->F.N * sizeof(double), cudaMemcpyHostToDevice, c->st));
     launch_kappa(c->st, c->F.N, c->cpa, nullptr, 0.0, c->cpa, c->t1.r, nullptr, c->kind, c->a);
-    launch_fine_flux(c->st, c->F, c->cpa, c->t1.r, c->g, c->sig0);
+    launch_fine_flux(c->st, c->F, c->cpa, c->t1.r, c->g, c->sig0, c->kind, c->a);
     CK(cudaMemcpyAsync(sigma_out, c->sig0, (size_t)c->F.nflux * sizeof(double), cudaMemcpyDeviceToHost, c->st));
     CK(cudaStreamSynchronize(c->st));
     return NLMG_OK;
@@ -1951,7 +1953,7 @@ nlmg_status nlmg_transfer(nlmg_ctx* c, int32_t level, int32_t op, const double* 
         if (level == 0) {
           need_data(c);
           launch_kappa(c->st, c->F.N, fin, nullptr, 0.0, fin, c->t1.r, nullptr, c->kind, c->a);
-          launch_fine_flux(c->st, c->F, fin, c->t1.r, c->g, c->sig0);
+          launch_fine_flux(c->st, c->F, fin, c->t1.r, c->g, c->sig0, c->kind, c->a);
           launch_csr(c->st, T.qs_n, T.qs_off, T.qs_col, T.qs_val, c->sig0, Bc.xt2, 1.0, 0.0);
         } else {
           launch_csr(c->st, T.qs_n, T.qs_off, T.qs_col, T.qs_val, fin, Bc.xt2, 1.0, 0.0);
@@ -1989,7 +1991,7 @@ nlmg_status nlmg_picard_update(nlmg_ctx* c, int32_t level, const double* x, cons
       CK(cudaMemcpyAsync(c->cpa, x, (size_t)c->F.N * sizeof(double), cudaMemcpyHostToDevice, c->st));
       fine_eval(c, c->cpa, nullptr, 0.0, c->t1);
       launch_residual(c->st, c->F, c->t1.p, c->t1.r, nullptr, c->g, c->rhs, c->t2.R, c->Tval, c->diagT, nullptr,
-                    c->red(S_NORM2B));
+                    c->red(S_NORM2B), c->kind, c->a);
       it = fine_pcg(c, c->t1.R, c->t1.r);
       CK(cudaMemcpyAsync(dx_out, c->cx, (size_t)c->F.N * sizeof(double), cudaMemcpyDeviceToHost, c->st));
     } else {
@@ -2022,7 +2024,7 @@ nlmg_status nlmg_precond_apply(nlmg_ctx* c, const double* p, const double* r, do
     CK(cudaMemcpyAsync(c->cpa, p, N * sizeof(double), cudaMemcpyHostToDevice, c->st));
     fine_eval(c, c->cpa, nullptr, 0.0, c->t1);
     launch_residual(c->st, c->F, c->t1.p, c->t1.r, nullptr, c->g, c->rhs, c->t2.R, c->Tval, c->diagT, nullptr,
-                    c->red(S_NORM2B));
+                    c->red(S_NORM2B), c->kind, c->a);
     mg_select_precision(c);
     mg_enqueue_setup(c->st, M, c->F, W, c->Tval, c->diagT, c->t1.r);
     CK(cudaMemcpyAsync(W.kb, r, N * sizeof(double), cudaMemcpyHostToDevice, c->st));

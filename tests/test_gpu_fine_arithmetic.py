@@ -1,0 +1,87 @@
+"""Rounding and range of the level-0 operators: transmissibilities, the exact Jacobian and the Newton system's solver."""
+import numpy as np
+import pytest
+
+from oracle import tpfa
+from synth.grids import cartesian_mesh
+
+pytestmark = pytest.mark.gpu
+
+
+def context(nlmg_lib, mesh, kind, a, g=None, f=None, **opts):
+    ctx = nlmg_lib.Context(mesh, kind, a, dict(dict(n_levels=1), **opts))
+    ctx.set_data(np.zeros(mesh.n_cells) if f is None else f, np.zeros(mesh.n_faces) if g is None else g)
+    return ctx
+
+
+def checkerboard(shape):
+    return (np.indices(shape).sum(0) % 2).T.reshape(-1).astype(float)
+
+
+def divided_residual(mesh, kind, a, p, g):
+    """The residual by the transmissibility ha (hb / (ha + hb)) of the two kappa-scaled halves, f = 0."""
+    with np.errstate(all="ignore"):
+        k = tpfa.kappa(p, kind, a)
+        K, L = mesh.face_cells.T
+        ha, hb = k[K] * mesh.half_trans[:, 0], k[L] * mesh.half_trans[:, 1]
+        T = np.where(mesh.face_bc == 0, ha * (hb / (ha + hb)), np.where(mesh.face_bc == 1, ha, 0.0))
+        flux = np.where(mesh.face_bc == 2, 0.0, T * (p[K] - np.where(mesh.face_bc == 0, p[L], g)))
+        r = np.zeros(mesh.n_cells)
+        np.add.at(r, K, flux)
+        np.add.at(r, L[mesh.face_bc == 0], -flux[mesh.face_bc == 0])
+    return r, flux[mesh.face_bc != 2]
+
+
+@pytest.mark.parametrize("shift", [-760.0, -720.0, -709.9, -500.0, -300.0, 300.0, 500.0, 700.0, 720.0])
+@pytest.mark.parametrize("cells", ["all", "one", "dirichlet"])
+def test_residual_keeps_its_range(nlmg_lib, shift, cells):
+    """kappa = exp(p) from zero to overflow, in all cells or in one: the residual and the fluxes are what the kappa-scaled
+    halves give, to the rounding of a subnormal kappa (2^-35 of it at -720), and infinities and NaN stand where they give
+    them."""
+    if cells == "dirichlet":
+        mesh = cartesian_mesh((1, 1), np.array([1.7]))
+        base = np.array([0.25])
+    else:
+        rng = np.random.default_rng(9)
+        mesh = cartesian_mesh((5, 4), rng.uniform(0.5, 2.0, 20))
+        base = rng.integers(-200, 200, 20) / 1024.0
+    where = np.zeros(mesh.n_cells, bool)
+    where[slice(None) if cells == "all" else 7 % mesh.n_cells] = True
+    p = base + np.where(where, shift, 0.0)
+    g = np.where(mesh.face_bc == 1, 0.5 if cells != "all" else shift + 0.5, 0.0)
+    want, flux = divided_residual(mesh, 0, 1.0, p, g)
+    ctx = context(nlmg_lib, mesh, 0, 1.0, g)
+    scale = np.abs(np.where(np.isfinite(want), want, 0.0)).max()
+    np.testing.assert_allclose(ctx.fine_residual(p), want, rtol=1e-9, atol=1e-9 * scale)
+    np.testing.assert_allclose(ctx.fine_flux(p), flux, rtol=1e-9, atol=1e-9 * scale)
+
+
+@pytest.mark.parametrize("shift", [-600, -500, -400, 400, 500, 600])
+def test_newton_update_does_not_depend_on_the_size_of_kappa(nlmg_lib, shift):
+    """kappa = exp(p): a shift of p and g scales the residual and the Jacobian by the same number, so the update is the
+    same (pressures are multiples of 1/1024, so the shift is exact; the linear solves stop at 1e-12 of the residual and
+    the scaled matrix has a condition below 1e3)."""
+    rng = np.random.default_rng(4)
+    mesh = cartesian_mesh((6, 5), rng.uniform(0.5, 2.0, 30))
+    p = rng.integers(0, 1024, 30) / 1024.0
+    g = rng.integers(0, 1024, mesh.n_faces) / 1024.0
+    dx = []
+    for s in (0, shift):
+        ctx = context(nlmg_lib, mesh, 0, 1.0, np.where(mesh.face_bc == 1, g + s, 0.0), newton_lin_tol=1e-12, lin_maxit=200)
+        dx.append(ctx.newton_update(p + s)[0])
+    assert np.linalg.norm(dx[1] - dx[0]) <= 1e-9 * np.linalg.norm(dx[0])
+
+
+@pytest.mark.parametrize("power", [150, 260, 300])
+def test_newton_update_scales_with_large_pressures(nlmg_lib, power):
+    """kappa = 1 / (1 + p^2) is p^-2 to the last bit from 2^30 on, where scaling p by a power of two scales the update by
+    it."""
+    rng = np.random.default_rng(6)
+    mesh = cartesian_mesh((6, 5), rng.uniform(0.5, 2.0, 30))
+    p = rng.uniform(1.0, 1.5, 30) * 2.0 ** 30
+    g = np.where(mesh.face_bc == 1, rng.uniform(1.0, 1.5, mesh.n_faces) * 2.0 ** 30, 0.0)
+    dx = []
+    for s in (1.0, 2.0 ** (power - 30)):
+        ctx = context(nlmg_lib, mesh, 1, 0.0, s * g, newton_lin_tol=1e-12, lin_maxit=200)
+        dx.append(ctx.newton_update(s * p)[0] / s)
+    assert np.linalg.norm(dx[1] - dx[0]) <= 1e-9 * np.linalg.norm(dx[0])
