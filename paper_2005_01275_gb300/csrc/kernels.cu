@@ -153,7 +153,7 @@ __device__ __noinline__ RowRare row_rare(const FineDev& F, int K, const double* 
   for (int j = 0; j < w; ++j, e += 32) {
     const int L = F.nbr[e];
     FaceRare f{0.0, 0.0, 0.0};
-    if (L != K) f = face_rare(qK, q[L], 1.0 / F.iu_s[e], 1.0 / F.iu_n[e], kind, a);
+    if (L != K) f = face_rare(qK, q[L], F.ups[e], F.ups[e] / F.upq[e], kind, a);
     const double td = f.T * (qK - q[L]);
     s.flux += td;
     s.dsum += f.T;
@@ -173,7 +173,7 @@ __device__ __noinline__ RowRare row_rare(const FineDev& F, int K, const double* 
 // R_K = sum_faces Ups_f (q_K - q_L) + sum_Dirichlet kappa_K Ups_K (q_K - g) - [f]_K  (eqs. TPFA_flux, FV_matrix).
 // MAT: also the frozen matrix entries Tval (= Ups_f) and its diagonal diagT; JAC: the exact Jacobian's diagonal jdiag and
 // entries Joff (null: not wanted), with diagT.
-// Bounded by FP64 issue: 7 operations an entry (2 for d, 3 for its reciprocal, the difference, the flux) and 1 for the
+// Bounded by FP64 issue: 7 operations an entry (d, 3 for its reciprocal, T, the difference, the flux) and 1 for the
 // diagonal. 10^6 cells: with a division, and a diagonal nobody asked for, an entry: 200 us; now about 110; its 125 MB would take 19.
 template <bool MAT, bool JAC>
 __global__ void __launch_bounds__(kThreads, 5) k_residual(const __grid_constant__ FineDev F,
@@ -192,24 +192,24 @@ __global__ void __launch_bounds__(kThreads, 5) k_residual(const __grid_constant_
     bool rare = false;   // some face's 1 / kappa is out of range
     const int w = F.sell_w[K >> 5];
     int e = F.sell_off[K >> 5] + (K & 31);
-#pragma unroll 2
+#pragma unroll 4
     for (int j = 0; j < w; ++j, e += 32) {
       const int L = F.nbr[e];
-      const double is = F.iu_s[e], in = F.iu_n[e], rL = r[L];
-      const double d = fma(rK, is, rL * in);
+      const double us = F.ups[e], uq = F.upq[e];
+      const double d = fma(r[L], uq, rK);
       rare |= !rcp_in_range(d);
-      double T = rcp_core(d);
-      if (L == K) T = 0.0;   // padding
+      const double y = rcp_core(d);
+      const double T = L == K ? 0.0 : us * y;   // 0: padding
       const double diff = qK - q[L];
       flux = fma(T, diff, flux);
       if (MAT || JAC) dsum += T;
       if (MAT) Tval[e] = T;
       if (JAC) {
-        // dT/dp_K = -T w_K with w_K = T r_K' / Ups_K (bounded by the kappa's rate, where T^2 leaves the range for kappas
-        // beyond 10^+-154), so dR_K/dp_K = T - T w_K (p_K - p_L), dR_K/dp_L = -T - T w_L (p_K - p_L)
+        // dT/dp_K = -T w_K with w_K = T r_K' / Ups_K = y r_K' (bounded by the kappa's rate, where T^2 leaves the range for
+        // kappas beyond 10^+-154), so dR_K/dp_K = T - T w_K (p_K - p_L), dR_K/dp_L = -T - T w_L (p_K - p_L)
         const double td = T * diff;
-        jd += fma(-td, T * is * drK, T);
-        if (Joff) Joff[e] = L == K ? 0.0 : -fma(td, T * in * dr[L], T);
+        jd += fma(-td, y * drK, T);
+        if (Joff) Joff[e] = -fma(td, y * uq * dr[L], T);
       }
     }
     const int d0 = F.dir_off[K], d1 = F.dir_off[K + 1];
@@ -283,10 +283,10 @@ __global__ void __launch_bounds__(kThreads, 6) k_fine_flux(FineDev F, const doub
   GRID_STRIDE(j, F.nflux) {
     const int K = F.fl_k[j], L = F.fl_l[j];
     const double rK = r[K], pK = p[K], pL = L >= 0 ? p[L] : g[F.fl_face[j]];
-    const double d = L >= 0 ? fma(rK, F.fl_u0[j], r[L] * F.fl_u1[j]) : rK * F.fl_u0[j];
-    double T = rcp_core(d);
+    const double u0 = F.fl_u0[j], u1 = F.fl_u1[j], d = L >= 0 ? fma(r[L], u1, rK) : rK;
+    double T = u0 * rcp_core(d);
     if (!rcp_in_range(d))
-      T = L >= 0 ? face_rare_T(pK, pL, 1.0 / F.fl_u0[j], 1.0 / F.fl_u1[j], kind, a) : kappa_of(pK, kind, a) / F.fl_u0[j];
+      T = L >= 0 ? face_rare_T(pK, pL, u0, u0 / u1, kind, a) : kappa_of(pK, kind, a) * u0;
     sigma[j] = T * (pK - pL);
   }
 }

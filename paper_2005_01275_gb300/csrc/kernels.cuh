@@ -27,14 +27,14 @@ struct FineDev {
   // interior neighbours per cell in SELL-32 layout: slice s = cells 32 s .. 32 s + 31, width sell_w[s]; entry j of
   // cell K sits at sell_off[s] + 32 j + (K & 31). Padding entries point to the cell itself (no face does).
   int *sell_off = nullptr, *sell_w = nullptr, *nbr = nullptr;
-  double *iu_s = nullptr, *iu_n = nullptr;         // 1 / own and 1 / neighbour half transmissibility per entry
+  double *ups = nullptr, *upq = nullptr;           // own half transmissibility per entry, and over the neighbour's
   int *dir_off = nullptr, *dir_face = nullptr;     // Dirichlet faces per cell (CSR)
   double* dir_ups = nullptr;
   int *neu_off = nullptr, *neu_face = nullptr;     // Neumann faces per cell (CSR)
   double* neu_area = nullptr;
   double* vol = nullptr;
   int *fl_k = nullptr, *fl_l = nullptr, *fl_face = nullptr;   // level-0 flux unknowns
-  double *fl_u0 = nullptr, *fl_u1 = nullptr;       // 1 / half transmissibilities (fl_u1: 0 on Dirichlet faces)
+  double *fl_u0 = nullptr, *fl_u1 = nullptr;       // K's half transmissibility, and over L's (0 on Dirichlet faces)
 };
 
 // The nonlinearity: kind 0 kappa = exp(a p), kind 1 kappa = (1 + p^2)^-1 (Sec. 4 examples), and its derivative.
@@ -49,9 +49,10 @@ __device__ __forceinline__ double inv_kappa_of(double p, int kind, double a) {
 __device__ __forceinline__ double kappa_rate(double p, int kind, double a) {
   return kind == 0 ? a : -2.0 * p / fma(p, p, 1.0);
 }
-// What the level-0 kernels carry per cell: r = 1 / kappa(p), whose face transmissibility 1 / (r_K / Ups_K + r_L / Ups_L)
+// What the level-0 kernels carry per cell: r = 1 / kappa(p), whose face transmissibility Ups_K / (r_K + r_L Ups_K / Ups_L)
 // needs one reciprocal and seven FP64 operations an entry (a division of kappas took sixteen), and r' = dr/dp where the
-// Jacobian is formed. Faces whose sum leaves the reciprocal's range (a kappa beyond 10^+-289) are formed from the kappas
+// Jacobian is formed. Where the two halves are equal nothing but the sum, the reciprocal and the product rounds
+// (1 / (r_K / Ups_K + r_L / Ups_L) costs as much, but rounds 1 / Ups first: on a uniform mesh an error with one sign). Faces whose sum leaves the reciprocal's range (a kappa beyond 10^+-289) are formed from the kappas
 // instead; r is not a number where kappa overflows, so that those are among them.
 __device__ __forceinline__ double level0_r(double p, int kind, double a) {
   const double r = inv_kappa_of(p, kind, a);

@@ -267,15 +267,15 @@ void upload_fine(nlmg_ctx* c) {
     soff[sl + 1] = soff[sl] + 32 * w;
   }
   std::vector<int> snbr(soff[F.nslice], 0);
-  std::vector<double> sus(soff[F.nslice], 1.0), sun(soff[F.nslice], 1.0);   // reciprocals
+  std::vector<double> sus(soff[F.nslice], 1.0), suq(soff[F.nslice], 1.0);
   for (int K = 0; K < N; ++K) {
     int sl = K >> 5, lane = K & 31, deg = off[K + 1] - off[K];
     for (int j = 0; j < sw[sl]; ++j) {
       int e = soff[sl] + 32 * j + lane;
       if (j < deg) {
         snbr[e] = nbr[off[K] + j];
-        sus[e] = 1.0 / us[off[K] + j];
-        sun[e] = 1.0 / un[off[K] + j];
+        sus[e] = us[off[K] + j];
+        suq[e] = us[off[K] + j] / un[off[K] + j];
       } else {
         snbr[e] = K;   // padding: the cell itself
       }
@@ -287,8 +287,8 @@ void upload_fine(nlmg_ctx* c) {
   F.sell_off = c->upload(soff);
   F.sell_w = c->upload(sw);
   F.nbr = c->upload(snbr);
-  F.iu_s = c->upload(sus);
-  F.iu_n = c->upload(sun);
+  F.ups = c->upload(sus);
+  F.upq = c->upload(suq);
   F.dir_off = c->upload(doff);
   F.dir_face = c->upload(dface);
   F.dir_ups = c->upload(dups);
@@ -304,8 +304,8 @@ void upload_fine(nlmg_ctx* c) {
     flk.push_back(fm.fk[f]);
     fll.push_back(fm.bc[f] == 0 ? fm.fl[f] : -1);
     flf.push_back(f);
-    u0.push_back(1.0 / fm.ups0[f]);
-    u1.push_back(fm.bc[f] == 0 ? 1.0 / fm.ups1[f] : 0.0);
+    u0.push_back(fm.ups0[f]);
+    u1.push_back(fm.bc[f] == 0 ? fm.ups0[f] / fm.ups1[f] : 0.0);
   }
   F.nflux = L0.n_flux;
   F.fl_k = c->upload(flk);
@@ -2154,7 +2154,7 @@ nlmg_status nlmg_profile_read(nlmg_ctx* c, int32_t kernel, int64_t* launches, do
     const double N = c->F.N, nnz = (double)c->sh->nnz_real;
     double b = 0.0;
     if (kernel != 2) b = c->prof.n[kernel] ? c->prof.bytes[kernel] / c->prof.n[kernel] : 0.0;
-    if (kernel == 2) b = 20.0 * nnz + 8.0 * N * 4;                          // nbr + 2 reciprocal halves, q, r, rhs, R
+    if (kernel == 2) b = 20.0 * nnz + 8.0 * N * 4;                          // nbr, the half and its ratio, q, r, rhs, R
     if (bytes_per_launch) *bytes_per_launch = b;
     if (flops_per_launch) *flops_per_launch = c->prof.n[kernel] ? c->prof.flops[kernel] / c->prof.n[kernel] : 0.0;
     return NLMG_OK;

@@ -18,6 +18,25 @@ def checkerboard(shape):
     return (np.indices(shape).sum(0) % 2).T.reshape(-1).astype(float)
 
 
+@pytest.mark.parametrize("k0", [3.0, 0.3, 0.7, 2.7, 9.9, 11.0, 19.4, 49.0, 7e5, 1e-3])
+def test_transmissibilities_of_a_uniform_field_are_exact(nlmg_lib, k0):
+    """Where both halves of a face are the same number u and kappa = 1, the transmissibility u / 2 is a number of the
+    format, and with pressures 0 and 1 in turn so is every flux. A cell adds up to four of them, whole multiples of u / 2,
+    with at most three roundings."""
+    mesh = cartesian_mesh((9, 9), np.full(81, k0))
+    u = k0 / 3.0
+    mesh.half_trans[:] = np.where(mesh.half_trans > 0, u, 0.0)
+    ctx = context(nlmg_lib, mesh, 0, 0.0)
+    p = checkerboard((9, 9))
+    K, L = mesh.face_cells[tpfa.flux_dofs(mesh)].T
+    flux = np.where(L >= 0, u / 2 * (p[K] - p[L]), u * p[K])
+    np.testing.assert_array_equal(ctx.fine_flux(p), flux)
+    want = np.zeros(81)
+    np.add.at(want, K, np.where(L >= 0, p[K] - p[L], 2 * p[K]))
+    np.add.at(want, L[L >= 0], -(p[K] - p[L])[L >= 0])
+    np.testing.assert_allclose(ctx.fine_residual(p), want * (u / 2), rtol=3 * 2.0 ** -53, atol=0)
+
+
 def divided_residual(mesh, kind, a, p, g):
     """The residual by the transmissibility ha (hb / (ha + hb)) of the two kappa-scaled halves, f = 0."""
     with np.errstate(all="ignore"):
