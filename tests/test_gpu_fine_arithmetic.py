@@ -104,3 +104,30 @@ def test_newton_update_scales_with_large_pressures(nlmg_lib, power):
         ctx = context(nlmg_lib, mesh, 1, 0.0, s * g, newton_lin_tol=1e-12, lin_maxit=200)
         dx.append(ctx.newton_update(s * p)[0] / s)
     assert np.linalg.norm(dx[1] - dx[0]) <= 1e-9 * np.linalg.norm(dx[0])
+
+
+def test_bicgstab_stops_at_its_tolerance_where_a_step_gains_much(nlmg_lib):
+    """Nearly decoupled cells: the first step leaves about 2^-16 of (s, s). The stopping test has to see (r, r) to a part
+    in 1e12 (rounding of the residual's entries, 2^-53 of s, gives about 5e-14), so a tolerance just above or below the
+    residual after one step decides whether there is a second."""
+    for seed in range(12):
+        rng = np.random.default_rng(seed)
+        mesh = cartesian_mesh((2, 40), np.ones(80))
+        inner = mesh.face_bc == 0
+        mesh.half_trans[inner] *= 1e-5 * rng.uniform(0.5, 1.5, (inner.sum(), 1))
+        p = rng.uniform(0, 1, 80)
+        g = np.zeros(mesh.n_faces)
+        J = tpfa.reduced_jacobian(mesh, 0, 0.0, p, g).toarray()
+        R = tpfa.reduced_residual(mesh, 0, 0.0, p, np.zeros(80), g)
+        S = 1.0 / np.sqrt(np.maximum(np.diag(J), 0.5 * tpfa.picard_diagonal(mesh, 0, 0.0, p)).astype(np.longdouble))
+        A, r = J * S[:, None] * S[None, :], -S * R
+        v = A @ r
+        alpha = (r @ r) / (r @ v)
+        s = r - alpha * v
+        t = A @ s
+        r1 = s - (t @ s) / (t @ t) * t
+        assert (r1 @ r1) < 2.0 ** -15 * (s @ s)
+        tol = float(np.sqrt((r1 @ r1) / (r @ r)))
+        for factor, steps in ((1 + 5e-13, {1}), (1 - 5e-13, {2, 3})):
+            ctx = context(nlmg_lib, mesh, 0, 0.0, g, newton_lin_tol=tol * factor, lin_maxit=50)
+            assert ctx.newton_update(p)[1] in steps, (seed, factor)
