@@ -777,11 +777,9 @@ cudaError_t launch_coarse_step(cudaStream_t st, const LevelDev& L, const double*
                                CoarseStepResult* res, bool* sell) {
   constexpr size_t kMaxDyn = 200 * 1024;
   const void* fns[kMaxU] = {(const void*)kp_coarse_step<1>, (const void*)kp_coarse_step<2>};
-  static const bool once = [&] {   // thread-safe one-time initialisation
-    for (const void* f : fns) cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDyn);
-    return true;
-  }();
-  (void)once;
+  static DeviceOnce limits[kMaxU];
+  for (int u = 0; u < kMaxU; ++u)
+    if (const cudaError_t e = raise_smem_limit(limits[u], fns[u], kMaxDyn)) return e;
   const int sms = coop_sms(gs.sm_cap);
   // A small level runs as one cluster of up to eight blocks, whose barrier costs a quarter of the grid's: worth it while
   // the FP64 work on eight SMs stays small beside it. In row entries and operations a lambda: 163 lambdas of a 2D level

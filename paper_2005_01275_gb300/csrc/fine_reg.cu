@@ -574,11 +574,8 @@ cudaError_t launch_cg(cudaStream_t st, const FShape& s, const FineDev& F, const 
                       const double* b, double bscale, double* dx, const FineCgBufs<T>& B, double* partial, GridSync gs,
                       double tol, int maxit, int replace, PcgResult* res) {
   const void* fn = (const void*)kp_fine_cg_reg<T, R>;
-  static const bool once = [&] {
-    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFDyn);
-    return true;
-  }();
-  (void)once;
+  static DeviceOnce limit;
+  if (const cudaError_t e = raise_smem_limit(limit, fn, kFDyn)) return e;
   const size_t eb = sizeof(T) + sizeof(int);
   gs.cluster = s.cluster ? 1 : 0;
   int staged = staged_entries(F, s, eb);
@@ -594,11 +591,8 @@ cudaError_t launch_bicg(cudaStream_t st, const FShape& s, const FineDev& F, cons
                         const double* jdiag, const double* D, const double* S, const double* b, double bscale, double* dx,
                         double* work, double* partial, GridSync gs, double tol, int maxit, PcgResult* res) {
   const void* fn = (const void*)kp_fine_bicgstab_reg<R>;
-  static const bool once = [&] {
-    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFDyn);
-    return true;
-  }();
-  (void)once;
+  static DeviceOnce limit;
+  if (const cudaError_t e = raise_smem_limit(limit, fn, kFDyn)) return e;
   gs.cluster = s.cluster ? 1 : 0;
   const size_t own = (size_t)3 * R * 32 * (s.warps + 1) * sizeof(double);
   int staged = staged_entries(F, s, sizeof(double) + sizeof(int), own);

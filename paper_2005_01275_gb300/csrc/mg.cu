@@ -15,6 +15,7 @@
 
 #include "isum.cuh"
 #include "mg.cuh"
+#include "persist.cuh"
 
 namespace nlmg {
 
@@ -2201,13 +2202,10 @@ cudaError_t mg_capture_apply(cudaStream_t st, const MgDev& M, const FineDev& F, 
   }, out);
 }
 
-void mg_set_smem_limits() {
-  static const bool once = [] {   // thread-safe one-time initialisation
-    cudaFuncSetAttribute(k_tail_cols<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmem);
-    cudaFuncSetAttribute(k_tail_cols<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmem);
-    return true;
-  }();
-  (void)once;
+cudaError_t mg_set_smem_limits() {
+  static DeviceOnce f32, bf16;
+  if (const cudaError_t e = raise_smem_limit(f32, (const void*)k_tail_cols<float>, kTailSmem)) return e;
+  return raise_smem_limit(bf16, (const void*)k_tail_cols<__nv_bfloat16>, kTailSmem);
 }
 
 }  // namespace nlmg

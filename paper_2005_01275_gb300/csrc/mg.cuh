@@ -149,7 +149,7 @@ cudaError_t mg_capture_bicgstab(cudaStream_t st, const MgDev& M, const FineDev& 
                                 const double* Joff, const double* wgt, cudaGraphExec_t* out);
 cudaError_t mg_capture_apply(cudaStream_t st, const MgDev& M, const FineDev& F, MgWork& W, cudaGraphExec_t* out);
 
-// Raises the dynamic shared-memory limit of the small levels' setup (once per process).
-void mg_set_smem_limits();
+// Raises the dynamic shared-memory limit of the small levels' setup (once per device).
+cudaError_t mg_set_smem_limits();
 
 }  // namespace nlmg

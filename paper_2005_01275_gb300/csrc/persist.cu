@@ -12,6 +12,7 @@
 // Reductions stay deterministic: each block writes one partial per value; after the barrier every block adds all
 // partials (in integers, isum.cuh) and derives the step lengths once, so all blocks take the same
 // decisions from bit-identical scalars and a run is bitwise reproducible for a given grid.
+#include <atomic>
 #include <cmath>
 
 #include "kernels.cuh"
@@ -382,14 +383,24 @@ cudaError_t launch_persistent(const void* fn, int grid, int threads, void** args
   return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
+cudaError_t raise_smem_limit(DeviceOnce& once, const void* fn, size_t bytes) {
+  int dev = -1;
+  if (const cudaError_t e = cudaGetDevice(&dev)) return e;
+  return once.run(dev, [&] { return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes); });
+}
+
 int coop_sms(int sm_cap) {
-  static const int sms = [] {
-    int dev = 0, n = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    return n;
-  }();
-  return sm_cap > 0 && sm_cap < sms ? sm_cap : sms;
+  static DeviceOnce once;
+  static std::atomic<int> count[DeviceOnce::kDevices];
+  int dev = 0, n = 0;
+  cudaGetDevice(&dev);
+  const auto ask = [&] {
+    const cudaError_t e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    if (dev < DeviceOnce::kDevices) count[dev].store(n);
+    return e;
+  };
+  if (once.run(dev, ask) == cudaSuccess && dev < DeviceOnce::kDevices) n = count[dev].load();
+  return sm_cap > 0 && sm_cap < n ? sm_cap : n;
 }
 
 template <class T>

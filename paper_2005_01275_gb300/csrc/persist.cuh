@@ -2,9 +2,13 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "device_once.hpp"
 #include "kernels.cuh"
 
 namespace nlmg {
+
+// Lets launches of a kernel use up to `bytes` of dynamic shared memory on the current device.
+cudaError_t raise_smem_limit(DeviceOnce& once, const void* fn, size_t bytes);
 
 // Results of a launch, in pinned host memory the kernel writes itself: the host sets err before the launch, and only a
 // launch whose barriers all completed clears it.

@@ -1227,7 +1227,7 @@ void alloc_mg(nlmg_ctx* c) {
   W.tail = c->dalloc<MgTailTab>(1);
   mg_fill_tail(c->st, M, W);
   CK(cudaGetLastError());
-  mg_set_smem_limits();
+  CK(mg_set_smem_limits());
 }
 
 // Transfers of the preconditioner in BF16 (lin_precision = 2) or FP32, and the level size from which the block levels
