@@ -20,9 +20,15 @@ __device__ __forceinline__ bool rcp_in_range(double x) {
   return ex - 63u < 1921u;
 }
 __device__ __forceinline__ double fast_rcp(double x) { return rcp_in_range(x) ? rcp_core(x) : 1.0 / x; }
-// a / b: the reciprocal's quotient with its residual added back (about half a division's chain of operations)
+// a / b: the reciprocal's quotient with its residual added back by a fused multiply-add (Markstein's correction; about half
+// a division's chain of operations). Both operands in 2^-480 .. 2^480, so that the quotient is far from the ends of the
+// range as well (an overflowing one would have an infinite residual), else the division.
+__device__ __forceinline__ bool div_in_range(double x) {
+  const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
+  return ex - 543u < 961u;
+}
 __device__ __forceinline__ double fast_div(double a, double b) {
-  if (!rcp_in_range(b) || !rcp_in_range(a)) return a / b;
+  if (!div_in_range(b) || !div_in_range(a)) return a / b;
   const double r = rcp_core(b), q = a * r;
   return fma(fma(-b, q, a), r, q);
 }

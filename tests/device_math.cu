@@ -90,3 +90,20 @@ extern "C" int grid_sums_host(const double* v, double* out, int blocks, int thre
   cudaFree(words);
   return r;
 }
+
+namespace {
+__global__ void k_scalar(const double* v, double* out, int n, int op) {   // v: a, then b
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const double a = v[i], b = v[n + i];
+  out[i] = op == 0 ? fast_rcp(a) : op == 1 ? fast_div(a, b) : op == 2 ? (double)narrow(a) : widen((float)a);
+}
+}  // namespace
+
+// op: 0 1 / a, 1 a / b, 2 the float next to a, 3 the double of a (a float)
+extern "C" int scalar_host(const double* v, double* out, int n, int op) {
+  return with_buffers(v, (size_t)2 * n, out, (size_t)n, [&](double* d, double* o) {
+    k_scalar<<<(n + 127) / 128, 128>>>(d, o, n, op);
+    return cudaGetLastError();
+  });
+}

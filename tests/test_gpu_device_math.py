@@ -160,3 +160,57 @@ def test_grid_sums_stay_within_their_bound(dev, blocks, cluster):
             err += (32 * 5 + 2 ** 9) * Fraction(2) ** (e - 63) + Fraction(9, 8) * abs(sum(parts)) / 2 ** 53
             err += max(0, -(-(blocks - 160) // 32)) * sum(abs(p) for p in parts) / 2 ** 53
             assert abs(Fraction(float(got[0, k])) - sum(parts)) <= err * Fraction(101, 100), name
+
+
+def scalar(dev, op, a, b=None):
+    a = np.ascontiguousarray(a, dtype=np.float64)
+    v = np.concatenate([a, a if b is None else np.asarray(b, dtype=np.float64)])
+    out = np.empty(a.size)
+    assert dev.scalar_host(ptr(v), ptr(out), a.size, op) == 0
+    return out
+
+
+def over_the_range(rng, n):
+    """Signed values of every exponent, and those next to the bounds of the short forms and of the format."""
+    x = rng.uniform(1, 2, n) * 2.0 ** rng.integers(-1022, 1024, n)
+    edges = [2.0 ** e for k in (-1022, -961, -960, -959, -481, -480, -1, 0, 1, 480, 481, 959, 960, 961, 1023)
+             for e in (k - 1, k) if e >= -1074]
+    x = np.concatenate([x, edges, np.nextafter(edges, 0), np.nextafter(edges, np.inf), [5e-324, 1e-310, np.inf, np.nan, 0.0]])
+    return np.where(rng.uniform(size=x.size) < 0.5, -x, x)
+
+
+def relative_error(got, num, den):
+    return abs(Fraction(float(got)) * Fraction(float(den)) - Fraction(float(num))) / abs(Fraction(float(num)))
+
+
+def test_reciprocal_and_quotient(dev):
+    """Within the short forms' ranges (2^-960 .. 2^960; both operands in 2^-480 .. 2^480): half a unit of the last place and
+    what the truncated series leaves, 2^-60, or the quotient's second-order terms. Outside them the plain operation."""
+    rng = np.random.default_rng(2)
+    a = over_the_range(rng, 4000)
+    with np.errstate(all="ignore"):
+        for got, num, den, top in ((scalar(dev, 0, a), np.ones_like(a), a, 961),):
+            for g, x, y in zip(got, num, den):
+                if 2.0 ** -960 <= abs(y) < 2.0 ** top:
+                    assert relative_error(g, x, y) <= Fraction(1, 2 ** 53) + Fraction(1, 2 ** 59), y
+                else:
+                    np.testing.assert_equal(g, x / y)
+        b = rng.permutation(over_the_range(rng, 4000))
+        a[:1000], b[:1000] = a[:1000] % 7 + 0.1, b[:1000] % 5 + 0.3
+        a, b = np.concatenate([a, [2.0 ** 900, 2.0 ** -900, 1.5 * 2.0 ** 700]]), np.concatenate([b, [2.0 ** -900, 2.0 ** 900, 2.0 ** -400]])
+        got = scalar(dev, 1, a, b)
+        short = (np.abs(a) >= 2.0 ** -480) & (np.abs(a) < 2.0 ** 481) & (np.abs(b) >= 2.0 ** -480) & (np.abs(b) < 2.0 ** 481)
+        np.testing.assert_array_equal(got[~short], (a / b)[~short])
+        assert short.sum() > 1000
+        for g, x, y in zip(got[short], a[short], b[short]):
+            assert relative_error(g, x, y) <= Fraction(1, 2 ** 53) + Fraction(1, 2 ** 80), (x, y)
+
+
+def test_conversions_by_bits(dev):
+    rng = np.random.default_rng(3)
+    a = np.concatenate([over_the_range(rng, 4000), rng.standard_normal(4000) * 2.0 ** rng.integers(-155, 130, 4000),
+                        np.float32(1.5) + np.arange(-4, 5) * 2.0 ** -25, [2.0 ** 128 - 2.0 ** 103, 2.0 ** 128 - 2.0 ** 104]])
+    with np.errstate(all="ignore"):
+        f = a.astype(np.float32)
+    np.testing.assert_array_equal(scalar(dev, 2, a), f.astype(np.float64))
+    np.testing.assert_array_equal(scalar(dev, 3, f.astype(np.float64)), f.astype(np.float64))
