@@ -43,7 +43,7 @@ DRAM_BYTES_64 = {}
 
 KERNELS = {0: ("kp_fine_cg_reg<double> (persistent register-resident pipelined Jacobi-scaled CG of the level-0 "
                "Picard step)", "kp_fine_cg* (level-0 Picard CG)"),
-           1: ("kp_coarse_step<double> (fused coarse Picard step: coarse operator evaluations, pipelined hybridized "
+           1: ("kp_coarse_step (fused coarse Picard step: coarse operator evaluations, pipelined hybridized "
                "CG, clamp and Algorithm 1 in one persistent launch)",) * 2,
            3: ("kp_fine_bicgstab* (persistent FP64 BiCGStab of the level-0 Newton step)",) * 2,
            5: ("level-0 CG preconditioned by the multigrid V-cycle (per-step Galerkin setup, then one CUDA graph "

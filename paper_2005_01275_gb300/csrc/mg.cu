@@ -624,14 +624,6 @@ __global__ void __launch_bounds__(kT, 6) k_cheb0_beta(FineDev F, const float* __
   }
 }
 
-// Loads of the vectors a V-cycle writes: ordinary loads, or (CG) through L2 with ld.global.cg for data another CTA
-// wrote in the same launch.
-template <bool CG>
-__device__ __forceinline__ float ldv(const float* p) {
-  if constexpr (CG) return __ldcg(p);
-  else return *p;
-}
-
 // (A x)_u of block-level cell c, one warp per cell: lane = slot * 8 + u, the four slots take every fourth block of
 // the row; a shuffle tree adds the slots, so every lane with component u < MB holds (A x)_u. The blocks are taken in
 // batches of RB per slot whose column indices, then matrix and vector entries, are all loaded before the first
@@ -653,7 +645,7 @@ struct RowBatch {
     }
   }
 };
-template <int MB, bool CG>
+template <int MB>
 __device__ __forceinline__ float row_ax(RowBatch<MB>& A, int q0, int q1, int lane, const int* __restrict__ col,
                                         const float* __restrict__ aval, const float* x) {
   constexpr int RB = RowBatch<MB>::RB;
@@ -665,7 +657,7 @@ __device__ __forceinline__ float row_ax(RowBatch<MB>& A, int q0, int q1, int lan
     for (int j = 0; j < RB; ++j) {
       const float* xd = x + (size_t)(A.cq[j] < 0 ? 0 : A.cq[j]) * MB;
 #pragma unroll
-      for (int v = 0; v < MB; ++v) xv[j][v] = A.cq[j] >= 0 ? ldv<CG>(xd + v) : 0.0f;
+      for (int v = 0; v < MB; ++v) xv[j][v] = A.cq[j] >= 0 ? xd[v] : 0.0f;
     }
 #pragma unroll
     for (int j = 0; j < RB; ++j)
@@ -682,26 +674,26 @@ __device__ __forceinline__ float row_ax(RowBatch<MB>& A, int q0, int q1, int lan
   ax += __shfl_xor_sync(0xffffffffu, ax, 16);
   return ax;
 }
-template <int MB, bool CG>
+template <int MB>
 __device__ __forceinline__ float row_ax(int c, int lane, const int* __restrict__ rowptr, const int* __restrict__ col,
                                         const float* __restrict__ aval, const float* x) {
   RowBatch<MB> A;
   const int q0 = rowptr[c], q1 = rowptr[c + 1];
   A.load(q0 + (lane >> 3), q1, lane & 7, col, aval);
-  return row_ax<MB, CG>(A, q0, q1, lane, col, aval, x);
+  return row_ax<MB>(A, q0, q1, lane, col, aval, x);
 }
 
 // One Chebyshev step on block level l (coefficients c1, c2 of step k): res = b - A x_in, d = c1 d + c2 D^-1 res,
 // x_out = x_in + d; warps w0, w0 + nw, ... take one cell each (see row_ax).
-template <int MB, bool CG>
+template <int MB>
 __device__ __forceinline__ void chebl_body(int w0, int nw, int nc, const int* __restrict__ rowptr,
                                            const int* __restrict__ col, const float* __restrict__ aval,
                                            const float* __restrict__ dinv, const float* b, const float* xin,
                                            float* xout, float* d, float c1, float c2, int k) {
   const int lane = threadIdx.x & 31, u = lane & 7;
   for (int c = w0; c < nc; c += nw) {
-    const float ax = row_ax<MB, CG>(c, lane, rowptr, col, aval, xin);
-    const float res = u < MB ? ldv<CG>(b + (size_t)c * MB + u) - ax : 0.0f;
+    const float ax = row_ax<MB>(c, lane, rowptr, col, aval, xin);
+    const float res = u < MB ? b[(size_t)c * MB + u] - ax : 0.0f;
     float s = 0.0f;
 #pragma unroll
     for (int v = 0; v < MB; ++v) {
@@ -710,29 +702,29 @@ __device__ __forceinline__ void chebl_body(int w0, int nw, int nc, const int* __
     }
     if (lane < MB) {
       const size_t i = (size_t)c * MB + u;
-      const float dn = (k == 0 ? 0.0f : c1 * ldv<CG>(d + i)) + c2 * s;
+      const float dn = (k == 0 ? 0.0f : c1 * d[i]) + c2 * s;
       d[i] = dn;
-      xout[i] = ldv<CG>(xin + i) + dn;
+      xout[i] = xin[i] + dn;
     }
   }
 }
 
 // Residual b - A x of a block level, one warp per cell.
-template <int MB, bool CG>
+template <int MB>
 __device__ __forceinline__ void resl_body(int w0, int nw, int nc, const int* __restrict__ rowptr,
                                           const int* __restrict__ col, const float* __restrict__ aval, const float* b,
                                           const float* x, float* res) {
   const int lane = threadIdx.x & 31;
   for (int c = w0; c < nc; c += nw) {
-    const float ax = row_ax<MB, CG>(c, lane, rowptr, col, aval, x);
-    if (lane < MB) res[(size_t)c * MB + lane] = ldv<CG>(b + (size_t)c * MB + lane) - ax;
+    const float ax = row_ax<MB>(c, lane, rowptr, col, aval, x);
+    if (lane < MB) res[(size_t)c * MB + lane] = b[(size_t)c * MB + lane] - ax;
   }
 }
 
 // Restriction of a residual (mbf per cell on level l) to level l+1 (mb per cell), one warp per level-(l+1) cell A:
 // lane = k * 8 + u takes component u of children k, k + 4, ...; a shuffle tree adds the lanes. `first` adds the first
 // Chebyshev step of level l+1 (x = c2 D^-1 b, d = x).
-template <class PT, bool CG>
+template <class PT>
 __device__ __forceinline__ void restr_body(int w0, int nw, int mbf, const float* res, const PT* __restrict__ Pl,
                                            const int* __restrict__ ch_off, const int* __restrict__ ch, int ncc,
                                            int mb, float* bc, const float* __restrict__ dinvc, float* xc, float* dc,
@@ -750,7 +742,7 @@ __device__ __forceinline__ void restr_body(int w0, int nw, int mbf, const float*
       for (int t = ch_off[A] + c0; t < t1; t += 2 * cstep) {
         const bool two = t + cstep < t1;
         const int ca = ch[t], cb = two ? ch[t + cstep] : ca;
-        const float ra = ldv<CG>(res + (size_t)ca * mbf + uu), rb = ldv<CG>(res + (size_t)cb * mbf + uu);
+        const float ra = res[(size_t)ca * mbf + uu], rb = res[(size_t)cb * mbf + uu];
         const size_t pa = ((size_t)ca * mbf + uu) * mb, pb = ((size_t)cb * mbf + uu) * mb;
         float Pa[kMaxM], Pb[kMaxM];
 #pragma unroll
@@ -793,26 +785,25 @@ __device__ __forceinline__ void restr_body(int w0, int nw, int mbf, const float*
 }
 
 // x += P e on a block level (one thread per cell and component; threads i0, i0 + ni, ...).
-template <class PT, bool CG>
+template <class PT>
 __device__ __forceinline__ void prol_body(long i0, long ni, int nc, int mbf, int mb, const PT* __restrict__ Pl,
                                           const int* __restrict__ agg, const float* e, float* x) {
   const long total = (long)nc * mbf;
   for (long i = i0; i < total; i += ni) {
     const int c = (int)(i / mbf);
     const float* ea = e + (size_t)agg[c] * mb;
-    float s = ldv<CG>(x + i);
-    for (int j = 0; j < mb; ++j) s = fmaf(pval(Pl, (size_t)i * mb + j), ldv<CG>(ea + j), s);
+    float s = x[i];
+    for (int j = 0; j < mb; ++j) s = fmaf(pval(Pl, (size_t)i * mb + j), ea[j], s);
     x[i] = s;
   }
 }
 
 // Coarsest level: x = C^-1 b with the dense inverse (threads i0, i0 + ni, ... take one row each).
-template <bool CG>
 __device__ __forceinline__ void coarse_solve_body(int i0, int ni, int n, const float* __restrict__ cinv,
                                                   const float* b, float* x) {
   for (int i = i0; i < n; i += ni) {
     float s = 0.0f;
-    for (int j = 0; j < n; ++j) s = fmaf(cinv[(size_t)i * n + j], ldv<CG>(b + j), s);
+    for (int j = 0; j < n; ++j) s = fmaf(cinv[(size_t)i * n + j], b[j], s);
     x[i] = s;
   }
 }
@@ -848,7 +839,7 @@ __global__ void k_chebl(int nc, const int* __restrict__ rowptr, const int* __res
     const size_t i = (size_t)c * MB + u;
     const bool own = lane < MB;
     const float bi = u < MB ? b[i] : 0.0f, di = own && k > 0 ? d[i] : 0.0f, xi = own ? xin[i] : 0.0f;
-    const float res = bi - row_ax<MB, false>(A, q0, q1, lane, col, aval, xin);
+    const float res = bi - row_ax<MB>(A, q0, q1, lane, col, aval, xin);
     float s = 0.0f;
 #pragma unroll
     for (int v = 0; v < MB; ++v) {
@@ -883,7 +874,7 @@ __global__ void k_resl(int nc, const int* __restrict__ rowptr, const int* __rest
   if (stop(done)) return;
   while (c < nc) {
     const float bi = lane < MB ? b[(size_t)c * MB + lane] : 0.0f;
-    const float ax = row_ax<MB, false>(A, q0, q1, lane, col, aval, x);
+    const float ax = row_ax<MB>(A, q0, q1, lane, col, aval, x);
     if (lane < MB) res[(size_t)c * MB + lane] = bi - ax;
     c += nwarps();
     if (c < nc) ahead();
@@ -899,7 +890,7 @@ __global__ void k_restr(int mbf, const float* __restrict__ res, const PT* __rest
   if (stop(done)) return;
   float c1 = 0.0f, c2 = 0.0f;
   if (first) cheb_tab(lam, lc, 0, c1, c2);
-  restr_body<PT, false>(gwarp(), nwarps(), mbf, res, Pl, ch_off, ch, ncc, mb, bc, dinvc, xc, dc, c2, first);
+  restr_body<PT>(gwarp(), nwarps(), mbf, res, Pl, ch_off, ch, ncc, mb, bc, dinvc, xc, dc, c2, first);
 }
 
 // The residual of a block level and its restriction in one pass: a block per cell A of the next level, a warp per child;
@@ -941,7 +932,7 @@ __global__ void __launch_bounds__(kT) k_res_restr(const int* __restrict__ rowptr
   if (stop(done)) return;
   while (t < t1) {
     const float bi = lane < MB ? b[(size_t)c * MB + lane] : 0.0f;
-    const float ax = row_ax<MB, false>(R, q0, q1, lane, col, aval, x);
+    const float ax = row_ax<MB>(R, q0, q1, lane, col, aval, x);
     const float res = lane < MB ? bi - ax : 0.0f;
 #pragma unroll
     for (int j = 0; j < kMaxM; ++j) acc[j] = fmaf(P[j], res, acc[j]);
@@ -998,7 +989,7 @@ __global__ void k_coarse_solve(int n, const float* __restrict__ cinv, const floa
                                float* __restrict__ x, const int* done) {
   pdl_start();
   if (stop(done)) return;
-  coarse_solve_body<false>(threadIdx.x, blockDim.x, n, cinv, b, x);
+  coarse_solve_body(threadIdx.x, blockDim.x, n, cinv, b, x);
 }
 
 // x_0 += P e on level 0 (per fine cell) and on a block level (per cell and component); the first item's transfer row and
@@ -1273,32 +1264,32 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail_cols(const MgTailTab* 
     float *xb[2] = {F32(T->o_x[l][0]), F32(T->o_x[l][1])}, *bl = F32(T->o_b[l]), *dl = F32(T->o_d[l]);
     for (int k = 1; k < kMgDegCoarse; ++k) {
       cheb_tab(coef, l, k, c1, c2);
-      MG_MB_SWITCH(M.mb[l], (chebl_body<MB, false>(w0, nw, M.nc[l], rp, cl, av, di, bl, xb[(k - 1) & 1], xb[k & 1],
+      MG_MB_SWITCH(M.mb[l], (chebl_body<MB>(w0, nw, M.nc[l], rp, cl, av, di, bl, xb[(k - 1) & 1], xb[k & 1],
                                                    dl, c1, c2, k)));
       __syncthreads();
     }
-    MG_MB_SWITCH(M.mb[l], (resl_body<MB, false>(w0, nw, M.nc[l], rp, cl, av, bl, xb[kDown], dl)));
+    MG_MB_SWITCH(M.mb[l], (resl_body<MB>(w0, nw, M.nc[l], rp, cl, av, bl, xb[kDown], dl)));
     __syncthreads();
     const int first = l + 1 < C ? 1 : 0;
     c2 = 0.0f;
     if (first) cheb_tab(coef, l + 1, 0, c1, c2);
-    restr_body<PT, false>(w0, nw, M.mb[l], dl, PL(l), I32(T->o_choff[l]), I32(T->o_ch[l]), M.nc[l + 1],
+    restr_body<PT>(w0, nw, M.mb[l], dl, PL(l), I32(T->o_choff[l]), I32(T->o_ch[l]), M.nc[l + 1],
                           M.mb[l + 1], F32(T->o_b[l + 1]), F32(T->o_dinv[l + 1]), F32(T->o_x[l + 1][0]),
                           F32(T->o_d[l + 1]), c2, first);
     __syncthreads();
   }
-  coarse_solve_body<false>(i0, ni, M.nc[C] * M.mb[C], F32(T->o_cinv), F32(T->o_b[C]), F32(T->o_x[C][0]));
+  coarse_solve_body(i0, ni, M.nc[C] * M.mb[C], F32(T->o_cinv), F32(T->o_b[C]), F32(T->o_x[C][0]));
   __syncthreads();
   for (int l = C - 1; l >= t; --l) {
     const int *rp = I32(T->o_rowptr[l]), *cl = I32(T->o_col[l]);
     const float *av = F32(T->o_aval[l]), *di = F32(T->o_dinv[l]);
     float *xb[2] = {F32(T->o_x[l][0]), F32(T->o_x[l][1])}, *bl = F32(T->o_b[l]), *dl = F32(T->o_d[l]);
-    prol_body<PT, false>(i0, ni, M.nc[l], M.mb[l], M.mb[l + 1], PL(l), I32(T->o_agg[l]),
+    prol_body<PT>(i0, ni, M.nc[l], M.mb[l], M.mb[l + 1], PL(l), I32(T->o_agg[l]),
                          F32(T->o_x[l + 1][l + 1 == C ? 0 : kUp]), xb[kDown]);
     __syncthreads();
     for (int k = 0; k < kMgDegCoarse; ++k) {
       cheb_tab(coef, l, k, c1, c2);
-      MG_MB_SWITCH(M.mb[l], (chebl_body<MB, false>(w0, nw, M.nc[l], rp, cl, av, di, bl, xb[(kDown + k) & 1],
+      MG_MB_SWITCH(M.mb[l], (chebl_body<MB>(w0, nw, M.nc[l], rp, cl, av, di, bl, xb[(kDown + k) & 1],
                                                    xb[(kDown + k + 1) & 1], dl, c1, c2, k)));
       __syncthreads();
     }
@@ -1367,10 +1358,10 @@ __device__ __forceinline__ void first_step0(int K, float r32, const float* __res
 }
 
 // PCG start: x = 0, r = bscale b, r32 = r, first smoothing step, rr0 = ||S r||^2 (S = diag(A)^-1/2).
-__global__ void k_pcg_init(int N, const double* __restrict__ b, double bscale, const double* __restrict__ diagT,
-                           double* __restrict__ x, double* __restrict__ r, float* __restrict__ r32,
-                           const float* __restrict__ a0dinv, float* __restrict__ x0, float* __restrict__ d0,
-                           const float* __restrict__ lam, double* part, MgScal* sc) {
+__global__ void k_pcg_init(int N, const double* __restrict__ b, double bscale, double* __restrict__ x,
+                           double* __restrict__ r, float* __restrict__ r32, const float* __restrict__ a0dinv,
+                           float* __restrict__ x0, float* __restrict__ d0, const float* __restrict__ lam, double* part,
+                           MgScal* sc) {
   pdl_start();
   float c1, c2;
   cheb_tab(lam, 0, 0, c1, c2);
@@ -1422,10 +1413,9 @@ __global__ void k_pcg_pq(FineDev F, const double* __restrict__ Tval, const doubl
 // x += alpha p, r -= alpha q, r32 = r with the first smoothing step of the next V-cycle; ||S r||^2 decides: the
 // iteration stops (conditional value 0) at ||S r||^2 <= tol^2 ||S r_0||^2, at maxit, or on a non-finite value.
 __global__ void k_pcg_update(int N, const double* __restrict__ p, const double* __restrict__ q,
-                             const double* __restrict__ diagT, double* __restrict__ x, double* __restrict__ r,
-                             float* __restrict__ r32, const float* __restrict__ a0dinv, float* __restrict__ x0,
-                             float* __restrict__ d0, const float* __restrict__ lam, double* part, MgScal* sc,
-                             cudaGraphConditionalHandle h) {
+                             double* __restrict__ x, double* __restrict__ r, float* __restrict__ r32,
+                             const float* __restrict__ a0dinv, float* __restrict__ x0, float* __restrict__ d0,
+                             const float* __restrict__ lam, double* part, MgScal* sc, cudaGraphConditionalHandle h) {
   pdl_start();
   if (stop(&sc->done)) {
     if (blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(h, 0);
@@ -1830,7 +1820,7 @@ void res_level(cudaStream_t st, const MgDev& M, const MgWork& W, int l, int cur,
 // (10^6 cells, 1,935 blocks: the CG iteration 250.8 -> 251.8 us; 64^3, 508 blocks: 98.0 -> 95.5), and aggregates are small
 // (with more than two children a warp few blocks walk a long chain).
 bool fused_restr(const MgDev& M, const MgWork& W, int l) {
-  return M.nc[l] < W.row_cells && M.nc[l + 1] <= kFusedMaxBlocks && M.nc[l] <= 16L * M.nc[l + 1];
+  return M.nc[l] < W.row_cells && M.nc[l + 1] <= W.fused_max && M.nc[l] <= 16L * M.nc[l + 1];
 }
 
 // b_(l+1) = P^T (b_l - A x_l), and (first) level l+1's first smoothing step.
@@ -2149,7 +2139,7 @@ cudaError_t mg_capture_pcg(cudaStream_t st, const MgDev& M, const FineDev& F, Mg
                            const double* diagT, cudaGraphExec_t* out) {
   const int gr = blocks_for(M.N, kMaxRedBlocks);
   cudaError_t e = capture_plain(st, [&]() {
-    launchk(st, gr, kT, 0, k_pcg_init, M.N, (const double*)W.kb, -1.0, diagT, W.kx, W.kr, W.b[0],
+    launchk(st, gr, kT, 0, k_pcg_init, M.N, (const double*)W.kb, -1.0, W.kx, W.kr, W.b[0],
             (const float*)W.a0dinv, W.x[0][0], W.d[0], (const float*)W.coef, W.part, W.sc);
   }, &out[0]);
   if (e != cudaSuccess) return e;
@@ -2158,7 +2148,7 @@ cudaError_t mg_capture_pcg(cudaStream_t st, const MgDev& M, const FineDev& F, Mg
   return capture_while(st, [&](cudaGraphConditionalHandle h) {
     const float* z = W.x[0][mg_enqueue_vcycle(st, M, F, W, nullptr, true)];   // its last step gives beta
     launchk(st, gr, kT, 0, k_pcg_pq, F, Tval, diagT, z, W.z[0], W.kp, W.kq, W.part, W.sc);
-    launchk(st, gr, kT, 0, k_pcg_update, M.N, (const double*)W.kp, (const double*)W.kq, diagT, W.kx, W.kr, W.b[0],
+    launchk(st, gr, kT, 0, k_pcg_update, M.N, (const double*)W.kp, (const double*)W.kq, W.kx, W.kr, W.b[0],
             (const float*)W.a0dinv, W.x[0][0], W.d[0], (const float*)W.coef, W.part, W.sc, h);
   }, &out[1]);
 }

@@ -25,7 +25,6 @@ constexpr int kMgDegFine = 2;       // Chebyshev steps before and after the coar
 constexpr int kMgDegCoarse = 2;     // the same on levels 1 .. L-2
 constexpr double kMgAlpha = 4.0;    // Chebyshev interval [lam / alpha, lam]
 constexpr int kMgMaxDeg = 4;        // Chebyshev steps per smoothing at most (coefficient table size)
-constexpr int kFusedMaxBlocks = 608;  // largest grid of the fused residual and restriction (see fused_restr)
 constexpr int kTailThreads = 1024;  // threads of a block of the small levels' setup (k_tail_cols)
 constexpr int kTailMaxUnknowns = 512;   // the small levels start at the first l >= 2 with at most this many unknowns ...
 constexpr size_t kTailSmem = 200 * 1024;   // ... whose data from there on fit this much shared memory
@@ -105,6 +104,7 @@ struct MgWork {
   int bf16 = 0;            // transfers in BF16 (FP32 accumulation) in the setup and V-cycle enqueued next
   int graphs_bf16 = -1;    // the transfer type the captured graphs use (-1: none captured)
   int grid0 = 4096;        // blocks of the level-0 streaming kernels: one full wave, SMs x 6 blocks of 256 threads
+  int fused_max = 608;     // largest grid of the fused residual and restriction: SMs x 4 blocks (see fused_restr)
   int row_cells = 16384;   // block levels with at least this many cells run the row-parallel kernels
   int graphs_row_cells = -1;   // the row_cells the captured graphs use (-1: none captured)
 };

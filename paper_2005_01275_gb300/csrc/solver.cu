@@ -142,7 +142,6 @@ struct nlmg_ctx {
   double r0_ref = 0.0;             // ||R(p_0)|| of the running solve (the Picard-then-Newton switch)
   bool newton_off = false;         // a Newton smoothing step of the running solve failed to halve the residual
   long long newton_steps = 0;      // level-0 Newton smoothing steps of the running solve
-  int last_fine_kind = 0;          // variant of the last level-0 CG launch (0 two-barrier, 1 pipelined, 2 registers)
   int auto_sm_cap = 0;            // SM share chosen by nlmg_solve_many while instances run side by side
   void reset_inner_tols() {
     sm_cap = opt.max_sms > 0 ? opt.max_sms : auto_sm_cap;
@@ -734,7 +733,6 @@ int fine_pcg(nlmg_ctx* c, const double* R, const double* r) {
     }
     CK(e);
   }
-  c->last_fine_kind = kind;
   c->prof_end(pi);
   count_launch(1);
   CK(cudaStreamSynchronize(c->st));
@@ -1197,6 +1195,7 @@ void alloc_mg(nlmg_ctx* c) {
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     W.grid0 = std::max(1, sms) * 6;   // the level-0 kernels are compiled for 6 blocks of 256 per SM
+    W.fused_max = std::max(1, sms) * 4;
   }
   W.a0off = c->dalloc<float>(c->F.nnz);
   W.a0diag = c->dalloc<float>(N);
