@@ -28,16 +28,18 @@ constexpr int kMaxU = 2;                          // lambdas a lane owns at most
 // so more lanes a row only pay until all sub-partitions are busy. The lane that owns a row keeps its CG state in
 // registers; the row's entries and columns lie in shared memory (sv, sc: entry j of a warp's rows at 32 (off + j) +
 // lane), so that the only loads an iteration waits for are the gathered values. A level whose entries do not fit there
-// streams them from the assembled SELL form (gsz = 1). Measured, microseconds per iteration before (rows gathered from
-// the per-cell blocks, every sum waited for) and after: 27,429 lambdas 14.0 -> 8.0 on 152 SMs, 3,597 lambdas 8.5 -> 5.0.
+// runs with its state in memory too (hyb_cg_mem), on all sixteen warps: this form with its entries streamed was slower in
+// every case measured (an iteration on 107,842 lambdas and 152 SMs 21.0 us instead of 15.7, 78,098 lambdas 18.8 instead
+// of 15.6, 27,429 lambdas on 38 SMs 20.3 instead of 15.4, rows of three flux unknowns an interface, 31,229 lambdas, 25.6
+// instead of 15.3). Measured, microseconds per iteration before (rows gathered from the per-cell blocks, every sum waited
+// for) and after: 27,429 lambdas 13.9 -> 8.1 on 152 SMs, 3,597 lambdas 8.6 -> 5.2.
 template <int U>
 struct HRows {
   int l[U];        // lambda (< 0: none)
   int n[U];        // entries a lane, the same in the whole warp
-  int off[U];      // shared memory: first entry / 32; SELL form: first entry
+  int off[U];      // first entry / 32
   const double* sv;
   const int* sc;
-  bool staged;
 };
 
 // (H v) of the warp's rows, in every lane of a row's group; entries, then the gathered v, eight at a time.
@@ -47,16 +49,15 @@ __device__ __forceinline__ void h_product(const HRows<U>& R, int gsz, const doub
 #pragma unroll
   for (int u = 0; u < U; ++u) {
     double a0 = 0.0;
-    const int e0 = R.staged ? 32 * R.off[u] + lane : R.off[u];
+    const int e0 = 32 * R.off[u] + lane;
     for (int j0 = 0; j0 < R.n[u]; j0 += 8) {
       double hv[8], xv[8];
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
         const bool in = j0 + q < R.n[u];
         const int e = e0 + 32 * (j0 + q);
-        const int c = in ? (R.staged ? R.sc[e] : __ldg(&R.sc[e])) : 0;
-        hv[q] = in ? (R.staged ? R.sv[e] : __ldcg(&R.sv[e])) : 0.0;
-        xv[q] = in ? __ldcg(&v[c]) : 0.0;
+        hv[q] = in ? R.sv[e] : 0.0;
+        xv[q] = in ? __ldcg(&v[R.sc[e]]) : 0.0;
       }
 #pragma unroll
       for (int q = 0; q < 8; ++q)
@@ -371,7 +372,7 @@ __device__ bool hyb_solve_dev(const LevelDev& L, const double* __restrict__ Hc, 
       ydiag[k] = kp * Hc[L.hc_off[c] + (k - k0) * ni + (k - k0)];
     }
   }
-  if (form == 2 && R.staged) {   // this kappa's H in shared memory
+  if (form == 2) {   // this kappa's H in shared memory
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int l = R.l[u];
@@ -678,29 +679,23 @@ __global__ void __launch_bounds__(kCThreads, 1) kp_coarse_step(LevelDev L, const
   {
     // rows of this thread: item i = ((warp + kCWarps u) gridDim + block) 32 + lane, gsz consecutive items a lambda
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    R.staged = staged > 0;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int i = (int)(((warp + kCWarps * u) * gridDim.x + blockIdx.x) * 32u) + lane;
       R.l[u] = form == 2 && warp < kCWarps && i < L.nlam * gsz ? i / gsz : -1;
       const int w = R.l[u] >= 0 ? (L.hs_w[R.l[u] >> 5] + gsz - 1) / gsz : 0;
       R.n[u] = __reduce_max_sync(0xffffffffu, w);
-      R.off[u] = R.l[u] >= 0 ? L.hs_off[R.l[u] >> 5] + (R.l[u] & 31) : 0;
       if (lane == 0 && warp < kCWarps) ew[u * kCWarps + warp] = R.n[u];
     }
-    R.sv = B.hsv;
-    R.sc = L.hs_col;
-    if (R.staged) {
-      __syncthreads();
+    __syncthreads();
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        int o = 0;
-        for (int k = 0; k < u * kCWarps + min(warp, kCWarps); ++k) o += ew[k];
-        R.off[u] = o;
-      }
-      R.sv = dyn;
-      R.sc = (const int*)(dyn + staged);
+    for (int u = 0; u < U; ++u) {
+      int o = 0;
+      for (int k = 0; k < u * kCWarps + min(warp, kCWarps); ++k) o += ew[k];
+      R.off[u] = o;
     }
+    R.sv = dyn;
+    R.sc = (const int*)(dyn + staged);
   }
   int iters = 0, steps = 0, evals = 0, trials = 0, bad = 0;
   StepScalars S{P.rn_in, P.rn_in, 0.0, false, false};
@@ -795,26 +790,21 @@ cudaError_t launch_coarse_step(cudaStream_t st, const LevelDev& L, const double*
     if (v > items) items = v;
   int grid = (int)std::max(1L, std::min((long)most, (items + 127) / 128));
   gs.cluster = cluster_grid(grid, sms) ? 1 : 0;
-  // form: registers when every lambda gets lanes in at most kMaxU passes of the grid (kept with its entries in shared
-  // memory when they fit, else streamed, one lane a row), else memory; two synchronisations when a tight solve is
-  // asked for
+  // form: registers when every lambda gets lanes in at most kMaxU passes of the grid and the rows' entries fit in shared
+  // memory, else memory; two synchronisations when a tight solve is asked for
   int form = B.pipe.ma ? 1 : 0, U = 1, staged = 0;
   if (form == 1 && L.nlam > 0 && (long)L.nlam <= (long)grid * 32 * kCWarps * kMaxU) {
-    form = 2;
-    long warps = ((long)L.nlam * gsz + 31) / 32;              // of rows
-    long per = (warps + grid - 1) / grid;                     // on one SM
+    const long warps = ((long)L.nlam * gsz + 31) / 32;              // of rows
+    const long per = (warps + grid - 1) / grid;                     // on one SM
     const long entries = per * 32 * ((L.hs_wmax + gsz - 1) / gsz);
     if ((size_t)entries * 12 <= kMaxDyn) {
+      form = 2;
       staged = (int)entries;
-    } else {
-      gsz = 1;
-      per = ((L.nlam + 31) / 32 + grid - 1) / grid;
+      U = per > kCWarps ? 2 : 1;
     }
-    U = per > kCWarps ? 2 : 1;
-  } else {
-    gsz = 1;
   }
-  if (sell) *sell = !staged;
+  if (form != 2) gsz = 1;
+  if (sell) *sell = form != 2;
   const void* fn = fns[U - 1];
   void* args[] = {(void*)&L, (void*)&Hc, (void*)&Sinv, (void*)&B, (void*)&P, (void*)&partial, (void*)&gs,
                   (void*)&form, (void*)&gsz, (void*)&staged, (void*)&res};
