@@ -14,7 +14,7 @@ namespace nlmg {
 namespace {
 
 // Warps that hold cells at most; one more, the server, adds up the sums (with 11 warps and more cells each, and with it
-// 168 registers a thread instead of 128, an iteration on 48^3 cells took 6.7 us instead of 5.3).
+// 168 registers a thread instead of 128, an iteration on 48^3 cells took 6.7 us instead of 5.7).
 constexpr int kFWarps = 15;
 constexpr int kFThreads = 32 * (kFWarps + 1);
 constexpr size_t kFDyn = 218 * 1024;             // shared memory for the rows at most
@@ -25,8 +25,13 @@ constexpr size_t kFDyn = 218 * 1024;             // shared memory for the rows a
 // other's neighbours, so a block also keeps its own cells' values of the vector it multiplies in shared memory (xl) and
 // gathers only the others' through L2: with every gather through L2 the product of 64^3 cells took 14.5k clocks, twice
 // its FP64 issue. The rows are copied once into shared memory, entry j of slice u of a warp at 32 (off + j) + lane, with
-// the column's index in xl, or the complement of its cell; rows that do not fit are read from memory (staged false).
-template <int R, class T>
+// the column's index in xl, or the complement of its cell. Rows that do not fit (ST false: unstructured meshes, small
+// shares of the SMs) are read from memory by the FP32 CG and the BiCGStab; the FP64 CG then runs the memory-resident
+// kernel, whose full blocks hide the reads better (microseconds an iteration of a Voronoi mesh, streamed and in memory:
+// FP64 85,184 cells 15.5 and 12.7, on 38 SMs 34.6 and 16.7; FP32 on 76 SMs 8.1 and 12.2; BiCGStab 27.7 and 30.4). A choice
+// per load instead of per kernel cost both: 20.8 and 53.9 (FP64), 18.4 (FP32), 42.1 (BiCGStab) for the same, and 10.9
+// instead of 10.0 on 64^3 cells in shared memory.
+template <int R, class T, bool ST>
 struct FRows {
   int K[R];        // cell (< 0: none)
   int n[R];        // entries of its slice
@@ -35,11 +40,11 @@ struct FRows {
   const T* v;
   const int* c;
   T* xl;           // the block's own values
-  bool staged;
+  static constexpr bool staged = ST;
 };
 
-template <int R, class T>
-__device__ __forceinline__ void rows_init(FRows<R, T>& X, const FineDev& F, int nw) {
+template <int R, class T, bool ST>
+__device__ __forceinline__ void rows_init(FRows<R, T, ST>& X, const FineDev& F, int nw) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int s0 = (int)((long long)F.nslice * blockIdx.x / gridDim.x);
   const int s1 = (int)((long long)F.nslice * (blockIdx.x + 1) / gridDim.x);
@@ -55,8 +60,8 @@ __device__ __forceinline__ void rows_init(FRows<R, T>& X, const FineDev& F, int 
 }
 
 // Copies the rows into shared memory, entries scaled by S_K S_L; every thread reads back only what it wrote.
-template <int R, class T>
-__device__ __forceinline__ void rows_stage(FRows<R, T>& X, const FineDev& F, const double* __restrict__ A,
+template <int R, class T, bool ST>
+__device__ __forceinline__ void rows_stage(FRows<R, T, ST>& X, const FineDev& F, const double* __restrict__ A,
                                            const double* __restrict__ S, T* dv, int* dc, int nw) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int own = 32 * (int)((long long)F.nslice * (blockIdx.x + 1) / gridDim.x) - X.K0;   // cells of the block
@@ -94,16 +99,16 @@ __device__ __forceinline__ float gather(const float* xl, const float* v, int c) 
 }
 
 // The gathered value of entry e of slice u, from xl (LOCAL) where the column is the block's own; entry e times x onto acc.
-template <int R, class T, bool LOCAL>
-__device__ __forceinline__ T row_value(const FRows<R, T>& X, const T* v, int u, int e) {
+template <bool LOCAL, int R, class T, bool ST>
+__device__ __forceinline__ T row_value(const FRows<R, T, ST>& X, const T* v, int u, int e) {
   if (X.staged) {
     const int c = X.c[e];
     return LOCAL ? gather(X.xl, v, c) : __ldcg(&v[c >= 0 ? c + X.K0 : ~c]);
   }
   return X.K[u] >= 0 ? __ldcg(&v[__ldg(&X.c[e])]) : (T)0;
 }
-template <int R, class T, bool DIAG>
-__device__ __forceinline__ T row_add(const FRows<R, T>& X, T acc, int u, int e, T x) {
+template <bool DIAG, int R, class T, bool ST>
+__device__ __forceinline__ T row_add(const FRows<R, T, ST>& X, T acc, int u, int e, T x) {
   const T a = X.staged ? X.v[e] : X.K[u] >= 0 ? __ldg(&X.v[e]) : (T)0;
   return DIAG ? fma(a, x, acc) : fma(-a, x, acc);
 }
@@ -114,8 +119,8 @@ __device__ __forceinline__ T row_add(const FRows<R, T>& X, T acc, int u, int e, 
 // FP32 has no such pipe to fill, and the registers of the second set cost more there than they save (5.8 -> 6.9 us an
 // iteration), and in the BiCGStab they spill (0.9 KB a thread, 46 instead of 28 us an iteration of 64^3 cells): those take a
 // slice's entries eight at a time.
-template <int R, class T, bool DIAG, bool LOCAL>
-__device__ __forceinline__ void rows_product(const FRows<R, T>& X, const T* v, const T (&own)[R], const T (&dg)[R],
+template <bool DIAG, bool LOCAL, int R, class T, bool ST>
+__device__ __forceinline__ void rows_product(const FRows<R, T, ST>& X, const T* v, const T (&own)[R], const T (&dg)[R],
                                              T (&out)[R]) {
   const int lane = threadIdx.x & 31;
   auto first = [&](int u) { return X.staged ? 32 * X.off[u] + lane : X.off[u]; };
@@ -125,7 +130,7 @@ __device__ __forceinline__ void rows_product(const FRows<R, T>& X, const T* v, c
     auto fetch = [&](int u, T(&y)[Q]) {
 #pragma unroll
       for (int q = 0; q < Q; ++q)
-        if (q < X.n[u]) y[q] = row_value<R, T, LOCAL>(X, v, u, first(u) + 32 * q);
+        if (q < X.n[u]) y[q] = row_value<LOCAL>(X, v, u, first(u) + 32 * q);
     };
     fetch(0, x[0]);
 #pragma unroll
@@ -135,9 +140,9 @@ __device__ __forceinline__ void rows_product(const FRows<R, T>& X, const T* v, c
       const int e0 = first(u);
 #pragma unroll
       for (int q = 0; q < Q; ++q)
-        if (q < X.n[u]) acc = row_add<R, T, DIAG>(X, acc, u, e0 + 32 * q, x[u & 1][q]);
+        if (q < X.n[u]) acc = row_add<DIAG>(X, acc, u, e0 + 32 * q, x[u & 1][q]);
       for (int j = Q; j < X.n[u]; ++j)   // wider rows
-        acc = row_add<R, T, DIAG>(X, acc, u, e0 + 32 * j, row_value<R, T, LOCAL>(X, v, u, e0 + 32 * j));
+        acc = row_add<DIAG>(X, acc, u, e0 + 32 * j, row_value<LOCAL>(X, v, u, e0 + 32 * j));
       out[u] = acc;
     }
   } else {
@@ -154,7 +159,7 @@ __device__ __forceinline__ void rows_product(const FRows<R, T>& X, const T* v, c
           x[q] = a[q] = (T)0;
           if (in) {
             a[q] = X.staged ? X.v[e] : __ldg(&X.v[e]);
-            x[q] = row_value<R, T, LOCAL>(X, v, u, e);
+            x[q] = row_value<LOCAL>(X, v, u, e);
           }
         }
 #pragma unroll
@@ -182,7 +187,7 @@ __device__ __forceinline__ double wide(float v) { return widen(v); }
 // so every `replace` iterations the residual and the auxiliary vectors are recomputed from their definitions --
 // r = b - A y and s = A p, then w = A r and z = A s (residual replacement, Cools and Vanroose) -- which costs four
 // products and two extra synchronisations.
-template <class T, int R>
+template <class T, int R, bool ST>
 __global__ void __launch_bounds__(kFThreads, 1) kp_fine_cg_reg(FineDev F, const double* __restrict__ Tval,
                                                                const T* __restrict__ Ts, const double* __restrict__ sdiag,
                                                                const double* __restrict__ b, double bscale,
@@ -195,10 +200,9 @@ __global__ void __launch_bounds__(kFThreads, 1) kp_fine_cg_reg(FineDev F, const 
   extern __shared__ double dyn[];
   const int server = (blockDim.x >> 5) - 1, warp = threadIdx.x >> 5;
   Grid g = grid_start(gs, partial, sm);
-  FRows<R, T> X;
+  FRows<R, T, ST> X;
   rows_init(X, F, server);
-  X.staged = staged > 0;
-  if (X.staged) {
+  if constexpr (ST) {
     X.xl = (T*)((int*)((T*)dyn + staged) + staged);
     rows_stage(X, F, Tval, sdiag, (T*)dyn, (int*)((T*)dyn + staged), server);
   } else {
@@ -219,7 +223,7 @@ __global__ void __launch_bounds__(kFThreads, 1) kp_fine_cg_reg(FineDev F, const 
     }
   }
   if (!grid_barrier(g)) return;
-  rows_product<R, T, false, true>(X, wn, r, r, w);
+  rows_product<false, true>(X, wn, r, r, w);
   __syncthreads();   // xl is read
   T t0 = (T)0, t1 = (T)0;
 #pragma unroll
@@ -255,7 +259,7 @@ __global__ void __launch_bounds__(kFThreads, 1) kp_fine_cg_reg(FineDev F, const 
       ig = t[0] != 0.0 ? fast_rcp(t[0]) : 0.0;
       ia = fast_rcp(alpha);
     } else {
-      rows_product<R, T, false, true>(X, wc, w, w, n);
+      rows_product<false, true>(X, wc, w, w, n);
       __syncthreads();
     }
     if (stop) break;
@@ -289,8 +293,8 @@ __global__ void __launch_bounds__(kFThreads, 1) kp_fine_cg_reg(FineDev F, const 
             B.p[X.K[u]] = p[u];
           }
         if (!grid_barrier(g)) return;
-        rows_product<R, T, false, false>(X, B.y, y, y, q);
-        rows_product<R, T, false, false>(X, B.p, p, p, sv);
+        rows_product<false, false>(X, B.y, y, y, q);
+        rows_product<false, false>(X, B.p, p, p, sv);
 #pragma unroll
         for (int u = 0; u < R; ++u) {
           const int K = X.K[u];
@@ -301,8 +305,8 @@ __global__ void __launch_bounds__(kFThreads, 1) kp_fine_cg_reg(FineDev F, const 
           }
         }
         if (!grid_barrier(g)) return;
-        rows_product<R, T, false, false>(X, B.r, r, r, w);
-        rows_product<R, T, false, false>(X, B.s, sv, sv, z);
+        rows_product<false, false>(X, B.r, r, r, w);
+        rows_product<false, false>(X, B.s, sv, sv, z);
         t0 = t1 = (T)0;
 #pragma unroll
         for (int u = 0; u < R; ++u)
@@ -349,7 +353,7 @@ __global__ void __launch_bounds__(kFThreads, 1) kp_fine_cg_reg(FineDev F, const 
 // |rh| |s| where the direct sum's are by |rh| |r|, as many; the sums themselves are more than a bit better than a tree's
 // (isum.cuh). That is one iteration in sixty on channelized fields. Bounded like the CG: 26 FP64 operations a cell, and
 // four synchronisations.
-template <int R>
+template <int R, bool ST>
 __global__ void __launch_bounds__(kFThreads, 1) kp_fine_bicgstab_reg(FineDev F, const double* __restrict__ Joff,
                                                                      const double* __restrict__ Js,
                                                                      const double* __restrict__ jdiag,
@@ -366,13 +370,12 @@ __global__ void __launch_bounds__(kFThreads, 1) kp_fine_bicgstab_reg(FineDev F, 
   extern __shared__ double dyn[];
   const int server = (blockDim.x >> 5) - 1, warp = threadIdx.x >> 5;
   Grid g = grid_start(gs, partial, sm);
-  FRows<R, double> X;
+  FRows<R, double, ST> X;
   rows_init(X, F, server);
-  X.staged = staged > 0;
   // per thread and slice: y, rh and the diagonal, then the rows
   const int T = blockDim.x;
   double *ys = dyn + threadIdx.x, *rhs = ys + R * T, *jds = rhs + R * T, *rows = dyn + 3 * R * T;
-  if (X.staged) {
+  if constexpr (ST) {
     X.xl = (double*)((int*)(rows + staged) + staged);
     rows_stage(X, F, Joff, S, rows, (int*)(rows + staged), server);
   } else {
@@ -421,7 +424,7 @@ __global__ void __launch_bounds__(kFThreads, 1) kp_fine_bicgstab_reg(FineDev F, 
     {
       double jd[R];
       diag(jd);
-      rows_product<R, double, true, true>(X, pg, p, jd, v);
+      rows_product<true, true>(X, pg, p, jd, v);
     }
     if (X.K[0] >= 0) {
 #pragma unroll
@@ -455,7 +458,7 @@ __global__ void __launch_bounds__(kFThreads, 1) kp_fine_bicgstab_reg(FineDev F, 
     {
       double jd[R];
       diag(jd);
-      rows_product<R, double, true, true>(X, sg, r, jd, t);
+      rows_product<true, true>(X, sg, r, jd, t);
     }
     if (X.K[0] >= 0) {
 #pragma unroll
@@ -569,34 +572,34 @@ int staged_entries(const FineDev& F, const FShape& s, size_t entry_bytes, size_t
   return n * entry_bytes + cells * (entry_bytes - sizeof(int)) + other <= kFDyn ? (int)n : 0;
 }
 
-template <class T, int R>
+template <class T, int R, bool ST>
 cudaError_t launch_cg(cudaStream_t st, const FShape& s, const FineDev& F, const double* Tval, T* Ts, const double* sdiag,
                       const double* b, double bscale, double* dx, const FineCgBufs<T>& B, double* partial, GridSync gs,
                       double tol, int maxit, int replace, PcgResult* res) {
-  const void* fn = (const void*)kp_fine_cg_reg<T, R>;
+  const void* fn = (const void*)kp_fine_cg_reg<T, R, ST>;
   static DeviceOnce limit;
   if (const cudaError_t e = raise_smem_limit(limit, fn, kFDyn)) return e;
   const size_t eb = sizeof(T) + sizeof(int);
   gs.cluster = s.cluster ? 1 : 0;
   int staged = staged_entries(F, s, eb);
-  if (!staged) launch_scale_sell<T>(st, F, Tval, sdiag, Ts);
+  if (!ST) launch_scale_sell<T>(st, F, Tval, sdiag, Ts);
   void* args[] = {(void*)&F, (void*)&Tval, (void*)&Ts, (void*)&sdiag, (void*)&b, (void*)&bscale, (void*)&dx, (void*)&B,
                   (void*)&partial, (void*)&gs, (void*)&tol, (void*)&maxit, (void*)&replace, (void*)&staged, (void*)&res};
   return launch_persistent(fn, s.grid, 32 * (s.warps + 1), args,
                            staged ? (size_t)staged * eb + (size_t)s.warps * s.R * 32 * sizeof(T) : 0, s.cluster, st);
 }
 
-template <int R>
+template <int R, bool ST>
 cudaError_t launch_bicg(cudaStream_t st, const FShape& s, const FineDev& F, const double* Joff, double* Js,
                         const double* jdiag, const double* D, const double* S, const double* b, double bscale, double* dx,
                         double* work, double* partial, GridSync gs, double tol, int maxit, PcgResult* res) {
-  const void* fn = (const void*)kp_fine_bicgstab_reg<R>;
+  const void* fn = (const void*)kp_fine_bicgstab_reg<R, ST>;
   static DeviceOnce limit;
   if (const cudaError_t e = raise_smem_limit(limit, fn, kFDyn)) return e;
   gs.cluster = s.cluster ? 1 : 0;
   const size_t own = (size_t)3 * R * 32 * (s.warps + 1) * sizeof(double);
   int staged = staged_entries(F, s, sizeof(double) + sizeof(int), own);
-  if (!staged) launch_scale_sell<double>(st, F, Joff, S, Js);
+  if (!ST) launch_scale_sell<double>(st, F, Joff, S, Js);
   double *pg = work, *sg = work + F.N;
   void* args[] = {(void*)&F, (void*)&Joff, (void*)&Js, (void*)&jdiag, (void*)&D, (void*)&S, (void*)&b, (void*)&bscale,
                   (void*)&dx, (void*)&pg, (void*)&sg, (void*)&partial, (void*)&gs, (void*)&tol, (void*)&maxit,
@@ -612,8 +615,13 @@ cudaError_t launch_fine_cg_reg(cudaStream_t st, const FineDev& F, const double* 
                                const double* b, double bscale, double* dx, const FineCgBufs<T>& B, double* partial,
                                GridSync gs, double tol, int maxit, int replace, PcgResult* res) {
   const FShape s = fine_shape(F, gs.sm_cap);
-#define NLMG_CG(RR) \
-  if (s.R <= RR) return launch_cg<T, RR>(st, s, F, Tval, Ts, sdiag, b, bscale, dx, B, partial, gs, tol, maxit, replace, res)
+  const bool fits = staged_entries(F, s, sizeof(T) + sizeof(int)) > 0;
+  constexpr bool kStream = std::is_same_v<T, float>;
+  if (!fits && !kStream) return cudaErrorNotSupported;
+#define NLMG_CG(RR)                                                                                                      \
+  if (s.R <= RR)                                                                                                         \
+  return (fits ? launch_cg<T, RR, true> : launch_cg<T, RR, !kStream>)(st, s, F, Tval, Ts, sdiag, b, bscale, dx, B,       \
+                                                                      partial, gs, tol, maxit, replace, res)
   NLMG_CG(1);
   NLMG_CG(2);
   NLMG_CG(3);
@@ -639,8 +647,11 @@ cudaError_t launch_fine_bicgstab_reg(cudaStream_t st, const FineDev& F, const do
                                      double bscale, double* dx, double* work, double* partial, GridSync gs, double tol,
                                      int maxit, PcgResult* res) {
   const FShape s = fine_shape(F, gs.sm_cap);
-#define NLMG_BICG(RR) \
-  if (s.R <= RR) return launch_bicg<RR>(st, s, F, Joff, Js, jdiag, D, S, b, bscale, dx, work, partial, gs, tol, maxit, res)
+  const bool fits = staged_entries(F, s, 12, (size_t)3 * s.R * 32 * (s.warps + 1) * sizeof(double)) > 0;
+#define NLMG_BICG(RR)                                                                                                    \
+  if (s.R <= RR)                                                                                                         \
+  return (fits ? launch_bicg<RR, true> : launch_bicg<RR, false>)(st, s, F, Joff, Js, jdiag, D, S, b, bscale, dx, work,   \
+                                                                 partial, gs, tol, maxit, res)
   NLMG_BICG(1);
   NLMG_BICG(2);
   NLMG_BICG(3);

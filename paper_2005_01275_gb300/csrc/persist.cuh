@@ -55,7 +55,8 @@ struct FineCgBufs {
 
 // Register-resident pipelined CG on the frozen matrix Tval scaled by sdiag (Ts: room for the scaled entries, used when
 // the rows do not fit in shared memory); T = float with residual replacement every `replace` iterations (0: never).
-// Returns cudaErrorNotSupported without launching when a thread would have to hold more than 5 (FP32: 9) cells.
+// Returns cudaErrorNotSupported without launching when a thread would have to hold more than 5 (FP32: 9) cells or, in FP64,
+// the rows do not fit in shared memory.
 template <class T>
 cudaError_t launch_fine_cg_reg(cudaStream_t st, const FineDev& F, const double* Tval, T* Ts, const double* sdiag,
                                const double* b, double bscale, double* dx, const FineCgBufs<T>& B, double* partial,

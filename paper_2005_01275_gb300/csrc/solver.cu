@@ -692,7 +692,7 @@ int fine_pcg(nlmg_ctx* c, const double* R, const double* r) {
   launch_sdiag(c->st, c->F.N, c->diagT, c->sdiag);
   const bool fp32 = c->opt.lin_precision == 1;
   // FP64 at loose tolerances: pipelined CG (one grid barrier per iteration), register-resident when every thread
-  // holds at most 5 cells. FP32: the pipelined CG with residual replacement every kReplace iterations (without it
+  // holds at most 5 cells and the matrix rows fit in shared memory. FP32: the pipelined CG with residual replacement every kReplace iterations (without it
   // the FP32 recurrences drift: measured 10,768 instead of 3,466 fine iterations on the 64^3 workload), registers
   // for at most 9 cells per thread; else the two-barrier CG in memory. Tight FP64 tolerances: the two-barrier CG, whose
   // updated residual tracks the true one more closely.
