@@ -37,9 +37,11 @@ CPU_SAMPLE_SCALE = 24      # side of the cpu_baseline sample
 
 
 # DRAM bytes (read + write) per launch on the 64^3 workload with the default options, from ncu captures of the
-# kernels as they are now: valid for that kernel, that workload and those options only, else the traffic is reported
-# as null (the register-resident kernels have no capture).
-DRAM_BYTES_64 = {}
+# kernels as they are now (averaged over the launches of one solve): valid for that kernel, that workload and those
+# options only, else the traffic is reported as null.
+DRAM_BYTES_64 = {0: 23.111e6,     # kp_fine_cg_reg<double, 4, true>, mean of the 8 launches of a solve
+                 1: 32.620e6,     # kp_coarse_step, mean of the 15 launches (10 on level 1, 5 coarsest solves)
+                 3: 27.341e6}     # kp_fine_bicgstab_reg<4, true>, mean of the 3 launches
 
 KERNELS = {0: ("kp_fine_cg_reg<double> (persistent register-resident pipelined Jacobi-scaled CG of the level-0 "
                "Picard step)", "kp_fine_cg* (level-0 Picard CG)"),

@@ -174,7 +174,8 @@ __device__ __noinline__ RowRare row_rare(const FineDev& F, int K, const double* 
 // MAT: also the frozen matrix entries Tval (= Ups_f) and its diagonal diagT; JAC: the exact Jacobian's diagonal jdiag and
 // entries Joff (null: not wanted), with diagT.
 // Bounded by FP64 issue: 7 operations an entry (d, 3 for its reciprocal, T, the difference, the flux) and 1 for the
-// diagonal. 10^6 cells: with a division, and a diagonal nobody asked for, an entry: 200 us; now about 110; its 125 MB would take 19.
+// diagonal. 10^6 cells: with a division, and a diagonal nobody asked for, an entry: 200 us; now about 105; its 125 MB would
+// take 19.
 template <bool MAT, bool JAC>
 __global__ void __launch_bounds__(kThreads, 5) k_residual(const __grid_constant__ FineDev F,
                                                        const double* __restrict__ q,

@@ -52,8 +52,9 @@ __device__ __forceinline__ double kappa_rate(double p, int kind, double a) {
 // What the level-0 kernels carry per cell: r = 1 / kappa(p), whose face transmissibility Ups_K / (r_K + r_L Ups_K / Ups_L)
 // needs one reciprocal and seven FP64 operations an entry (a division of kappas took sixteen), and r' = dr/dp where the
 // Jacobian is formed. Where the two halves are equal nothing but the sum, the reciprocal and the product rounds
-// (1 / (r_K / Ups_K + r_L / Ups_L) costs as much, but rounds 1 / Ups first: on a uniform mesh an error with one sign). Faces whose sum leaves the reciprocal's range (a kappa beyond 10^+-289) are formed from the kappas
-// instead; r is not a number where kappa overflows, so that those are among them.
+// (1 / (r_K / Ups_K + r_L / Ups_L) costs as much, but rounds 1 / Ups first: on a uniform mesh an error with one sign).
+// Faces whose sum leaves the reciprocal's range (a kappa beyond 10^+-289) are formed from the kappas instead; r is not a
+// number where kappa overflows, so that those are among them.
 __device__ __forceinline__ double level0_r(double p, int kind, double a) {
   const double r = inv_kappa_of(p, kind, a);
   return r < 0x1p-1024 ? __longlong_as_double(0x7ff8000000000000ll) : r;   // 1 / DBL_MAX rounds to 2^-1024

@@ -90,8 +90,9 @@ __device__ __forceinline__ bool grid_barrier(Grid& g, unsigned long long spin_li
 
 // Grid sums of NV values, in two halves, for a block whose warp `server` does the serial part (it may hold values too).
 // grid_sum_arrive: warp sums, the block's sums to the partial buffer, then the grid barrier; on return every block's
-// earlier writes and partials are visible. The other warps run `meanwhile` (on registers) while the server waits. grid_sum_finish, by the server warp alone: every block's partials added
-// (all blocks get bit-identical sums, so they take the same decisions); every lane of that warp returns the sums.
+// earlier writes and partials are visible. The other warps run `meanwhile` (on registers) while the server waits.
+// grid_sum_finish, by the server warp alone: every block's partials added (all blocks get bit-identical sums, so they take
+// the same decisions); every lane of that warp returns the sums.
 // Consecutive reductions use the two partial buffers in turn: a block can only overwrite a buffer after every block
 // has passed the next barrier, i.e. has finished reading it.
 template <int NV>
